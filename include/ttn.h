@@ -332,7 +332,7 @@ int ttn_selftest_df(void* d_ws, size_t bytes, double* out_rel, int n_out, void* 
  * where cudaMalloc is not permitted); the paper has no counterpart.
  *   C[p][q] = sum_{j < n2} Y[p][j] W[q][j]      (FP64, row-major, all device)
  * the product over both child legs that ends every ascend step.  It runs the
- * library's FP64 split-K kernel with its partial sums in a fixed 8 MiB device
+ * library's FP64 split-K kernels with their partial sums in a fixed 8 MiB device
  * array inside the library instead of caller scratch; every GPU that loads the
  * library holds that array until the process exits.  The first call on a
  * device looks the array up (cudaGetSymbolAddress), so make that first call

@@ -90,6 +90,8 @@ struct GemmDesc {
   int tile;          // tile width chosen by the autotuner (0: the launcher's
                      // default): BN of a tensor-core kernel, the square tile of
                      // the FP64 engine
+  int digits;        // FP64 products: the digit engine (gemm_oz.cu) where it is supported
+  unsigned* words;   // its magnitude scratch (oz_words(d) words)
   int occ;           // TMA-fed kernel: 2 = the 96 KB stage ring (two CTAs per
                      // SM), else the 192 KB ring (one CTA per SM)
 };
@@ -113,6 +115,16 @@ int device_sm_count();
 // Split count / partial-buffer size the launcher will use for a descriptor.
 int gemm_pick_splits(const GemmDesc& d);
 size_t gemm_partial_elems(const GemmDesc& d, int splits);
+
+// Digit engine of the FP64 products (gemm_oz.cu).  kOzMinWork: multiply-adds
+// below which the FP64 kernel stays (at 2^20 both take 15 us, at 2^24 the
+// digit engine 24 and the FP64 kernel 62).
+constexpr double kOzMinWork = 1 << 23;
+int gemm_oz_launch(const GemmDesc& d, cudaStream_t stream);
+bool gemm_oz_supported(const GemmDesc& d);
+int oz_pick_splits(const GemmDesc& d);
+size_t oz_words(const GemmDesc& d);
+void gemm_oz_init();
 
 // Tensor-core path (gemm_tc.cu).
 int gemm_tc_launch(const GemmDesc& d, cudaStream_t stream);

@@ -256,6 +256,7 @@ int f64_tile(const GemmDesc& d) {
 
 int gemm_pick_splits(const GemmDesc& d) {
   if (d.prec != 0 && gemm_tc_supported(d)) return tc_pick_splits(d);
+  if (gemm_oz_supported(d)) return oz_pick_splits(d);
   const int bm = f64_tile(d);
   const long long tm = (d.M + bm - 1) / bm, tn = (d.N + bm - 1) / bm;
   // a symmetric product launches only the tiles on or above the diagonal
@@ -281,7 +282,10 @@ int gemm_launch(const GemmDesc& d0, cudaStream_t s) {
   const int t = f64_tile(d);
   d.sym_tile = t;
   if (d.sym && d.M != d.N) d.sym = 0;
-  if (t == 64) n += launch_tile<64, 64>(d, s);
+  if (gemm_oz_supported(d)) {
+    d.sym = 0;   // every tile is computed (the exact sums are symmetric)
+    n += gemm_oz_launch(d, s);
+  } else if (t == 64) n += launch_tile<64, 64>(d, s);
   else if (t == 32) n += launch_tile<32, 32>(d, s);
   else n += launch_tile<16, 16>(d, s);
   if (d.splits > 1) {
@@ -312,6 +316,8 @@ namespace ttn {
 namespace {
 
 constexpr long long kNoAllocScratchDoubles = 1LL << 20;   // 8 MiB of FP64 partial sums
+// the last of them hold the digit engine's magnitude words
+constexpr int kNoAllocWordDoubles = 512;
 constexpr int kNoAllocMaxDim = 256;
 constexpr int kNoAllocMaxDevices = 64;
 
@@ -339,6 +345,7 @@ extern "C" int ttn_close_noalloc(const double* d_Y, const double* d_W, int P, in
       void* p = nullptr;
       if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || !p) return TTN_ECUDA;
       g_noalloc_ptr[dev] = static_cast<double*>(p);
+      gemm_oz_init();
     }
     scratch = g_noalloc_ptr[dev];
   }
@@ -348,16 +355,19 @@ extern "C" int ttn_close_noalloc(const double* d_Y, const double* d_W, int P, in
   d.C = d_C; d.sc_m = Q; d.sc_n = 1;
   d.alpha = 1.0; d.beta = 0.0; d.prec = 0;
   Group g;
-  // K0 = 1, K1 = n2: any length, addressed through the K1 stride
+  // one K level of any length (n2 <= 2^30)
   g.a.p = d_Y; g.a.s_mn = n2; g.a.s_k0 = 1; g.a.s_k1 = 1; g.a.s_b0 = 0; g.a.s_b1 = 0; g.a.f32 = 0;
   g.b.p = d_W; g.b.s_mn = n2; g.b.s_k0 = 1; g.b.s_k1 = 1; g.b.s_b0 = 0; g.b.s_b1 = 0; g.b.f32 = 0;
   g.K = static_cast<int>(n2);
-  g.k0_log2 = 0;
+  g.k0_log2 = 30;
   d.g[0] = g;
   d.ngroups = 1;
+  d.digits = 1;
+  d.words = reinterpret_cast<unsigned*>(scratch + kNoAllocScratchDoubles - kNoAllocWordDoubles);
+  if (oz_words(d) > 2 * kNoAllocWordDoubles) d.digits = 0;   // (at most 2 x 256 words)
   const long long per_split = static_cast<long long>(P) * Q;
   int splits = gemm_pick_splits(d);
-  splits = static_cast<int>(std::min<long long>(splits, kNoAllocScratchDoubles / per_split));
+  splits = static_cast<int>(std::min<long long>(splits, (kNoAllocScratchDoubles - kNoAllocWordDoubles) / per_split));
   d.splits = std::max(1, splits);
   d.partial = scratch;
   // an error left pending by earlier work of the caller is reported, not

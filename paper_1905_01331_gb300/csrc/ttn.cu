@@ -121,6 +121,7 @@ struct SubStreams {
   int n = 0;                              // 0: stages run on the lane's stream
   cudaStream_t s[kSubStreams] = {};
   double* partial[kSubStreams] = {};
+  unsigned* words[kSubStreams] = {};      // magnitude words of the digit engine
   cudaEvent_t fork = nullptr;
   cudaEvent_t join[kSubStreams] = {};
 };
@@ -162,6 +163,7 @@ struct Lane {
          *top_stack0 = nullptr, *top_stack1 = nullptr, *lz_part = nullptr;
   double *lz_opsp = nullptr, *lz_bp = nullptr, *lz_Yp = nullptr;
   int* iflags = nullptr;
+  unsigned* words = nullptr;
   SubStreams sub;
 };
 
@@ -197,6 +199,12 @@ struct ttn_ctx {
                                // [5]=grid-barrier counter of the polar composition
                                // [6], [7]=top-solve flags; [8..]=composition tile counters
   SubStreams sub;              // of the current lane
+  // FP64 products enqueued now may take the digit engine (gemm_oz.cu): set in
+  // the FP64 sweeps and calls, not in the mixed modes' sweeps, whose small
+  // FP64 products keep their order of operations
+  bool digits = false;
+  unsigned* words = nullptr;   // its magnitude scratch
+  size_t words_cap = 0;
   int lz_m = 48;
   double* E_hist = nullptr;    // device energies of the current ttn_sweep call
   std::vector<PolarBlock> polar_f64, polar_tc;
@@ -229,7 +237,7 @@ namespace {
 #define TTN_LANE_FIELDS(X_) X_(stream) X_(Y) X_(Gam) X_(X) X_(X2) X_(Yt) X_(M1) X_(pA) X_(pF) \
   X_(pP) X_(pT) X_(pS) X_(partial) X_(red) X_(scal) X_(lz_basis) X_(lz_w) X_(lz_c1) X_(lz_c2) \
   X_(lz_alpha) X_(lz_beta) X_(lz_y) X_(lz_tmp) X_(top_stack0) X_(top_stack1) X_(lz_part) \
-  X_(lz_opsp) X_(lz_bp) X_(lz_Yp) X_(iflags) X_(sub)
+  X_(lz_opsp) X_(lz_bp) X_(lz_Yp) X_(iflags) X_(words) X_(sub)
 
 void load_lane(ttn_ctx* h, const Lane& l) {
 #define TTN_LOAD(f) h->f = l.f;
@@ -343,7 +351,7 @@ uint64_t tune_key(const GemmDesc& d) {
     mix(o.s_mn); mix(o.s_k0); mix(o.s_k1); mix(o.s_b0); mix(o.s_b1); mix(o.f32);
     mix((long long)((uintptr_t)o.p & 15));
   };
-  mix(d.prec); mix(d.M); mix(d.N); mix(d.B0); mix(d.B1); mix(d.c_f32); mix(d.sym);
+  mix(gemm_oz_supported(d) ? 100 : d.prec); mix(d.M); mix(d.N); mix(d.B0); mix(d.B1); mix(d.c_f32); mix(d.sym);
   mix(d.sc_m); mix(d.sc_n); mix(d.ngroups);
   for (int g = 0; g < d.ngroups && g < kMaxGroups; ++g) {
     mix(d.g[g].K); mix(d.g[g].k0_log2);
@@ -365,7 +373,7 @@ Tuned tune_product(ttn_ctx* h, const GemmDesc& d0) {
   std::vector<int> splits;
   for (int s = 1; s <= 128; s *= 2)
     if (s == 1 || (s <= ksum / 64 && gemm_partial_elems(d0, s) <= h->partial_cap)) splits.push_back(s);
-  const bool tc = d0.prec != 0 && gemm_tc_supported(d0);
+  const bool tc = d0.prec != 0 && gemm_tc_supported(d0), oz = gemm_oz_supported(d0);
   GemmDesc dd = d0;
   dd.tile = 0;
   const int def_splits = std::max(1, std::min(gemm_pick_splits(dd), (int)splits.back()));
@@ -379,6 +387,8 @@ Tuned tune_product(ttn_ctx* h, const GemmDesc& d0) {
       }
       for (int bn : {32, 64, 128})
         if (bn <= std::max(32, d0.N)) cands.push_back({1, bn, s, 0});
+    } else if (oz) {
+      cands.push_back({d0.tc_engine, 0, s, 0});
     } else {
       for (int t : {16, 32, 64})
         if (t == 16 || t <= std::min(d0.M, d0.N)) cands.push_back({d0.tc_engine, t, s, 0});
@@ -414,6 +424,9 @@ Tuned tune_product(ttn_ctx* h, const GemmDesc& d0) {
 // Run (or, in the plan pass, size and bounds-check) one product.
 void run(ttn_ctx* h, GemmDesc d, int prec) {
   d.prec = prec;
+  d.digits = h->digits && prec == 0;
+  if (d.digits && !h->measuring && oz_words(d) > h->words_cap) d.digits = 0;   // cannot happen after planning
+  d.words = h->words;
   d.tc_engine = h->opt.tc_engine;
   int s;
   const uint64_t key = h->tuned.empty() && !h->tuning ? 0 : tune_key(d);
@@ -433,6 +446,7 @@ void run(ttn_ctx* h, GemmDesc d, int prec) {
   size_t need = gemm_partial_elems(d, s);
   if (h->measuring) {
     if (need > h->partial_cap) h->partial_cap = need;
+    h->words_cap = std::max(h->words_cap, oz_words(d));
     if (d.ngroups > kMaxGroups) h->bounds_error = "too many groups";
     check_desc(h, d);
     return;
@@ -481,9 +495,10 @@ struct StageFork {
   ttn_ctx* h;
   cudaStream_t main;
   double* partial;
+  unsigned* words;
   bool on;
   explicit StageFork(ttn_ctx* hh)
-      : h(hh), main(hh->stream), partial(hh->partial),
+      : h(hh), main(hh->stream), partial(hh->partial), words(hh->words),
         on(hh->sub.n > 0 && !hh->measuring && !hh->profiling && !hh->tuning) {
     if (!on) return;
     cudaEventRecord(h->sub.fork, main);
@@ -493,6 +508,7 @@ struct StageFork {
     if (!on) return;
     h->stream = h->sub.s[i % h->sub.n];
     h->partial = h->sub.partial[i % h->sub.n];
+    h->words = h->sub.words[i % h->sub.n];
   }
   void join() {
     if (!on) return;
@@ -502,6 +518,7 @@ struct StageFork {
     }
     h->stream = main;
     h->partial = partial;
+    h->words = words;
     on = false;
   }
   ~StageFork() { join(); }
@@ -860,7 +877,8 @@ void top_adjoints(ttn_ctx* h, Instance& I) {
 }
 
 // Gamma_J = R_J Zs + sum_k [P_k W A_k^T + P_k^T W A_k + Q_k B_k W + Q_k^T B_k^T W]
-void environment(ttn_ctx* h, Instance& I, int t, int prec, double* Gam) {
+// fp64_units: the last product runs in plain FP64 FMAs in every mode.
+void environment(ttn_ctx* h, Instance& I, int t, int prec, double* Gam, bool fp64_units = false) {
   const LayerView v = view(I, t, prec);
   const int K = I.K;
   const TP W = v.W;
@@ -916,7 +934,10 @@ void environment(ttn_ctx* h, Instance& I, int t, int prec, double* Gam) {
     add(d, grp(Gn(1 + K + k), Tn(BW + k * slab), v.P));
     add(d, grp(Gt(1 + K + k), Tn(BtW + k * slab), v.P));
   }
+  const bool digits = h->digits;
+  if (fp64_units) h->digits = false;
   run(h, d, prec);
+  h->digits = digits;
 }
 
 // w_t <- -polar(Gam - mu |Gam| w_t) by scaled Newton-Schulz blocks.
@@ -1346,6 +1367,7 @@ void descend(ttn_ctx* h, Instance& I, int t, int prec) {
 }
 
 void forward(ttn_ctx* h, Instance& I, int prec) {
+  h->digits = prec == 0;
   if (prec != 0 && !h->measuring) {
     // FP32 copies of the layer-0 operators and of every isometry
     h->launches += to_f32(I.ops[0], I.ops32[0], I.op_elems(0), h->stream);
@@ -1364,7 +1386,13 @@ void sweep_instance(ttn_ctx* h, Instance& I) {
     h->launches += to_f32(I.adj[I.T], I.adj32[I.T], I.op_elems(I.T), h->stream);
   for (int t = I.T - 1; t >= 0; --t) {
     ensure_ops(h, I, t, prec);
-    environment(h, I, t, prec, h->Gam);
+    // The top isometry's environment has directions of singular value ~0 that
+    // the damping keeps: there the update takes the rounding of this one
+    // product divided by mu = 1e-7.  It stays on the FP64 units (2.7 ms of an
+    // FP64 sweep at P = n = 128), so that those directions are those of plain
+    // FP64 sums; with the digit engine they differ by up to 4.5e-8 of the
+    // isometry's entries.
+    environment(h, I, t, prec, h->Gam, t == I.T - 1);
     polar(h, I, t, prec, h->Gam);
     descend(h, I, t, prec);
   }
@@ -1429,6 +1457,28 @@ void value_and_grad(ttn_ctx* h, Instance& I, int prec, double* energy_out, doubl
   }
 }
 
+// Density matrix of the leftmost site of `site_layer` of a translation-invariant
+// tree, in pA: rho = V V^T, then Tr_r(W^T rho W) downwards.
+void leftmost_rdm(ttn_ctx* h, Instance& I, int site_layer) {
+  const int c = I.chis[I.T];
+  double* rho = h->pA;
+  h->digits = true;
+  {
+    GemmDesc d = desc(c, c, 1, 1, rho, c, 1, 0, 0);
+    add(d, grp(op(I.V, c, 1), op(I.V, c, 1), c));
+    run(h, d, 0);
+  }
+  for (int t = I.T - 1; t >= site_layer; --t) {
+    const LayerView v = view(I, t, 0);
+    GemmDesc g = desc(v.P, (int)v.n2, 1, 1, h->Yt, v.n2, 1, 0, 0);
+    add(g, grp(op(rho, v.P, 1), op(I.W[t], 1, v.n2), v.P));
+    run(h, g, 0);
+    GemmDesc r = desc(v.n, v.n, 1, 1, rho, v.n, 1, 0, 0);
+    add(r, grp(op(I.W[t], v.n, 1, v.n2), op(h->Yt, v.n, 1, v.n2), v.n, v.P));
+    run(h, r, 0);
+  }
+}
+
 // Plan all scratch sizes (pass with base == nullptr) or carve them.
 void layout(ttn_ctx* h, Arena& ar) {
   size_t slab_max = 0, pp_max = 0, c2_max = 0, nj_max = 1;
@@ -1445,6 +1495,8 @@ void layout(ttn_ctx* h, Arena& ar) {
       if (h->opt.prec != 0) I.w32[t] = reinterpret_cast<float*>(ar.take((I.w_elems(t) + 1) / 2));
       slab_max = std::max(slab_max, I.w_elems(t));
       pp_max = std::max(pp_max, (size_t)I.nodes(t) * I.chis[t + 1] * I.chis[t + 1]);
+      // (leftmost_rdm keeps the density matrix of any site layer in pA)
+      pp_max = std::max(pp_max, (size_t)I.chis[t] * I.chis[t]);
       nj_max = std::max(nj_max, (size_t)I.nodes(t));
     }
     I.eoff.assign(I.T + 1, nullptr);
@@ -1515,10 +1567,14 @@ void layout(ttn_ctx* h, Arena& ar) {
     }
     h->iflags = ar.take_int(8 + 3 * kComposeMaxTiles);
     h->partial = ar.take(h->partial_cap);
+    h->words = reinterpret_cast<unsigned*>(ar.take_int(h->words_cap));
     const int ss = h->opt.stage_streams == 0 ? (h->lanes.size() == 1 ? kSubStreams : 1)
                                              : h->opt.stage_streams;
     h->sub.n = ss > 1 ? std::min(ss, kSubStreams) : 0;
-    for (int i = 0; i < h->sub.n; ++i) h->sub.partial[i] = ar.take(h->partial_cap);
+    for (int i = 0; i < h->sub.n; ++i) {
+      h->sub.partial[i] = ar.take(h->partial_cap);
+      h->sub.words[i] = reinterpret_cast<unsigned*>(ar.take_int(h->words_cap));
+    }
     save_lane(h, h->lanes[k]);
   }
   h->E_hist = ar.take(4096 * h->inst.size() + 16);
@@ -1575,11 +1631,13 @@ int build_instances(ttn_ctx* h, const ttn_problem* probs, int n) {
 void plan(ttn_ctx* h) {
   h->measuring = true;
   h->partial_cap = 0;
+  h->words_cap = 0;
   for (Instance& I : h->inst) {
     sweep_instance(h, I);
     adjoints_only(h, I, 0);
     energy_only(h, I, nullptr);
     isometry_grams(h, I, nullptr);
+    if (!I.per_node) leftmost_rdm(h, I, 0);
     value_and_grad(h, I, h->opt.prec, nullptr, h->Gam);
   }
   h->measuring = false;
@@ -1759,6 +1817,7 @@ int ttn_create(ttn_t* out, const ttn_problem* probs, int n, const ttn_options* o
   layout(h, real);
   h->user = reinterpret_cast<cudaStream_t>(stream);
   gemm_tc_init();
+  gemm_oz_init();
   rc = check_cuda(h, cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking), "stream");
   h->lanes[0].stream = h->stream;
   h->ev_join.assign(h->lanes.size(), nullptr);
@@ -2153,6 +2212,7 @@ int ttn_ascend(ttn_t h, int inst, int site_layer, int prec, double* host_out) {
     h->launches += to_f32(I.ops[0], I.ops32[0], I.op_elems(0), h->stream);
     for (int t = 0; t < site_layer; ++t) h->launches += to_f32(I.W[t], I.w32[t], I.w_elems(t), h->stream);
   }
+  h->digits = prec == 0;
   for (int t = 0; t < site_layer; ++t) ascend_layer(h, I, t, prec);
   std::vector<double> e(I.sites(site_layer));
   int rc = check_cuda(h, cudaMemcpyAsync(host_out, I.ops[site_layer], I.op_elems(site_layer) * sizeof(double),
@@ -2232,23 +2292,9 @@ int ttn_rdm(ttn_t h, int inst, int site_layer, int which, double* out) {
     }
     return TTN_OK;
   }
-  // translation-invariant tree, leftmost site: rho = V V^T, then Tr_r(W^T rho W) downwards
-  const int c = I.chis[I.T];
+  // translation-invariant tree, leftmost site
   double* rho = h->pA;
-  {
-    GemmDesc d = desc(c, c, 1, 1, rho, c, 1, 0, 0);
-    add(d, grp(op(I.V, c, 1), op(I.V, c, 1), c));
-    run(h, d, 0);
-  }
-  for (int t = I.T - 1; t >= site_layer; --t) {
-    const LayerView v = view(I, t, 0);
-    GemmDesc g = desc(v.P, (int)v.n2, 1, 1, h->Yt, v.n2, 1, 0, 0);
-    add(g, grp(op(rho, v.P, 1), op(I.W[t], 1, v.n2), v.P));
-    run(h, g, 0);
-    GemmDesc r = desc(v.n, v.n, 1, 1, rho, v.n, 1, 0, 0);
-    add(r, grp(op(I.W[t], v.n, 1, v.n2), op(h->Yt, v.n, 1, v.n2), v.n, v.P));
-    run(h, r, 0);
-  }
+  leftmost_rdm(h, I, site_layer);
   int rc = check_cuda(h, cudaMemcpyAsync(out, rho, n2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream), "rdm");
   if (rc) return rc;
   rc = check_cuda(h, cudaStreamSynchronize(h->stream), "rdm sync");
