@@ -725,6 +725,7 @@ struct TmaParams {
   int a_mn[kMaxGroups], b_mn[kMaxGroups];     // 1: MN index contiguous (transposed boxes)
   int a_use[kMaxGroups], b_use[kMaxGroups];   // bit i: map dim i is a real index (else coordinate 0)
   int total_tiles;
+  int nacc;    // K splits summed inside the CTA (accumulators side by side in TMEM)
   int* err;
 };
 
@@ -883,6 +884,17 @@ __device__ __forceinline__ void store_row16(const GemmDesc& d, int b, int b0, in
     if (n + j < d.N) store_out(d, cb + static_cast<long long>(n + j) * d.sc_n, __uint_as_float(r[j]), af, bf);
 }
 
+// Sixteen accumulator columns of the warp's 32 rows.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 template <bool kSplit, int BN, int kRing>
 __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
     gemm_tma_kernel(const GemmDesc d, const __grid_constant__ TmaParams tp) {
@@ -917,6 +929,8 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
   const int t_hi =
       static_cast<int>(static_cast<long long>(tp.total_tiles) * (split_id + 1) / d.splits);
   const int nk = t_hi - t_lo;
+  const int nacc = tp.nacc;
+  const uint32_t ncols = nacc <= 1 ? BN : (nacc == 2 ? 2 * BN : 4 * BN);   // TMEM columns
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
@@ -932,7 +946,7 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_slot)),
-                 "r"(BN));
+                 "r"(ncols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -994,8 +1008,17 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
     if (lane == 0) {
       // ---- MMA issuer ----
       bool ok = true;
+      // accumulator q takes the K tiles [nk q / nacc, nk (q + 1) / nacc)
+      int q = 0, q_end = nacc > 1 ? static_cast<int>(static_cast<long long>(nk) / nacc) : nk, q_begin = 0;
+      uint32_t dcol = tmem;
       for (int kt = 0; kt < nk; ++kt) {
         const int s = kt % S, u = kt / S;
+        if (kt == q_end) {
+          ++q;
+          q_begin = kt;
+          q_end = static_cast<int>(static_cast<long long>(nk) * (q + 1) / nacc);
+          dcol += BN;
+        }
         if (!mbar_wait_ab(&conv_bar[s], u & 1, abort_v)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t a_hi = smem_u32(smem + s * kStageBytes);
@@ -1004,13 +1027,13 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint32_t off = j * 32;   // 8 TF32 values of K per instruction
-          const uint32_t acc = (kt > 0 || j > 0) ? 1u : 0u;
+          const uint32_t acc = (kt > q_begin || j > 0) ? 1u : 0u;
           if constexpr (kSplit) {
-            mma<false>(tmem, smem_desc(a_lo + off), smem_desc(b_hi + off), kIdesc, acc);
-            mma<false>(tmem, smem_desc(a_hi + off), smem_desc(b_lo + off), kIdesc, 1u);
-            mma<false>(tmem, smem_desc(a_hi + off), smem_desc(b_hi + off), kIdesc, 1u);
+            mma<false>(dcol, smem_desc(a_lo + off), smem_desc(b_hi + off), kIdesc, acc);
+            mma<false>(dcol, smem_desc(a_hi + off), smem_desc(b_lo + off), kIdesc, 1u);
+            mma<false>(dcol, smem_desc(a_hi + off), smem_desc(b_hi + off), kIdesc, 1u);
           } else {
-            mma<false>(tmem, smem_desc(a_hi + off), smem_desc(b_hi + off), kIdesc, acc);
+            mma<false>(dcol, smem_desc(a_hi + off), smem_desc(b_hi + off), kIdesc, acc);
           }
         }
         mma_commit(&empty_bar[s]);
@@ -1068,13 +1091,25 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
           for (int j = 0; j < 16; ++j) r[j] = 0u;
         } else {
           const uint32_t taddr = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + c0;
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
-                "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-              : "r"(taddr));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          tmem_ld16(taddr, r);
+          if (nacc > 1) {
+            // the FP32 pair sum of splitk_reduce_tc (one split per group of
+            // eight, in order), so that both give the same bits
+            float th[16], tl[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) { th[j] = 0.f + __uint_as_float(r[j]); tl[j] = 0.f; }
+            for (int q = 1; q < nacc; ++q) {
+              tmem_ld16(taddr + q * BN, r);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const float x = __uint_as_float(r[j]), s = th[j] + x, bb = s - th[j];
+                tl[j] += (th[j] - (s - bb)) + (x - bb);
+                th[j] = s;
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(th[j] + tl[j]);
+          }
         }
         if (m < d.M && n0 + c0 < d.N) store_row16(d, b, b0, b1, split_id, m, n0 + c0, r, af, bf);
       }
@@ -1085,7 +1120,7 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(BN));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
 }
 
 template <bool kSplit, int BN, int kRing>
@@ -1182,7 +1217,7 @@ bool encode_operand(const Operand& o, int k0_log2, int K, int rows, int B0, int 
 // Returns 1 (launched) or 0 (a tensor map could not be encoded: the caller
 // runs the thread-staged kernel instead).
 template <bool kSplit, int BN, int kRing>
-int launch_tma(const GemmDesc& d, cudaStream_t s) {
+int launch_tma(const GemmDesc& d, cudaStream_t s, int in_cta) {
   static TmaParams tp;   // host staging of the kernel parameter (launch copies it)
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
@@ -1195,6 +1230,7 @@ int launch_tma(const GemmDesc& d, cudaStream_t s) {
       return 0;
   }
   tp.total_tiles = tc_total_tiles(d, 32);
+  tp.nacc = in_cta;
   tp.err = d.err;
   const int tiles = ((d.M + kBM - 1) / kBM) * ((d.N + BN - 1) / BN);
   dim3 grid(tiles, d.B0 * d.B1, d.splits);
@@ -1204,16 +1240,32 @@ int launch_tma(const GemmDesc& d, cudaStream_t s) {
 
 // d.occ == 2 selects the 96 KB ring (two CTAs per SM) where a stage still
 // fits twice: BN = 64 in both forms, BN = 128 without the split.
-int launch_tma_bn(const GemmDesc& d, cudaStream_t s) {
+int launch_tma_bn(const GemmDesc& d, cudaStream_t s, int in_cta) {
   const bool split = d.prec == 2;
   const int bn = (d.tile == 64 || d.tile == 128) ? d.tile : tma_bn(d.N);
   const bool two = d.occ == 2 && !(split && bn == 128);
   if (bn == 128) {
-    if (split) return launch_tma<true, 128, kTSmem>(d, s);
-    return two ? launch_tma<false, 128, kTSmem2>(d, s) : launch_tma<false, 128, kTSmem>(d, s);
+    if (split) return launch_tma<true, 128, kTSmem>(d, s, in_cta);
+    return two ? launch_tma<false, 128, kTSmem2>(d, s, in_cta) : launch_tma<false, 128, kTSmem>(d, s, in_cta);
   }
-  if (split) return two ? launch_tma<true, 64, kTSmem2>(d, s) : launch_tma<true, 64, kTSmem>(d, s);
-  return two ? launch_tma<false, 64, kTSmem2>(d, s) : launch_tma<false, 64, kTSmem>(d, s);
+  if (split) return two ? launch_tma<true, 64, kTSmem2>(d, s, in_cta) : launch_tma<true, 64, kTSmem>(d, s, in_cta);
+  return two ? launch_tma<false, 64, kTSmem2>(d, s, in_cta) : launch_tma<false, 64, kTSmem>(d, s, in_cta);
+}
+
+// K splits that one CTA sums itself: a product whose output tiles alone fill
+// at least half of the SMs gains nothing from more CTAs per tile, while its
+// partial sums and their reduction cost a write and a read of the whole output
+// per split.  The K ranges and the order of the sums are those of the split
+// product (same bits).  Measured for 128 x 16384 outputs, K = 128, two splits:
+// the reduction alone took 100 us, the product 18 us.
+int tma_in_cta(const GemmDesc& d) {
+  if (d.splits < 2 || d.splits > 4 || tc_total_tiles(d, 32) < d.splits) return 1;
+  const int bn = (d.tile == 64 || d.tile == 128) ? d.tile : tma_bn(d.N);
+  const long long base = static_cast<long long>((d.M + kBM - 1) / kBM) * ((d.N + bn - 1) / bn) * d.B0 * d.B1;
+  if (2 * base < device_sm_count()) return 1;
+  // (two CTAs per SM share the 512 TMEM columns)
+  const int cols = (d.splits == 2 ? 2 : 4) * bn;
+  return cols <= (d.occ == 2 ? 256 : 512) ? d.splits : 1;
 }
 
 int tc_bn(int N) { return N >= 64 ? 64 : 32; }
@@ -1281,7 +1333,13 @@ int tc_pick_splits(const GemmDesc& d) {
 
 int gemm_tc_launch(const GemmDesc& d, cudaStream_t s) {
   int n = 0;
-  if (d.tc_engine != 1 && tma_eligible(d)) n = launch_tma_bn(d, s);
+  if (d.tc_engine != 1 && tma_eligible(d)) {
+    const int in_cta = tma_in_cta(d);
+    GemmDesc e = d;
+    if (in_cta > 1) e.splits = 1;
+    n = launch_tma_bn(e, s, in_cta);
+    if (n && in_cta > 1) return n;
+  }
   if (n == 0)
   switch (d.prec) {
     case 1: n = launch_tc_bn<false, false>(d, s, d.err); break;
