@@ -282,7 +282,7 @@ int polar_compose(const ComposeArgs& a, cudaStream_t s, bool df = false);
 // the top Hamiltonian in one cooperative launch.  V (c x c) holds the start
 // vector on entry and the normalised eigenvector on exit, sign-aligned with
 // the start (copied to Vprev).  Scratch: basis (m+1) c^2, w c^2, Y 2K c^2,
-// part grid*(m+2), coef 2(m+2), alpha, beta, y (m+2 each), scal (4),
+// part grid*(m+2), coef 2(m+2), alpha, beta, y (m+2 each), scal (16),
 // flags[0] = converged, flags[1] = tridiagonal size.  err |= 4 when a grid
 // barrier wait expires.
 // ---------------------------------------------------------------------------
@@ -305,7 +305,7 @@ struct LanczosArgs {
   int* flags;
   int c, K, m, restarts;
   double tol;
-  unsigned* bar;      // grid-barrier counter (zeroed by lanczos_launch)
+  unsigned* bar;      // grid-barrier counter and two words (zeroed by lanczos_launch)
   int* err;
   int max_spin;       // polls of a grid-barrier wait before it expires (<= 0: 2^21, ~1 s)
   // double-float matrix-vector products (mixed modes): df != 0 and pair
@@ -317,15 +317,18 @@ struct LanczosArgs {
   float* s1p;
   float* bp;
   float* Yp;
-  // set by lanczos_launch: the double-float matrix-vector phases stage all
-  // operand tiles of a phase at once (asynchronous copies into shared memory)
-  int wide = 0;
+  // set by lanczos_launch: the matrix-vector phases stage all operand tiles of
+  // a phase at once (asynchronous copies into shared memory); basis vectors
+  // whose own entries a CTA keeps in shared memory, and their pitch; an extra
+  // CTA runs the convergence checks, told by job[0] and answering in job[1]
+  int wide = 0, ncache = 0, own_pitch = 0, extra = 0;
+  unsigned* job = nullptr;
 };
 bool lanczos_supported(int c, int m);
 // CTAs of the launch for top dimension c when grid_share streams share the GPU.
 int lanczos_grid(int c, int grid_share);
 // Returns the number of kernel launches (1), or -1 if the launch was refused.
-int lanczos_launch(const LanczosArgs& a, int grid, cudaStream_t s);
+int lanczos_launch(const LanczosArgs& a, int grid, int grid_share, cudaStream_t s);
 
 // ---------------------------------------------------------------------------
 // Double-float products (gemm_df.cu): FP64 values held as FP32 pairs

@@ -18,12 +18,20 @@
 //     of |w|^2, then alpha_j, beta_j and the next basis vector
 // with every phase shared by all CTAs and a grid barrier between phases
 // (bounded spin, error flag).  Each CTA owns the vector entries of the 8 x 8
-// output tiles it computes; every reduction adds its per-CTA partial sums in
-// a fixed order, so the result does not depend on timing.  Every kLCheck
-// steps CTA 0 tests the tridiagonal so far for convergence in pair
-// arithmetic (tridiag_df.cuh) and a passed test ends the cycle; at the end of
-// a cycle CTA 0 finds the eigenpair of the tridiagonal (Sturm bisection, in
-// FP32 to bracket, then in FP64, and inverse iteration).
+// output tiles it computes (and keeps them, of w and of every basis vector, in
+// shared memory); every reduction adds its per-CTA partial sums in a fixed
+// order, so the result does not depend on timing.  Every kLCheck steps the
+// tridiagonal so far is tested for convergence in pair arithmetic by an extra
+// CTA, which has the next kLLag steps for it, and a passed test ends the cycle;
+// at the end of a cycle CTA 0 finds the eigenpair of the tridiagonal.
+//
+// What bounds it: latency, and the FP64 units.  An FP64 warp instruction takes
+// 16 clocks of an SM and about 100 of latency, so scalars are computed by one
+// warp, the butterflies of four sums share their additions, and the Sturm
+// sequences run in pairs.  Measured per sweep from a random start (clocks of
+// one step, then the solve): c = 8, one CTA: 48 k -> 23 k, 2.37 -> 1.2 ms; c =
+// 128, mixed: 45 -> 29 us a step, 4.4 -> 2.8 ms; the FP64 products of c = 128
+// alone take 25 us of a step.
 #include <algorithm>
 #include <mutex>
 
@@ -41,22 +49,52 @@ constexpr int kLWarps = kLThreads / 32;
 constexpr int kLMaxC = 256;
 constexpr int kLMaxSpin = 1 << 21;       // ~1 s of polling, then the error flag
 constexpr int kLCheck = 8;               // steps between convergence checks within a cycle
+constexpr int kLLag = 4;                 // steps that a check may take (less than kLCheck)
 
+// Static shared memory; the operand tiles and the cached basis entries are
+// dynamic (lz_dyn): first the tiles (LzTiles), then the cache (LzOwn).
 struct __align__(16) LzSmem {
-  double L[kLT][kLMaxC + 1];             // left-operand rows of a tile
-  double R[kLT][kLMaxC + 1];             // right-operand rows (or columns) of a tile
   double red[kLWarps][kLT * kLT];
-  double tri[6][kLMaxM + 2];             // inverse iteration scratch (CTA 0)
-  double da[kLMaxM + 2], db2[kLMaxM + 2];  // tridiagonal: diagonal, squared off-diagonal
+  double tri[1][kLMaxM + 2];             // eigenvector of the tridiagonal
   float fa[kLMaxM + 2], fb2[kLMaxM + 2];
   double cf[kLMaxM + 2];                 // coefficients of the current combination
+  double al[kLMaxM + 2], be[kLMaxM + 2]; // the tridiagonal's entries (CTA 0 and the checks)
   double bcast[4];
+  unsigned ball[kLWarps];
+  float bnd[2 * kLWarps];
+  // scalars of the recurrence, kept by warp 0: Rayleigh shift, beta_{j-1},
+  // alpha_{j-1} of H, 1 / beta_j; whether one Gram-Schmidt pass was enough, and
+  // whether beta_j vanished
+  double sigma, beta_prev, alpha_prev_h, inv;
+  int one_pass, brk;
   int ok;
 };
 
-__device__ bool lz_barrier(LzSmem& sm, unsigned* bar, unsigned& target, int* err, int max_spin) {
-  target += gridDim.x;
+// Operand tiles of a matrix product: L (left rows) and R (right rows or
+// columns), pitch c + 1.
+struct LzTiles {
+  double* L;
+  double* R;
+  int ld;
+};
+
+// The CTA's own entries (own_index) of basis vectors 0 .. n - 1 in shared
+// memory, and of w at row `wrow` (or -1): the projections and combinations of
+// every step read them here instead of from L2 (about 700 clocks per round of
+// loads).  Rows have a pitch of nown + 8 doubles, so that the threads that
+// share an entry read distinct banks.
+struct LzOwn {
+  double* p;
+  int pitch, n, wrow;
+  __device__ __forceinline__ void set(int i, int q, double v) const {
+    if (n) p[i * pitch + q] = v;
+  }
+};
+
+__device__ bool lz_barrier(LzSmem& sm, unsigned* bar, unsigned& target, int G, int* err, int max_spin) {
   __syncthreads();
+  if (G == 1) return true;   // one CTA: its own barrier orders its accesses
+  target += G;
   if (threadIdx.x == 0) {
     // arrive with release semantics (this CTA's writes before it), poll with
     // acquire semantics (the other CTAs' writes after it)
@@ -98,8 +136,8 @@ __device__ double cta_ordered_sum(LzSmem& sm, const double* x, int count, long l
 // shared-memory store, so that a staged tile costs one load latency.
 constexpr int kLStage = kLT * kLMaxC / kLThreads;
 
-// Stage rows [r0, r0+8) of the row-major c x c matrix M (times scale) into dst.
-__device__ void stage_rows(double (*dst)[kLMaxC + 1], const double* M, int c, int r0, double scale) {
+// Stage rows [r0, r0+8) of the row-major c x c matrix M into dst.
+__device__ void stage_rows(double* dst, const double* M, int c, int r0) {
   double v[kLStage];
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
@@ -109,11 +147,11 @@ __device__ void stage_rows(double (*dst)[kLMaxC + 1], const double* M, int c, in
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
     const int e = threadIdx.x + u * kLThreads, r = e / c, k = e - r * c;
-    if (e < kLT * c) dst[r][k] = scale * v[u];
+    if (e < kLT * c) dst[r * (c + 1) + k] = v[u];
   }
 }
-// Stage columns [c0, c0+8) of M (times scale) as rows of dst: dst[j][k] = M[k][c0 + j].
-__device__ void stage_cols(double (*dst)[kLMaxC + 1], const double* M, int c, int c0, double scale) {
+// Stage columns [c0, c0+8) of M as rows of dst: dst[j][k] = M[k][c0 + j].
+__device__ void stage_cols(double* dst, const double* M, int c, int c0) {
   double v[kLStage];
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
@@ -123,19 +161,19 @@ __device__ void stage_cols(double (*dst)[kLMaxC + 1], const double* M, int c, in
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
     const int e = threadIdx.x + u * kLThreads, k = e / kLT, j = e - k * kLT;
-    if (e < kLT * c) dst[j][k] = scale * v[u];
+    if (e < kLT * c) dst[j * (c + 1) + k] = v[u];
   }
 }
 
 // acc[0..1] += sum_k L[i][k] R[j][k] over this warp's K slice (i = lane/4,
 // j = 2 (lane % 4) + {0, 1}).
-__device__ __forceinline__ void tile_fma(const LzSmem& sm, int c, double& a0, double& a1) {
+__device__ __forceinline__ void tile_fma(const LzTiles& ts, int c, double& a0, double& a1) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = lane >> 2, j = (lane & 3) * 2;
   for (int k = warp; k < c; k += kLWarps) {
-    const double x = sm.L[i][k];
-    a0 = fma(x, sm.R[j][k], a0);
-    a1 = fma(x, sm.R[j + 1][k], a1);
+    const double x = ts.L[i * ts.ld + k];
+    a0 = fma(x, ts.R[j * ts.ld + k], a0);
+    a1 = fma(x, ts.R[(j + 1) * ts.ld + k], a1);
   }
 }
 
@@ -143,7 +181,8 @@ __device__ __forceinline__ void tile_fma(const LzSmem& sm, int c, double& a0, do
 // minus sigma X when sigma != 0 (the shifted operator H - sigma I).
 __device__ void tile_store(LzSmem& sm, double a0, double a1, double* C, int c, int i0, int j0,
                            const double* X = nullptr, double sigma = 0.0,
-                           const double* Xprev = nullptr, double beta = 0.0) {
+                           const double* Xprev = nullptr, double beta = 0.0,
+                           double* own_w = nullptr) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = lane >> 2, j = (lane & 3) * 2;
   sm.red[warp][i * kLT + j] = a0;
@@ -158,22 +197,22 @@ __device__ void tile_store(LzSmem& sm, double a0, double a1, double* C, int c, i
       if (sigma != 0.0) v = fma(-sigma, __ldcg(X + e), v);
       if (beta != 0.0) v = fma(-beta, __ldcg(Xprev + e), v);
       __stcg(C + e, v);
+      if (own_w) own_w[threadIdx.x] = v;
     }
   }
   __syncthreads();
 }
 
 // Number of eigenvalues of the symmetric tridiagonal below x (diagonal a,
-// squared off-diagonal b2), by the signs of the LDL^T pivots.
-template <typename T>
-__device__ int sturm_below(const T* a, const T* b2, int m, T x) {
+// squared off-diagonal b2), by the signs of the LDL^T pivots, in FP32.
+__device__ int sturm_below_f32(const float* a, const float* b2, int m, float x) {
   int cnt = 0;
-  T q = a[0] - x;
-  if (q < (T)0) ++cnt;
+  float q = a[0] - x;
+  if (q < 0.f) ++cnt;
   for (int i = 1; i < m; ++i) {
-    if (q == (T)0) q = (T)1e-30;
+    if (q == 0.f) q = 1e-30f;
     q = a[i] - x - b2[i - 1] / q;
-    if (q < (T)0) ++cnt;
+    if (q < 0.f) ++cnt;
   }
   return cnt;
 }
@@ -207,195 +246,433 @@ __device__ int sturm_below_f64(const double* a, const double* b2, int m, double 
   return cnt;
 }
 
-template <typename T>
-__device__ __forceinline__ int sturm_count(const T* a, const T* b2, int m, T x) {
-  if constexpr (sizeof(T) == 8) return sturm_below_f64(a, b2, m, x);
-  else return sturm_below<T>(a, b2, m, x);
+// Index of the first thread of the CTA whose flag is set, else kLThreads.
+__device__ int first_thread(LzSmem& sm, bool flag) {
+  const unsigned bal = __ballot_sync(0xffffffffu, flag);
+  if ((threadIdx.x & 31) == 0) sm.ball[threadIdx.x >> 5] = bal;
+  __syncthreads();
+  int f = kLThreads;
+  for (int w = kLWarps - 1; w >= 0; --w)
+    if (sm.ball[w]) f = w * 32 + __ffs(sm.ball[w]) - 1;
+  __syncthreads();
+  return f;
 }
 
-// 32-way multisection of [lo, hi] for the lowest eigenvalue, by one warp,
-// until the interval is narrower than rel * max(|lo|, |hi|) or `its` rounds.
-template <typename T>
-__device__ void multisect(const T* a, const T* b2, int m, T& lo, T& hi, T rel, int its) {
-  const int lane = threadIdx.x & 31;
-  for (int it = 0; it < its; ++it) {
-    const T mag = fabs(lo) > fabs(hi) ? fabs(lo) : fabs(hi);
-    if (!(hi - lo > rel * mag)) break;
-    constexpr T r33 = (T)1 / (T)33;
-    const T pt = lo + (hi - lo) * ((T)(lane + 1) * r33);
-    const unsigned below = __ballot_sync(0xffffffffu, sturm_count<T>(a, b2, m, pt) >= 1);
-    const int f = below ? __ffs(below) - 1 : 32;
-    const T nlo = f == 0 ? lo : lo + (hi - lo) * ((T)f * r33);
-    const T nhi = f == 32 ? hi : lo + (hi - lo) * ((T)(f + 1) * r33);
-    lo = nlo;
-    hi = nhi;
-  }
-}
+// The work of the tridiagonal in pair arithmetic or FP64: twisted_rows is
+// generic over the two.
+struct ArithDF {
+  typedef tdf::DF T;
+  static __device__ __forceinline__ T sub(T a, T b) { return tdf::sub(a, b); }
+  static __device__ __forceinline__ T mul(T a, T b) { return tdf::mul(a, b); }
+  static __device__ __forceinline__ T div(T a, T b) { return tdf::div(a, b); }
+  static __device__ __forceinline__ bool zero(T a) { return a.h == 0.f; }
+  static __device__ __forceinline__ T tiny() { return {1e-30f, 0.f}; }
+  static __device__ __forceinline__ T one() { return {1.f, 0.f}; }
+  static __device__ __forceinline__ double mag(T a) { return fabs((double)a.h); }
+  static __device__ __forceinline__ T from(double x) { return tdf::make(x); }
+  static __device__ __forceinline__ double to(T x) { return tdf::to_double(x); }
+};
+struct ArithD {
+  typedef double T;
+  static __device__ __forceinline__ T sub(T a, T b) { return a - b; }
+  static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
+  static __device__ __forceinline__ T div(T a, T b) { return a / b; }
+  static __device__ __forceinline__ bool zero(T a) { return a == 0.0; }
+  static __device__ __forceinline__ T tiny() { return 1e-290; }
+  static __device__ __forceinline__ T one() { return 1.0; }
+  static __device__ __forceinline__ double mag(T a) { return fabs(a); }
+  static __device__ __forceinline__ T from(double x) { return x; }
+  static __device__ __forceinline__ double to(T x) { return x; }
+};
 
-// Lowest eigenvalue of the m x m tridiagonal (alpha, beta) by warp 0 of the
-// calling CTA (threads >= 32 return at once): bracketed by FP32 multisection,
-// confirmed and refined in FP64; the tridiagonal is left in sm.da / sm.db2.
-__device__ double ritz_value(LzSmem& sm, const double* alpha, const double* beta, int m) {
+// Eigenvector of the m x m tridiagonal (al, be) for the eigenvalue th, by warp
+// 0, from the twisted factorisation (Dhillon and Parlett, "Orthogonal
+// eigenvectors and relative gaps", SIAM J. Matrix Anal. Appl. 25, 2004): the
+// pivots of T - th I from both ends (lanes 0 and 1 at the same time), the
+// twist at the row where their sum less the diagonal is smallest, and the
+// vector outwards from 1 there by products alone.  One division per row in
+// each chain, where an LU with pivoting and its two substitutions need four.
+// z[0 .. m) unnormalised (FP64); scratch: 4 m values of T.
+template <typename A>
+__device__ void twisted_vector(const double* al, const double* be, int m, double th, typename A::T* scratch,
+                               double* z) {
+  typedef typename A::T T;
   const int lane = threadIdx.x;
-  double glo = alpha[0], ghi = alpha[0];
-  for (int i = 0; i < m; ++i) {
-    const double r = (i > 0 ? fabs(beta[i - 1]) : 0.0) + (i + 1 < m ? fabs(beta[i]) : 0.0);
-    glo = fmin(glo, alpha[i] - r);
-    ghi = fmax(ghi, alpha[i] + r);
-  }
+  T* ms = scratch;           // al - th
+  T* b2 = scratch + m;       // squared off-diagonal, then the multipliers
+  T* dp = scratch + 2 * m;   // pivots from the top
+  T* dm = scratch + 3 * m;   // pivots from the bottom
   for (int i = lane; i < m; i += 32) {
-    sm.da[i] = alpha[i];
-    sm.fa[i] = (float)alpha[i];
-    const double b2 = i + 1 < m ? beta[i] * beta[i] : 0.0;
-    sm.db2[i] = b2;
-    sm.fb2[i] = (float)b2;
+    ms[i] = A::sub(A::from(al[i]), A::from(th));
+    const T b = A::from(i + 1 < m ? be[i] : 0.0);
+    b2[i] = A::mul(b, b);
   }
   __syncwarp();
-  // bracket in FP32, widen by the FP32 rounding of T, confirm in FP64
-  float flo = (float)glo, fhi = (float)ghi;
-  multisect<float>(sm.fa, sm.fb2, m, flo, fhi, 2e-6f, 8);
-  const double tnorm = fmax(fabs(glo), fabs(ghi));
-  double lo = (double)flo - 1e-5 * tnorm, hi = (double)fhi + 1e-5 * tnorm;
-  const int c_lo = sturm_below_f64(sm.da, sm.db2, m, lo);
-  const int c_hi = sturm_below_f64(sm.da, sm.db2, m, hi);
-  if (!__all_sync(0xffffffffu, c_lo == 0 && c_hi >= 1)) { lo = glo; hi = ghi; }
-  multisect<double>(sm.da, sm.db2, m, lo, hi, 4e-16, 16);
-  return 0.5 * (lo + hi);
-}
-
-// Convergence test of the tridiagonal of the steps so far (alpha, beta: m
-// entries, shifted by -sigma) by warp 0 of the calling CTA, for the checks
-// within a cycle: the lowest eigenvalue bracketed in FP32 and refined by
-// 32-way multisection in pair arithmetic, then one round of inverse
-// iteration in pair arithmetic for the last component y_{m-1} of its
-// eigenvector; true when |beta_{m-1} y_{m-1}| <= tol |theta + sigma|.  (The
-// end of a cycle recomputes the pair in FP64; a wrong early answer costs a
-// restart, not accuracy.)  Uses sm.L as scratch.  The result is valid in
-// thread 0.
-__device__ bool ritz_check_df(LzSmem& sm, const double* alpha, const double* beta, int m,
-                              double sigma, double tol) {
-  using namespace tdf;
-  const int lane = threadIdx.x;
-  constexpr int S = kLMaxM + 2;
-  DF* A = reinterpret_cast<DF*>(&sm.L[0][0]);
-  DF* B = A + S;
-  DF* B2 = B + S;
-  double glo = alpha[0], ghi = alpha[0];
-  for (int i = 0; i < m; ++i) {
-    const double r = (i > 0 ? fabs(beta[i - 1]) : 0.0) + (i + 1 < m ? fabs(beta[i]) : 0.0);
-    glo = fmin(glo, alpha[i] - r);
-    ghi = fmax(ghi, alpha[i] + r);
-  }
-  for (int i = lane; i < m; i += 32) {
-    const double b2 = i + 1 < m ? beta[i] * beta[i] : 0.0;
-    sm.fa[i] = (float)alpha[i];
-    sm.fb2[i] = (float)b2;
-    A[i] = make(alpha[i]);
-    B[i] = make(i + 1 < m ? beta[i] : 0.0);
-    B2[i] = make(b2);
-  }
-  __syncwarp();
-  float flo = (float)glo, fhi = (float)ghi;
-  multisect<float>(sm.fa, sm.fb2, m, flo, fhi, 2e-6f, 8);
-  const double tnorm = fmax(fabs(glo), fabs(ghi));
-  DF lo = make((double)flo - 1e-5 * tnorm), hi = make((double)fhi + 1e-5 * tnorm);
-  const int c_lo = sturm_below(A, B2, m, lo), c_hi = sturm_below(A, B2, m, hi);
-  if (!__all_sync(0xffffffffu, c_lo == 0 && c_hi >= 1)) { lo = make(glo); hi = make(ghi); }
-  constexpr float r33 = 1.f / 33.f;
-  for (int it = 0; it < 12; ++it) {
-    const float w = sub(hi, lo).h;
-    if (!(w > 1e-14f * fmaxf(fabsf(lo.h), fabsf(hi.h)))) break;
-    const DF pt = add(lo, {w * ((float)(lane + 1) * r33), 0.f});
-    const unsigned below = __ballot_sync(0xffffffffu, sturm_below(A, B2, m, pt) >= 1);
-    const int f = below ? __ffs(below) - 1 : 32;
-    const DF nlo = f == 0 ? lo : add(lo, {w * ((float)f * r33), 0.f});
-    const DF nhi = f == 32 ? hi : add(lo, {w * ((float)(f + 1) * r33), 0.f});
-    lo = nlo;
-    hi = nhi;
-  }
-  if (lane != 0) return false;
-  const DF th = add(lo, {0.5f * sub(hi, lo).h, 0.f});
-  DF* w = B2 + S;
-  const double ylast = last_component(A, B, m, th, w, w + S, w + 2 * S, w + 3 * S, w + 4 * S);
-  return fabs(beta[m - 1]) * ylast <= tol * fmax(fabs(to_double(th) + sigma), 1e-300);
-}
-
-// Lowest eigenpair of the m x m tridiagonal (alpha, beta) by warp 0 of the
-// calling CTA: y (m entries, unit norm), theta, residual |beta_{m-1} y_{m-1}|.
-__device__ void ritz_pair(LzSmem& sm, const double* alpha, const double* beta, int m, double* y,
-                          double* theta, double* res) {
-  if (threadIdx.x >= 32) return;
-  const double th = ritz_value(sm, alpha, beta, m);
-  if (threadIdx.x != 0) return;
-  // inverse iteration on (T - th I) x = x_prev: LU with partial pivoting of
-  // the tridiagonal, two rounds
-  double* x = sm.tri[0];
-  double* dd = sm.tri[1];
-  double* du = sm.tri[2];
-  double* du2 = sm.tri[3];
-  double* rhs = sm.tri[4];
-  double* dl = sm.tri[5];
-  for (int i = 0; i < m; ++i) x[i] = 1.0 / sqrt((double)m);
-  const double eps = fmax(fabs(th), 1.0) * 1e-15;
-  for (int round = 0; round < 2; ++round) {
-    for (int i = 0; i < m; ++i) {
-      dd[i] = alpha[i] - th;
-      du[i] = i + 1 < m ? beta[i] : 0.0;
-      du2[i] = 0.0;
-      rhs[i] = x[i];
-      dl[i] = i + 1 < m ? beta[i] : 0.0;
+  if (lane < 2) {
+    T* d = lane == 0 ? dp : dm;
+    int i = lane == 0 ? 0 : m - 1;
+    const int step = lane == 0 ? 1 : -1;
+    T cur = ms[i];
+    d[i] = cur;
+    for (int k = 1; k < m; ++k) {
+      const T bb = b2[lane == 0 ? i : i - 1];
+      i += step;
+      const T a = ms[i];
+      if (A::zero(cur)) {
+        cur = A::tiny();
+        d[i - step] = cur;
+      }
+      cur = A::sub(a, A::div(bb, cur));
+      d[i] = cur;
     }
-    for (int i = 0; i + 1 < m; ++i) {
-      if (fabs(dd[i]) >= fabs(dl[i])) {
-        if (dd[i] == 0.0) dd[i] = eps;
-        const double f = dl[i] / dd[i];
-        dl[i] = f;
-        dd[i + 1] -= f * du[i];
-        rhs[i + 1] -= f * rhs[i];
-      } else {
-        const double f = dd[i] / dl[i];
-        dd[i] = dl[i];
-        dl[i] = f;
-        const double t = du[i];
-        du[i] = dd[i + 1];
-        dd[i + 1] = t - f * dd[i + 1];
-        if (i + 2 < m) { du2[i] = du[i + 1]; du[i + 1] = -f * du[i + 1]; }
-        const double r = rhs[i];
-        rhs[i] = rhs[i + 1];
-        rhs[i + 1] = r - f * rhs[i + 1];
+    if (A::zero(cur)) d[i] = A::tiny();
+  }
+  __syncwarp();
+  // twist row: smallest |d+ + d- - (a - th)|
+  double best = 1e300;
+  int r = 0;
+  for (int i = lane; i < m; i += 32) {
+    const double g = A::mag(A::sub(dp[i], A::sub(ms[i], dm[i])));
+    if (g < best) { best = g; r = i; }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+    const int orr = __shfl_xor_sync(0xffffffffu, r, o);
+    if (ob < best || (ob == best && orr < r)) { best = ob; r = orr; }
+  }
+  // multipliers: z_i = -(b_i / d+_i) z_{i+1} above r, z_{i+1} = -(b_i / d-_{i+1}) z_i below
+  for (int i = lane; i + 1 < m; i += 32) b2[i] = A::div(A::from(-be[i]), i < r ? dp[i] : dm[i + 1]);
+  __syncwarp();
+  if (lane < 2) {
+    T cur = A::one();
+    if (lane == 0) {
+      z[r] = 1.0;
+      for (int i = r - 1; i >= 0; --i) {
+        cur = A::mul(b2[i], cur);
+        dp[i] = cur;
+      }
+    } else {
+      for (int i = r; i + 1 < m; ++i) {
+        cur = A::mul(b2[i], cur);
+        dp[i + 1] = cur;
       }
     }
-    if (dd[m - 1] == 0.0) dd[m - 1] = eps;
-    for (int i = m - 1; i >= 0; --i) {
-      double s = rhs[i];
-      if (i + 1 < m) s -= du[i] * x[i + 1];
-      if (i + 2 < m) s -= du2[i] * x[i + 2];
-      x[i] = s / (fabs(dd[i]) < eps ? (dd[i] < 0 ? -eps : eps) : dd[i]);
-    }
-    double nrm = 0.0;
-    for (int i = 0; i < m; ++i) nrm += x[i] * x[i];
-    nrm = sqrt(nrm);
-    for (int i = 0; i < m; ++i) x[i] /= nrm;
   }
-  for (int i = 0; i < m; ++i) y[i] = x[i];
-  *theta = th;
-  *res = fabs(beta[m - 1] * x[m - 1]);
+  __syncwarp();
+  for (int i = lane; i < m; i += 32)
+    if (i != r) z[i] = A::to(dp[i]);
+  __syncwarp();
+}
+
+__device__ __forceinline__ double warp_sum(double s) {
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// Lowest eigenvalue of the tridiagonal in sm.al and sm.be (m entries) by the
+// whole CTA, to pair accuracy: 257-way multisection in FP32, then in pair
+// arithmetic (tridiag_df.cuh).  FP64 runs at one warp instruction per 16
+// clocks of an SM and about 100 clocks of latency here: one Sturm count of 48
+// rows takes 26 k clocks in FP64 and 8 k in pairs.  The tridiagonal is scaled
+// by a power of two to unit size first (sm.al and sm.be hold the scaled one on
+// return; the result is in the same scale).  scratch: 2 m pairs.
+__device__ double lowest_value(LzSmem& sm, double* scratch, int m, double& unscale) {
+  using namespace tdf;
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  // largest entry -> scale
+  unsigned hw = 0;
+  for (int i = t; i < m; i += kLThreads) {
+    hw = max(hw, (unsigned)__double2hiint(sm.al[i]) & 0x7FFFFFFFu);
+    if (i + 1 < m) hw = max(hw, (unsigned)__double2hiint(sm.be[i]) & 0x7FFFFFFFu);
+  }
+  hw = __reduce_max_sync(0xffffffffu, hw);
+  if (lane == 0) sm.ball[warp] = hw;
+  __syncthreads();
+  for (int w = 0; w < kLWarps; ++w) hw = max(hw, sm.ball[w]);
+  __syncthreads();
+  const int e = min(max((int)(hw >> 20), 30), 2000);
+  const double sc = __hiloint2double((2046 - e) << 20, 0);     // 2^(1023 - e)
+  unscale = __hiloint2double(e << 20, 0);                       // 2^(e - 1023)
+  DF* A = reinterpret_cast<DF*>(scratch);
+  DF* B2 = A + m;
+  for (int i = t; i < m; i += kLThreads) {
+    const double al = sm.al[i] * sc, be = i + 1 < m ? sm.be[i] * sc : 0.0;
+    sm.al[i] = al;
+    sm.be[i] = be;
+    A[i] = make(al);
+    const DF b = make(be);
+    B2[i] = mul(b, b);
+    sm.fa[i] = (float)al;
+    sm.fb2[i] = (float)be;
+  }
+  __syncthreads();
+  // Gershgorin bounds in FP32 (entries of size <= 2, margins far above rounding)
+  float glo = 3.4e38f, ghi = -3.4e38f;
+  for (int i = t; i < m; i += kLThreads) {
+    const float r = (i > 0 ? fabsf(sm.fb2[i - 1]) : 0.f) + fabsf(sm.fb2[i]);
+    glo = fminf(glo, sm.fa[i] - r);
+    ghi = fmaxf(ghi, sm.fa[i] + r);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    glo = fminf(glo, __shfl_xor_sync(0xffffffffu, glo, o));
+    ghi = fmaxf(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
+  }
+  if (lane == 0) { sm.bnd[warp] = glo; sm.bnd[kLWarps + warp] = ghi; }
+  __syncthreads();
+  for (int w = 0; w < kLWarps; ++w) {
+    glo = fminf(glo, sm.bnd[w]);
+    ghi = fmaxf(ghi, sm.bnd[kLWarps + w]);
+  }
+  const float tn = fmaxf(fabsf(glo), fabsf(ghi));
+  glo -= 1e-5f * tn;
+  ghi += 1e-5f * tn;
+  __syncthreads();
+  for (int i = t; i < m; i += kLThreads) sm.fb2[i] = sm.fb2[i] * sm.fb2[i];
+  __syncthreads();
+  float flo = glo, fhi = ghi;
+  constexpr float kR = 1.f / (kLThreads + 1);
+  for (int it = 0; it < 4; ++it) {
+    if (!(fhi - flo > 2e-6f * fmaxf(fabsf(flo), fabsf(fhi)))) break;
+    const float pt = flo + (fhi - flo) * ((float)(t + 1) * kR);
+    const int f = first_thread(sm, sturm_below_f32(sm.fa, sm.fb2, m, pt) >= 1);
+    const float nlo = f == 0 ? flo : flo + (fhi - flo) * ((float)f * kR);
+    const float nhi = f == kLThreads ? fhi : flo + (fhi - flo) * ((float)(f + 1) * kR);
+    flo = nlo;
+    fhi = nhi;
+  }
+  // widen by the FP32 rounding of T, confirm in pairs (half of the CTA each)
+  DF lo = {flo - 1e-5f * tn, 0.f}, hi = {fhi + 1e-5f * tn, 0.f};
+  const int cnt = sturm_below(A, B2, m, t < kLThreads / 2 ? lo : hi);
+  if (!__syncthreads_and(t < kLThreads / 2 ? cnt == 0 : cnt >= 1)) {
+    lo = {glo, 0.f};
+    hi = {ghi, 0.f};
+  }
+  for (int it = 0; it < 8; ++it) {
+    const float w = sub(hi, lo).h;
+    if (!(w > 1e-14f * fmaxf(fabsf(lo.h), fabsf(hi.h)))) break;
+    const DF pt = add(lo, {w * ((float)(t + 1) * kR), 0.f});
+    const int f = first_thread(sm, sturm_below(A, B2, m, pt) >= 1);
+    const DF nlo = f == 0 ? lo : add(lo, {w * ((float)f * kR), 0.f});
+    const DF nhi = f == kLThreads ? hi : add(lo, {w * ((float)(f + 1) * kR), 0.f});
+    lo = nlo;
+    hi = nhi;
+  }
+  return to_double(add(lo, {0.5f * sub(hi, lo).h, 0.f}));
+}
+
+// The first m entries of the tridiagonal into sm.al and sm.be (whole CTA).
+__device__ __forceinline__ void load_tridiagonal(const LanczosArgs& a, LzSmem& sm, int m) {
+  __syncthreads();
+  for (int i = threadIdx.x; i < m; i += kLThreads) {
+    sm.al[i] = __ldcg(a.alpha + i);
+    sm.be[i] = __ldcg(a.beta + i);
+  }
+  __syncthreads();
+}
+
+// Convergence test of the tridiagonal of the steps so far (sm.al, sm.be: m
+// entries, shifted by -sigma; both are scaled on return): |beta_{m-1} y_{m-1}|
+// <= tol |theta + sigma| for its lowest eigenpair (theta, y) in pair
+// arithmetic.  (The end of a cycle recomputes the pair; a wrong early answer
+// costs a restart, not accuracy.)  scratch: 6 m doubles of shared memory.
+// Valid in thread 0.
+__device__ bool ritz_check_df(LzSmem& sm, double* scratch, int m, double sigma, double tol) {
+  const double blast = sm.be[m - 1];
+  double unscale;
+  const double th = lowest_value(sm, scratch, m, unscale);
+  if (threadIdx.x >= 32) return false;
+  double* z = sm.tri[0];
+  twisted_vector<ArithDF>(sm.al, sm.be, m, th, reinterpret_cast<tdf::DF*>(scratch), z);
+  double s = 0.0;
+  for (int i = threadIdx.x; i < m; i += 32) s = fma(z[i], z[i], s);
+  s = warp_sum(s);
+  return fabs(blast) * fabs(z[m - 1]) <= tol * fmax(fabs(th * unscale + sigma), 1e-300) * sqrt(s);
+}
+
+// Lowest eigenpair of the m x m tridiagonal (sm.al, sm.be; scaled on return) by
+// the calling CTA: y (m entries, unit norm), theta, residual |beta_{m-1}
+// y_{m-1}|.  The eigenvalue and a first vector in pair arithmetic, the
+// eigenvalue's FP64 digits as their Rayleigh quotient, and the vector again in
+// FP64: 45 k clocks of FP64 chain instead of 570 k for a multisection and two
+// rounds of inverse iteration in FP64 (m = 48).  For the mixed modes.
+__device__ void ritz_pair(LzSmem& sm, double* scratch, int m, double* y, double* theta, double* res) {
+  const double blast = sm.be[m - 1];
+  double unscale;
+  const double th0 = lowest_value(sm, scratch, m, unscale);
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  double* z = sm.tri[0];
+  twisted_vector<ArithDF>(sm.al, sm.be, m, th0, reinterpret_cast<tdf::DF*>(scratch), z);
+  // Rayleigh quotient of (T - th0) z, added to th0
+  double nn = 0.0, rq = 0.0;
+  for (int i = lane; i < m; i += 32) {
+    nn = fma(z[i], z[i], nn);
+    double tz = (sm.al[i] - th0) * z[i];
+    if (i + 1 < m) tz = fma(2.0 * sm.be[i], z[i + 1], tz);
+    rq = fma(z[i], tz, rq);
+  }
+  nn = warp_sum(nn);
+  rq = warp_sum(rq);
+  const double th = th0 + rq / nn;
+  twisted_vector<ArithD>(sm.al, sm.be, m, th, scratch, z);
+  double s = 0.0;
+  for (int i = lane; i < m; i += 32) s = fma(z[i], z[i], s);
+  const double inv = sqrt(warp_sum(s));
+  for (int i = lane; i < m; i += 32) y[i] = z[i] / inv;
+  if (lane == 0) {
+    *theta = th * unscale;
+    *res = fabs(blast * z[m - 1] / inv);
+  }
+}
+
+// The same in FP64 mode, all of whose result is FP64: bracketing in FP32,
+// 32-way FP64 multisection to 4e-16 and two rounds of inverse iteration.  A
+// count whose point lies 1e-13 |T| or more from the pair-accurate eigenvalue is
+// known without its Sturm sequence (26 k clocks in FP64; most rounds have no
+// other), so the result is that of the full multisection.
+__device__ void ritz_pair_f64(LzSmem& sm, const LanczosArgs& a, double* scratch, int m, double* y, double* theta,
+                              double* res) {
+  double unscale;
+  const double near = lowest_value(sm, scratch, m, unscale) * unscale;
+  load_tridiagonal(a, sm, m);    // (lowest_value scaled it)
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  const double *al = sm.al, *be = sm.be;
+  double* db2 = scratch;
+  double *x = scratch + m, *dd = x + m, *du = dd + m, *du2 = du + m, *rhs = du2 + m, *dl = rhs + m;
+  double glo = al[0], ghi = al[0];
+  for (int i = lane; i < m; i += 32) {
+    const double r = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i + 1 < m ? fabs(be[i]) : 0.0);
+    glo = fmin(glo, al[i] - r);
+    ghi = fmax(ghi, al[i] + r);
+    const double b2 = i + 1 < m ? be[i] * be[i] : 0.0;
+    db2[i] = b2;
+    sm.fa[i] = (float)al[i];
+    sm.fb2[i] = (float)b2;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
+    ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
+  }
+  __syncwarp();
+  const double tnorm = fmax(fabs(glo), fabs(ghi)), margin = 1e-13 * tnorm;
+  // whether an eigenvalue lies below p (all lanes call it)
+  auto below = [&](double p) {
+    bool r = p > near;
+    const bool close = !(fabs(p - near) > margin);
+    if (__any_sync(0xffffffffu, close)) {
+      const int cnt = sturm_below_f64(al, db2, m, p);
+      if (close) r = cnt >= 1;
+    }
+    return r;
+  };
+  float flo = (float)glo, fhi = (float)ghi;
+  for (int it = 0; it < 8; ++it) {
+    const float mag = fabsf(flo) > fabsf(fhi) ? fabsf(flo) : fabsf(fhi);
+    if (!(fhi - flo > 2e-6f * mag)) break;
+    constexpr float r33 = 1.f / 33.f;
+    const float pt = flo + (fhi - flo) * ((float)(lane + 1) * r33);
+    const unsigned bal = __ballot_sync(0xffffffffu, sturm_below_f32(sm.fa, sm.fb2, m, pt) >= 1);
+    const int f = bal ? __ffs(bal) - 1 : 32;
+    const float nlo = f == 0 ? flo : flo + (fhi - flo) * ((float)f * r33);
+    const float nhi = f == 32 ? fhi : flo + (fhi - flo) * ((float)(f + 1) * r33);
+    flo = nlo;
+    fhi = nhi;
+  }
+  double lo = (double)flo - 1e-5 * tnorm, hi = (double)fhi + 1e-5 * tnorm;
+  const bool b_lo = below(lo), b_hi = below(hi);
+  if (!__all_sync(0xffffffffu, !b_lo && b_hi)) { lo = glo; hi = ghi; }
+  for (int it = 0; it < 16; ++it) {
+    const double mag = fabs(lo) > fabs(hi) ? fabs(lo) : fabs(hi);
+    if (!(hi - lo > 4e-16 * mag)) break;
+    constexpr double r33 = 1.0 / 33.0;
+    const double pt = lo + (hi - lo) * ((double)(lane + 1) * r33);
+    const unsigned bal = __ballot_sync(0xffffffffu, below(pt));
+    const int f = bal ? __ffs(bal) - 1 : 32;
+    const double nlo = f == 0 ? lo : lo + (hi - lo) * ((double)f * r33);
+    const double nhi = f == 32 ? hi : lo + (hi - lo) * ((double)(f + 1) * r33);
+    lo = nlo;
+    hi = nhi;
+  }
+  const double th = 0.5 * (lo + hi);
+  // inverse iteration on (T - th I) x = x_prev: LU with partial pivoting of
+  // the tridiagonal, two rounds.  The elimination is one chain (lane 0, its
+  // running row in registers); rows are set up and scaled by all lanes.
+  const double x0 = 1.0 / sqrt((double)m);
+  for (int i = lane; i < m; i += 32) x[i] = x0;
+  const double eps = fmax(fabs(th), 1.0) * 1e-15;
+  for (int round = 0; round < 2; ++round) {
+    for (int i = lane; i < m; i += 32) {
+      dd[i] = al[i] - th;
+      du[i] = i + 1 < m ? be[i] : 0.0;
+      du2[i] = 0.0;
+      rhs[i] = x[i];
+      dl[i] = i + 1 < m ? be[i] : 0.0;
+    }
+    __syncwarp();
+    if (lane == 0) {
+      double cd = dd[0], cu = du[0], cr = rhs[0];   // row i: diagonal, first off-diagonal, right side
+      for (int i = 0; i + 1 < m; ++i) {
+        double nd = dd[i + 1], nu = du[i + 1], nr = rhs[i + 1];
+        const double l = dl[i];
+        if (fabs(cd) >= fabs(l)) {
+          if (cd == 0.0) cd = eps;
+          const double f = l / cd;
+          nd -= f * cu;
+          nr -= f * cr;
+          dd[i] = cd;
+          du[i] = cu;
+          rhs[i] = cr;
+        } else {
+          const double f = cd / l;
+          dd[i] = l;
+          du[i] = nd;
+          rhs[i] = nr;
+          nd = cu - f * nd;
+          if (i + 2 < m) { du2[i] = nu; nu = -f * nu; }
+          nr = cr - f * nr;
+        }
+        cd = nd;
+        cu = nu;
+        cr = nr;
+      }
+      if (cd == 0.0) cd = eps;
+      dd[m - 1] = cd;
+      du[m - 1] = cu;
+      rhs[m - 1] = cr;
+      double x1 = 0.0, x2 = 0.0, nrm = 0.0;
+      for (int i = m - 1; i >= 0; --i) {
+        double s = rhs[i];
+        if (i + 1 < m) s -= du[i] * x1;
+        if (i + 2 < m) s -= du2[i] * x2;
+        const double d = dd[i];
+        x2 = x1;
+        x1 = s / (fabs(d) < eps ? (d < 0 ? -eps : eps) : d);
+        x[i] = x1;
+      }
+      for (int i = 0; i < m; ++i) nrm += x[i] * x[i];
+      sm.bcast[3] = sqrt(nrm);
+    }
+    __syncwarp();
+    const double nrm = sm.bcast[3];
+    for (int i = lane; i < m; i += 32) x[i] /= nrm;
+    __syncwarp();
+  }
+  for (int i = lane; i < m; i += 32) y[i] = x[i];
+  if (lane == 0) {
+    *theta = th;
+    *res = fabs(be[m - 1] * x[m - 1]);
+  }
 }
 
 // Double-float matrix-vector products (mixed modes): matrices and vectors as
 // FP32 pairs (hi block of n floats, then lo block), tiles staged into the
 // shared arrays L and R reinterpreted as hi/lo float rows.
-using FRow = float[kLMaxC + 1];
-
-__device__ __forceinline__ FRow* frows(double (*d)[kLMaxC + 1], int half) {
-  return reinterpret_cast<FRow*>(&d[0][0]) + half * kLT;
-}
-
+// (pitch c + 1 floats; hi rows, then lo rows)
 // rows [r0, r0+8) of the pair matrix M (hi at M, lo at M + n)
-__device__ void stage_rows_p(double (*dst)[kLMaxC + 1], const float* M, long long n, int c,
-                             int r0) {
-  FRow* h = frows(dst, 0);
-  FRow* l = frows(dst, 1);
+__device__ void stage_rows_p(double* dst, const float* M, long long n, int c, int r0) {
+  float* h = reinterpret_cast<float*>(dst);
+  float* l = h + kLT * (c + 1);
   float vh[kLStage], vl[kLStage];
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
@@ -408,14 +685,13 @@ __device__ void stage_rows_p(double (*dst)[kLMaxC + 1], const float* M, long lon
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
     const int e = threadIdx.x + u * kLThreads, r = e / c, k = e - r * c;
-    if (e < kLT * c) { h[r][k] = vh[u]; l[r][k] = vl[u]; }
+    if (e < kLT * c) { h[r * (c + 1) + k] = vh[u]; l[r * (c + 1) + k] = vl[u]; }
   }
 }
 // columns [c0, c0+8) of M as rows: dst[j][k] = M[k][c0 + j]
-__device__ void stage_cols_p(double (*dst)[kLMaxC + 1], const float* M, long long n, int c,
-                             int c0) {
-  FRow* h = frows(dst, 0);
-  FRow* l = frows(dst, 1);
+__device__ void stage_cols_p(double* dst, const float* M, long long n, int c, int c0) {
+  float* h = reinterpret_cast<float*>(dst);
+  float* l = h + kLT * (c + 1);
   float vh[kLStage], vl[kLStage];
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
@@ -428,23 +704,24 @@ __device__ void stage_cols_p(double (*dst)[kLMaxC + 1], const float* M, long lon
 #pragma unroll
   for (int u = 0; u < kLStage; ++u) {
     const int e = threadIdx.x + u * kLThreads, k = e / kLT, j = e - k * kLT;
-    if (e < kLT * c) { h[j][k] = vh[u]; l[j][k] = vl[u]; }
+    if (e < kLT * c) { h[j * (c + 1) + k] = vh[u]; l[j * (c + 1) + k] = vl[u]; }
   }
 }
 
-__device__ __forceinline__ void tile_fma_p(LzSmem& sm, int c, float& a0h, float& a0l, float& a1h,
-                                           float& a1l) {
+__device__ __forceinline__ void tile_fma_p(const LzTiles& ts, int c, float& a0h, float& a0l,
+                                           float& a1h, float& a1l) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = lane >> 2, j = (lane & 3) * 2;
-  const FRow* Lh = frows(sm.L, 0);
-  const FRow* Ll = frows(sm.L, 1);
-  const FRow* Rh = frows(sm.R, 0);
-  const FRow* Rl = frows(sm.R, 1);
+  const int ld = c + 1;
+  const float* Lh = reinterpret_cast<const float*>(ts.L) + i * ld;
+  const float* Ll = Lh + kLT * ld;
+  const float* Rh = reinterpret_cast<const float*>(ts.R) + j * ld;
+  const float* Rl = Rh + kLT * ld;
   int cnt = 0;
   for (int k = warp; k < c; k += kLWarps) {
-    const float xh = Lh[i][k], xl = Ll[i][k];
-    pair_mac(xh, xl, Rh[j][k], Rl[j][k], a0h, a0l);
-    pair_mac(xh, xl, Rh[j + 1][k], Rl[j + 1][k], a1h, a1l);
+    const float xh = Lh[k], xl = Ll[k];
+    pair_mac(xh, xl, Rh[k], Rl[k], a0h, a0l);
+    pair_mac(xh, xl, Rh[ld + k], Rl[ld + k], a1h, a1l);
     if (++cnt == 8) {
       cnt = 0;
       pair_renorm(a0h, a0l);
@@ -460,7 +737,8 @@ __device__ __forceinline__ void tile_fma_p(LzSmem& sm, int c, float& a0h, float&
 __device__ void tile_store_p(LzSmem& sm, float a0h, float a0l, float a1h, float a1l, float* Cp,
                              double* Cd, long long n, int c, int i0, int j0,
                              const double* X = nullptr, double sigma = 0.0,
-                             const double* Xprev = nullptr, double beta = 0.0) {
+                             const double* Xprev = nullptr, double beta = 0.0,
+                             double* own_w = nullptr) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = lane >> 2, j = (lane & 3) * 2;
   float* rh = reinterpret_cast<float*>(&sm.red[0][0]);
@@ -482,35 +760,37 @@ __device__ void tile_store_p(LzSmem& sm, float a0h, float a0l, float a1h, float 
         if (sigma != 0.0) v = fma(-sigma, __ldcg(X + e), v);
         if (beta != 0.0) v = fma(-beta, __ldcg(Xprev + e), v);
         __stcg(Cd + e, v);
+        if (own_w) own_w[threadIdx.x] = v;
       }
     }
   }
   __syncthreads();
 }
 
-// Wide staging (double-float mode, c <= kLWideMaxC, c a multiple of 8): every
+// Wide staging (c <= kLWideMaxC, c a multiple of 8): every
 // operand tile of a matrix-vector phase is requested at once by 16-byte
 // asynchronous copies (cp.async.cg: L2 only, like the loads above) into
-// kLWideSlots slots of 16 rows of ldw = c + 4 floats (slots 0 and 1 reuse
-// sm.L and sm.R, the others are dynamic shared memory), so that a phase costs
+// kLWideSlots slots of 16 rows of ldw = c + 4 floats, so that a phase costs
 // one L2 latency instead of one per term.  A row tile holds rows [r0, r0+8)
 // of a pair matrix (hi rows 0-7, lo rows 8-15); a column tile holds columns
 // [c0, c0+8) untransposed (hi: c rows of 8 floats, then lo).  The products
-// below take the same operands in the same order as tile_fma_p, so both
-// stagings give the same bits.
+// below take the same operands in the same order as tile_fma_p and tile_fma, so
+// both stagings give the same bits.  In FP64 mode a slot holds 8 rows of c + 2
+// doubles (or a column tile of c rows of 8).
 constexpr int kLWideMaxC = 128;
 constexpr int kLWideSlots = 8;
 
 __host__ __device__ __forceinline__ int lz_wide_ld(int c) { return c + 4; }
+__host__ __device__ __forceinline__ int lz_slot_floats(int c) { return 2 * kLT * (c + 4); }
 
-size_t lz_wide_dyn_bytes(int c) {
-  return (size_t)(kLWideSlots - 2) * 2 * kLT * lz_wide_ld(c) * sizeof(float);
+// Doubles of the operand tiles: the wide slots, or L and R.
+__host__ __device__ __forceinline__ int lz_tile_doubles(int c, int wide) {
+  const int t = wide ? kLWideSlots * lz_slot_floats(c) / 2 : 2 * kLT * (c + 1);
+  return t > 8 * (kLMaxM + 2) ? t : 8 * (kLMaxM + 2);   // also the checks' scratch
 }
 
-__device__ __forceinline__ float* wide_slot(LzSmem& sm, float* dyn, int s, int ldw) {
-  if (s == 0) return reinterpret_cast<float*>(&sm.L[0][0]);
-  if (s == 1) return reinterpret_cast<float*>(&sm.R[0][0]);
-  return dyn + (long long)(s - 2) * 2 * kLT * ldw;
+__device__ __forceinline__ float* wide_slot(float* dyn, int s, int c) {
+  return dyn + s * lz_slot_floats(c);
 }
 
 __device__ __forceinline__ void cp_async16(float* dst, const float* src) {
@@ -578,6 +858,39 @@ __device__ __forceinline__ void wide_fma(const float* L, const float* R, bool rc
   pair_renorm(a1h, a1l);
 }
 
+// The same three for FP64 tiles (row pitch c + 2 doubles).
+__device__ void wide_rows_d(float* slot, const double* M, int c, int r0) {
+  double* dst = reinterpret_cast<double*>(slot);
+  const int q2 = c >> 1;
+  for (int q = threadIdx.x; q < kLT * q2; q += kLThreads) {
+    const int r = q / q2, k2 = (q - r * q2) << 1;
+    cp_async16(reinterpret_cast<float*>(dst + r * (c + 2) + k2),
+               reinterpret_cast<const float*>(M + (long long)(r0 + r) * c + k2));
+  }
+}
+__device__ void wide_cols_d(float* slot, const double* M, int c, int c0) {
+  double* dst = reinterpret_cast<double*>(slot);
+  for (int q = threadIdx.x; q < 4 * c; q += kLThreads) {
+    const int k = q >> 2, j2 = (q & 3) << 1;
+    cp_async16(reinterpret_cast<float*>(dst + k * kLT + j2),
+               reinterpret_cast<const float*>(M + (long long)k * c + c0 + j2));
+  }
+}
+__device__ __forceinline__ void wide_fma_d(const float* Ls, const float* Rs, bool rcol, int c,
+                                           double& a0, double& a1) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int i = lane >> 2, j = (lane & 3) * 2;
+  const double* L = reinterpret_cast<const double*>(Ls) + i * (c + 2);
+  const double* R = reinterpret_cast<const double*>(Rs) + (rcol ? j : j * (c + 2));
+  const int rk = rcol ? kLT : 1, rj = rcol ? 1 : c + 2;
+#pragma unroll 4
+  for (int k = warp; k < c; k += kLWarps) {
+    const double x = L[k];
+    a0 = fma(x, R[k * rk], a0);
+    a1 = fma(x, R[k * rk + rj], a1);
+  }
+}
+
 // FP64 value and its pair at index e of a vector (pair vector: hi at P, lo at P + n)
 __device__ __forceinline__ void store_both(double* D, float* P, long long n, long long e, double v) {
   __stcg(D + e, v);
@@ -626,8 +939,8 @@ __device__ double own_dot(LzSmem& sm, const double* a, const double* b, int nown
 // part[bid][nslot] = |w|^2 when nslot >= 0.  Warp w takes the vectors
 // 4w .. 4w+3, 4w+32 .. (their loads issued together); each sum runs over the
 // owned entries lane by lane, then a fixed butterfly.
-__device__ void own_projections(const LanczosArgs& a, double* part, int ldp, int j, int nslot,
-                                int nown, int bid, int G, int nt, int c, long long n) {
+__device__ void own_projections(const LanczosArgs& a, const LzOwn& own, double* part, int ldp, int j,
+                                int nslot, int nown, int bid, int G, int nt, int c, long long n) {
   constexpr int U = 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nv = j + 1 + (nslot >= 0 ? 1 : 0);
@@ -638,22 +951,55 @@ __device__ void own_projections(const LanczosArgs& a, double* part, int ldp, int
     for (int q = lane; q < nown; q += 32) {
       const long long e = own_index(q, bid, G, nt, c);
       if (e < 0) continue;
+      const double wv = own.wrow >= 0 ? own.p[own.wrow * own.pitch + q] : __ldcg(a.w + e);
       double bv[U];
+      if (own.n) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int i = i0 + u;
-        bv[u] = i < nv ? __ldcg((i > j ? a.w : a.basis + (long long)i * n) + e) : 0.0;
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u;
+          bv[u] = i < nv ? own.p[(i > j ? own.wrow : i) * own.pitch + q] : 0.0;
+        }
+      } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int i = i0 + u;
+          bv[u] = i < nv ? __ldcg((i > j ? a.w : a.basis + (long long)i * n) + e) : 0.0;
+        }
       }
-      const double wv = __ldcg(a.w + e);
 #pragma unroll
       for (int u = 0; u < U; ++u) s[u] = fma(bv[u], wv, s[u]);
     }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      for (int o = 16; o > 0; o >>= 1) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
-      const int i = i0 + u;
-      if (lane == 0 && i < nv) __stcg(part + (long long)bid * ldp + (i > j ? nslot : i), s[u]);
-    }
+    // the butterfly of every sum, four of them together: each exchange halves
+    // the number of values a lane holds (6 additions instead of 20 -- an FP64
+    // warp instruction takes 16 clocks of the SM -- in the same tree, so the
+    // same bits)
+    static_assert(U == 4, "four sums share a butterfly");
+    const bool h16 = lane & 16, h8 = lane & 8;
+    double r0 = h16 ? s[1] : s[0], r1 = h16 ? s[3] : s[2];
+    r0 += __shfl_xor_sync(0xffffffffu, h16 ? s[0] : s[1], 16);
+    r1 += __shfl_xor_sync(0xffffffffu, h16 ? s[2] : s[3], 16);
+    double r = h8 ? r1 : r0;
+    r += __shfl_xor_sync(0xffffffffu, h8 ? r0 : r1, 8);
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    const int i = i0 + (h8 ? 2 : 0) + (h16 ? 1 : 0);
+    if ((lane & 7) == 0 && i < nv) __stcg(part + (long long)bid * ldp + (i > j ? nslot : i), r);
+  }
+}
+
+// out[i] = the sum over the CTAs of their partial sums of coefficient i (i = nn:
+// at *out_n instead), in the order of cta_ordered_sum; warp by warp, so that a
+// small grid's CTA sums eight coefficients at a time.
+__device__ void sum_coefs(const double* part, int ldp, int nn, int nslot, int G, int bid, double* out,
+                          double* out_n) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int i = bid + G * warp; i <= nn; i += G * kLWarps) {
+    const double* x = part + (i == nn ? nslot : i);
+    double s = 0.0;
+    for (int q = lane; q < G; q += 32) s += __ldcg(x + (long long)q * ldp);
+    // (lanes without a CTA hold 0: their additions change nothing)
+    for (int o = 16; o > 0; o >>= 1)
+      if (o < G) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) __stcg(i == nn ? out_n : out + i, s);
   }
 }
 
@@ -664,13 +1010,13 @@ __device__ __forceinline__ void load_coefs(LzSmem& sm, const double* cf, int cnt
   __syncthreads();
 }
 
-// For every owned entry e: f(e, base[e] + sgn * sum_{i < cnt} sm.cf[i] basis_i[e])
-// (base may be null: 0).  S = 1, 2 or 4 threads share an entry, each summing
+// For every owned entry e (local index q): f(q, e, base[e] + sgn * sum_{i < cnt}
+// sm.cf[i] basis_i[e]) (base: w, or null: 0).  S = 1, 2 or 4 threads share an entry, each summing
 // the terms i = sub, sub + S, ... with eight loads in flight; the S partial
 // sums are added in a fixed order.
 template <typename Fn>
-__device__ void owned_combine(const LanczosArgs& a, const LzSmem& sm, int cnt, const double* base,
-                              double sgn, int nown, int bid, int G, int nt, int c, long long n,
+__device__ void owned_combine(const LanczosArgs& a, const LzSmem& sm, const LzOwn& own, int cnt,
+                              const double* base, double sgn, int nown, int bid, int G, int nt, int c, long long n,
                               Fn f) {
   const int S = nown >= kLThreads ? 1 : (nown > kLThreads / 4 ? 2 : 4);
   const int per = kLThreads / S, sub = threadIdx.x % S;
@@ -683,24 +1029,80 @@ __device__ void owned_combine(const LanczosArgs& a, const LzSmem& sm, int cnt, c
       for (; i + 7 * S < cnt; i += 8 * S) {
         double b[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) b[u] = __ldcg(a.basis + (long long)(i + u * S) * n + e);
+        for (int u = 0; u < 8; ++u)
+          b[u] = own.n ? own.p[(i + u * S) * own.pitch + q] : __ldcg(a.basis + (long long)(i + u * S) * n + e);
 #pragma unroll
         for (int u = 0; u < 8; ++u) s = fma(sm.cf[i + u * S], b[u], s);
       }
-      for (; i < cnt; i += S) s = fma(sm.cf[i], __ldcg(a.basis + (long long)i * n + e), s);
+      for (; i < cnt; i += S) s = fma(sm.cf[i], own.n ? own.p[i * own.pitch + q] : __ldcg(a.basis + (long long)i * n + e), s);
     }
     if (S >= 2) s += __shfl_down_sync(0xffffffffu, s, 1);
     if (S >= 4) s += __shfl_down_sync(0xffffffffu, s, 2);
-    if (sub == 0 && e >= 0) f(e, (base ? __ldcg(base + e) : 0.0) + sgn * s);
+    if (sub == 0 && e >= 0) {
+      const double bv = !base ? 0.0 : (own.wrow >= 0 ? own.p[own.wrow * own.pitch + q] : __ldcg(base + e));
+      f(q, e, bv + sgn * s);
+    }
   }
 }
 
-__global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs a) {
-  __shared__ LzSmem sm;
-  extern __shared__ __align__(16) float lz_dyn[];
+// Poll a word until test(v), at most `limit` times and not after *err was
+// raised, by thread 0; the word is returned to every thread (ok: whether the
+// wait succeeded).
+template <typename Test>
+__device__ unsigned lz_wait_word(LzSmem& sm, const unsigned* w, Test test, int* err, int limit, bool raise,
+                                 bool& ok) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned v = 0;
+    int good = 0;
+    for (int spins = 0; spins <= limit; ++spins) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(w) : "memory");
+      if (test(v)) { good = 1; break; }
+      if (*reinterpret_cast<volatile int*>(err)) break;
+      __nanosleep(64);
+    }
+    if (!good && raise) atomicOr(err, 4);
+    sm.ok = good;
+    sm.bcast[1] = __longlong_as_double((long long)v);
+  }
+  __syncthreads();
+  ok = sm.ok != 0;
+  const unsigned v = (unsigned)__double_as_longlong(sm.bcast[1]);
+  __syncthreads();
+  return v;
+}
+
+constexpr unsigned kLQuit = 0xFFFFFFFFu;
+
+// The extra CTA of a launch with a.extra: it runs the convergence checks of
+// the tridiagonal while the others take the next step.  A job (a.job[0]) is
+// number << 8 | m; its answer (a.job[1]) is number << 1 | passed.
+__device__ void lz_checker(const LanczosArgs& a, LzSmem& sm, double* dyn) {
+  unsigned seen = 0;
+  const int limit = max(a.max_spin, 1 << 23);   // between jobs it only idles
+  while (true) {
+    bool ok;
+    const unsigned v = lz_wait_word(sm, a.job, [&](unsigned w) { return w != seen; }, a.err, limit, false, ok);
+    if (!ok || v == kLQuit) return;
+    seen = v;
+    const int m = (int)(v & 0xFFu);
+    load_tridiagonal(a, sm, m);
+    {
+      const bool pass = ritz_check_df(sm, dyn, m, __ldcg(a.scal + 8), a.tol);
+      if (threadIdx.x == 0)
+        asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.job + 1), "r"((v >> 8) << 1 | (pass ? 1u : 0u)) : "memory");
+    }
+  }
+}
+
+__device__ __forceinline__ void lz_post(const LanczosArgs& a, unsigned v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.job), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, float* lz_dyn, int G) {
   const int c = a.c, K = a.K, m = a.m;
   const long long n = (long long)c * c;
-  const int G = gridDim.x, bid = blockIdx.x;
+  const int bid = blockIdx.x;
   const int nt = (c + kLT - 1) / kLT;
   const int ntiles = nt * nt;
   const int nown = (bid < ntiles ? (ntiles - bid + G - 1) / G : 0) * 64;
@@ -711,8 +1113,21 @@ __global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs
   unsigned target = 0;
 
   const bool df = a.df != 0;
-  const bool wide = df && a.wide != 0;
+  const bool wide = a.wide != 0;
   const int ldw = lz_wide_ld(c);
+  double* dynd = reinterpret_cast<double*>(lz_dyn);
+  const LzTiles ts{dynd, dynd + kLT * (c + 1), c + 1};
+  LzOwn own;
+  own.p = dynd + lz_tile_doubles(c, a.wide);
+  own.pitch = a.own_pitch;
+  own.n = a.ncache;
+  own.wrow = a.ncache > 0 ? a.ncache : -1;
+  unsigned jobs = 0;          // checks posted to the extra CTA
+  bool ok = true;
+  const int wlimit = max(a.max_spin > 0 ? a.max_spin : kLMaxSpin, 1 << 16);
+  auto answer = [&](bool& good) {
+    return lz_wait_word(sm, a.job + 1, [&](unsigned w) { return (w >> 1) == jobs; }, a.err, wlimit, true, good);
+  };
   float* bp0 = df ? a.bp : nullptr;          // pairs of basis_0
   // start: the operators as pairs (double-float mode), Vprev = V, basis_0 = V / |V|
   if (df) {
@@ -738,26 +1153,29 @@ __global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs
     const double s = own_dot(sm, a.V, a.V, nown, bid, G, nt, c);
     if (threadIdx.x == 0) __stcg(part + (long long)bid * ldp, s);
   }
-  if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+  if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
   double inv = 1.0 / sqrt(cta_ordered_sum(sm, part, G, ldp));
   for (int q = threadIdx.x; q < nown; q += kLThreads) {
     const long long e = own_index(q, bid, G, nt, c);
-    if (e >= 0) store_both(a.basis, bp0, n, e, __ldcg(a.V + e) * inv);
+    if (e >= 0) {
+      const double v = __ldcg(a.V + e) * inv;
+      store_both(a.basis, bp0, n, e, v);
+      own.set(0, q, v);
+    }
   }
-  if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+  if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
   const float* s0p = a.s0p;
   const float* s1p = a.s1 == a.s0 ? a.s0p : a.s1p;
 
   int conv = 0;
   for (int cyc = 0; cyc < a.restarts && !conv; ++cyc) {
     int tdim = 0;
-    double beta_prev = 0.0;
+    int due = -1, due_m = 0;    // step whose end reads the pending check's answer, its size
     // Steps j >= 1 run on H - sigma I with sigma = alpha_0, the Rayleigh
     // quotient of the start vector (the same Krylov space; the tridiagonal is
     // shifted by -sigma, its first entry 0).  Without the shift |w|^2 ~ E^2
     // would dwarf beta_j^2 and every step would need the second
     // Gram-Schmidt pass.
-    double sigma = 0.0;
     // Step j >= 1 also subtracts, while w is stored, the two recurrence terms
     // it knows: sigma_j x_j with sigma_j = alpha_{j-1} of H (the previous
     // step's diagonal entry, close to this one's) and beta_{j-1} x_{j-1}.  The
@@ -766,32 +1184,44 @@ __global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs
     // the second Gram-Schmidt pass with its two grid barriers is skipped.  The
     // tridiagonal keeps the single shift sigma: its entry j is
     // c_j + sigma_j - sigma.
-    double alpha_prev_h = 0.0;
     for (int j = 0; j < m; ++j) {
       const double* x = a.basis + (long long)j * n;
-      const double sigma_j = j == 0 ? 0.0 : (j == 1 ? sigma : alpha_prev_h);
+      const double sigma_j = j == 0 ? 0.0 : (j == 1 ? sm.sigma : sm.alpha_prev_h);
       const double* xprev = j > 0 ? x - n : nullptr;
-      const double beta_j1 = j > 0 ? beta_prev : 0.0;
+      const double beta_j1 = j > 0 ? sm.beta_prev : 0.0;
       // phase A: Y_b = Op_b x for the 2K operators A_k0, B_k0 (stored after o_0)
       const float* xp = df ? a.bp + 2 * (long long)j * n : nullptr;
       // wide staging: all 2K products of a tile by its CTA, the columns of x
-      // staged once, the operator rows two at a time
+      // staged once, the operator rows up to seven at a time
       for (int t = bid; t < ntiles && wide; t += G) {
         const int i0 = (t / nt) * kLT, j0 = (t % nt) * kLT;
-        for (int b0 = 0; b0 < 2 * K; b0 += 2) {
-          const int nb = min(2, 2 * K - b0);
-          if (b0 == 0) wide_cols(wide_slot(sm, lz_dyn, 0, ldw), xp, n, c, j0);
-          for (int u = 0; u < nb; ++u)
-            wide_rows(wide_slot(sm, lz_dyn, 1 + u, ldw), s0p + 2 * (long long)(1 + b0 + u) * n, n,
-                      c, i0, ldw);
+        constexpr int kRows = kLWideSlots - 1;
+        for (int b0 = 0; b0 < 2 * K; b0 += kRows) {
+          const int nb = min(kRows, 2 * K - b0);
+          if (df) {
+            if (b0 == 0) wide_cols(wide_slot(lz_dyn, 0, c), xp, n, c, j0);
+            for (int u = 0; u < nb; ++u)
+              wide_rows(wide_slot(lz_dyn, 1 + u, c), s0p + 2 * (long long)(1 + b0 + u) * n, n, c,
+                        i0, ldw);
+          } else {
+            if (b0 == 0) wide_cols_d(wide_slot(lz_dyn, 0, c), x, c, j0);
+            for (int u = 0; u < nb; ++u)
+              wide_rows_d(wide_slot(lz_dyn, 1 + u, c), a.s0 + (long long)(1 + b0 + u) * n, c, i0);
+          }
           cp_async_wait_all();
           __syncthreads();
           for (int u = 0; u < nb; ++u) {
-            float a0h = 0.f, a0l = 0.f, a1h = 0.f, a1l = 0.f;
-            wide_fma(wide_slot(sm, lz_dyn, 1 + u, ldw), wide_slot(sm, lz_dyn, 0, ldw), true, c, ldw,
-                     a0h, a0l, a1h, a1l);
-            tile_store_p(sm, a0h, a0l, a1h, a1l, a.Yp + 2 * (long long)(b0 + u) * n, nullptr, n, c,
-                         i0, j0);
+            if (df) {
+              float a0h = 0.f, a0l = 0.f, a1h = 0.f, a1l = 0.f;
+              wide_fma(wide_slot(lz_dyn, 1 + u, c), wide_slot(lz_dyn, 0, c), true, c, ldw, a0h, a0l,
+                       a1h, a1l);
+              tile_store_p(sm, a0h, a0l, a1h, a1l, a.Yp + 2 * (long long)(b0 + u) * n, nullptr, n,
+                           c, i0, j0);
+            } else {
+              double a0 = 0.0, a1 = 0.0;
+              wide_fma_d(wide_slot(lz_dyn, 1 + u, c), wide_slot(lz_dyn, 0, c), true, c, a0, a1);
+              tile_store(sm, a0, a1, a.Y + (long long)(b0 + u) * n, c, i0, j0);
+            }
           }
         }
       }
@@ -799,219 +1229,279 @@ __global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs
         const int b = it / ntiles, t = it % ntiles;
         const int i0 = (t / nt) * kLT, j0 = (t % nt) * kLT;
         if (df) {
-          stage_rows_p(sm.L, s0p + 2 * (long long)(1 + b) * n, n, c, i0);
-          stage_cols_p(sm.R, xp, n, c, j0);
+          stage_rows_p(ts.L, s0p + 2 * (long long)(1 + b) * n, n, c, i0);
+          stage_cols_p(ts.R, xp, n, c, j0);
           __syncthreads();
           float a0h = 0.f, a0l = 0.f, a1h = 0.f, a1l = 0.f;
-          tile_fma_p(sm, c, a0h, a0l, a1h, a1l);
+          tile_fma_p(ts, c, a0h, a0l, a1h, a1l);
           tile_store_p(sm, a0h, a0l, a1h, a1l, a.Yp + 2 * (long long)b * n, nullptr, n, c, i0, j0);
           continue;
         }
-        stage_rows(sm.L, a.s0 + (long long)(1 + b) * n, c, i0, 1.0);
-        stage_cols(sm.R, x, c, j0, 1.0);
+        stage_rows(ts.L, a.s0 + (long long)(1 + b) * n, c, i0);
+        stage_cols(ts.R, x, c, j0);
         __syncthreads();
         double a0 = 0.0, a1 = 0.0;
-        tile_fma(sm, c, a0, a1);
+        tile_fma(ts, c, a0, a1);
         tile_store(sm, a0, a1, a.Y + (long long)b * n, c, i0, j0);
       }
-      if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+      if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
       // phase B: w = o_0 x + x o_1^T + sum_k Y_k B_k1^T + Y_{K+k} A_k1^T on the
       // owned tiles, then their projections on basis_0..j and |w|^2
       // wide staging: the operand tiles of up to four terms in one round
       for (int t = bid; t < ntiles && wide; t += G) {
         const int i0 = (t / nt) * kLT, j0 = (t % nt) * kLT;
         float a0h = 0.f, a0l = 0.f, a1h = 0.f, a1l = 0.f;
+        double a0 = 0.0, a1 = 0.0;
         const int nterms = 2 + 2 * K;
         for (int t0 = 0; t0 < nterms; t0 += kLWideSlots / 2) {
           const int tn = min(kLWideSlots / 2, nterms - t0);
           for (int u = 0; u < tn; ++u) {
             const int term = t0 + u;
-            float* Ls = wide_slot(sm, lz_dyn, 2 * u, ldw);
-            float* Rs = wide_slot(sm, lz_dyn, 2 * u + 1, ldw);
-            if (term == 0) {
-              wide_rows(Ls, s0p, n, c, i0, ldw);
-              wide_cols(Rs, xp, n, c, j0);
-            } else if (term == 1) {
-              wide_rows(Ls, xp, n, c, i0, ldw);
-              wide_rows(Rs, s1p, n, c, j0, ldw);
+            float* Ls = wide_slot(lz_dyn, 2 * u, c);
+            float* Rs = wide_slot(lz_dyn, 2 * u + 1, c);
+            const int q = term - 2;            // Y_q with q < K: B_{q,1}; else A_{q-K,1}
+            const long long rop = q < K ? (long long)(1 + K + q) : (long long)(1 + q - K);
+            if (df) {
+              if (term == 0) {
+                wide_rows(Ls, s0p, n, c, i0, ldw);
+                wide_cols(Rs, xp, n, c, j0);
+              } else if (term == 1) {
+                wide_rows(Ls, xp, n, c, i0, ldw);
+                wide_rows(Rs, s1p, n, c, j0, ldw);
+              } else {
+                wide_rows(Ls, a.Yp + 2 * (long long)q * n, n, c, i0, ldw);
+                wide_rows(Rs, s1p + 2 * rop * n, n, c, j0, ldw);
+              }
             } else {
-              const int q = term - 2;          // Y_q with q < K: B_{q,1}; else A_{q-K,1}
-              const long long rop = q < K ? (long long)(1 + K + q) : (long long)(1 + q - K);
-              wide_rows(Ls, a.Yp + 2 * (long long)q * n, n, c, i0, ldw);
-              wide_rows(Rs, s1p + 2 * rop * n, n, c, j0, ldw);
+              if (term == 0) {
+                wide_rows_d(Ls, a.s0, c, i0);
+                wide_cols_d(Rs, x, c, j0);
+              } else if (term == 1) {
+                wide_rows_d(Ls, x, c, i0);
+                wide_rows_d(Rs, a.s1, c, j0);
+              } else {
+                wide_rows_d(Ls, a.Y + (long long)q * n, c, i0);
+                wide_rows_d(Rs, a.s1 + rop * n, c, j0);
+              }
             }
           }
           cp_async_wait_all();
           __syncthreads();
-          for (int u = 0; u < tn; ++u)
-            wide_fma(wide_slot(sm, lz_dyn, 2 * u, ldw), wide_slot(sm, lz_dyn, 2 * u + 1, ldw),
-                     t0 + u == 0, c, ldw, a0h, a0l, a1h, a1l);
+          for (int u = 0; u < tn; ++u) {
+            if (df)
+              wide_fma(wide_slot(lz_dyn, 2 * u, c), wide_slot(lz_dyn, 2 * u + 1, c), t0 + u == 0, c,
+                       ldw, a0h, a0l, a1h, a1l);
+            else
+              wide_fma_d(wide_slot(lz_dyn, 2 * u, c), wide_slot(lz_dyn, 2 * u + 1, c), t0 + u == 0,
+                         c, a0, a1);
+          }
           __syncthreads();
         }
-        tile_store_p(sm, a0h, a0l, a1h, a1l, nullptr, a.w, n, c, i0, j0, x, sigma_j, xprev,
-                     beta_j1);
+        double* ow = own.wrow >= 0 ? own.p + own.wrow * own.pitch + ((t - bid) / G) * 64 : nullptr;
+        if (df)
+          tile_store_p(sm, a0h, a0l, a1h, a1l, nullptr, a.w, n, c, i0, j0, x, sigma_j, xprev,
+                       beta_j1, ow);
+        else
+          tile_store(sm, a0, a1, a.w, c, i0, j0, x, sigma_j, xprev, beta_j1, ow);
       }
       for (int t = bid; t < ntiles && df && !wide; t += G) {
         const int i0 = (t / nt) * kLT, j0 = (t % nt) * kLT;
         float a0h = 0.f, a0l = 0.f, a1h = 0.f, a1l = 0.f;
         for (int term = 0; term < 2 + 2 * K; ++term) {
           if (term == 0) {
-            stage_rows_p(sm.L, s0p, n, c, i0);
-            stage_cols_p(sm.R, xp, n, c, j0);
+            stage_rows_p(ts.L, s0p, n, c, i0);
+            stage_cols_p(ts.R, xp, n, c, j0);
           } else if (term == 1) {
-            stage_rows_p(sm.L, xp, n, c, i0);
-            stage_rows_p(sm.R, s1p, n, c, j0);
+            stage_rows_p(ts.L, xp, n, c, i0);
+            stage_rows_p(ts.R, s1p, n, c, j0);
           } else {
             const int q = term - 2;            // Y_q with q < K: B_{q,1}; else A_{q-K,1}
             const long long rop = q < K ? (long long)(1 + K + q) : (long long)(1 + q - K);
-            stage_rows_p(sm.L, a.Yp + 2 * (long long)q * n, n, c, i0);
-            stage_rows_p(sm.R, s1p + 2 * rop * n, n, c, j0);
+            stage_rows_p(ts.L, a.Yp + 2 * (long long)q * n, n, c, i0);
+            stage_rows_p(ts.R, s1p + 2 * rop * n, n, c, j0);
           }
           __syncthreads();
-          tile_fma_p(sm, c, a0h, a0l, a1h, a1l);
+          tile_fma_p(ts, c, a0h, a0l, a1h, a1l);
           __syncthreads();
         }
-        tile_store_p(sm, a0h, a0l, a1h, a1l, nullptr, a.w, n, c, i0, j0, x, sigma_j, xprev,
-                     beta_j1);
+        tile_store_p(sm, a0h, a0l, a1h, a1l, nullptr, a.w, n, c, i0, j0, x, sigma_j, xprev, beta_j1,
+                     own.wrow >= 0 ? own.p + own.wrow * own.pitch + ((t - bid) / G) * 64 : nullptr);
       }
-      for (int t = bid; t < ntiles && !df; t += G) {
+      for (int t = bid; t < ntiles && !df && !wide; t += G) {
         const int i0 = (t / nt) * kLT, j0 = (t % nt) * kLT;
         double a0 = 0.0, a1 = 0.0;
         for (int term = 0; term < 2 + 2 * K; ++term) {
           if (term == 0) {
-            stage_rows(sm.L, a.s0, c, i0, 1.0);
-            stage_cols(sm.R, x, c, j0, 1.0);
+            stage_rows(ts.L, a.s0, c, i0);
+            stage_cols(ts.R, x, c, j0);
           } else if (term == 1) {
-            stage_rows(sm.L, x, c, i0, 1.0);
-            stage_rows(sm.R, a.s1, c, j0, 1.0);
+            stage_rows(ts.L, x, c, i0);
+            stage_rows(ts.R, a.s1, c, j0);
           } else {
             const int q = term - 2;            // Y_q with q < K: B_{q,1}; else A_{q-K,1}
             const long long rop = q < K ? (long long)(1 + K + q) * n : (long long)(1 + q - K) * n;
-            stage_rows(sm.L, a.Y + (long long)q * n, c, i0, 1.0);
-            stage_rows(sm.R, a.s1 + rop, c, j0, 1.0);
+            stage_rows(ts.L, a.Y + (long long)q * n, c, i0);
+            stage_rows(ts.R, a.s1 + rop, c, j0);
           }
           __syncthreads();
-          tile_fma(sm, c, a0, a1);
+          tile_fma(ts, c, a0, a1);
           __syncthreads();
         }
-        tile_store(sm, a0, a1, a.w, c, i0, j0, x, sigma_j, xprev, beta_j1);
+        tile_store(sm, a0, a1, a.w, c, i0, j0, x, sigma_j, xprev, beta_j1,
+                   own.wrow >= 0 ? own.p + own.wrow * own.pitch + ((t - bid) / G) * 64 : nullptr);
       }
-      own_projections(a, part, ldp, j, nslot, nown, bid, G, nt, c, n);
-      if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
-      // coefficients of the first Gram-Schmidt pass and |w|^2 (one CTA each)
-      for (int i = bid; i <= j + 1; i += G) {
-        const double s = cta_ordered_sum(sm, part + (i > j ? nslot : i), G, ldp);
-        if (threadIdx.x == 0) __stcg(i > j ? wn2 : a.coef + i, s);
+      own_projections(a, own, part, ldp, j, nslot, nown, bid, G, nt, c, n);
+      if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+      // coefficients of the first Gram-Schmidt pass and |w|^2 (one warp each)
+      sum_coefs(part, ldp, j + 1, nslot, G, bid, a.coef, wn2);
+      if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+      if (j == due) {
+        // the answer to the check posted kLLag steps ago, which ran meanwhile:
+        // when it passed, the cycle ends with that step's tridiagonal and the
+        // steps since are dropped (they only extended the basis)
+        const unsigned v = answer(ok);
+        if (!ok) return;
+        due = -1;
+        if (v & 1u) {
+          tdim = due_m;
+          break;
+        }
       }
-      if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
       // |w - sum c_i b_i|^2 = |w|^2 - sum c_i^2 for orthonormal b_i; when at
       // least a quarter of |w|^2 remains, one pass is accurate to rounding
       // (the second pass of "twice is enough" is needed only after heavy
       // cancellation), and the norm needs no further reduction
-      const double w2 = __ldcg(wn2);
       load_coefs(sm, a.coef, j + 1);
-      // sum of c_i^2 in a fixed order (lane-strided, then a butterfly): the
-      // same value, and the same one-pass decision, in every CTA
+      // warp 0 takes the step's scalars (the FP64 square root and division are
+      // long: eight warps repeating them cost 4 k clocks a step): the sum of
+      // c_i^2 in a fixed order (lane-strided, then a butterfly), so the same
+      // one-pass decision in every CTA, then alpha_j, beta_j, 1 / beta_j
+      const bool check = (j + 1) % kLCheck == 0 && j + 1 < m;
+      auto scalars = [&](double alpha_j, double beta_j) {   // lane 0
+        if (j == 0) {
+          sm.sigma = alpha_j;
+          alpha_j = 0.0;
+        } else {
+          alpha_j += sigma_j - sm.sigma;
+        }
+        const double ah = alpha_j + sm.sigma;
+        sm.alpha_prev_h = ah;
+        const bool brk = !(beta_j > 1e-12 * fmax(fabs(ah) + beta_j1, 1e-300));
+        sm.brk = brk;
+        if (bid == 0) {
+          __stcg(a.alpha + j, alpha_j);
+          __stcg(a.beta + j, brk ? 0.0 : beta_j);
+          if (check && a.extra && !brk) {
+            __stcg(a.scal + 8, sm.sigma);
+            lz_post(a, (jobs + 1) << 8 | (unsigned)(j + 1));
+          }
+        }
+        sm.beta_prev = beta_j;
+        sm.inv = 1.0 / beta_j;
+      };
       if (threadIdx.x < 32) {
+        const double w2 = __ldcg(wn2);
         double t = 0.0;
         for (int i = threadIdx.x; i <= j; i += 32) t = fma(sm.cf[i], sm.cf[i], t);
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        if (threadIdx.x == 0) sm.bcast[2] = t;
+        const bool one = w2 - t > 0.25 * w2;
+        if (threadIdx.x == 0) {
+          sm.one_pass = one;
+          if (one) scalars(sm.cf[j], sqrt(w2 - t));
+        }
       }
       __syncthreads();
-      const double c2 = sm.bcast[2];
-      const bool one_pass = w2 - c2 > 0.25 * w2;
-      double alpha_j = sm.cf[j];
-      double beta_j;
-      if (one_pass) {
-        beta_j = sqrt(w2 - c2);
-      } else {
+      if (!sm.one_pass) {
         // second pass: w1 = w - sum c_i b_i, then d_i = <b_i, w1> and |w1|^2 in
         // one reduction; |w1 - sum d_i b_i|^2 = |w1|^2 - sum d_i^2 (the d_i are
         // rounding-sized), and basis_{j+1} below subtracts sum d_i b_i
-        owned_combine(a, sm, j + 1, a.w, -1.0, nown, bid, G, nt, c, n,
-                      [&](long long e, double v) { __stcg(a.w + e, v); });
+        const double alpha1 = sm.cf[j];
+        owned_combine(a, sm, own, j + 1, a.w, -1.0, nown, bid, G, nt, c, n,
+                      [&](int q, long long e, double v) {
+                        __stcg(a.w + e, v);
+                        if (own.wrow >= 0) own.p[own.wrow * own.pitch + q] = v;
+                      });
         __syncthreads();
-        own_projections(a, part, ldp, j, nslot, nown, bid, G, nt, c, n);
-        if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
-        for (int i = bid; i <= j + 1; i += G) {
-          const double s = cta_ordered_sum(sm, part + (i > j ? nslot : i), G, ldp);
-          if (threadIdx.x == 0) __stcg(a.coef + ldp + i, s);
-        }
-        if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+        own_projections(a, own, part, ldp, j, nslot, nown, bid, G, nt, c, n);
+        if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+        sum_coefs(part, ldp, j + 1, nslot, G, bid, a.coef + ldp, a.coef + ldp + j + 1);
+        if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
         load_coefs(sm, a.coef + ldp, j + 2);
         if (threadIdx.x < 32) {
           double t = 0.0;
           for (int i = threadIdx.x; i <= j; i += 32) t = fma(sm.cf[i], sm.cf[i], t);
           for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-          if (threadIdx.x == 0) sm.bcast[2] = t;
+          if (threadIdx.x == 0) scalars(alpha1 + sm.cf[j], sqrt(fmax(sm.cf[j + 1] - t, 0.0)));
         }
         __syncthreads();
-        alpha_j += sm.cf[j];
-        beta_j = sqrt(fmax(sm.cf[j + 1] - sm.bcast[2], 0.0));
       }
-      if (j == 0) {
-        sigma = alpha_j;
-        alpha_j = 0.0;
-      } else {
-        alpha_j += sigma_j - sigma;
-      }
-      alpha_prev_h = alpha_j + sigma;
+      // every kLCheck steps the tridiagonal so far is tested for convergence
+      // (pair arithmetic): by the extra CTA during the next kLLag steps, or by
+      // CTA 0 while the others wait
+      const bool breakdown = sm.brk != 0;
       tdim = j + 1;
-      const bool breakdown = !(beta_j > 1e-12 * fmax(fabs(alpha_j + sigma) + beta_prev, 1e-300));
-      if (bid == 0 && threadIdx.x == 0) {
-        a.alpha[j] = alpha_j;
-        a.beta[j] = breakdown ? 0.0 : beta_j;
+      if (breakdown) {
+        if (due >= 0) {
+          const unsigned v = answer(ok);
+          if (!ok) return;
+          if (v & 1u) tdim = due_m;
+        }
+        break;
       }
-      if (breakdown) break;
-      beta_prev = beta_j;
+      if (check && a.extra) {
+        ++jobs;
+        due = min(j + kLLag, m - 1);
+        due_m = j + 1;
+      }
       // basis_{j+1} = (w - sum c_i b_i) / beta_j, or (w1 - sum d_i b_i) / beta_j
-      inv = 1.0 / beta_j;
+      const double binv = sm.inv;
       double* nb = a.basis + (long long)(j + 1) * n;
       float* nbp = df ? a.bp + 2 * (long long)(j + 1) * n : nullptr;
       // (sm.cf holds the c_i of the one-pass path or the d_i of the second pass)
-      owned_combine(a, sm, j + 1, a.w, -1.0, nown, bid, G, nt, c, n,
-                    [&](long long e, double v) { store_both(nb, nbp, n, e, v * inv); });
-      // every kLCheck steps CTA 0 tests the tridiagonal so far (pair
-      // arithmetic); the cycle ends early once its Ritz pair passes the
-      // convergence test
-      const bool check = (j + 1) % kLCheck == 0 && j + 1 < m;
-      if (check && bid == 0) {
-        __syncthreads();
-        if (threadIdx.x < 32) {
-          const bool ok = ritz_check_df(sm, a.alpha, a.beta, j + 1, sigma, a.tol);
-          if (threadIdx.x == 0) __stcg(a.scal + 3, ok ? 1.0 : 0.0);
-        }
+      owned_combine(a, sm, own, j + 1, a.w, -1.0, nown, bid, G, nt, c, n,
+                    [&](int q, long long e, double v) {
+                      const double x1 = v * binv;
+                      store_both(nb, nbp, n, e, x1);
+                      own.set(j + 1, q, x1);
+                    });
+      // (without the extra CTA: CTA 0's check, while the others wait)
+      const bool inline_check = check && !a.extra;
+      if (inline_check && bid == 0) {
+        load_tridiagonal(a, sm, j + 1);
+        const bool pass = ritz_check_df(sm, dynd, j + 1, sm.sigma, a.tol);
+        if (threadIdx.x == 0) __stcg(a.scal + 3, pass ? 1.0 : 0.0);
         __syncthreads();
       }
-      if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
-      if (check && __ldcg(a.scal + 3) != 0.0) break;
+      if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+      if (inline_check && __ldcg(a.scal + 3) != 0.0) break;
     }
     // Ritz pair of the tridiagonal (CTA 0), then V = sum_i y_i basis_i
-    if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+    if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
     if (bid == 0) {
-      ritz_pair(sm, a.alpha, a.beta, tdim, a.y, a.scal + 1, a.scal + 2);
+      load_tridiagonal(a, sm, tdim);
+      if (df) ritz_pair(sm, dynd, tdim, a.y, a.scal + 1, a.scal + 2);
+      else ritz_pair_f64(sm, a, dynd, tdim, a.y, a.scal + 1, a.scal + 2);
       __syncthreads();
       if (threadIdx.x == 0) {
         // Ritz value of H: the tridiagonal's plus the shift
-        const double theta = *(volatile double*)(a.scal + 1) + sigma;
+        const double theta = *(volatile double*)(a.scal + 1) + sm.sigma;
         a.scal[1] = theta;
         a.flags[1] = tdim;
         a.flags[0] = *(volatile double*)(a.scal + 2) <= a.tol * fmax(fabs(theta), 1e-300);
         __threadfence();
       }
     }
-    if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+    if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
     conv = __ldcg(a.flags);
     load_coefs(sm, a.y, tdim);
-    owned_combine(a, sm, tdim, nullptr, 1.0, nown, bid, G, nt, c, n,
-                  [&](long long e, double v) { __stcg(a.V + e, v); });
+    owned_combine(a, sm, own, tdim, nullptr, 1.0, nown, bid, G, nt, c, n,
+                  [&](int, long long e, double v) { __stcg(a.V + e, v); });
     __syncthreads();
     {
       const double s = own_dot(sm, a.V, a.V, nown, bid, G, nt, c);
       if (threadIdx.x == 0) __stcg(part + (long long)bid * ldp, s);
     }
-    if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+    if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
     inv = 1.0 / sqrt(cta_ordered_sum(sm, part, G, ldp));
     for (int q = threadIdx.x; q < nown; q += kLThreads) {
       const long long e = own_index(q, bid, G, nt, c);
@@ -1019,21 +1509,37 @@ __global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs
       const double t = __ldcg(a.V + e) * inv;
       __stcg(a.V + e, t);
       store_both(a.basis, bp0, n, e, t);
+      own.set(0, q, t);
     }
-    if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+    if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
   }
   // sign: <V, Vprev> >= 0
   {
     const double s = own_dot(sm, a.V, a.Vprev, nown, bid, G, nt, c);
     if (threadIdx.x == 0) __stcg(part + (long long)bid * ldp + 1, s);
   }
-  if (!lz_barrier(sm, a.bar, target, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+  if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
   if (cta_ordered_sum(sm, part + 1, G, ldp) < 0.0)
     for (int q = threadIdx.x; q < nown; q += kLThreads) {
       const long long e = own_index(q, bid, G, nt, c);
       if (e >= 0) __stcg(a.V + e, -__ldcg(a.V + e));
     }
 }
+
+__global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs a) {
+  __shared__ LzSmem sm;
+  extern __shared__ __align__(16) float lz_dyn[];
+  const int G = (int)gridDim.x - (a.extra ? 1 : 0);
+  if ((int)blockIdx.x == G) {
+    lz_checker(a, sm, reinterpret_cast<double*>(lz_dyn));
+    return;
+  }
+  lanczos_body(a, sm, lz_dyn, G);
+  if (a.extra && blockIdx.x == 0 && threadIdx.x == 0) lz_post(a, kLQuit);
+}
+
+// Dynamic shared memory of a CTA at most (two CTAs per SM).
+constexpr int kLMaxDyn = 96 * 1024;
 
 struct LzGrid {
   int sms = 0, per_sm = 0;
@@ -1049,8 +1555,7 @@ int lanczos_grid_cap() {
   if (!g.sms) {
     int sms = 0, occ = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    // (with the wide staging's dynamic shared memory at its largest)
-    const int dyn = (int)lz_wide_dyn_bytes(kLWideMaxC);
+    const int dyn = kLMaxDyn;
     if (cudaFuncSetAttribute(lanczos_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) !=
         cudaSuccess)
       return 0;
@@ -1076,17 +1581,26 @@ int lanczos_grid(int c, int grid_share) {
   return (int)std::max<long long>(1, std::min<long long>(std::min(cap, kLMaxGrid), n / 64));
 }
 
-int lanczos_launch(const LanczosArgs& a0, int grid, cudaStream_t s) {
+int lanczos_launch(const LanczosArgs& a0, int grid, int grid_share, cudaStream_t s) {
   if (!lanczos_supported(a0.c, a0.m) || grid < 1 || grid > kLMaxGrid) return -1;
   // the grid cap also sets the kernel's dynamic shared-memory limit
   if (lanczos_grid_cap() <= 0) return -1;
   LanczosArgs a = a0;
-  a.wide = a.df != 0 && a.c <= kLWideMaxC && a.c % 8 == 0 ? 1 : 0;
-  cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s);
+  a.wide = a.c <= kLWideMaxC && a.c % 8 == 0 ? 1 : 0;
+  // shared-memory copies of the CTA's entries of the basis vectors, if all fit
+  const int nt = (a.c + kLT - 1) / kLT;
+  const int tiles = lz_tile_doubles(a.c, a.wide);
+  a.own_pitch = (nt * nt + grid - 1) / grid * 64 + 8;
+  a.ncache = a.m + 1 <= (kLMaxDyn / 8 - tiles) / a.own_pitch - 1 ? a.m + 1 : 0;
+  // the checks run in a CTA of their own when one more is co-resident
+  a.extra = grid + 1 <= lanczos_grid_cap() / std::max(1, grid_share) ? 1 : 0;
+  const size_t dyn = 8 * ((size_t)tiles + (a.ncache > 0 ? (size_t)(a.ncache + 1) * a.own_pitch : 0));
+  a.job = a.bar + 1;
+  cudaMemsetAsync(a.bar, 0, 3 * sizeof(unsigned), s);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = dim3(grid + a.extra);
   cfg.blockDim = dim3(kLThreads);
-  cfg.dynamicSmemBytes = a.wide ? lz_wide_dyn_bytes(a.c) : 0;
+  cfg.dynamicSmemBytes = dyn;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;

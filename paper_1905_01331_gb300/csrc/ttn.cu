@@ -744,7 +744,8 @@ void top_solve(ttn_ctx* h, Instance& I, double* energy_out) {
       a.flags = h->iflags + 6;
       a.c = c; a.K = I.K; a.m = m; a.restarts = h->opt.lanczos_restarts;
       a.tol = lanczos_tolerance(h);
-      a.bar = reinterpret_cast<unsigned*>(h->iflags + 5);
+      // (three words of the composition's counters, idle now)
+      a.bar = reinterpret_cast<unsigned*>(h->iflags + 8);
       a.err = h->iflags + 4;
       a.max_spin = h->opt.wait_polls;
       a.df = h->opt.prec != 0 && h->opt.double_float;
@@ -752,14 +753,15 @@ void top_solve(ttn_ctx* h, Instance& I, double* energy_out) {
       a.s1p = a.s0p + 2 * (ll)(1 + 2 * I.K) * n;
       a.bp = reinterpret_cast<float*>(h->lz_bp);
       a.Yp = reinterpret_cast<float*>(h->lz_Yp);
-      const int grid = lanczos_grid(c, h->profiling ? 1 : (int)h->lanes.size());
+      const int share = h->profiling ? 1 : (int)h->lanes.size();
+      const int grid = lanczos_grid(c, share);
       cudaEvent_t ev[2];
       if (h->profiling) {
         cudaEventCreate(&ev[0]);
         cudaEventCreate(&ev[1]);
         cudaEventRecord(ev[0], h->stream);
       }
-      const int nl = grid > 0 ? lanczos_launch(a, grid, h->stream) : -1;
+      const int nl = grid > 0 ? lanczos_launch(a, grid, share, h->stream) : -1;
       if (nl < 0) h->compose_refused = true;
       else h->launches += nl;
       if (h->profiling) {
