@@ -133,8 +133,8 @@ typedef struct {
                                the FP32 pipes; 0: FP64 */
   int tc_engine;            /* tensor-core products: 0 (default) the TMA-fed,
                                warp-specialised kernel wherever the operand
-                               layouts allow it (FP32, K or MN index contiguous;
-                               TF32 modes), else the thread-staged kernel;
+                               layouts allow it (FP32, K or MN index contiguous),
+                               else the thread-staged kernel;
                                1: the thread-staged kernel for every product */
   int wait_polls;           /* polls of a grid-barrier wait in the persistent
                                kernels before it expires and the sweep reports

@@ -129,8 +129,8 @@ void gemm_oz_init();
 // Tensor-core path (gemm_tc.cu).
 int gemm_tc_launch(const GemmDesc& d, cudaStream_t stream);
 bool gemm_tc_supported(const GemmDesc& d);
-// The TMA-fed kernel can run this product (TF32 modes, FP32 operands with a
-// contiguous K or MN index, aligned strides).
+// The TMA-fed kernel can run this product (FP32 operands with a contiguous K or
+// MN index, aligned strides; BF16 modes: K a multiple of 64).
 bool gemm_tma_eligible(const GemmDesc& d);
 int tc_pick_splits(const GemmDesc& d);
 void gemm_tc_init();

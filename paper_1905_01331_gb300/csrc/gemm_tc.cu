@@ -53,6 +53,12 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr) {
   return d;
 }
 
+// K-major, 64-byte swizzle: rows of 64 bytes, 8-row atoms every 512 bytes.
+__device__ __forceinline__ uint64_t smem_desc64(uint32_t saddr) {
+  return static_cast<uint64_t>((saddr >> 4) & 0x3FFF) | (1ull << 16) |
+         (static_cast<uint64_t>(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
+}
+
 // Instruction descriptor: D = F32, A/B format fmt (2 = TF32, 1 = BF16), both
 // K-major, N >> 3 at bit 17, M >> 4 at bit 24.
 __host__ __device__ constexpr uint32_t instr_desc(uint32_t fmt, int M, int N) {
@@ -695,14 +701,17 @@ __global__ void splitk_reduce_tc(const GemmDesc d) {
 
 
 // ---------------------------------------------------------------------------
-// TMA-fed, warp-specialised variant for the TF32 modes with FP32 operands
-// whose K index or MN index is contiguous (every full-layer product of the
-// sweep).  Per CTA one 128 x BN output tile and a ring of S stages; a stage
+// TMA-fed, warp-specialised variant for FP32 operands whose K index or MN index
+// is contiguous (every full-layer product of the sweep).  Per CTA one 128 x BN output tile and a ring of S stages; a stage
 // holds the raw FP32 tiles of A (128 x 32) and B (BN x 32), loaded by TMA
 // (SWIZZLE_128B: the K-major canonical layout of the MMA; an MN-contiguous
 // operand arrives as 32 x 32 boxes and is transposed), converted in place to
 // TF32 heads by four converter warps, which also write the tails of the
-// split form; one thread issues the tcgen05.mma of the stage and commits its
+// split form (BF16 modes: heads and tails as separate tiles of half the size
+// after the raw ones, 64-byte swizzle; the thread-staged kernel took 615 us for
+// the mean product of a chi = 256 Heisenberg sweep, this one 270, in the same
+// order of MMAs per K tile: same bits); one thread issues the tcgen05.mma of the
+// stage and commits its
 // completion to the stage's "empty" barrier, which frees it for the next TMA.
 //   warp 0: TMA producer (one thread)       warp 1: TMEM owner, MMA issuer
 //   warps 2-5: converters, then the epilogue (TMEM lanes 32 (w % 4) ..)
@@ -884,6 +893,58 @@ __device__ __forceinline__ void store_row16(const GemmDesc& d, int b, int b0, in
     if (n + j < d.N) store_out(d, cb + static_cast<long long>(n + j) * d.sc_n, __uint_as_float(r[j]), af, bf);
 }
 
+// BF16 modes: eight consecutive K values of row r (chunk c of four) as heads
+// and tails in rows of 64 bytes with the 64-byte swizzle.
+template <bool kSplit>
+__device__ __forceinline__ void store_bf16(uint8_t* hi, uint8_t* lo, int r, int c, const float* x) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const __nv_bfloat162 hh = __floats2bfloat162_rn(x[2 * q], x[2 * q + 1]);
+    h[q] = *reinterpret_cast<const uint32_t*>(&hh);
+    if constexpr (kSplit) {
+      const __nv_bfloat162 ll =
+          __floats2bfloat162_rn(x[2 * q] - __uint_as_float(h[q] << 16),
+                                x[2 * q + 1] - __uint_as_float(h[q] & 0xFFFF0000u));
+      l[q] = *reinterpret_cast<const uint32_t*>(&ll);
+    }
+  }
+  const int off = r * 64 + ((c ^ ((r >> 1) & 3)) << 4);
+  *reinterpret_cast<uint4*>(hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
+  if constexpr (kSplit) *reinterpret_cast<uint4*>(lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+// Raw FP32 tile of ROWS rows x 32 K values (either TMA layout) -> BF16 tiles.
+template <bool kSplit, int ROWS>
+__device__ __forceinline__ void convert_bf16(const uint8_t* raw, bool mn, uint8_t* hi, uint8_t* lo, int ct) {
+  if (!mn) {
+#pragma unroll 2
+    for (int i = ct; i < ROWS * 4; i += kTConv) {
+      const int r = i >> 2, c = i & 3;
+      float x[8];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(raw + r * 128 + (((2 * c + q) ^ (r & 7)) << 4));
+        x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
+      }
+      store_bf16<kSplit>(hi, lo, r, c, x);
+    }
+  } else if (ct < ROWS) {
+    const int j = ct >> 5, c = (ct & 31) >> 2, e = ct & 3;
+    const uint8_t* box = raw + 4096 * j;
+#pragma unroll
+    for (int kc = 0; kc < 4; ++kc) {
+      float x[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int k = 8 * kc + q;
+        x[q] = *reinterpret_cast<const float*>(box + 128 * k + ((c ^ (k & 7)) << 4) + 4 * e);
+      }
+      store_bf16<kSplit>(hi, lo, ct, kc, x);
+    }
+  }
+}
+
 // Sixteen accumulator columns of the warp's 32 rows.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
   asm volatile(
@@ -895,7 +956,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-template <bool kSplit, int BN, int kRing>
+template <bool kBF16, bool kSplit, int BN, int kRing>
 __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
     gemm_tma_kernel(const GemmDesc d, const __grid_constant__ TmaParams tp) {
   pdl_wait();
@@ -903,9 +964,11 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
   constexpr int kA = kBM * 128;                     // raw A tile: 128 rows x 32 FP32
   constexpr int kB = BN * 128;
   constexpr int kHi = kA + kB;                      // raw tiles, TF32 heads after conversion
-  constexpr int kStageBytes = (kSplit ? 2 : 1) * kHi;
+  // TF32: heads in place of the raw tiles, tails after them; BF16: heads, then
+  // tails, after the raw tiles (half of their size each)
+  constexpr int kStageBytes = kBF16 ? kHi + (kSplit ? 2 : 1) * (kHi / 2) : (kSplit ? 2 : 1) * kHi;
   constexpr int S = kRing / kStageBytes < 8 ? kRing / kStageBytes : 8;
-  constexpr uint32_t kIdesc = instr_desc(2u, kBM, BN);
+  constexpr uint32_t kIdesc = instr_desc(kBF16 ? 1u : 2u, kBM, BN);
   static_assert(S >= 2, "stage ring");
   static_assert(BN == 64 || BN == 128, "tile width");
 
@@ -925,9 +988,12 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
   const int b0 = b % d.B0, b1 = b / d.B0;
   const int split_id = blockIdx.z;
   const int m0 = tm * kBM, n0 = tn * BN;
-  const int t_lo = static_cast<int>(static_cast<long long>(tp.total_tiles) * split_id / d.splits);
+  // (a split is a whole number of K tiles: 32 values, in the BF16 modes 64, two
+  // stages, as in the thread-staged kernel)
+  constexpr int kUnit = kBF16 ? 2 : 1;
+  const int t_lo = kUnit * static_cast<int>(static_cast<long long>(tp.total_tiles / kUnit) * split_id / d.splits);
   const int t_hi =
-      static_cast<int>(static_cast<long long>(tp.total_tiles) * (split_id + 1) / d.splits);
+      kUnit * static_cast<int>(static_cast<long long>(tp.total_tiles / kUnit) * (split_id + 1) / d.splits);
   const int nk = t_hi - t_lo;
   const int nacc = tp.nacc;
   const uint32_t ncols = nacc <= 1 ? BN : (nacc == 2 ? 2 * BN : 4 * BN);   // TMEM columns
@@ -1008,15 +1074,15 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
     if (lane == 0) {
       // ---- MMA issuer ----
       bool ok = true;
-      // accumulator q takes the K tiles [nk q / nacc, nk (q + 1) / nacc)
-      int q = 0, q_end = nacc > 1 ? static_cast<int>(static_cast<long long>(nk) / nacc) : nk, q_begin = 0;
+      // accumulator q takes the q-th of nacc parts of the K tiles
+      int q = 0, q_end = nacc > 1 ? kUnit * (nk / kUnit / nacc) : nk, q_begin = 0;
       uint32_t dcol = tmem;
       for (int kt = 0; kt < nk; ++kt) {
         const int s = kt % S, u = kt / S;
         if (kt == q_end) {
           ++q;
           q_begin = kt;
-          q_end = static_cast<int>(static_cast<long long>(nk) * (q + 1) / nacc);
+          q_end = kUnit * static_cast<int>(static_cast<long long>(nk / kUnit) * (q + 1) / nacc);
           dcol += BN;
         }
         if (!mbar_wait_ab(&conv_bar[s], u & 1, abort_v)) { ok = false; break; }
@@ -1024,6 +1090,21 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
         const uint32_t a_hi = smem_u32(smem + s * kStageBytes);
         const uint32_t b_hi = a_hi + kA;
         const uint32_t a_lo = a_hi + kHi, b_lo = a_lo + kA;
+        if constexpr (kBF16) {
+          const uint32_t ah = a_hi + kHi, bh = ah + kA / 2, al = ah + kHi / 2, bl = al + kA / 2;
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const uint32_t off = j * 32;   // 16 BF16 values of K per instruction
+            const uint32_t acc = (kt > q_begin || j > 0) ? 1u : 0u;
+            if constexpr (kSplit) {
+              mma<true>(dcol, smem_desc64(al + off), smem_desc64(bh + off), kIdesc, acc);
+              mma<true>(dcol, smem_desc64(ah + off), smem_desc64(bl + off), kIdesc, 1u);
+              mma<true>(dcol, smem_desc64(ah + off), smem_desc64(bh + off), kIdesc, 1u);
+            } else {
+              mma<true>(dcol, smem_desc64(ah + off), smem_desc64(bh + off), kIdesc, acc);
+            }
+          }
+        } else
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
           const uint32_t off = j * 32;   // 8 TF32 values of K per instruction
@@ -1060,10 +1141,16 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
         // all converter threads take the same decision (their named barriers follow)
         if (!conv_vote(mbar_wait_ab(&full_bar[s], u & 1, abort_v))) { ok = false; break; }
         uint8_t* st = smem + s * kStageBytes;
-        if (amn) convert_mnmajor<kSplit, kBM>(st, st + kHi, ct);
-        else convert_kmajor<kSplit, kBM>(st, st + kHi, ct);
-        if (bmn) convert_mnmajor<kSplit, BN>(st + kA, st + kHi + kA, ct);
-        else convert_kmajor<kSplit, BN>(st + kA, st + kHi + kA, ct);
+        if constexpr (kBF16) {
+          uint8_t* hi = st + kHi;
+          convert_bf16<kSplit, kBM>(st, amn, hi, hi + kHi / 2, ct);
+          convert_bf16<kSplit, BN>(st + kA, bmn, hi + kA / 2, hi + kHi / 2 + kA / 2, ct);
+        } else {
+          if (amn) convert_mnmajor<kSplit, kBM>(st, st + kHi, ct);
+          else convert_kmajor<kSplit, kBM>(st, st + kHi, ct);
+          if (bmn) convert_mnmajor<kSplit, BN>(st + kA, st + kHi + kA, ct);
+          else convert_kmajor<kSplit, BN>(st + kA, st + kHi + kA, ct);
+        }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(&conv_bar[s]);
         ++kt;
@@ -1123,9 +1210,9 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols));
 }
 
-template <bool kSplit, int BN, int kRing>
+template <bool kBF16, bool kSplit, int BN, int kRing>
 void tma_configure() {
-  cudaFuncSetAttribute(gemm_tma_kernel<kSplit, BN, kRing>,
+  cudaFuncSetAttribute(gemm_tma_kernel<kBF16, kSplit, BN, kRing>,
                        cudaFuncAttributeMaxDynamicSharedMemorySize, kRing + 1024);
 }
 
@@ -1167,10 +1254,14 @@ bool tma_operand_ok(const Operand& o, int k0_log2) {
 }
 
 bool tma_eligible(const GemmDesc& d) {
-  if (d.prec != 1 && d.prec != 2) return false;
-  for (int g = 0; g < d.ngroups; ++g)
+  if (d.prec < 1 || d.prec > 4) return false;
+  for (int g = 0; g < d.ngroups; ++g) {
     if (!tma_operand_ok(d.g[g].a, d.g[g].k0_log2) || !tma_operand_ok(d.g[g].b, d.g[g].k0_log2))
       return false;
+    // BF16: whole K tiles of 64, so that the K ranges of the splits are those of
+    // the thread-staged kernel
+    if (d.prec >= 3 && d.g[g].K % 64 != 0) return false;
+  }
   return d.ngroups > 0 && d.ngroups <= kMaxGroups;
 }
 
@@ -1216,7 +1307,7 @@ bool encode_operand(const Operand& o, int k0_log2, int K, int rows, int B0, int 
 
 // Returns 1 (launched) or 0 (a tensor map could not be encoded: the caller
 // runs the thread-staged kernel instead).
-template <bool kSplit, int BN, int kRing>
+template <bool kBF16, bool kSplit, int BN, int kRing>
 int launch_tma(const GemmDesc& d, cudaStream_t s, int in_cta) {
   static TmaParams tp;   // host staging of the kernel parameter (launch copies it)
   static std::mutex mu;
@@ -1234,22 +1325,23 @@ int launch_tma(const GemmDesc& d, cudaStream_t s, int in_cta) {
   tp.err = d.err;
   const int tiles = ((d.M + kBM - 1) / kBM) * ((d.N + BN - 1) / BN);
   dim3 grid(tiles, d.B0 * d.B1, d.splits);
-  launch_k(gemm_tma_kernel<kSplit, BN, kRing>, grid, kTThreads, kRing + 1024, s, d, tp);
+  launch_k(gemm_tma_kernel<kBF16, kSplit, BN, kRing>, grid, kTThreads, kRing + 1024, s, d, tp);
   return 1;
 }
 
 // d.occ == 2 selects the 96 KB ring (two CTAs per SM) where a stage still
 // fits twice: BN = 64 in both forms, BN = 128 without the split.
+template <bool kBF16>
 int launch_tma_bn(const GemmDesc& d, cudaStream_t s, int in_cta) {
-  const bool split = d.prec == 2;
+  const bool split = d.prec == 2 || d.prec == 4;
   const int bn = (d.tile == 64 || d.tile == 128) ? d.tile : tma_bn(d.N);
   const bool two = d.occ == 2 && !(split && bn == 128);
   if (bn == 128) {
-    if (split) return launch_tma<true, 128, kTSmem>(d, s, in_cta);
-    return two ? launch_tma<false, 128, kTSmem2>(d, s, in_cta) : launch_tma<false, 128, kTSmem>(d, s, in_cta);
+    if (split) return launch_tma<kBF16, true, 128, kTSmem>(d, s, in_cta);
+    return two ? launch_tma<kBF16, false, 128, kTSmem2>(d, s, in_cta) : launch_tma<kBF16, false, 128, kTSmem>(d, s, in_cta);
   }
-  if (split) return two ? launch_tma<true, 64, kTSmem2>(d, s, in_cta) : launch_tma<true, 64, kTSmem>(d, s, in_cta);
-  return two ? launch_tma<false, 64, kTSmem2>(d, s, in_cta) : launch_tma<false, 64, kTSmem>(d, s, in_cta);
+  if (split) return two ? launch_tma<kBF16, true, 64, kTSmem2>(d, s, in_cta) : launch_tma<kBF16, true, 64, kTSmem>(d, s, in_cta);
+  return two ? launch_tma<kBF16, false, 64, kTSmem2>(d, s, in_cta) : launch_tma<kBF16, false, 64, kTSmem>(d, s, in_cta);
 }
 
 // K splits that one CTA sums itself: a product whose output tiles alone fill
@@ -1259,7 +1351,7 @@ int launch_tma_bn(const GemmDesc& d, cudaStream_t s, int in_cta) {
 // product (same bits).  Measured for 128 x 16384 outputs, K = 128, two splits:
 // the reduction alone took 100 us, the product 18 us.
 int tma_in_cta(const GemmDesc& d) {
-  if (d.splits < 2 || d.splits > 4 || tc_total_tiles(d, 32) < d.splits) return 1;
+  if (d.splits < 2 || d.splits > 4 || tc_total_tiles(d, d.prec >= 3 ? 64 : 32) < d.splits) return 1;
   const int bn = (d.tile == 64 || d.tile == 128) ? d.tile : tma_bn(d.N);
   const long long base = static_cast<long long>((d.M + kBM - 1) / kBM) * ((d.N + bn - 1) / bn) * d.B0 * d.B1;
   if (2 * base < device_sm_count()) return 1;
@@ -1299,10 +1391,14 @@ int launch_tc_bn(const GemmDesc& d, cudaStream_t s, int* err) {
 }  // namespace
 
 void gemm_tc_init() {
-  tma_configure<false, 64, kTSmem>(); tma_configure<false, 128, kTSmem>();
-  tma_configure<true, 64, kTSmem>(); tma_configure<true, 128, kTSmem>();
-  tma_configure<false, 64, kTSmem2>(); tma_configure<false, 128, kTSmem2>();
-  tma_configure<true, 64, kTSmem2>();
+  tma_configure<false, false, 64, kTSmem>(); tma_configure<false, false, 128, kTSmem>();
+  tma_configure<false, true, 64, kTSmem>(); tma_configure<false, true, 128, kTSmem>();
+  tma_configure<false, false, 64, kTSmem2>(); tma_configure<false, false, 128, kTSmem2>();
+  tma_configure<false, true, 64, kTSmem2>();
+  tma_configure<true, false, 64, kTSmem>(); tma_configure<true, false, 128, kTSmem>();
+  tma_configure<true, true, 64, kTSmem>(); tma_configure<true, true, 128, kTSmem>();
+  tma_configure<true, false, 64, kTSmem2>(); tma_configure<true, false, 128, kTSmem2>();
+  tma_configure<true, true, 64, kTSmem2>();
   tc_configure<false, false, 32>(); tc_configure<false, false, 64>(); tc_configure<false, false, 128>();
   tc_configure<false, true, 32>(); tc_configure<false, true, 64>(); tc_configure<false, true, 128>();
   tc_configure<true, false, 32>(); tc_configure<true, false, 64>(); tc_configure<true, false, 128>();
@@ -1321,7 +1417,7 @@ bool gemm_tc_supported(const GemmDesc& d) {
 
 int tc_pick_splits(const GemmDesc& d) {
   const int BK = (d.prec == 3 || d.prec == 4) ? 64 : 32;
-  const int bn = (d.tc_engine != 1 && tma_eligible(d)) ? tma_bn(d.N) : tc_bn(d.N);
+  const int bn = (d.tc_engine != 1 && tma_eligible(d) && d.prec < 3) ? tma_bn(d.N) : tc_bn(d.N);
   const long long base = static_cast<long long>((d.M + kBM - 1) / kBM) *
                          ((d.N + bn - 1) / bn) * d.B0 * d.B1;
   const int kt = tc_total_tiles(d, BK);
@@ -1337,7 +1433,7 @@ int gemm_tc_launch(const GemmDesc& d, cudaStream_t s) {
     const int in_cta = tma_in_cta(d);
     GemmDesc e = d;
     if (in_cta > 1) e.splits = 1;
-    n = launch_tma_bn(e, s, in_cta);
+    n = d.prec >= 3 ? launch_tma_bn<true>(e, s, in_cta) : launch_tma_bn<false>(e, s, in_cta);
     if (n && in_cta > 1) return n;
   }
   if (n == 0)

@@ -383,7 +383,7 @@ Tuned tune_product(ttn_ctx* h, const GemmDesc& d0) {
       if (gemm_tma_eligible(d0)) {
         for (int bn : {64, 128})
           for (int occ : {1, 2})
-            if (!(occ == 2 && bn == 128 && d0.prec == 2)) cands.push_back({0, bn, s, occ});
+            if (!(occ == 2 && bn == 128 && (d0.prec == 2 || d0.prec == 4))) cands.push_back({0, bn, s, occ});
       }
       for (int bn : {32, 64, 128})
         if (bn <= std::max(32, d0.N)) cands.push_back({1, bn, s, 0});
