@@ -79,47 +79,86 @@ __global__ void __launch_bounds__(kThreads) gemm_f64_kernel(const GemmDesc d, in
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = 0.0;
 
-  int t_global = 0;
-  for (int g = 0; g < d.ngroups && t_global < t_hi; ++g) {
+  // K tiles of this split, over all groups: the next one is loaded into
+  // registers while the current one is multiplied
+  constexpr int LA = BM * kBK / kThreads, LB = BN * kBK / kThreads;
+  double ra[LA], rb[LB];
+  int g = 0, t = 0;
+  {
+    int skip = t_lo;
+    while (g < d.ngroups) {
+      const int nt = (d.g[g].K + kBK - 1) / kBK;
+      if (skip < nt) break;
+      skip -= nt;
+      ++g;
+    }
+    t = skip;
+  }
+  auto load = [&]() {
     const Group& G = d.g[g];
-    const int nt = (G.K + kBK - 1) / kBK;
-    if (t_global + nt <= t_lo) { t_global += nt; continue; }
     const long long abase = b0 * G.a.s_b0 + (long long)b1 * G.a.s_b1;
     const long long bbase = b0 * G.b.s_b0 + (long long)b1 * G.b.s_b1;
-    const int first = max(0, t_lo - t_global), last = min(nt, t_hi - t_global);
-    const bool a_kfast = (G.a.s_k0 == 1);
-    const bool b_kfast = (G.b.s_k0 == 1);
-    for (int t = first; t < last; ++t) {
-      const int kb = t * kBK;
-      // stage A tile (BM x kBK) and B tile (kBK x BN)
-      for (int e = threadIdx.x; e < BM * kBK; e += kThreads) {
-        int mi, ki;
-        if (a_kfast) { ki = e % kBK; mi = e / kBK; } else { mi = e % BM; ki = e / BM; }
-        const int m = m0 + mi, k = kb + ki;
-        As[ki][mi] = (m < d.M && k < G.K) ? ld_operand(G.a, G.k0_log2, abase, m, k) : 0.0;
-      }
-      for (int e = threadIdx.x; e < BN * kBK; e += kThreads) {
-        int ni, ki;
-        if (b_kfast) { ki = e % kBK; ni = e / kBK; } else { ni = e % BN; ki = e / BN; }
-        const int n = n0 + ni, k = kb + ki;
-        Bs[ki][ni] = (n < d.N && k < G.K) ? ld_operand(G.b, G.k0_log2, bbase, n, k) : 0.0;
-      }
-      __syncthreads();
+    const bool a_kfast = (G.a.s_k0 == 1), b_kfast = (G.b.s_k0 == 1);
+    const int kb = t * kBK;
 #pragma unroll
-      for (int kk = 0; kk < kBK; ++kk) {
-        double av[TM], bv[TN];
-#pragma unroll
-        for (int i = 0; i < TM; ++i) av[i] = As[kk][ty + 16 * i];
-#pragma unroll
-        for (int j = 0; j < TN; ++j) bv[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-        for (int i = 0; i < TM; ++i)
-#pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
-      }
-      __syncthreads();
+    for (int i = 0; i < LA; ++i) {
+      const int e = threadIdx.x + i * kThreads;
+      const int mi = a_kfast ? e / kBK : e % BM, ki = a_kfast ? e % kBK : e / BM;
+      const int m = m0 + mi, k = kb + ki;
+      ra[i] = (m < d.M && k < G.K) ? ld_operand(G.a, G.k0_log2, abase, m, k) : 0.0;
     }
-    t_global += nt;
+#pragma unroll
+    for (int i = 0; i < LB; ++i) {
+      const int e = threadIdx.x + i * kThreads;
+      const int ni = b_kfast ? e / kBK : e % BN, ki = b_kfast ? e % kBK : e / BN;
+      const int n = n0 + ni, k = kb + ki;
+      rb[i] = (n < d.N && k < G.K) ? ld_operand(G.b, G.k0_log2, bbase, n, k) : 0.0;
+    }
+  };
+  // a warp without a row inside the matrix has nothing to add (an FP64 warp
+  // instruction takes 16 clocks of the SM's two FP64 units, used or not)
+  const bool rows_in = m0 + (threadIdx.x / 32) * 2 < d.M;
+  if (t_lo < t_hi) load();
+  for (int it = t_lo; it < t_hi; ++it) {
+    const Group& G = d.g[g];
+    const bool a_kfast = (G.a.s_k0 == 1), b_kfast = (G.b.s_k0 == 1);
+    const int kmax = min(kBK, G.K - t * kBK);
+#pragma unroll
+    for (int i = 0; i < LA; ++i) {
+      const int e = threadIdx.x + i * kThreads;
+      if (a_kfast) As[e % kBK][e / kBK] = ra[i];
+      else As[e / BM][e % BM] = ra[i];
+    }
+#pragma unroll
+    for (int i = 0; i < LB; ++i) {
+      const int e = threadIdx.x + i * kThreads;
+      if (b_kfast) Bs[e % kBK][e / kBK] = rb[i];
+      else Bs[e / BN][e % BN] = rb[i];
+    }
+    __syncthreads();
+    ++t;
+    if (t * kBK >= G.K) { ++g; t = 0; }
+    if (it + 1 < t_hi) load();
+    auto step = [&](int kk) {
+      double av[TM], bv[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) av[i] = As[kk][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < TN; ++j) bv[j] = Bs[kk][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) acc[i][j] = fma(av[i], bv[j], acc[i][j]);
+    };
+    if (rows_in) {
+      if (kmax == kBK) {
+#pragma unroll
+        for (int kk = 0; kk < kBK; ++kk) step(kk);
+      } else {
+        for (int kk = 0; kk < kmax; ++kk) step(kk);
+      }
+    }
+    __syncthreads();
   }
 
   if (d.splits == 1) {
@@ -241,8 +280,9 @@ int device_sm_count() {
   return cache[dev];
 }
 
-// 64 x 64 tiles when they alone give two waves, else 32 x 32 or 16 x 16.
-int f64_tile(const GemmDesc& d) {
+// 64 x 64 tiles when they alone give two waves, else 32 x 32 or 16 x 16: the
+// tile that the split count is computed for.
+int f64_split_tile(const GemmDesc& d) {
   if (d.tile == 16 || d.tile == 32 || d.tile == 64) return d.tile;
   const long long b = (long long)d.B0 * d.B1;
   const long long wave2 = 2LL * device_sm_count();
@@ -254,10 +294,21 @@ int f64_tile(const GemmDesc& d) {
   return 16;
 }
 
+// The tile that runs: 16 x 16 where the tiles above leave SMs idle.  Every SM has
+// two FP64 units, so a product of few tiles is bound by the FMAs of one tile;
+// a smaller one changes no sum (the K order and the splits stay).  A product of
+// 1024 x 32 by 32 took 14.6 us as 32 tiles on 32 SMs.
+int f64_tile(const GemmDesc& d) {
+  const int t = f64_split_tile(d);
+  if (d.tile || t == 16) return t;
+  const long long n = (long long)((d.M + t - 1) / t) * ((d.N + t - 1) / t) * d.B0 * d.B1 * std::max(1, d.splits);
+  return n < device_sm_count() ? 16 : t;
+}
+
 int gemm_pick_splits(const GemmDesc& d) {
   if (d.prec != 0 && gemm_tc_supported(d)) return tc_pick_splits(d);
   if (gemm_oz_supported(d)) return oz_pick_splits(d);
-  const int bm = f64_tile(d);
+  const int bm = f64_split_tile(d);
   const long long tm = (d.M + bm - 1) / bm, tn = (d.N + bm - 1) / bm;
   // a symmetric product launches only the tiles on or above the diagonal
   const long long tiles = (d.sym && d.M == d.N) ? tm * (tm + 1) / 2 : tm * tn;
