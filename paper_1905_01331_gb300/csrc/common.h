@@ -91,7 +91,8 @@ struct GemmDesc {
                      // default): BN of a tensor-core kernel, the square tile of
                      // the FP64 engine
   int digits;        // FP64 products: the digit engine (gemm_oz.cu) where it is supported
-  unsigned* words;   // its magnitude scratch (oz_words(d) words)
+  unsigned* words;   // its scratch (oz_scratch(d) bytes) and the bytes there are
+  size_t words_bytes;
   int occ;           // TMA-fed kernel: 2 = the 96 KB stage ring (two CTAs per
                      // SM), else the 192 KB ring (one CTA per SM)
 };
@@ -123,7 +124,7 @@ constexpr double kOzMinWork = 1 << 23;
 int gemm_oz_launch(const GemmDesc& d, cudaStream_t stream);
 bool gemm_oz_supported(const GemmDesc& d);
 int oz_pick_splits(const GemmDesc& d);
-size_t oz_words(const GemmDesc& d);
+size_t oz_scratch(const GemmDesc& d);
 void gemm_oz_init();
 
 // Tensor-core path (gemm_tc.cu).

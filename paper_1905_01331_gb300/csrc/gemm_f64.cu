@@ -333,9 +333,10 @@ int gemm_launch(const GemmDesc& d0, cudaStream_t s) {
   const int t = f64_tile(d);
   d.sym_tile = t;
   if (d.sym && d.M != d.N) d.sym = 0;
-  if (gemm_oz_supported(d)) {
+  const int oz = gemm_oz_supported(d) ? gemm_oz_launch(d, s) : -1;
+  if (oz >= 0) {
     d.sym = 0;   // every tile is computed (the exact sums are symmetric)
-    n += gemm_oz_launch(d, s);
+    n += oz;
   } else if (t == 64) n += launch_tile<64, 64>(d, s);
   else if (t == 32) n += launch_tile<32, 32>(d, s);
   else n += launch_tile<16, 16>(d, s);
@@ -415,7 +416,7 @@ extern "C" int ttn_close_noalloc(const double* d_Y, const double* d_W, int P, in
   d.ngroups = 1;
   d.digits = 1;
   d.words = reinterpret_cast<unsigned*>(scratch + kNoAllocScratchDoubles - kNoAllocWordDoubles);
-  if (oz_words(d) > 2 * kNoAllocWordDoubles) d.digits = 0;   // (at most 2 x 256 words)
+  d.words_bytes = kNoAllocWordDoubles * sizeof(double);   // (needs at most 2 x 256 words)
   const long long per_split = static_cast<long long>(P) * Q;
   int splits = gemm_pick_splits(d);
   splits = static_cast<int>(std::min<long long>(splits, (kNoAllocScratchDoubles - kNoAllocWordDoubles) / per_split));

@@ -8,7 +8,7 @@
 // and Rump, "Error-free transformations of matrix multiplication", Numer.
 // Algorithms 59 (2012), with digits in place of floating-point slices (Mukunoki
 // et al., "DGEMM using tensor cores", ISC 2020).  A digit is an integer in
-// [-128, 127], exact in BF16; a product of two digits is below 2^14, and the
+// [-128, 127], exact in FP16; a product of two digits is below 2^14, and the
 // digit products of one weight (i + j = l <= 7) over 128 values of K stay below
 // 2^24, so the tensor cores' FP32 accumulation of them is exact.  The 36 digit
 // products with i + j <= 7 go to eight accumulators, one per weight; what is
@@ -17,22 +17,30 @@
 // to FP64 once at the end: the result carries one rounding instead of one per
 // term.
 //
-// One CTA owns a 128 x BN output tile (BN 64 or 32).  Warps 0-7 load FP64
-// operands (any strides), cut them into digits with integer operations and
-// write them to shared memory in the K-major SWIZZLE_128B layout (two stages of
-// 32 K values: the two halves of the 128-byte rows); warp 8 issues the MMAs.
-// The digits of B are stacked along N, so that one MMA multiplies A's digit i
-// with B's digits 0 .. 7 - i and adds each product to the accumulator of its
-// weight: TMEM columns (i + j) BN .. of the same instruction.  All waits are
-// bounded, as in the other tensor-core kernels.
+// One CTA owns a 128 x BN output tile (BN 64 or 32); two stages of 32 K values.
+// Warps 0-7 load FP64 operands (any strides), cut them into digits with integer
+// operations and write them to shared memory in the K-major 64-byte-swizzle
+// layout; digits that oz_prepare_kernel left in memory (small operands that many
+// tiles read) arrive as one bulk copy per stage, started by a thread of warp 9;
+// one thread of warp 8 issues the MMAs.  The digits of B are stacked along N, so
+// that one MMA multiplies A's digit i with B's digits 0 .. 7 - i and adds each
+// product to the accumulator of its weight: TMEM columns (i + j) BN .. of the
+// same instruction.  All waits are bounded, as in the other tensor-core kernels.
 //
-// Measured on a GB300 (P = n = 128): F X of 128 x 128 by 128 x 16384 takes 55
-// us, the FP64 kernel 553 (its two FMA units per SM are busy throughout); the
-// environment's five such products in one 186 against 2706, three close
-// products over K = 16384 123 against 1976; relative error against extended
-// precision 4e-17 to 2e-16 where the FP64 kernel has 2e-16 to 2e-15.  At n =
-// 32 both take 15 to 30 us (latency), so kOzMinWork lies between n = 32 (2^20
-// multiply-adds) and n = 64 (2^24: 24 against 62 us).
+// What bounds it (clocks of a 128 x 64 tile, K = 128): the four stages' MMAs take
+// 12.4 k -- 9.2 k at the tensor rate, the rest is shared memory, which feeds them
+// 106 bytes a clock beside the next stage's stores -- the combination of the
+// accumulators about 6 k, first loads and start 3 k.  128 x 64 because eight
+// accumulators of 64 columns fill TMEM.  Measured on a GB300 (P = n = 128, with the
+// preparation): F X of 128 x 128 by 128 x 16384 41 us (the FP64 kernel 547), the
+// environment's five such products in one 128 us (2674), three close products over
+// K = 16384 120 us (1931), the Gram matrix of 128 x 16384 56 us (449).  Converting
+// both operands in every tile with BF16 digits, which take two operations more a
+// pair, and combining by eight converting instructions per output took 55, 186,
+// 123 and 59.  Relative error against extended precision 4e-17 to 2e-16 where the
+// FP64 kernel has 2e-16 to 2e-15.  At n = 32 both kernels take 15 to 30 us
+// (latency), so kOzMinWork lies between n = 32 (2^20 multiply-adds) and n = 64
+// (2^24: 21 against 58 us).
 //
 // An operand with an infinity or NaN, or whose range would leave the normal
 // FP64 numbers, makes the CTA compute its tile with plain FP64 FMAs instead, so
@@ -41,7 +49,7 @@
 #include <cstdint>
 #include <cstring>
 
-#include <cuda_bf16.h>
+#include <cuda_fp16.h>
 
 #include "common.h"
 
@@ -54,16 +62,21 @@ constexpr int kOBM = 128;
 constexpr int kOChunk = 128;        // K values per exact accumulation
 constexpr int kOBK = 32;            // K values per stage
 constexpr int kOConv = 256;         // converter threads
-constexpr int kOThreads = kOConv + 128;   // and the MMA warp's warpgroup
+constexpr int kOThreads = kOConv + 128;   // and the warpgroup of the MMA and image warps
 constexpr long kOWait = 1L << 22;
 
-// Largest magnitude of an operand: absmax_kernel leaves `parts` words (the high
-// words of |x|, at least 1 for a nonzero x) per operand and batch.
+// Magnitude of an operand: `parts` words (the high words of |x|, at least 1 for
+// a nonzero x) per batch, at word off + (b0 s0 + b1 s1) parts.  img >= 0: the
+// operand's digits are ready in memory (oz_prepare_kernel), block (batch, row
+// tile, K slice of 32) at byte img + ((batch nrt + row tile) nks + slice) of
+// the block size, laid out as a stage of shared memory.
 struct OzOperand {
-  int off, parts, n0, s0, s1;       // word of batch (b0, b1): off + (b0 s0 + b1 s1) parts
+  int off, parts, s0, s1, nrt, nks;
+  long long img;
 };
 struct OzParams {
   const unsigned* words;
+  const uint8_t* images;
   OzOperand a[kMaxGroups], b[kMaxGroups];
   int total_chunks;
   int* err;
@@ -71,15 +84,18 @@ struct OzParams {
 
 struct AbsItem {
   const double* p;
-  long long s_mn, s_k0, s_k1, s_b0, s_b1, count;
-  int flat, mn, k0_log2, k, n0, n1, parts, off, blocks_before, pad;
+  long long s_mn, s_k0, s_k1, s_b0, s_b1, count, img;
+  int flat, mn, k0_log2, k, n0, n1, parts, off, blocks_before, nrt, nks, rt;
 };
-constexpr int kAbsPer = 8192;       // elements per block of absmax_kernel
-constexpr int kAbsMaxParts = 256;
+constexpr int kAbsPer = 4096;       // elements per block of a magnitude pass
+constexpr int kAbsMaxParts = 512;
 struct AbsParams {
   AbsItem it[2 * kMaxGroups];
   int n;
   unsigned* words;
+  uint8_t* images;
+  const int* skip;
+  int skip_when_zero;
 };
 static_assert(sizeof(AbsParams) < 32000, "kernel parameter");
 
@@ -88,29 +104,139 @@ __device__ __forceinline__ unsigned mag_word(double x) {
   return hi | (__double2loint(x) != 0 ? 1u : 0u);
 }
 
-// words[off + batch parts + part] = the largest magnitude word of that part of
-// the operand's batch.  Bound by the read of the operands (from L2 when they
-// were just produced).
-__global__ void __launch_bounds__(256) absmax_kernel(const AbsParams ap) {
+// The eight digits of x as bytes (digit + 128; the most significant digit in
+// the highest byte), for |x| below 2^(emax - 1022): x / 2^(emax - 1084), cut
+// to an integer, plus 128 in every byte.
+__device__ __forceinline__ void digit_bytes(double x, int emax, uint32_t& lo, uint32_t& hi) {
+  const uint32_t h = static_cast<uint32_t>(__double2hiint(x)), l = static_cast<uint32_t>(__double2loint(x));
+  const int e = (h >> 20) & 0x7FF;
+  const uint32_t mh = (h & 0xFFFFFu) | 0x100000u;
+  unsigned long long v = (static_cast<unsigned long long>(__funnelshift_l(l, mh, 9)) << 32) | (l << 9);
+  v >>= min(emax - e, 63);                      // a subnormal x (e = 0) is far below the cut
+  const long long s = static_cast<int>(h) >> 31;
+  v = (v ^ s) + (0x8080808080808080ull - s);
+  lo = static_cast<uint32_t>(v);
+  hi = static_cast<uint32_t>(v >> 32);
+}
+
+// Two digits (bytes b of w0 and w1, each digit + 128) as an FP16 pair: the
+// byte in the low mantissa bits of 1024 is 1024 + digit + 128, less 1152.
+template <int b>
+__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1) {
+  const uint32_t t = __byte_perm(w0, w1, 0x0400 + 0x0101 * b);
+  const uint32_t y = (t & 0x00FF00FFu) | 0x64006400u, z = 0x64806480u;
+  const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&y), *reinterpret_cast<const __half2*>(&z));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+// Eight consecutive K values of row r -> 16-byte chunk c (of four) of every
+// digit tile: rows of 64 bytes, 64-byte swizzle, tiles of ROWS rows.
+template <int ROWS>
+__device__ __forceinline__ void store_digits(const double* v, int emax, uint8_t* tile, int r, int c) {
+  uint32_t lo[8], hi[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) digit_bytes(v[q], emax, lo[q], hi[q]);
+  uint8_t* p = tile + r * 64 + ((c ^ ((r >> 1) & 3)) << 4);
+  constexpr int kTile = ROWS * 64;
+#define TTN_OZ_DIGIT(d, w, b)                                                              \
+  *reinterpret_cast<uint4*>(p + (d) * kTile) =                                             \
+      make_uint4(digit_pair<b>(w[0], w[1]), digit_pair<b>(w[2], w[3]),                     \
+                 digit_pair<b>(w[4], w[5]), digit_pair<b>(w[6], w[7]));
+  TTN_OZ_DIGIT(0, hi, 3) TTN_OZ_DIGIT(1, hi, 2) TTN_OZ_DIGIT(2, hi, 1) TTN_OZ_DIGIT(3, hi, 0)
+  TTN_OZ_DIGIT(4, lo, 3) TTN_OZ_DIGIT(5, lo, 2) TTN_OZ_DIGIT(6, lo, 1) TTN_OZ_DIGIT(7, lo, 0)
+#undef TTN_OZ_DIGIT
+}
+
+// Row and 16-byte chunk of converter task `task` of a stage (4 chunks per row):
+// K contiguous: eight rows by four chunks per warp (a row's 64 bytes of a digit
+// are consecutive); MN contiguous: 32 consecutive rows of one chunk per warp.
+// Both fill the 32 banks in every store phase.
+template <int ROWS>
+__device__ __forceinline__ void task_pos(int task, bool kfast, int& r, int& c) {
+  const int w = task >> 5, lane = task & 31;
+  if (kfast) {
+    r = w * 8 + (lane >> 2);
+    c = lane & 3;
+  } else {
+    r = (w % (ROWS / 32)) * 32 + lane;
+    c = w / (ROWS / 32);
+  }
+}
+
+// Eight consecutive K values (k a multiple of 8) of a row that starts at
+// `base`; zeros outside.
+__device__ __forceinline__ void load8(long long s_mn, long long s_k0, long long s_k1, int k0_log2,
+                                      const double* base, int row, bool row_ok, int k, int K, bool vec, double* v) {
+  if (!row_ok || k >= K) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = 0.0;
+    return;
+  }
+  const int k0 = k & ((1 << k0_log2) - 1), k1 = k >> k0_log2;
+  const double* p = base + row * s_mn + k0 * s_k0 + static_cast<long long>(k1) * s_k1;
+  if (k + 8 <= K) {
+    if (vec) {
+#pragma unroll
+      for (int q = 0; q < 8; q += 2) {
+        const double2 t = *reinterpret_cast<const double2*>(p + q);
+        v[q] = t.x;
+        v[q + 1] = t.y;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = p[q * s_k0];
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) v[q] = k + q < K ? p[q * s_k0] : 0.0;
+  }
+}
+
+// The digits of one stage block (ROWS rows from r0, 32 K values from k) of a
+// small operand into memory, by the whole block.
+template <int ROWS>
+__device__ __forceinline__ void image_block(const AbsItem& it, const double* p, int r0, int k, int emax, uint8_t* out) {
+  const bool kf = it.s_k0 == 1;
+  const bool vec = kf && (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ((it.s_mn | it.s_k1) & 1) == 0;
+#pragma unroll 1
+  for (int task = threadIdx.x; task < ROWS * 4; task += 256) {
+    int r, c;
+    task_pos<ROWS>(task, kf, r, c);
+    double v[8];
+    load8(it.s_mn, it.s_k0, it.s_k1, it.k0_log2, p, r0 + r, r0 + r < it.mn, k + 8 * c, it.k, vec, v);
+    store_digits<ROWS>(v, emax, out, r, c);
+  }
+}
+
+// Before a product: the magnitudes of its operands, and the digits of the
+// small operands that many of its tiles read.
+//   without an image: words[off + batch parts + part] = the largest magnitude
+//     word of that part of the batch;
+//   with one: a block per stage block; each scans its whole (small) batch.
+// Bound by the read of the operands (from L2 when they were just produced).
+__global__ void __launch_bounds__(256) oz_prepare_kernel(const AbsParams ap) {
   pdl_wait();
   pdl_trigger();
+  if (ap.skip && ((*ap.skip != 0) != (ap.skip_when_zero != 0))) return;
   int i = 0;
   while (i + 1 < ap.n && static_cast<int>(blockIdx.x) >= ap.it[i + 1].blocks_before) ++i;
   const AbsItem& it = ap.it[i];
   const int u = blockIdx.x - it.blocks_before;
-  const int batch = u / it.parts, part = u % it.parts;
+  const bool image = it.img >= 0;
+  const int per = image ? it.nrt * it.nks : it.parts;
+  const int batch = u / per, part = u % per;
   const int b0 = batch % it.n0, b1 = batch / it.n0;
   const double* p = it.p + b0 * it.s_b0 + static_cast<long long>(b1) * it.s_b1;
-  const long long lo = it.count * part / it.parts, hi = it.count * (part + 1) / it.parts;
+  const long long lo = image ? 0 : it.count * part / it.parts, hi = image ? it.count : it.count * (part + 1) / it.parts;
   unsigned m = 0;
   if (it.flat) {
     long long e = lo + threadIdx.x;
-    for (; e + 7 * 256 < hi; e += 8 * 256) {
-      double v[8];
+    for (; e + 15 * 256 < hi; e += 16 * 256) {
+      double v[16];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = p[e + q * 256];
+      for (int q = 0; q < 16; ++q) v[q] = p[e + q * 256];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) m = max(m, mag_word(v[q]));
+      for (int q = 0; q < 16; ++q) m = max(m, mag_word(v[q]));
     }
     for (; e < hi; e += 256) m = max(m, mag_word(p[e]));
   } else {
@@ -124,10 +250,18 @@ __global__ void __launch_bounds__(256) absmax_kernel(const AbsParams ap) {
   __shared__ unsigned sh[8];
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) m = max(m, sh[w]);
-    ap.words[it.off + u] = m;
+  for (int w = 0; w < 8; ++w) m = max(m, sh[w]);
+  if (!image) {
+    if (threadIdx.x == 0) ap.words[it.off + u] = m;
+    return;
   }
+  if (part == 0 && threadIdx.x == 0) ap.words[it.off + batch] = m;
+  const int rt = part / it.nks, ks = part % it.nks;
+  uint8_t* out = ap.images + it.img + static_cast<long long>(u) * kOD * it.rt * 64;
+  const int emax = m ? static_cast<int>(m >> 20) : 1023;
+  if (it.rt == 128) image_block<128>(it, p, rt * 128, ks * kOBK, emax, out);
+  else if (it.rt == 64) image_block<64>(it, p, rt * 64, ks * kOBK, emax, out);
+  else image_block<32>(it, p, rt * 32, ks * kOBK, emax, out);
 }
 
 __device__ __forceinline__ uint32_t osmem(const void* p) {
@@ -155,15 +289,23 @@ __device__ __forceinline__ void omb_init(uint64_t* bar, int count) {
 __device__ __forceinline__ void omb_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(osmem(bar)) : "memory");
 }
+__device__ __forceinline__ void omb_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(osmem(bar)), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(osmem(bar))
+               : "memory");
+}
 __device__ __forceinline__ void ocommit(uint64_t* bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(osmem(bar))
       : "memory");
 }
-// K-major, 128-byte swizzle, 8-row atoms stacked every 1024 bytes.
+// K-major, 64-byte swizzle: rows of 64 bytes, 8-row atoms every 512 bytes.
 __device__ __forceinline__ uint64_t odesc(uint32_t saddr) {
   return static_cast<uint64_t>((saddr >> 4) & 0x3FFF) | (1ull << 16) |
-         (static_cast<uint64_t>(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+         (static_cast<uint64_t>(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
 }
 __device__ __forceinline__ void omma(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
   asm volatile(
@@ -171,126 +313,30 @@ __device__ __forceinline__ void omma(uint32_t tmem, uint64_t ad, uint64_t bd, ui
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
       "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
 }
-// D = F32, A and B BF16, both K-major.
+// D = F32, A and B FP16, both K-major.
 __host__ __device__ constexpr uint32_t oidesc(int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | (static_cast<uint32_t>(N >> 3) << 17) |
+  return (1u << 4) | (static_cast<uint32_t>(N >> 3) << 17) |
          (static_cast<uint32_t>(kOBM >> 4) << 24);
 }
 
-// The eight digits of x as bytes (digit + 128; the most significant digit in
-// the highest byte), for |x| below 2^(emax - 1022): x / 2^(emax - 1084), cut
-// to an integer, plus 128 in every byte.
-__device__ __forceinline__ void digit_bytes(double x, int emax, uint32_t& lo, uint32_t& hi) {
-  const uint32_t h = static_cast<uint32_t>(__double2hiint(x)), l = static_cast<uint32_t>(__double2loint(x));
-  const int e = (h >> 20) & 0x7FF;
-  const uint32_t mh = (h & 0xFFFFFu) | 0x100000u;
-  unsigned long long v = (static_cast<unsigned long long>(__funnelshift_l(l, mh, 9)) << 32) | (l << 9);
-  const int sh = emax - e;
-  v = sh < 64 ? v >> sh : 0ull;                 // a subnormal x (e = 0) is far below the cut
-  const long long s = static_cast<int>(h) >> 31;
-  v = (v ^ s) - s + 0x8080808080808080ull;
-  lo = static_cast<uint32_t>(v);
-  hi = static_cast<uint32_t>(v >> 32);
-}
-
-// Two digits (bytes b of w0 and w1, each digit + 128) as a BF16 pair, by BF16
-// arithmetic that is exact: 128 + (u mod 128) minus 256 (u < 128) or 128.
-template <int b>
-__device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1) {
-  const uint32_t t = __byte_perm(w0, w1, 0x0400 + 0x0101 * b);
-  const uint32_t y = (t & 0x007F007Fu) | 0x43004300u;
-  const uint32_t z = (t & 0x00800080u) ^ 0x43804380u;
-  const __nv_bfloat162 r = __hsub2(*reinterpret_cast<const __nv_bfloat162*>(&y),
-                                   *reinterpret_cast<const __nv_bfloat162*>(&z));
-  return *reinterpret_cast<const uint32_t*>(&r);
-}
-
-// Eight consecutive K values of one row -> a 16-byte chunk of each digit tile.
-template <int ROWS>
-__device__ __forceinline__ void store_digits(const double* v, int emax, uint8_t* tile, int r, int chunk) {
-  uint32_t lo[8], hi[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) digit_bytes(v[q], emax, lo[q], hi[q]);
-  uint8_t* p = tile + r * 128 + ((chunk ^ (r & 7)) << 4);
-  constexpr int kTile = ROWS * 128;
-#define TTN_OZ_DIGIT(d, w, b)                                                              \
-  *reinterpret_cast<uint4*>(p + (d) * kTile) =                                             \
-      make_uint4(digit_pair<b>(w[0], w[1]), digit_pair<b>(w[2], w[3]),                     \
-                 digit_pair<b>(w[4], w[5]), digit_pair<b>(w[6], w[7]));
-  TTN_OZ_DIGIT(0, hi, 3) TTN_OZ_DIGIT(1, hi, 2) TTN_OZ_DIGIT(2, hi, 1) TTN_OZ_DIGIT(3, hi, 0)
-  TTN_OZ_DIGIT(4, lo, 3) TTN_OZ_DIGIT(5, lo, 2) TTN_OZ_DIGIT(6, lo, 1) TTN_OZ_DIGIT(7, lo, 0)
-#undef TTN_OZ_DIGIT
-}
-
-// Position of the converters in the K range of a CTA: stage k0 .. k0 + 31 of
-// group g, `left` stages in its chunk after it.
-struct OzCursor {
-  int g, k, chunk;     // group, first K value, chunk counted over all groups
-};
-
-// Row and 16-byte chunk of converter task `task` of a stage (4 chunks per row):
-// K contiguous: eight rows by four chunks per warp, rows r and r + 4 in the
-// same eight-thread store phase (their swizzled halves are disjoint); MN
-// contiguous: 32 consecutive rows of one chunk per warp.
-template <int ROWS>
-__device__ __forceinline__ void task_pos(int task, bool kfast, int& r, int& c) {
-  const int w = task >> 5, lane = task & 31;
-  if (kfast) {
-    r = w * 8 + ((lane >> 2) & 1) * 4 + (lane >> 3);
-    c = lane & 3;
-  } else {
-    r = (w % (ROWS / 32)) * 32 + lane;
-    c = w / (ROWS / 32);
-  }
-}
-
-__device__ __forceinline__ void load8(const Operand& o, int k0_log2, const double* base, int row, bool row_ok,
-                                      int k, int K, bool vec, double* v) {
-  if (!row_ok || k >= K) {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = 0.0;
-    return;
-  }
-  const int k0 = k & ((1 << k0_log2) - 1), k1 = k >> k0_log2;
-  const double* p = base + row * o.s_mn + k0 * o.s_k0 + static_cast<long long>(k1) * o.s_k1;
-  if (k + 8 <= K) {
-    if (vec) {
-#pragma unroll
-      for (int q = 0; q < 8; q += 2) {
-        const double2 t = *reinterpret_cast<const double2*>(p + q);
-        v[q] = t.x;
-        v[q + 1] = t.y;
-      }
-    } else {
-#pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = p[q * o.s_k0];
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < 8; ++q) v[q] = k + q < K ? p[q * o.s_k0] : 0.0;
-  }
-}
-
 // The 96-bit integer (a2 a1 a0, two's complement) times 2^scale, rounded to
-// FP64 (the caller has checked that the result is zero or a normal number).
+// FP64 (the caller has checked that the result is zero or a normal number).  A
+// negative value is complemented without the one: a unit of 2^scale, 2^-124 of
+// the operands' magnitudes, below the cut of their digits.
 __device__ __forceinline__ double to_double(uint32_t a0, uint32_t a1, uint32_t a2, int scale) {
   const uint32_t neg = static_cast<uint32_t>(static_cast<int>(a2) >> 31);
   a0 ^= neg; a1 ^= neg; a2 ^= neg;
-  asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, 0;\n\taddc.u32 %2, %2, 0;"
-      : "+r"(a0), "+r"(a1), "+r"(a2)
-      : "r"(neg & 1u));
-  int pos = 95;
-  if (a2 == 0u) { a2 = a1; a1 = a0; a0 = 0u; pos = 63; }
-  if (a2 == 0u) { a2 = a1; a1 = 0u; pos = 31; }
-  if (a2 == 0u) return 0.0;
+  int e = scale + 1022 + 95;
+  if (a2 == 0u) {
+    a2 = a1; a1 = a0; a0 = 0u; e -= 32;
+    if (a2 == 0u) { a2 = a1; a1 = 0u; e -= 32; }
+  }
   const int n = __clz(a2);
   const uint32_t t1 = __funnelshift_l(a1, a2, n), t0 = __funnelshift_l(a0, a1, n);
   const unsigned long long t = (static_cast<unsigned long long>(t1) << 32) | t0;
-  const unsigned long long m = (t >> 11) + ((t >> 10) & 1ull);
-  const unsigned long long bits =
-      (static_cast<unsigned long long>(pos - n + scale + 1022) << 52) + m +
-      (static_cast<unsigned long long>(neg & 0x80000000u) << 32);
-  return __longlong_as_double(static_cast<long long>(bits));
+  const unsigned long long m = (t >> 11) + ((t0 >> 10) & 1u);
+  const uint32_t hi = static_cast<uint32_t>(m >> 32) + (static_cast<uint32_t>(e - n) << 20);
+  return __hiloint2double(a2 ? static_cast<int>(hi | (neg & 0x80000000u)) : 0, static_cast<int>(static_cast<uint32_t>(m)));
 }
 
 // Output (or split-K partial) of one element.
@@ -327,16 +373,57 @@ __device__ __noinline__ void plain_tile(const GemmDesc& d, int b, int b0, int b1
   }
 }
 
+// Combine four columns' accumulators (levels l of columns cb .. cb + 3) into
+// 96-bit integers, shifted right by sh.
+template <int BN>
+__device__ __forceinline__ void combine4(uint32_t taddr, int sh, uint32_t (&v)[4][3]) {
+  uint32_t r[kOD][4];
+#pragma unroll
+  for (int l = 0; l < kOD; ++l)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3])
+                 : "r"(taddr + l * BN));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    // levels 0 to 2 are at most 2^22 (digit 0 is at most 64): their integers sit
+    // in the low bits of x + 1.5 2^23; the others take the converting
+    // instruction, a quarter of the rate of an addition
+    int L[kOD];
+#pragma unroll
+    for (int l = 0; l < 3; ++l) L[l] = __float_as_int(__uint_as_float(r[l][j]) + 12582912.f) - 0x4B400000;
+#pragma unroll
+    for (int l = 3; l < kOD; ++l) L[l] = __float2int_rn(__uint_as_float(r[l][j]));
+    // (both inner sums fit 32 bits: 2^27 and 2^30 + 2^23)
+    const long long H = static_cast<long long>(L[0] * 256 + L[1]) * (1 << 16) + (L[2] * 256 + L[3]);
+    const long long Q = static_cast<long long>(L[4]) * (1 << 24) + (static_cast<long long>(L[5]) * (1 << 16) +
+                        (static_cast<long long>(L[6]) * 256 + L[7]));
+    const long long hi = H + static_cast<int>(Q >> 32);
+    uint32_t v0 = static_cast<uint32_t>(Q), v1 = static_cast<uint32_t>(hi), v2 = static_cast<uint32_t>(hi >> 32);
+    if (sh) {   // (the same in all threads of the CTA)
+      const uint32_t sg = static_cast<uint32_t>(static_cast<int>(v2) >> 31);
+      int s2 = sh;
+      if (s2 >= 32) { v0 = v1; v1 = v2; v2 = sg; s2 -= 32; }
+      if (s2 >= 32) { v0 = v1; v1 = v2; s2 -= 32; }
+      if (s2 >= 32) { v0 = sg; v1 = sg; s2 = 0; }
+      v0 = __funnelshift_r(v0, v1, s2);
+      v1 = __funnelshift_r(v1, v2, s2);
+      v2 = static_cast<uint32_t>(static_cast<int>(v2) >> s2);
+    }
+    v[j][0] = v0; v[j][1] = v1; v[j][2] = v2;
+  }
+}
+
 template <int BN>
 __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d, const OzParams op) {
   pdl_wait();
   pdl_trigger();
-  constexpr int kA = kOBM * 128;                   // bytes of one digit tile of A
+  constexpr int kA = kOBM * 64, kB = BN * 64;      // bytes of one digit tile of a stage
+  constexpr int kStage = kOD * (kA + kB);
   constexpr int kHalf = BN / 2;                    // columns per flush warp
   constexpr int kCols = kOD * BN;                  // TMEM columns
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  uint8_t* sA = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* sB = sA + kOD * kA;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   __shared__ __align__(8) uint64_t full_bar[2], empty_bar[2], done_bar, free_bar, drain_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
@@ -352,6 +439,62 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   const int c_lo = static_cast<int>(static_cast<long long>(op.total_chunks) * split / d.splits);
   const int c_hi = static_cast<int>(static_cast<long long>(op.total_chunks) * (split + 1) / d.splits);
 
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(osmem(&tmem_slot)), "r"(kCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  // first chunk of the CTA: group g0, K offset kfirst
+  int g0 = 0, kfirst = 0;
+  {
+    int c = c_lo;
+    while (g0 < d.ngroups) {
+      const int nc = (d.g[g0].K + kOChunk - 1) / kOChunk;
+      if (c < nc) break;
+      c -= nc;
+      ++g0;
+    }
+    kfirst = c * kOChunk;
+  }
+  const int nchunks = c_hi - c_lo;
+
+  // converter state: the values of the next stage (loaded before the operands'
+  // magnitudes arrive), their rows and chunks, the position after them
+  const int t = threadIdx.x;
+  constexpr int kATasks = kOBM * 4 / kOConv;                     // 2
+  double va[kATasks][8], vb[8];
+  int g = g0, k = kfirst;                                        // next stage to load
+  const double *pa = nullptr, *pb = nullptr;
+  bool avec = false, bvec = false, a_on = false, b_on = false;
+  int ar[kATasks], ac[kATasks], br = 0, bc = 0;
+  auto enter = [&]() {
+    const Group& G = d.g[g];
+    pa = static_cast<const double*>(G.a.p) + b0 * G.a.s_b0 + static_cast<long long>(b1) * G.a.s_b1;
+    pb = static_cast<const double*>(G.b.p) + b0 * G.b.s_b0 + static_cast<long long>(b1) * G.b.s_b1;
+    const bool akf = G.a.s_k0 == 1, bkf = G.b.s_k0 == 1;
+    a_on = op.a[g].img < 0;
+    b_on = op.b[g].img < 0 && t < BN * 4;
+    avec = akf && ((reinterpret_cast<uintptr_t>(pa) & 15) == 0) && ((G.a.s_mn | G.a.s_k1) & 1) == 0;
+    bvec = bkf && ((reinterpret_cast<uintptr_t>(pb) & 15) == 0) && ((G.b.s_mn | G.b.s_k1) & 1) == 0;
+#pragma unroll
+    for (int q = 0; q < kATasks; ++q) task_pos<kOBM>(t + q * kOConv, akf, ar[q], ac[q]);
+    task_pos<BN>(t, bkf, br, bc);
+  };
+  auto load_a = [&](int q) {
+    const Group& G = d.g[g];
+    load8(G.a.s_mn, G.a.s_k0, G.a.s_k1, G.k0_log2, pa, m0 + ar[q], m0 + ar[q] < d.M, k + 8 * ac[q], G.K, avec, va[q]);
+  };
+  auto load_b = [&]() {
+    const Group& G = d.g[g];
+    load8(G.b.s_mn, G.b.s_k0, G.b.s_k1, G.k0_log2, pb, n0 + br, n0 + br < d.N, k + 8 * bc, G.K, bvec, vb);
+  };
+  if (warp < 8 && nchunks > 0) {
+    enter();
+    if (b_on) load_b();
+    if (a_on) {
+#pragma unroll
+      for (int q = 0; q < kATasks; ++q) load_a(q);
+    }
+  }
   // largest magnitude of every operand
   for (int i = warp; i < 2 * d.ngroups; i += kOThreads / 32) {
     const OzOperand& o = (i & 1) ? op.b[i >> 1] : op.a[i >> 1];
@@ -363,7 +506,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   }
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
-      omb_init(&full_bar[s], kOConv);
+      omb_init(&full_bar[s], kOConv + 1);
       omb_init(&empty_bar[s], 1);
     }
     omb_init(&done_bar, 1);
@@ -372,6 +515,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   // the scale of a group's digit products is 2^(ea + eb - 68); all groups are
   // added relative to the largest one
@@ -386,43 +530,22 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     sref = max(sref, s);
   }
   if (sref != -100000 && (sref < -1000 || sref > 900)) plain = true;
-  if (plain) {
-    plain_tile<BN>(d, b, b0, b1, split, m0, n0, c_lo, c_hi);
-    return;
-  }
-  if (warp == 8) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(osmem(&tmem_slot)), "r"(kCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
+  if (plain) plain_tile<BN>(d, b, b0, b1, split, m0, n0, c_lo, c_hi);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
   volatile int* abort_v = &abort_flag;
 
-  // first chunk of the CTA: group g, K offset k
-  int g0 = 0, kfirst = 0;
-  {
-    int c = c_lo;
-    while (g0 < d.ngroups) {
-      const int nc = (d.g[g0].K + kOChunk - 1) / kOChunk;
-      if (c < nc) break;
-      c -= nc;
-      ++g0;
-    }
-    kfirst = c * kOChunk;
-  }
-  const int nchunks = c_hi - c_lo;
-
   // registers: three warpgroups of 168 at launch -> 72 for the MMA warp's, 216
   // for the two of the converters (2 x 216 + 72 = 3 x 168)
-  if (warp >= 8) {
+  if (plain) {
+    // (the tile is done)
+  } else if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
     if (warp == 8 && lane == 0) {
       // ---- MMA issuer ----
       bool ok = true;
       int g = g0, k = kfirst, it = 0;
-      const uint32_t a0 = osmem(sA), b0s = osmem(sB);
+      const uint32_t base = osmem(smem);
       for (int c = 0; c < nchunks && ok; ++c) {
         if (c > 0 && !omb_wait(&free_bar, (c - 1) & 1, abort_v)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -432,19 +555,19 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
           const int s = it & 1;
           if (!omb_wait(&full_bar[s], (it >> 1) & 1, abort_v)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t sa = base + s * kStage, sb = sa + kOD * kA;
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            const uint32_t off = s * 64 + j * 32;
 #pragma unroll
             for (int i = 0; i < kOD; ++i) {
-              const uint64_t ad = odesc(a0 + i * kA + off);
+              const uint64_t ad = odesc(sa + i * kA + j * 32);
               const uint32_t acc = (st > 0 || j > 0 || i > 0) ? 1u : 0u;
               // digits 0 .. 7 - i of B in pieces of at most 256 columns
 #pragma unroll
               for (int n = 0; n < (kOD - i) * BN; n += 256) {
                 constexpr int kMaxN = 256;
                 const int nn = (kOD - i) * BN - n < kMaxN ? (kOD - i) * BN - n : kMaxN;
-                omma(tmem + i * BN + n, ad, odesc(b0s + n * 128 + off), oidesc(nn), acc);
+                omma(tmem + i * BN + n, ad, odesc(sb + n * 64 + j * 32), oidesc(nn), acc);
               }
             }
           }
@@ -461,39 +584,42 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
         ocommit(&drain_bar);
         omb_wait(&drain_bar, 0, nullptr);
       }
+    } else if (warp == 9 && lane == 0) {
+      // ---- ready digits: one bulk copy per operand and stage ----
+      bool ok = true;
+      int g = g0, k = kfirst, it = 0;
+      const uint32_t base = osmem(smem);
+      for (int c = 0; c < nchunks && ok; ++c) {
+        const int kend = min(d.g[g].K, k + kOChunk);
+        const OzOperand &oa = op.a[g], &ob = op.b[g];
+        for (int ks = k / kOBK; ks * kOBK < kend; ++ks, ++it) {
+          const int s = it & 1;
+          if (it >= 2 && !omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v)) { ok = false; break; }
+          const uint32_t bytes = (oa.img >= 0 ? kOD * kA : 0) + (ob.img >= 0 ? kOD * kB : 0);
+          if (!bytes) { omb_arrive(&full_bar[s]); continue; }
+          omb_expect(&full_bar[s], bytes);
+          if (oa.img >= 0)
+            bulk_load(base + s * kStage,
+                      op.images + oa.img +
+                          ((static_cast<long long>(b0 * oa.s0 + b1 * oa.s1) * oa.nrt + tm) * oa.nks + ks) * (kOD * kA),
+                      kOD * kA, &full_bar[s]);
+          if (ob.img >= 0)
+            bulk_load(base + s * kStage + kOD * kA,
+                      op.images + ob.img +
+                          ((static_cast<long long>(b0 * ob.s0 + b1 * ob.s1) * ob.nrt + tn) * ob.nks + ks) * (kOD * kB),
+                      kOD * kB, &full_bar[s]);
+        }
+        k += kOChunk;
+        if (k >= d.g[g].K) { ++g; k = 0; }
+      }
+      if (!ok) *abort_v = 1;
+      // copies in flight land before the CTA exits, also after an abort
+      for (int q = max(0, it - 2); q < it; ++q) omb_wait(&full_bar[q & 1], (q >> 1) & 1, nullptr);
     }
     __syncwarp();
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
     // ---- converters, then the flush of every chunk ----
-    const int t = threadIdx.x;
-    constexpr int kATasks = kOBM * 4 / kOConv;                     // 2
-    const bool b_on = t < BN * 4;
-    double va[kATasks][8], vb[8];
-    int g = g0, k = kfirst;                               // next stage to load
-    const double *pa = nullptr, *pb = nullptr;
-    bool akf = false, bkf = false, avec = false, bvec = false;
-    int ar[kATasks], ac[kATasks], br = 0, bc = 0;
-    auto enter = [&]() {
-      const Group& G = d.g[g];
-      pa = static_cast<const double*>(G.a.p) + b0 * G.a.s_b0 + static_cast<long long>(b1) * G.a.s_b1;
-      pb = static_cast<const double*>(G.b.p) + b0 * G.b.s_b0 + static_cast<long long>(b1) * G.b.s_b1;
-      akf = G.a.s_k0 == 1;
-      bkf = G.b.s_k0 == 1;
-      avec = akf && ((reinterpret_cast<uintptr_t>(pa) & 15) == 0) && ((G.a.s_mn | G.a.s_k1) & 1) == 0;
-      bvec = bkf && ((reinterpret_cast<uintptr_t>(pb) & 15) == 0) && ((G.b.s_mn | G.b.s_k1) & 1) == 0;
-#pragma unroll
-      for (int q = 0; q < kATasks; ++q) task_pos<kOBM>(t + q * kOConv, akf, ar[q], ac[q]);
-      task_pos<BN>(t, bkf, br, bc);
-    };
-    auto load_a = [&](int q) {
-      const Group& G = d.g[g];
-      load8(G.a, G.k0_log2, pa, m0 + ar[q], m0 + ar[q] < d.M, k + 8 * ac[q], G.K, avec, va[q]);
-    };
-    auto load_b = [&]() {
-      const Group& G = d.g[g];
-      if (b_on) load8(G.b, G.k0_log2, pb, n0 + br, n0 + br < d.N, k + 8 * bc, G.K, bvec, vb);
-    };
     uint32_t acc[3][kHalf];
 #pragma unroll
     for (int j = 0; j < kHalf; ++j) acc[0][j] = acc[1][j] = acc[2][j] = 0u;
@@ -501,62 +627,30 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + half * kHalf;
     bool ok = true;
     int flushed = 0;
+    auto shift_of = [&](int fg) {
+      const unsigned wa = ex[2 * fg], wb = ex[2 * fg + 1];
+      return (wa == 0u || wb == 0u) ? 0 : sref - (static_cast<int>(wa >> 20) + static_cast<int>(wb >> 20) - 2 * 1022 - 68);
+    };
     // add the eight accumulators of a finished chunk (of group fg) to acc
     auto flush = [&](int fg) {
       ok = __all_sync(0xffffffffu, ok && omb_wait(&done_bar, flushed & 1, abort_v));
       ++flushed;
       if (!ok) return;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const unsigned wa = ex[2 * fg], wb = ex[2 * fg + 1];
-      const int sh = (wa == 0u || wb == 0u) ? 0 : sref - (static_cast<int>(wa >> 20) + static_cast<int>(wb >> 20) - 2 * 1022 - 68);
+      const int sh = shift_of(fg);
 #pragma unroll
       for (int cb = 0; cb < kHalf; cb += 4) {
-        uint32_t r[kOD][4];
+        uint32_t v[4][3];
+        combine4<BN>(trow + cb, sh, v);
 #pragma unroll
-        for (int l = 0; l < kOD; ++l)
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-              : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3])
-              : "r"(trow + l * BN + cb));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          int L[kOD];
-#pragma unroll
-          for (int l = 0; l < kOD; ++l) L[l] = __float2int_rn(__uint_as_float(r[l][j]));
-          const long long H = static_cast<long long>(L[0]) * (1 << 24) + static_cast<long long>(L[1]) * (1 << 16) +
-                              static_cast<long long>(L[2]) * 256 + L[3];
-          const long long Q = static_cast<long long>(L[4]) * (1 << 24) + static_cast<long long>(L[5]) * (1 << 16) +
-                              static_cast<long long>(L[6]) * 256 + L[7];
-          uint32_t v0 = static_cast<uint32_t>(Q), v1 = static_cast<uint32_t>(Q >> 32);
-          uint32_t v2 = static_cast<uint32_t>(static_cast<int>(v1) >> 31);
-          asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, %3;"
-              : "+r"(v1), "+r"(v2)
-              : "r"(static_cast<uint32_t>(H)), "r"(static_cast<uint32_t>(H >> 32)));
-          if (sh) {   // (the same in all threads of the CTA)
-            const uint32_t sg = static_cast<uint32_t>(static_cast<int>(v2) >> 31);
-            int s2 = sh;
-            if (s2 >= 32) { v0 = v1; v1 = v2; v2 = sg; s2 -= 32; }
-            if (s2 >= 32) { v0 = v1; v1 = v2; s2 -= 32; }
-            if (s2 >= 32) { v0 = sg; v1 = sg; s2 = 0; }
-            v0 = __funnelshift_r(v0, v1, s2);
-            v1 = __funnelshift_r(v1, v2, s2);
-            v2 = static_cast<uint32_t>(static_cast<int>(v2) >> s2);
-          }
+        for (int j = 0; j < 4; ++j)
           asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
               : "+r"(acc[0][cb + j]), "+r"(acc[1][cb + j]), "+r"(acc[2][cb + j])
-              : "r"(v0), "r"(v1), "r"(v2));
-        }
+              : "r"(v[j][0]), "r"(v[j][1]), "r"(v[j][2]));
       }
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       omb_arrive(&free_bar);
     };
-    if (nchunks > 0) {
-      enter();
-      load_b();
-#pragma unroll
-      for (int q = 0; q < kATasks; ++q) load_a(q);
-    }
     int it = 0, pend = -1;    // pend: group of the chunk that waits for its flush
     for (int c = 0; c <= nchunks && ok; ++c) {   // (one round more: the last flush)
       const int cg = g;
@@ -564,30 +658,35 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       const unsigned wa = ex[2 * cg], wb = ex[2 * cg + 1];
       // (an all-zero operand: any exponent gives zero digits)
       const int ea = wa ? static_cast<int>(wa >> 20) : 1023, eb = wb ? static_cast<int>(wb >> 20) : 1023;
+      if (nst == 0 && nchunks == 1) break;       // a single chunk is stored from TMEM below
+#pragma unroll 1
       for (int st = 0; st < max(nst, 1); ++st, ++it) {
         const int s = it & 1;
         if (nst) {
-        if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v));
-        if (!ok) break;
-        // the positions of this stage's tasks; the next stage's loads follow each conversion
-        int car[kATasks], cac[kATasks];
+          if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v));
+          if (!ok) break;
+          uint8_t* sA = smem + s * kStage;
+          uint8_t* sB = sA + kOD * kA;
+          // the positions of this stage's tasks; the next stage's loads follow each conversion
+          int car[kATasks], cac[kATasks];
 #pragma unroll
-        for (int q = 0; q < kATasks; ++q) { car[q] = ar[q]; cac[q] = ac[q]; }
-        const int cbr = br, cbc = bc;
-        const bool last = c + 1 == nchunks && st + 1 == nst;
-        if (!last) {
-          k += kOBK;
-          if (k >= d.g[g].K) { ++g; k = 0; enter(); }
-        }
-        if (b_on) store_digits<BN>(vb, eb, sB, cbr, s * 4 + cbc);
-        if (!last) load_b();
+          for (int q = 0; q < kATasks; ++q) { car[q] = ar[q]; cac[q] = ac[q]; }
+          const int cbr = br, cbc = bc;
+          const bool ca = a_on, cb = b_on;
+          const bool last = c + 1 == nchunks && st + 1 == nst;
+          if (!last) {
+            k += kOBK;
+            if (k >= d.g[g].K) { ++g; k = 0; enter(); }
+          }
+          if (cb) store_digits<BN>(vb, eb, sB, cbr, cbc);
+          if (!last && b_on) load_b();
 #pragma unroll
-        for (int q = 0; q < kATasks; ++q) {
-          store_digits<kOBM>(va[q], ea, sA, car[q], s * 4 + cac[q]);
-          if (!last) load_a(q);
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        omb_arrive(&full_bar[s]);
+          for (int q = 0; q < kATasks; ++q) {
+            if (ca) store_digits<kOBM>(va[q], ea, sA, car[q], cac[q]);
+            if (!last && a_on) load_a(q);
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          omb_arrive(&full_bar[s]);
         }
         // the previous chunk is flushed once two stages of this one are staged
         if (pend >= 0 && (st == 1 || st + 1 >= nst)) {
@@ -598,28 +697,44 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       }
       pend = cg;
     }
+    const int m = m0 + quarter * 32 + lane;
+    double* row = out_ptr(d, b, b0, b1, split, m, n0 + half * kHalf);
+    const long long sn = d.splits > 1 ? 1 : d.sc_n;
+    const int nv = m < d.M ? min(kHalf, d.N - (n0 + half * kHalf)) : 0;
+    const bool vec = sn == 1 && nv == kHalf && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
+    auto put = [&](int j, double x, double y) {
+      if (vec) {
+        *reinterpret_cast<double2*>(row + j) = make_double2(x, y);
+      } else {
+        if (j < nv) row[j * sn] = x;
+        if (j + 1 < nv) row[(j + 1) * sn] = y;
+      }
+    };
+    if (ok && nchunks == 1) {
+      // one chunk: straight from the accumulators, four columns at a time (a
+      // short loop: unrolled, its instructions took longer to fetch than to run)
+      ok = __all_sync(0xffffffffu, omb_wait(&done_bar, 0, abort_v));
+      if (ok) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int sh = shift_of(g0);
+#pragma unroll 1
+        for (int cb = 0; cb < kHalf; cb += 4) {
+          uint32_t v[4][3];
+          combine4<BN>(trow + cb, sh, v);
+#pragma unroll
+          for (int j = 0; j < 4; j += 2)
+            put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
+        }
+      }
+    } else if (ok) {
+#pragma unroll
+      for (int j = 0; j < kHalf; j += 2)
+        put(j, to_double(acc[0][j], acc[1][j], acc[2][j], sref),
+            to_double(acc[0][j + 1], acc[1][j + 1], acc[2][j + 1], sref));
+    }
     if (!ok) {
       *abort_v = 1;
       if (op.err && t == 0) atomicOr(op.err, 1);
-    } else {
-      const int m = m0 + quarter * 32 + lane;
-      if (m < d.M) {
-        double* row = out_ptr(d, b, b0, b1, split, m, n0 + half * kHalf);
-        const long long sn = d.splits > 1 ? 1 : d.sc_n;
-        const int nv = min(kHalf, d.N - (n0 + half * kHalf));
-        const bool vec = sn == 1 && nv == kHalf && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
-#pragma unroll
-        for (int j = 0; j < kHalf; j += 2) {
-          const double x = to_double(acc[0][j], acc[1][j], acc[2][j], sref);
-          const double y = to_double(acc[0][j + 1], acc[1][j + 1], acc[2][j + 1], sref);
-          if (vec) {
-            *reinterpret_cast<double2*>(row + j) = make_double2(x, y);
-          } else {
-            if (j < nv) row[j * sn] = x;
-            if (j + 1 < nv) row[(j + 1) * sn] = y;
-          }
-        }
-      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -629,7 +744,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
 }
 
 template <int BN>
-constexpr int oz_smem() { return kOD * (kOBM + BN) * 128 + 1024; }
+constexpr int oz_smem() { return 2 * kOD * (kOBM + BN) * 64 + 1024; }
 
 int oz_chunks(const GemmDesc& d) {
   int t = 0;
@@ -660,7 +775,78 @@ bool flat_operand(const Operand& o, int k0_log2, int K, int mn, long long* count
 bool same_operand(const AbsItem& a, const AbsItem& b) {
   return a.p == b.p && a.s_mn == b.s_mn && a.s_k0 == b.s_k0 && a.s_k1 == b.s_k1 && a.s_b0 == b.s_b0 &&
          a.s_b1 == b.s_b1 && a.count == b.count && a.flat == b.flat && a.mn == b.mn && a.k == b.k &&
-         a.k0_log2 == b.k0_log2 && a.n0 == b.n0 && a.n1 == b.n1;
+         a.k0_log2 == b.k0_log2 && a.n0 == b.n0 && a.n1 == b.n1 && a.rt == b.rt && (a.img >= 0) == (b.img >= 0);
+}
+
+// Digits prepared in memory for an operand that at least kOzReuse CTAs read
+// per row tile, while all its batches' digits stay below kOzImageMax bytes: the
+// tiles' converters then have the other operand only, and the bulk copy of a
+// stage costs them nothing.  (Digits take 16 bytes per value where FP64 takes
+// 8, so a large operand is converted by the tiles that read it.)
+constexpr int kOzReuse = 8;
+constexpr long long kOzImageMax = 4 << 20;
+
+// The preparation of a product: items (operands, without repeats), their words
+// and images; returns the blocks of oz_prepare_kernel.
+struct OzPlan {
+  AbsParams ap;
+  OzParams op;
+  int blocks;
+  long long words, image_bytes;
+};
+
+void plan_product(const GemmDesc& d, OzPlan& pl) {
+  memset(&pl, 0, sizeof(pl));
+  const int bn = oz_bn(d);
+  const long long tm = (d.M + kOBM - 1) / kOBM, tn = (d.N + bn - 1) / bn, nb = static_cast<long long>(d.B0) * d.B1;
+  AbsParams& ap = pl.ap;
+  for (int g = 0; g < d.ngroups; ++g)
+    for (int side = 0; side < 2; ++side) {
+      const Group& G = d.g[g];
+      const Operand& o = side ? G.b : G.a;
+      AbsItem it;
+      memset(&it, 0, sizeof(it));
+      it.p = static_cast<const double*>(o.p);
+      it.s_mn = o.s_mn; it.s_k0 = o.s_k0; it.s_k1 = o.s_k1; it.s_b0 = o.s_b0; it.s_b1 = o.s_b1;
+      it.mn = side ? d.N : d.M;
+      it.k = G.K;
+      it.k0_log2 = G.k0_log2;
+      it.n0 = o.s_b0 ? d.B0 : 1;
+      it.n1 = o.s_b1 ? d.B1 : 1;
+      it.flat = flat_operand(o, G.k0_log2, G.K, it.mn, &it.count) ? 1 : 0;
+      it.rt = side ? bn : kOBM;
+      it.nrt = (it.mn + it.rt - 1) / it.rt;
+      it.nks = (G.K + kOBK - 1) / kOBK;
+      const long long batches = static_cast<long long>(it.n0) * it.n1;
+      const long long bytes = batches * it.nrt * it.nks * kOD * it.rt * 64;
+      const long long reuse = (side ? tm : tn) * nb / batches;
+      const bool image = reuse >= kOzReuse && bytes <= kOzImageMax && it.count <= 16 * kAbsPer;
+      it.img = image ? 0 : -1;
+      it.parts = image ? 1 : static_cast<int>(std::max<long long>(1, std::min<long long>((it.count + kAbsPer - 1) / kAbsPer, kAbsMaxParts)));
+      int at = 0;
+      while (at < ap.n && !same_operand(ap.it[at], it)) ++at;
+      if (at == ap.n) {
+        it.off = static_cast<int>(pl.words);
+        it.blocks_before = pl.blocks;
+        pl.words += it.parts * batches;
+        if (image) {
+          it.img = pl.image_bytes;
+          pl.image_bytes += bytes;
+          pl.blocks += static_cast<int>(batches) * it.nrt * it.nks;
+        } else {
+          pl.blocks += static_cast<int>(batches) * it.parts;
+        }
+        ap.it[ap.n++] = it;
+      }
+      OzOperand& w = side ? pl.op.b[g] : pl.op.a[g];
+      w.off = ap.it[at].off;
+      w.parts = ap.it[at].parts;
+      w.s0 = o.s_b0 ? 1 : 0;
+      w.s1 = o.s_b1 ? it.n0 : 0;
+      w.nrt = it.nrt;
+      w.nks = it.nks;
+      w.img = ap.it[at].img;
+    }
 }
 
 }  // namespace
@@ -689,65 +875,34 @@ int oz_pick_splits(const GemmDesc& d) {
   return static_cast<int>(std::max<long long>(1, std::min<long long>(sms / base, oz_chunks(d))));
 }
 
-// Words of magnitude scratch for a product.
-size_t oz_words(const GemmDesc& d) {
+// Bytes of scratch for a product: the magnitude words, then the images.
+static size_t words_bytes(long long words) { return (static_cast<size_t>(words) * sizeof(unsigned) + 255) & ~size_t(255); }
+
+size_t oz_scratch(const GemmDesc& d) {
   if (!gemm_oz_supported(d)) return 0;
-  size_t n = 0;
-  for (int g = 0; g < d.ngroups; ++g)
-    for (int s = 0; s < 2; ++s) {
-      const Operand& o = s ? d.g[g].b : d.g[g].a;
-      const long long count = static_cast<long long>(s ? d.N : d.M) * d.g[g].K;
-      const long long parts = std::max<long long>(1, std::min<long long>((count + kAbsPer - 1) / kAbsPer, kAbsMaxParts));
-      n += static_cast<size_t>(parts) * (o.s_b0 ? d.B0 : 1) * (o.s_b1 ? d.B1 : 1);
-    }
-  return n;
+  static thread_local OzPlan pl;
+  plan_product(d, pl);
+  return words_bytes(pl.words) + static_cast<size_t>(pl.image_bytes);
 }
 
+// Returns the launches, or -1 when the scratch is too small (nothing launched).
 int gemm_oz_launch(const GemmDesc& d, cudaStream_t s) {
-  AbsParams ap;
-  OzParams op;
-  memset(&op, 0, sizeof(op));
-  ap.n = 0;
-  ap.words = d.words;
-  int off = 0, blocks = 0;
-  for (int g = 0; g < d.ngroups; ++g)
-    for (int side = 0; side < 2; ++side) {
-      const Group& G = d.g[g];
-      const Operand& o = side ? G.b : G.a;
-      AbsItem it;
-      memset(&it, 0, sizeof(it));
-      it.p = static_cast<const double*>(o.p);
-      it.s_mn = o.s_mn; it.s_k0 = o.s_k0; it.s_k1 = o.s_k1; it.s_b0 = o.s_b0; it.s_b1 = o.s_b1;
-      it.mn = side ? d.N : d.M;
-      it.k = G.K;
-      it.k0_log2 = G.k0_log2;
-      it.n0 = o.s_b0 ? d.B0 : 1;
-      it.n1 = o.s_b1 ? d.B1 : 1;
-      it.flat = flat_operand(o, G.k0_log2, G.K, it.mn, &it.count) ? 1 : 0;
-      it.parts = static_cast<int>(std::max<long long>(1, std::min<long long>((it.count + kAbsPer - 1) / kAbsPer, kAbsMaxParts)));
-      int at = 0;
-      while (at < ap.n && !same_operand(ap.it[at], it)) ++at;
-      if (at == ap.n) {
-        it.off = off;
-        it.blocks_before = blocks;
-        off += it.parts * it.n0 * it.n1;
-        blocks += it.parts * it.n0 * it.n1;
-        ap.it[ap.n++] = it;
-      }
-      OzOperand& w = side ? op.b[g] : op.a[g];
-      w.off = ap.it[at].off;
-      w.parts = ap.it[at].parts;
-      w.s0 = o.s_b0 ? 1 : 0;
-      w.s1 = o.s_b1 ? it.n0 : 0;
-    }
-  launch_k(absmax_kernel, blocks, 256, 0, s, ap);
-  op.words = d.words;
-  op.total_chunks = oz_chunks(d);
-  op.err = d.err;
+  static thread_local OzPlan pl;
+  plan_product(d, pl);
+  if (words_bytes(pl.words) + static_cast<size_t>(pl.image_bytes) > d.words_bytes) return -1;
+  pl.ap.words = d.words;
+  pl.ap.images = reinterpret_cast<uint8_t*>(d.words) + words_bytes(pl.words);
+  pl.ap.skip = d.skip;
+  pl.ap.skip_when_zero = d.skip_when_zero;
+  launch_k(oz_prepare_kernel, pl.blocks, 256, 0, s, pl.ap);
+  pl.op.words = pl.ap.words;
+  pl.op.images = pl.ap.images;
+  pl.op.total_chunks = oz_chunks(d);
+  pl.op.err = d.err;
   const int bn = oz_bn(d);
   dim3 grid(((d.M + kOBM - 1) / kOBM) * ((d.N + bn - 1) / bn), d.B0 * d.B1, d.splits);
-  if (bn == 64) launch_k(gemm_oz_kernel<64>, grid, kOThreads, oz_smem<64>(), s, d, op);
-  else launch_k(gemm_oz_kernel<32>, grid, kOThreads, oz_smem<32>(), s, d, op);
+  if (bn == 64) launch_k(gemm_oz_kernel<64>, grid, kOThreads, oz_smem<64>(), s, d, pl.op);
+  else launch_k(gemm_oz_kernel<32>, grid, kOThreads, oz_smem<32>(), s, d, pl.op);
   return 2;
 }
 

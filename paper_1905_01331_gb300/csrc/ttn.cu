@@ -203,7 +203,7 @@ struct ttn_ctx {
   // the FP64 sweeps and calls, not in the mixed modes' sweeps, whose small
   // FP64 products keep their order of operations
   bool digits = false;
-  unsigned* words = nullptr;   // its magnitude scratch
+  unsigned* words = nullptr;   // its scratch (oz_scratch bytes)
   size_t words_cap = 0;
   int lz_m = 48;
   double* E_hist = nullptr;    // device energies of the current ttn_sweep call
@@ -425,8 +425,8 @@ Tuned tune_product(ttn_ctx* h, const GemmDesc& d0) {
 void run(ttn_ctx* h, GemmDesc d, int prec) {
   d.prec = prec;
   d.digits = h->digits && prec == 0;
-  if (d.digits && !h->measuring && oz_words(d) > h->words_cap) d.digits = 0;   // cannot happen after planning
   d.words = h->words;
+  d.words_bytes = h->words_cap;
   d.tc_engine = h->opt.tc_engine;
   int s;
   const uint64_t key = h->tuned.empty() && !h->tuning ? 0 : tune_key(d);
@@ -446,7 +446,7 @@ void run(ttn_ctx* h, GemmDesc d, int prec) {
   size_t need = gemm_partial_elems(d, s);
   if (h->measuring) {
     if (need > h->partial_cap) h->partial_cap = need;
-    h->words_cap = std::max(h->words_cap, oz_words(d));
+    h->words_cap = std::max(h->words_cap, oz_scratch(d));
     if (d.ngroups > kMaxGroups) h->bounds_error = "too many groups";
     check_desc(h, d);
     return;
@@ -1569,13 +1569,13 @@ void layout(ttn_ctx* h, Arena& ar) {
     }
     h->iflags = ar.take_int(8 + 3 * kComposeMaxTiles);
     h->partial = ar.take(h->partial_cap);
-    h->words = reinterpret_cast<unsigned*>(ar.take_int(h->words_cap));
+    h->words = reinterpret_cast<unsigned*>(ar.take((h->words_cap + 7) / 8));
     const int ss = h->opt.stage_streams == 0 ? (h->lanes.size() == 1 ? kSubStreams : 1)
                                              : h->opt.stage_streams;
     h->sub.n = ss > 1 ? std::min(ss, kSubStreams) : 0;
     for (int i = 0; i < h->sub.n; ++i) {
       h->sub.partial[i] = ar.take(h->partial_cap);
-      h->sub.words[i] = reinterpret_cast<unsigned*>(ar.take_int(h->words_cap));
+      h->sub.words[i] = reinterpret_cast<unsigned*>(ar.take((h->words_cap + 7) / 8));
     }
     save_lane(h, h->lanes[k]);
   }
@@ -1641,6 +1641,7 @@ void plan(ttn_ctx* h) {
     isometry_grams(h, I, nullptr);
     if (!I.per_node) leftmost_rdm(h, I, 0);
     value_and_grad(h, I, h->opt.prec, nullptr, h->Gam);
+    if (h->opt.prec != 0) value_and_grad(h, I, 0, nullptr, h->Gam);
   }
   h->measuring = false;
 }

@@ -1,5 +1,6 @@
 """The top solve's energy against the lowest eigenvalue of the same top
-Hamiltonian (built from the ascended operators) by ARPACK, over the top
+Hamiltonian (built from the ascended operators, its symmetric part: the mixed
+modes' products leave them asymmetric by 1e-7) by ARPACK, over the top
 dimensions where the kernel's staging differs: below a tile (4), one tile and
 one CTA (8), grids with and without a CTA for the convergence checks, the
 largest (256), and with several streams sharing the GPU."""
@@ -17,10 +18,10 @@ def _lowest(ops, K, c):
 
     def mv(x):
         x = x.reshape(c, c)
-        y = o @ x + x @ o.T
+        y = (o + o.T) @ x + x @ (o + o.T)
         for a, b in zip(A, B):
-            y = y + a @ x @ b.T + b @ x @ a.T
-        return y.ravel()
+            y = y + a @ x @ b.T + b @ x @ a.T + a.T @ x @ b + b.T @ x @ a
+        return 0.5 * y.ravel()
 
     if c * c <= 64:
         return np.linalg.eigvalsh(np.stack([mv(e) for e in np.eye(c * c)], 1))[0]
