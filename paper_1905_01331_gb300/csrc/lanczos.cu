@@ -770,22 +770,24 @@ __device__ void tile_store_p(LzSmem& sm, float a0h, float a0l, float a1h, float 
 // Wide staging (c <= kLWideMaxC, c a multiple of 8): every
 // operand tile of a matrix-vector phase is requested at once by 16-byte
 // asynchronous copies (cp.async.cg: L2 only, like the loads above) into
-// kLWideSlots slots of 16 rows of ldw = c + 4 floats, so that a phase costs
+// lz_slots(c) slots of 16 rows of ldw = c + 4 floats, so that a phase costs
 // one L2 latency instead of one per term.  A row tile holds rows [r0, r0+8)
 // of a pair matrix (hi rows 0-7, lo rows 8-15); a column tile holds columns
 // [c0, c0+8) untransposed (hi: c rows of 8 floats, then lo).  The products
 // below take the same operands in the same order as tile_fma_p and tile_fma, so
 // both stagings give the same bits.  In FP64 mode a slot holds 8 rows of c + 2
 // doubles (or a column tile of c rows of 8).
-constexpr int kLWideMaxC = 128;
-constexpr int kLWideSlots = 8;
+// (eight slots up to c = 128; five at c = 256, where two CTAs per SM have no
+// room for more)
+constexpr int kLWideMaxC = kLMaxC;
+__host__ __device__ __forceinline__ int lz_slots(int c) { return c <= 128 ? 8 : 5; }
 
 __host__ __device__ __forceinline__ int lz_wide_ld(int c) { return c + 4; }
 __host__ __device__ __forceinline__ int lz_slot_floats(int c) { return 2 * kLT * (c + 4); }
 
 // Doubles of the operand tiles: the wide slots, or L and R.
 __host__ __device__ __forceinline__ int lz_tile_doubles(int c, int wide) {
-  const int t = wide ? kLWideSlots * lz_slot_floats(c) / 2 : 2 * kLT * (c + 1);
+  const int t = wide ? lz_slots(c) * lz_slot_floats(c) / 2 : 2 * kLT * (c + 1);
   return t > 8 * (kLMaxM + 2) ? t : 8 * (kLMaxM + 2);   // also the checks' scratch
 }
 
@@ -1192,12 +1194,12 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
       // phase A: Y_b = Op_b x for the 2K operators A_k0, B_k0 (stored after o_0)
       const float* xp = df ? a.bp + 2 * (long long)j * n : nullptr;
       // wide staging: all 2K products of a tile by its CTA, the columns of x
-      // staged once, the operator rows up to seven at a time
+      // staged once, the operator rows as many at a time as there are slots
       for (int t = bid; t < ntiles && wide; t += G) {
         const int i0 = (t / nt) * kLT, j0 = (t % nt) * kLT;
-        constexpr int kRows = kLWideSlots - 1;
-        for (int b0 = 0; b0 < 2 * K; b0 += kRows) {
-          const int nb = min(kRows, 2 * K - b0);
+        const int rows = lz_slots(c) - 1;
+        for (int b0 = 0; b0 < 2 * K; b0 += rows) {
+          const int nb = min(rows, 2 * K - b0);
           if (df) {
             if (b0 == 0) wide_cols(wide_slot(lz_dyn, 0, c), xp, n, c, j0);
             for (int u = 0; u < nb; ++u)
@@ -1247,14 +1249,15 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
       if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
       // phase B: w = o_0 x + x o_1^T + sum_k Y_k B_k1^T + Y_{K+k} A_k1^T on the
       // owned tiles, then their projections on basis_0..j and |w|^2
-      // wide staging: the operand tiles of up to four terms in one round
+      // wide staging: the operand tiles of several terms in one round
       for (int t = bid; t < ntiles && wide; t += G) {
         const int i0 = (t / nt) * kLT, j0 = (t % nt) * kLT;
         float a0h = 0.f, a0l = 0.f, a1h = 0.f, a1l = 0.f;
         double a0 = 0.0, a1 = 0.0;
         const int nterms = 2 + 2 * K;
-        for (int t0 = 0; t0 < nterms; t0 += kLWideSlots / 2) {
-          const int tn = min(kLWideSlots / 2, nterms - t0);
+        const int terms = lz_slots(c) / 2;
+        for (int t0 = 0; t0 < nterms; t0 += terms) {
+          const int tn = min(terms, nterms - t0);
           for (int u = 0; u < tn; ++u) {
             const int term = t0 + u;
             float* Ls = wide_slot(lz_dyn, 2 * u, c);
