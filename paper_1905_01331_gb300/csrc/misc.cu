@@ -120,13 +120,16 @@ __global__ void polar_start_kernel(const double* G, const double* W, double* X, 
       a += __shfl_xor_sync(0xffffffffu, a, o);
       c += __shfl_xor_sync(0xffffffffu, c, o);
     }
-    if (threadIdx.x == 0) { sums[0] = a; sums[1] = c; }
+    // the two scalars by one warp: repeated by all eight, the square roots and
+    // the division took longer than the elements (an FP64 warp instruction
+    // occupies the SM's two FP64 units for 16 clocks)
+    const double f2 = a;
+    const double s = mu * sqrt(f2);
+    const double nrm2 = f2 - 2.0 * s * c + s * s * P;
+    if (threadIdx.x == 0) { sums[0] = s; sums[1] = nrm2 > 0.0 ? 1.0 / sqrt(nrm2) : 0.0; }
   }
   __syncthreads();
-  const double f2 = sums[0];
-  const double s = mu * sqrt(f2);
-  const double nrm2 = f2 - 2.0 * s * sums[1] + s * s * P;
-  const double inv = nrm2 > 0.0 ? 1.0 / sqrt(nrm2) : 0.0;
+  const double s = sums[0], inv = sums[1];
   const double* g = G + b * elems;
   const double* w = W + b * elems;
   double* x = X + b * elems;
