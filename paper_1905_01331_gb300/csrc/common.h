@@ -93,6 +93,7 @@ struct GemmDesc {
   int digits;        // FP64 products: the digit engine (gemm_oz.cu) where it is supported
   unsigned* words;   // its scratch (oz_scratch(d) bytes) and the bytes there are
   size_t words_bytes;
+  float* c32;        // digit engine: also the FP32 copy of C (may be null; splits == 1)
   int occ;           // TMA-fed kernel: 2 = the 96 KB stage ring (two CTAs per
                      // SM), else the 192 KB ring (one CTA per SM)
 };
@@ -156,6 +157,7 @@ int dot_self_and_cross_partial(const double* x, const double* y, long long n, lo
 // Polar start: per batch b (P x N rows), with fro2 = |G|^2 and gw = <G, W>
 // summed from the partial sums `part` of dot_self_and_cross_partial:
 //   s = mu * sqrt(fro2);  X = (G - s W) / sqrt(fro2 - 2 s gw + s^2 P).
+// both: X in FP64 as well as its pairs.
 // zero (may be null): set to 0 by the launch (a flag that later kernels OR into).
 // With xh, xl (one batch only) X is written as FP32 pairs for the double-float
 // products instead (xh = fl32(X), xl = fl32(X - xh); X itself is not written).
@@ -164,7 +166,7 @@ int dot_self_and_cross_partial(const double* x, const double* y, long long n, lo
 int polar_start(const double* G, const double* W, double* X, long long elems, int nb,
                 int P, double mu, const double* part, cudaStream_t s, float* xh = nullptr,
                 float* xl = nullptr, int* zero = nullptr, const int* try_first = nullptr,
-                int* run_full = nullptr, int* zero2 = nullptr);
+                int* run_full = nullptr, int* zero2 = nullptr, bool both = false);
 
 // For one P x P matrix A: (ph, pl) = FP32 pair of a I - c A (a = 0, c = -1:
 // of A itself, as df_split), with flag: flag |= 1 when max |A - I| > thr, and
@@ -251,6 +253,7 @@ struct ComposeArgs {
   // returns at once (the block is then one Newton-Schulz step, corrected on
   // the tensor cores)
   const int* shortcut = nullptr;
+  double* F64 = nullptr;   // double-float kernel (NJ = 1): F also as FP64 (may be null)
 };
 bool compose_supported(int P, int nsteps);
 
@@ -355,6 +358,13 @@ struct GramCheck {
   double thr2 = 0.0;     // flag2 |= 1 when max |C - I| > thr2 (flag2 may be null)
   int* flag2 = nullptr;
 };
+// C (P x P, FP64) = X X^T for X (P x n2, FP64) on the digit engine, with the
+// check over C in the split-K reduction; scratch as in GemmDesc.  oz_gram_ok:
+// whether the size is one for it.  Returns the launches, or -1 (scratch too
+// small: nothing launched).
+bool oz_gram_ok(int P, long long n2);
+GemmDesc oz_gram_desc(const double* X, int P, long long n2, double* C);
+int oz_gram(GemmDesc d, const int* run_if, const GramCheck& chk, cudaStream_t s);
 // C (P x P, FP64) = X X^T for X (P x n2, row-major) given as (Xh, Xl).
 // run_if (device, may be null): when it points to 0 the launches return at once.
 // chk (may be null): also the check_split pass over C, with the same results

@@ -15,6 +15,7 @@
 // Newton-Schulz step in the same arithmetic brings the isometry defect to
 // ~1e-14.
 #include <algorithm>
+#include <cstring>
 
 #include "common.h"
 #include "f64_bits.cuh"
@@ -308,6 +309,37 @@ int df_gram(const float* Xh, const float* Xl, int P, long long n2, double* C, do
             cudaStream_t s, const int* run_if, const GramCheck* chk) {
   return gram_launch<kGramB, kGramT, 2>(Xh, Xl, P, n2, C, part, df_gram_splits(P, (int)n2), s,
                                         run_if, chk);
+}
+
+GemmDesc oz_gram_desc(const double* X, int P, long long n2, double* C) {
+  GemmDesc d;
+  memset(&d, 0, sizeof(d));
+  d.M = P; d.N = P; d.B0 = 1; d.B1 = 1;
+  d.C = C; d.sc_m = P; d.sc_n = 1;
+  d.alpha = 1.0; d.splits = 1; d.digits = 1;
+  Group& g = d.g[0];
+  g.a.p = X; g.a.s_mn = n2; g.a.s_k0 = 1;
+  g.b = g.a;
+  g.K = (int)n2;
+  g.k0_log2 = 30;
+  d.ngroups = 1;
+  return d;
+}
+
+bool oz_gram_ok(int P, long long n2) {
+  const GemmDesc d = oz_gram_desc(nullptr, P, n2, nullptr);
+  return n2 <= (1LL << 30) && gemm_oz_supported(d) && oz_pick_splits(d) > 1;
+}
+
+int oz_gram(GemmDesc d, const int* run_if, const GramCheck& chk, cudaStream_t s) {
+  d.splits = oz_pick_splits(d);
+  d.skip = run_if;
+  d.skip_when_zero = 1;
+  const int n = gemm_oz_launch(d, s);
+  if (n < 0) return n;
+  launch_k(df_reduce_kernel, (int)std::min<long long>(((long long)d.M * d.N + 31) / 32, 8192), 256, 0, s, d.partial,
+           d.splits, d.M, d.N, 1, 0, static_cast<double*>(d.C), (long long)d.N, run_if, chk);
+  return n + 1;
 }
 
 int df_apply(const float* Fh, const float* Fl, const float* Xh, const float* Xl, int P,

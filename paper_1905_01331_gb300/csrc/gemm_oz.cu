@@ -52,6 +52,7 @@
 #include <cuda_fp16.h>
 
 #include "common.h"
+#include "f64_bits.cuh"
 
 namespace ttn {
 
@@ -369,7 +370,9 @@ __device__ __noinline__ void plain_tile(const GemmDesc& d, int b, int b0, int b1
                   pb[k0 * G.b.s_k0 + static_cast<long long>(k1) * G.b.s_k1], acc);
       }
     }
-    *out_ptr(d, b, b0, b1, split, m, n) = acc;
+    double* out = out_ptr(d, b, b0, b1, split, m, n);
+    *out = acc;
+    if (d.c32) d.c32[out - static_cast<double*>(d.C)] = static_cast<float>(acc);
   }
 }
 
@@ -702,7 +705,12 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     const long long sn = d.splits > 1 ? 1 : d.sc_n;
     const int nv = m < d.M ? min(kHalf, d.N - (n0 + half * kHalf)) : 0;
     const bool vec = sn == 1 && nv == kHalf && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
+    float* row32 = d.c32 ? d.c32 + (row - static_cast<double*>(d.C)) : nullptr;   // (splits == 1)
     auto put = [&](int j, double x, double y) {
+      if (row32) {
+        if (j < nv) row32[j * sn] = f64b::to_f32(x);
+        if (j + 1 < nv) row32[(j + 1) * sn] = f64b::to_f32(y);
+      }
       if (vec) {
         *reinterpret_cast<double2*>(row + j) = make_double2(x, y);
       } else {

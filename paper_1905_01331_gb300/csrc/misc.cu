@@ -96,7 +96,7 @@ __global__ void dot_final_kernel(const double* partial, int nb, double* out, con
 __global__ void polar_start_kernel(const double* G, const double* W, double* X, long long elems,
                                    int P, double mu, const double* part, int nb, float* xh,
                                    float* xl, int* zero, const int* try_first, int* run_full,
-                                   int* zero2) {
+                                   int* zero2, bool both) {
   pdl_wait();
   pdl_trigger();
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
@@ -136,12 +136,10 @@ __global__ void polar_start_kernel(const double* G, const double* W, double* X, 
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < elems;
        i += (long long)gridDim.x * blockDim.x) {
     const double v = (g[i] - s * w[i]) * inv;
-    // mixed modes (one batch): only the FP32 pair of X, which is all that the
-    // double-float products read (X itself is not written)
-    if (xh)
-      f64b::split(v, xh[i], xl[i]);
-    else
-      x[i] = v;
+    // mixed modes (one batch): the FP32 pair of X, which the double-float
+    // products read; X itself too when a first try on the digit engine follows
+    if (xh) f64b::split(v, xh[i], xl[i]);
+    if (!xh || both) x[i] = v;
   }
 }
 
@@ -625,11 +623,11 @@ int dot_self_and_cross_partial(const double* x, const double* y, long long n, lo
 
 int polar_start(const double* G, const double* W, double* X, long long elems, int nb, int P,
                 double mu, const double* part, cudaStream_t s, float* xh, float* xl, int* zero,
-                const int* try_first, int* run_full, int* zero2) {
+                const int* try_first, int* run_full, int* zero2, bool both) {
   if (nb != 1) xh = xl = nullptr;
   if (!try_first) run_full = nullptr;
   launch_k(polar_start_kernel, dim3(grid_for(elems, 256, 512), nb), 256, 0, s, G, W, X, elems, P,
-           mu, part, nb, xh, xl, zero, try_first, run_full, zero2);
+           mu, part, nb, xh, xl, zero, try_first, run_full, zero2, both);
   return 1;
 }
 

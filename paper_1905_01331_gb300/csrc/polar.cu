@@ -264,10 +264,11 @@ __device__ __forceinline__ void xform_elem(float& mh, float& ml, int i, int k, f
 //   pass issued before any of them is transformed and stored;
 //   OU = P-rows x U-columns when U, OV = R-rows x V-columns when V (each K
 //   range cut into 8 interleaved slices, one per warp, added in warp order);
-//   OE (when given) = the tile of Pm itself (F_1 = Pm_0).
+//   OE (when given) = the tile of Pm itself (F_1 = Pm_0); O64 (when given): the
+//   tile of OU also in FP64.
 __device__ void df_item(const DFSmem& sm, int P, int ld, const float* A, bool wantR,
                         const float* U, const float* V, float dh, float dl, float sh, float sl,
-                        int i0, int j0, float* OU, float* OV, float* OE) {
+                        int i0, int j0, float* OU, float* OV, float* OE, double* O64) {
   constexpr int kBatch = 4;
   const long long PP = (long long)P * P;
   const int total = kCT * P;
@@ -373,6 +374,7 @@ __device__ void df_item(const DFSmem& sm, int P, int ld, const float* A, bool wa
         pair_add(rh, rl, red[w * kT2 + e], red[(kCWarps + w) * kT2 + e], rh, rl);
       __stcg(out + (long long)gi * P + gj, rh);
       __stcg(out + PP + (long long)gi * P + gj, rl);
+      if (O64 && q == 0) O64[(long long)gi * P + gj] = f64b::from_f32(rh) + f64b::from_f32(rl);
     }
   } else if (q == 2 && OE && gi < P && gj < P) {
     __stcg(OE + (long long)gi * P + gj, sm.Ph[(e / kCT) * ld + gj]);
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(kCThreads) polar_compose_df_kernel(const Compo
       df_item(sm, P, ld, Aj + b * P2, !last, j > 0 ? Fj + b * P2 : nullptr,
               last ? nullptr : Aj + b * P2, alh, all, mbh, mbl, ti * kCT, tj * kCT,
               j > 0 ? Fn + b * P2 : nullptr, last ? nullptr : T + b * P2,
-              j == 0 ? Fn + b * P2 : nullptr);
+              j == 0 ? Fn + b * P2 : nullptr, last && j > 0 ? a.F64 : nullptr);
       if (!last) df_signal(cT + tj, nullptr);
       else __syncthreads();   // the staged rows are read by the stores above
     }
@@ -461,7 +463,7 @@ __global__ void __launch_bounds__(kCThreads) polar_compose_df_kernel(const Compo
       const int b = it / ntt, ti = (it % ntt) / nt, tj = it % nt;
       if (!df_wait(sm, cT + tj, per_block * (j + 1), nullptr, 0, a.err, max_spin)) return;
       df_item(sm, P, ld, Aj + b * P2, false, T + b * P2, nullptr, alh, all, mbh, mbl, ti * kCT,
-              tj * kCT, An + b * P2, nullptr, nullptr);
+              tj * kCT, An + b * P2, nullptr, nullptr, nullptr);
       df_signal(rA + ti, cA + tj);
     }
   }

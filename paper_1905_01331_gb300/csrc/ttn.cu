@@ -969,7 +969,7 @@ void df_end(ttn_ctx* h, int launches, double flops, const int* cond = nullptr) {
 // only, device, may be null): when it holds 0 the block is one Newton-Schulz
 // step instead.
 void compose_block(ttn_ctx* h, const PolarBlock& blk, int P, int NJ, bool df,
-                   const int* shortcut = nullptr) {
+                   const int* shortcut = nullptr, double* F64 = nullptr) {
   ComposeArgs a;
   // double-float: A_0 arrives as pairs in pP (split from the FP64 Gram in pA)
   a.A0 = df ? h->pP : h->pA; a.A1 = df ? h->pA : h->pP;
@@ -985,6 +985,7 @@ void compose_block(ttn_ctx* h, const PolarBlock& blk, int P, int NJ, bool df,
   a.max_spin = h->opt.wait_polls;
   a.grid_share = h->profiling ? 1 : (int)h->lanes.size();
   a.shortcut = df ? shortcut : nullptr;
+  a.F64 = df ? F64 : nullptr;
   cudaEvent_t ev[2];
   if (h->profiling) {
     cudaEventCreate(&ev[0]);
@@ -1050,6 +1051,12 @@ void polar(ttn_ctx* h, Instance& I, int t, int prec, const double* Gam) {
   const int nT = std::max(I.T, 1);
   int* try_flag = I.ppred + t;
   int* run_full = try_first ? I.ppred + nT + t : nullptr;
+  // The first try's products over X on the digit engine (gemm_oz.cu), where the
+  // layer is large enough for it: a well-conditioned factor is the same to
+  // 1e-13, at 56 (Gram) and 41 us (apply) where the double-float products take 88
+  // and 127 (P = 128, N = 16384).  The full schedule keeps the double-float
+  // products: the directions it amplifies by up to 1e7 carry their rounding.
+  const bool oz_try = try_first && oz_gram_ok(P, N);
   if (df_ok && !h->measuring && !adaptive)
     h->launches += store_ints(full, nullptr, 1, 1, h->stream);
   // X as FP32 pairs for the double-float products (hi at Xp, lo at Xp + PN),
@@ -1078,7 +1085,7 @@ void polar(ttn_ctx* h, Instance& I, int t, int prec, const double* Gam) {
     h->launches += polar_start(Gam, W, X, PN, NJ, P, h->opt.polar_damping, h->red, h->stream,
                                df_ok ? Xp : nullptr, df_ok ? Xp + PN : nullptr,
                                adaptive ? full : nullptr, try_first ? try_flag : nullptr,
-                               run_full, adaptive ? I.pfar + t : nullptr);
+                               run_full, adaptive ? I.pfar + t : nullptr, oz_try);
   }
   // Mixed modes, layers with P < 32 (short blocks): the whole factor in one
   // CTA in pair arithmetic (small_polar) instead of a Gram, a composition and
@@ -1107,7 +1114,46 @@ void polar(ttn_ctx* h, Instance& I, int t, int prec, const double* Gam) {
   }
   if (df_ok && h->measuring)
     h->partial_cap = std::max<size_t>(h->partial_cap, (size_t)df_gram_splits(P, (int)N) * PP);
-  if (try_first && !h->measuring) {
+  if (oz_try) {
+    // (the same steps on the digit engine: X_0 and X_A in FP64, F in FP64 from
+    // the composition, the head of X_A for the correction's product)
+    double* F64 = h->Yt + PP + (PN + 1) / 2;   // after F's pairs and Corr
+    auto gram = [&](const double* Xg, const GramCheck& c) {
+      GemmDesc d = oz_gram_desc(Xg, P, N, h->pA);
+      if (h->measuring) {
+        h->partial_cap = std::max(h->partial_cap, gemm_partial_elems(d, oz_pick_splits(d)));
+        h->words_cap = std::max(h->words_cap, oz_scratch(d));
+        return;
+      }
+      d.partial = h->partial;
+      d.words = h->words;
+      d.words_bytes = h->words_cap;
+      d.err = h->iflags + 4;
+      df_begin(h);
+      const int n = oz_gram(d, try_flag, c, h->stream);
+      if (n < 0) h->compose_refused = true;   // cannot happen after planning
+      df_end(h, std::max(n, 0), 2.0 * P * P * (double)N, try_flag);
+    };
+    GramCheck g0;
+    g0.ph = reinterpret_cast<float*>(h->pP);
+    g0.pl = g0.ph + PP;
+    gram(X, g0);
+    if (!h->measuring) compose_block(h, h->polar_first[0], P, NJ, true, try_flag, F64);
+    GemmDesc f = desc(P, (int)N, 1, 1, X2, N, 1, 0, 0);
+    add(f, grp(op(F64, P, 1), op(X, 1, N), P));
+    f.skip = try_flag;
+    f.skip_when_zero = 1;
+    f.c32 = Xp2;
+    const bool digits = h->digits;
+    h->digits = true;
+    run(h, f, 0);
+    h->digits = digits;
+    GramCheck g1 = g0;
+    g1.thr = kPolarNear;
+    g1.flag = run_full;
+    g1.d32 = Dc;
+    gram(X2, g1);
+  } else if (try_first && !h->measuring) {
     // The first try (every launch returns at once unless *try_flag): Gram
     // matrix of X_0 (its pairs for the composition), the short block's
     // composition, X_A = F X_0 into X2 and Xp2 (X_0 stays in Xp for the full
