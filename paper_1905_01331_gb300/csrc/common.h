@@ -216,6 +216,11 @@ int add_identity_part(void* Z, const void* W, int f32, long long elems, int node
 // identity-free operators.
 int top_grad(double* out, const double* w, const double* v, long long n, const double* e,
              int per_node, cudaStream_t s);
+// dst[off + i] = src[i] for i < n, where *slot holds dst (device): the gradient of
+// a captured pass goes to the caller's buffer of each call.
+int store_at(double* const* slot, long long off, const double* src, long long n, cudaStream_t s);
+// *slot = p
+int set_slot(double** slot, double* p, cudaStream_t s);
 // y = sign * x / sqrt(nrm2[0]).
 int scale_normalise(const double* x, double* y, long long n, const double* nrm2, double sign,
                     cudaStream_t s);

@@ -758,6 +758,35 @@ int scale_normalise(const double* x, double* y, long long n, const double* nrm2,
   return 1;
 }
 
+namespace {
+__global__ void store_at_kernel(double* const* slot, long long off, const double* src, long long n) {
+  pdl_wait();
+  pdl_trigger();
+  double* dst = *slot + off;
+  const long long step = (long long)gridDim.x * blockDim.x;
+  long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  for (; i + 3 * step < n; i += 4 * step) {
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = src[i + q * step];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) dst[i + q * step] = v[q];
+  }
+  for (; i < n; i += step) dst[i] = src[i];
+}
+__global__ void set_slot_kernel(double** slot, double* p) { *slot = p; }
+}  // namespace
+
+int store_at(double* const* slot, long long off, const double* src, long long n, cudaStream_t s) {
+  launch_k(store_at_kernel, grid_for(n, 256, 1216), 256, 0, s, slot, off, src, n);
+  return 1;
+}
+
+int set_slot(double** slot, double* p, cudaStream_t s) {
+  set_slot_kernel<<<1, 1, 0, s>>>(slot, p);
+  return 1;
+}
+
 int top_grad(double* out, const double* w, const double* v, long long n, const double* e,
              int per_node, cudaStream_t s) {
   launch_k(top_grad_kernel, grid_for(n), 256, 0, s, out, w, v, n, e, per_node);

@@ -167,8 +167,18 @@ struct Lane {
   SubStreams sub;
 };
 
+// A captured energy or gradient pass: the first call of a kind runs eagerly, the
+// second is captured, later ones replay it.
+struct PassGraph {
+  int calls = 0;
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+};
+
 struct ttn_ctx {
   ttn_options opt;
+  std::map<int, PassGraph> passes;    // by pass_key
+  double** grad_slot = nullptr;       // device: where the current gradient goes
   std::vector<Lane> lanes;            // lanes[0].stream == stream
   std::vector<int> lane_of;           // lane of each instance
   cudaEvent_t ev_fork = nullptr;
@@ -1477,7 +1487,8 @@ void adjoints_only(ttn_ctx* h, Instance& I, int down_to) {
 // respect to every tensor (laid out as ttn_env with layer -1), with the
 // contractions of the ascend, environment and descend in precision prec (the
 // top contraction, the top adjoints and the energy FP64).
-void value_and_grad(ttn_ctx* h, Instance& I, int prec, double* energy_out, double* grad) {
+// The gradient goes to the buffer whose address h->grad_slot holds.
+void value_and_grad(ttn_ctx* h, Instance& I, int prec, double* energy_out, bool grad) {
   forward(h, I, prec);
   energy_only(h, I, energy_out);
   if (!grad) return;
@@ -1486,8 +1497,9 @@ void value_and_grad(ttn_ctx* h, Instance& I, int prec, double* energy_out, doubl
   for (int t = 0; t < I.T; ++t) off += I.w_elems(t);
   if (!h->measuring) {
     top_matvec(h, I, I.V, h->lz_w, nullptr);
-    h->launches += top_grad(grad + off, h->lz_w, I.V, c2, I.eoff[I.T], I.per_node ? 1 : 0,
+    h->launches += top_grad(h->lz_tmp, h->lz_w, I.V, c2, I.eoff[I.T], I.per_node ? 1 : 0,
                             h->stream);
+    h->launches += store_at(h->grad_slot, off, h->lz_tmp, c2, h->stream);
   } else {
     top_matvec(h, I, I.V, h->lz_w, nullptr);
   }
@@ -1498,9 +1510,7 @@ void value_and_grad(ttn_ctx* h, Instance& I, int prec, double* energy_out, doubl
     off -= I.w_elems(t);
     ensure_ops(h, I, t, prec);
     environment(h, I, t, prec, h->Gam);
-    if (!h->measuring)
-      cudaMemcpyAsync(grad + off, h->Gam, I.w_elems(t) * sizeof(double), cudaMemcpyDeviceToDevice,
-                      h->stream);
+    if (!h->measuring) h->launches += store_at(h->grad_slot, off, h->Gam, I.w_elems(t), h->stream);
     if (t > 0) descend(h, I, t, prec);
   }
 }
@@ -1626,6 +1636,7 @@ void layout(ttn_ctx* h, Arena& ar) {
     save_lane(h, h->lanes[k]);
   }
   h->E_hist = ar.take(4096 * h->inst.size() + 16);
+  h->grad_slot = reinterpret_cast<double**>(ar.take(1));
   load_lane(h, h->lanes[0]);
 }
 
@@ -1638,6 +1649,49 @@ int check_cuda(ttn_ctx* h, cudaError_t e, const char* what) {
   if (e == cudaSuccess) return TTN_OK;
   return fail(h, TTN_ECUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
+
+void destroy_passes(ttn_ctx* h) {
+  for (auto& kv : h->passes) {
+    if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
+    if (kv.second.graph) cudaGraphDestroy(kv.second.graph);
+  }
+  h->passes.clear();
+}
+
+// Run a pass of many small launches (`body` enqueues it on h->stream): eagerly
+// the first time, so that a context used once pays no capture; captured on the
+// second call of its kind and replayed from then on (launches of 2 us instead
+// of 4 to 5, branches in parallel).  A pass that cannot be captured stays eager.
+template <typename Body>
+int run_pass(ttn_ctx* h, int key, Body body) {
+  PassGraph& pg = h->passes[key];
+  ++pg.calls;
+  if (!h->opt.use_graph || pg.calls == 1 || (!pg.exec && pg.calls > 2)) {
+    body();
+    return TTN_OK;
+  }
+  if (!pg.exec) {
+    if (cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) {
+      cudaGetLastError();
+      body();
+      return TTN_OK;
+    }
+    body();
+    if (cudaStreamEndCapture(h->stream, &pg.graph) != cudaSuccess ||
+        cudaGraphInstantiate(&pg.exec, pg.graph, 0) != cudaSuccess) {
+      cudaGetLastError();
+      if (pg.graph) cudaGraphDestroy(pg.graph);
+      pg.graph = nullptr;
+      pg.exec = nullptr;
+      body();
+      return TTN_OK;
+    }
+  }
+  return check_cuda(h, cudaGraphLaunch(pg.exec, h->stream), "graph launch");
+}
+
+// kind 0: energy, 1: energy in precision prec, 2: energy and gradient
+int pass_key(int inst, int prec, int kind) { return (inst * 8 + prec) * 4 + kind; }
 
 int build_instances(ttn_ctx* h, const ttn_problem* probs, int n) {
   for (int i = 0; i < n; ++i) {
@@ -1686,8 +1740,8 @@ void plan(ttn_ctx* h) {
     energy_only(h, I, nullptr);
     isometry_grams(h, I, nullptr);
     if (!I.per_node) leftmost_rdm(h, I, 0);
-    value_and_grad(h, I, h->opt.prec, nullptr, h->Gam);
-    if (h->opt.prec != 0) value_and_grad(h, I, 0, nullptr, h->Gam);
+    value_and_grad(h, I, h->opt.prec, nullptr, true);
+    if (h->opt.prec != 0) value_and_grad(h, I, 0, nullptr, true);
   }
   h->measuring = false;
 }
@@ -2285,8 +2339,11 @@ int ttn_energy(ttn_t h, int inst, double* E) {
   if (!h || !E || inst < 0 || inst >= (int)h->inst.size()) return TTN_EINVAL;
   sync_user(h);
   Instance& I = h->inst[inst];
-  forward(h, I, 0);
-  energy_only(h, I, h->scal + 5);
+  int prc = run_pass(h, pass_key(inst, 0, 0), [&] {
+    forward(h, I, 0);
+    energy_only(h, I, h->scal + 5);
+  });
+  if (prc) return prc;
   int rc = check_cuda(h, cudaMemcpyAsync(E, h->scal + 5, sizeof(double), cudaMemcpyDeviceToHost,
                                          h->stream), "energy");
   if (rc) return rc;
@@ -2301,7 +2358,10 @@ int ttn_value_and_grad(ttn_t h, int inst, int prec, double* E, double* d_grad) {
     return fail(h, TTN_EINVAL, "context was created for FP64 only");
   sync_user(h);
   Instance& I = h->inst[inst];
-  value_and_grad(h, I, prec, h->scal + 5, d_grad);
+  if (d_grad) h->launches += set_slot(h->grad_slot, d_grad, h->stream);
+  const int prc = run_pass(h, pass_key(inst, prec, d_grad ? 2 : 1),
+                           [&] { value_and_grad(h, I, prec, h->scal + 5, d_grad != nullptr); });
+  if (prc) return prc;
   int rc = check_cuda(h, cudaMemcpyAsync(E, h->scal + 5, sizeof(double), cudaMemcpyDeviceToHost,
                                          h->stream), "value_and_grad");
   if (rc) return rc;
@@ -2536,6 +2596,7 @@ int ttn_autotune(ttn_t h, int reps, void* blob, size_t* blob_bytes) {
     // the captured sweep used the previous configurations: capture again
     if (h->exec) { cudaGraphExecDestroy(h->exec); h->exec = nullptr; }
     if (h->graph) { cudaGraphDestroy(h->graph); h->graph = nullptr; }
+    destroy_passes(h);
     if (rc) return rc;
   }
   if (blob_bytes) {
@@ -2570,6 +2631,7 @@ void ttn_destroy(ttn_t h) {
   if (!h) return;
   if (h->exec) cudaGraphExecDestroy(h->exec);
   if (h->graph) cudaGraphDestroy(h->graph);
+  destroy_passes(h);
   if (h->stream) cudaStreamSynchronize(h->stream);
   for (size_t k = 1; k < h->lanes.size(); ++k)
     if (h->lanes[k].stream) {
