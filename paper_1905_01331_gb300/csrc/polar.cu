@@ -45,40 +45,45 @@ struct ComposeSmem {
   int ok;
 };
 
+// x / 2 by the exponent field (the FP64 multiply takes the two FP64 units).
+__device__ __forceinline__ double half_of(double x) {
+  const int hi = __double2hiint(x), e = (hi >> 20) & 0x7FF;
+  if (e <= 1 || e == 0x7FF) return 0.5 * x;     // zero, subnormal, infinite or NaN
+  return __hiloint2double(hi - 0x100000, __double2loint(x));
+}
+
 // Element (r, c) = (tid / 8, tid % 8) of the tile (i0, j0) of X' Y', for
 // threads tid < 64 (0 elsewhere): sum_k X'[i0 + r][k] Y'[k][j0 + c] with
 //     X' = dx I + sx S_x(X),   Y' = dy I + sy S_y(Y),
 // S(M) = (M + M^T)/2 when the flag is set, else M, formed while rows of X and
-// columns of Y are staged.  The K range is cut into 8 interleaved slices (one
-// per warp) whose partial sums are added in warp order.
-__device__ double tile_product(ComposeSmem& sm, const double* X, double dx, double sx, bool symx,
-                               const double* Y, double dy, double sy, bool symy, int P, int i0,
-                               int j0) {
+// columns of Y are staged (scalex, scaley: whether d or s differ from the
+// identity map; staging 2048 values took as long in the FP64 units as the
+// tile's 8192 FMAs do on half of them, so it multiplies only where it must).
+// The K range is cut into 8 interleaved slices (one per warp) whose partial
+// sums are added in warp order.
+__device__ double tile_product(ComposeSmem& sm, const double* X, double dx, double sx, bool scalex,
+                               bool symx, const double* Y, double dy, double sy, bool scaley,
+                               bool symy, int P, int i0, int j0) {
   for (int e = threadIdx.x; e < kCT * P; e += kCThreads) {
-    // rows of X: element (r, k), consecutive threads along k
-    {
-      const int r = e / P, k = e - (e / P) * P;
-      const int gi = i0 + r;
-      double v = 0.0;
-      if (gi < P) {
-        const double x = __ldcg(X + (long long)gi * P + k);
-        const double m = symx ? 0.5 * (x + __ldcg(X + (long long)k * P + gi)) : x;
-        v = sx * m + (gi == k ? dx : 0.0);
-      }
-      sm.X[r][k] = v;
+    // rows of X: element (r, k), consecutive threads along k; columns of Y:
+    // element (k2, c), consecutive threads along c; all loads first
+    const int r = e / P, k = e - (e / P) * P, gi = i0 + r;
+    const int k2 = e / kCT, c = e - (e / kCT) * kCT, gj = j0 + c;
+    double x = 0.0, xt = 0.0, y = 0.0, yt = 0.0;
+    if (gi < P) {
+      x = __ldcg(X + (long long)gi * P + k);
+      if (symx) xt = __ldcg(X + (long long)k * P + gi);
     }
-    // columns of Y: element (k, c), consecutive threads along c
-    {
-      const int k = e / kCT, c = e - (e / kCT) * kCT;
-      const int gj = j0 + c;
-      double v = 0.0;
-      if (gj < P) {
-        const double y = __ldcg(Y + (long long)k * P + gj);
-        const double m = symy ? 0.5 * (y + __ldcg(Y + (long long)gj * P + k)) : y;
-        v = sy * m + (gj == k ? dy : 0.0);
-      }
-      sm.Y[c][k] = v;
+    if (gj < P) {
+      y = __ldcg(Y + (long long)k2 * P + gj);
+      if (symy) yt = __ldcg(Y + (long long)gj * P + k2);
     }
+    if (symx) x = half_of(x + xt);
+    if (scalex) x = gi < P ? sx * x + (gi == k ? dx : 0.0) : 0.0;
+    if (symy) y = half_of(y + yt);
+    if (scaley) y = gj < P ? sy * y + (gj == k2 ? dy : 0.0) : 0.0;
+    sm.X[r][k] = x;
+    sm.Y[c][k2] = y;
   }
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -154,9 +159,10 @@ __global__ void __launch_bounds__(kCThreads) polar_compose_kernel(const ComposeA
       const int ti = (u % ntt) / nt, tj = (u % ntt) % nt;
       const double* Ab = Aj + b * PP;
       const double v = isF
-          ? tile_product(sm, Ab, al, -be, true, Fbuf(j) + b * PP, 0.0, 1.0, false, P, ti * kCT,
-                         tj * kCT)
-          : tile_product(sm, Ab, 0.0, 1.0, true, Ab, al, -be, true, P, ti * kCT, tj * kCT);
+          ? tile_product(sm, Ab, al, -be, true, true, Fbuf(j) + b * PP, 0.0, 1.0, false, false, P,
+                         ti * kCT, tj * kCT)
+          : tile_product(sm, Ab, 0.0, 1.0, false, true, Ab, al, -be, true, true, P, ti * kCT,
+                         tj * kCT);
       store_tile((isF ? Fn : a.T) + b * PP, P, ti, tj, v);
     }
     if (j == 0) {
@@ -175,8 +181,8 @@ __global__ void __launch_bounds__(kCThreads) polar_compose_kernel(const ComposeA
     const int items2 = ntt * a.NJ;
     for (int it = blockIdx.x; it < items2; it += gridDim.x) {
       const int b = it / ntt, ti = (it % ntt) / nt, tj = (it % ntt) % nt;
-      const double v = tile_product(sm, Aj + b * PP, al, -be, true, a.T + b * PP, 0.0, 1.0, false,
-                                    P, ti * kCT, tj * kCT);
+      const double v = tile_product(sm, Aj + b * PP, al, -be, true, true, a.T + b * PP, 0.0, 1.0,
+                                    false, false, P, ti * kCT, tj * kCT);
       store_tile(An + b * PP, P, ti, tj, v);
     }
     target += gridDim.x;
