@@ -909,8 +909,10 @@ int gemm_oz_launch(const GemmDesc& d, cudaStream_t s) {
   pl.op.err = d.err;
   const int bn = oz_bn(d);
   dim3 grid(((d.M + kOBM - 1) / kOBM) * ((d.N + bn - 1) / bn), d.B0 * d.B1, d.splits);
-  if (bn == 64) launch_k(gemm_oz_kernel<64>, grid, kOThreads, oz_smem<64>(), s, d, pl.op);
-  else launch_k(gemm_oz_kernel<32>, grid, kOThreads, oz_smem<32>(), s, d, pl.op);
+  // always with programmatic serialisation: its only predecessor is the
+  // preparation, so its CTAs wait for nothing else
+  if (bn == 64) launch_attr(true, gemm_oz_kernel<64>, grid, kOThreads, oz_smem<64>(), s, d, pl.op);
+  else launch_attr(true, gemm_oz_kernel<32>, grid, kOThreads, oz_smem<32>(), s, d, pl.op);
   return 2;
 }
 
