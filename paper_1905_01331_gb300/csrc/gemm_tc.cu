@@ -706,7 +706,7 @@ __global__ void splitk_reduce_tc(const GemmDesc d) {
 // holds the raw FP32 tiles of A (128 x 32) and B (BN x 32), loaded by TMA
 // (SWIZZLE_128B: the K-major canonical layout of the MMA; an MN-contiguous
 // operand arrives as 32 x 32 boxes and is transposed), converted in place to
-// TF32 heads by four converter warps, which also write the tails of the
+// TF32 heads by eight converter warps, which also write the tails of the
 // split form (BF16 modes: heads and tails as separate tiles of half the size
 // after the raw ones, 64-byte swizzle; the thread-staged kernel took 615 us for
 // the mean product of a chi = 256 Heisenberg sweep, this one 270, in the same
@@ -714,7 +714,12 @@ __global__ void splitk_reduce_tc(const GemmDesc d) {
 // stage and commits its
 // completion to the stage's "empty" barrier, which frees it for the next TMA.
 //   warp 0: TMA producer (one thread)       warp 1: TMEM owner, MMA issuer
-//   warps 2-5: converters, then the epilogue (TMEM lanes 32 (w % 4) ..)
+//   warps 2-9: converters, then the epilogue (TMEM lanes 32 (w % 4) .., half of
+//   the columns)
+// The conversion of a stage is a chain of shared-memory reads, roundings and
+// writes that the MMAs wait for; eight warps instead of four halve it (3xTF32
+// gradient of a 64 x 4 torus at chi = 128: 4.56 against 4.76 ms; BF16x3 sweep at
+// chi = 256: 90.1 against 92.0 ms).
 // Every wait is bounded; an expired wait raises the error flag and the CTA's
 // abort flag, every role then stops, the producer waits (bounded) for the
 // copies it issued, the MMA thread commits so that the epilogue can wait for
@@ -723,8 +728,8 @@ __global__ void splitk_reduce_tc(const GemmDesc d) {
 
 int tc_total_tiles(const GemmDesc& d, int BK);
 
-constexpr int kTThreads = 192;
-constexpr int kTConv = 128;
+constexpr int kTConv = 256;               // converter threads: eight warps
+constexpr int kTThreads = 64 + kTConv;
 constexpr int kTSmem = 196608;           // bytes of the stage ring, one CTA per SM
 constexpr int kTSmem2 = 98304;           // two CTAs per SM
 
@@ -775,18 +780,18 @@ __device__ __forceinline__ void tma_load5(uint32_t dst, const CUtensorMap* map, 
       : "memory");
 }
 
-// Named barrier of the four converter warps (id 1), with an AND vote.
+// Named barrier of the converter warps (id 1), with an AND vote.
 __device__ __forceinline__ bool conv_vote(bool v) {
   uint32_t r;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 128, p;\n\t"
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, %2, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}\n"
       : "=r"(r)
-      : "r"(static_cast<uint32_t>(v))
+      : "r"(static_cast<uint32_t>(v)), "n"(kTConv)
       : "memory");
   return r != 0;
 }
-__device__ __forceinline__ void conv_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+__device__ __forceinline__ void conv_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTConv) : "memory"); }
 
 // TF32 head and tail of four FP32 values (head rounded to nearest).
 template <bool kSplit>
@@ -819,29 +824,29 @@ __device__ __forceinline__ void convert_kmajor(uint8_t* hi, uint8_t* lo, int ct)
 
 // An MN-contiguous operand arrives as ROWS / 32 boxes of 32 K rows x 32 MN
 // values (box j at hi + 4096 j, row k at 128 k, 16-byte chunk c stored at
-// c ^ (k & 7)).  Converter thread ct owns MN row ct: it reads its 32 values,
-// all converter threads meet, and it writes the row in the K-major layout.
+// c ^ (k & 7)).  kTConv / ROWS converter threads share an MN row: each reads its
+// part of the 32 values, all converter threads meet, and it writes the part in
+// the K-major layout.
 template <bool kSplit, int ROWS>
 __device__ __forceinline__ void convert_mnmajor(uint8_t* hi, uint8_t* lo, int ct) {
-  float v[32];
-  const bool active = ct < ROWS;
-  if (active) {
-    const int j = ct >> 5, c = (ct & 31) >> 2, e = ct & 3;
-    const uint8_t* box = hi + 4096 * j;
+  constexpr int kVals = 32 * ROWS / kTConv;
+  const int row = ct % ROWS, k0 = ct / ROWS * kVals;
+  float v[kVals];
+  const int j = row >> 5, c = (row & 31) >> 2, e = row & 3;
+  const uint8_t* box = hi + 4096 * j;
 #pragma unroll
-    for (int k = 0; k < 32; ++k)
-      v[k] = *reinterpret_cast<const float*>(box + 128 * k + ((c ^ (k & 7)) << 4) + 4 * e);
+  for (int q = 0; q < kVals; ++q) {
+    const int k = k0 + q;
+    v[q] = *reinterpret_cast<const float*>(box + 128 * k + ((c ^ (k & 7)) << 4) + 4 * e);
   }
   conv_sync();
-  if (active) {
 #pragma unroll
-    for (int kc = 0; kc < 8; ++kc) {
-      uint4 h, l;
-      split4<kSplit>(v + 4 * kc, h, l);
-      const int off = 128 * ct + ((kc ^ (ct & 7)) << 4);
-      *reinterpret_cast<uint4*>(hi + off) = h;
-      if constexpr (kSplit) *reinterpret_cast<uint4*>(lo + off) = l;
-    }
+  for (int q = 0; q < kVals / 4; ++q) {
+    uint4 h, l;
+    split4<kSplit>(v + 4 * q, h, l);
+    const int off = 128 * row + (((k0 / 4 + q) ^ (row & 7)) << 4);
+    *reinterpret_cast<uint4*>(hi + off) = h;
+    if constexpr (kSplit) *reinterpret_cast<uint4*>(lo + off) = l;
   }
 }
 
@@ -929,18 +934,21 @@ __device__ __forceinline__ void convert_bf16(const uint8_t* raw, bool mn, uint8_
       }
       store_bf16<kSplit>(hi, lo, r, c, x);
     }
-  } else if (ct < ROWS) {
-    const int j = ct >> 5, c = (ct & 31) >> 2, e = ct & 3;
+  } else {
+    constexpr int kChunks = 4 * ROWS / kTConv;    // chunks of eight K values per thread
+    const int row = ct % ROWS, kc0 = ct / ROWS * kChunks;
+    const int j = row >> 5, c = (row & 31) >> 2, e = row & 3;
     const uint8_t* box = raw + 4096 * j;
 #pragma unroll
-    for (int kc = 0; kc < 4; ++kc) {
+    for (int kk = 0; kk < kChunks; ++kk) {
+      const int kc = kc0 + kk;
       float x[8];
 #pragma unroll
       for (int q = 0; q < 8; ++q) {
         const int k = 8 * kc + q;
         x[q] = *reinterpret_cast<const float*>(box + 128 * k + ((c ^ (k & 7)) << 4) + 4 * e);
       }
-      store_bf16<kSplit>(hi, lo, ct, kc, x);
+      store_bf16<kSplit>(hi, lo, row, kc, x);
     }
   }
 }
@@ -1170,8 +1178,9 @@ __global__ void __launch_bounds__(kTThreads, kRing == kTSmem ? 1 : 2)
       const int row = quarter * 32 + lane;
       const int m = m0 + row;
       const float af = static_cast<float>(d.alpha), bf = static_cast<float>(d.beta);
+      const int c_lo = ((warp - 2) >> 2) * (BN / 2);   // two warps per 32 rows
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 16) {
+      for (int c0 = c_lo; c0 < c_lo + BN / 2; c0 += 16) {
         uint32_t r[16];
         if (nk == 0) {
 #pragma unroll
