@@ -48,6 +48,7 @@
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
+#include <utility>
 
 #include <cuda_fp16.h>
 
@@ -65,6 +66,7 @@ constexpr int kOBK = 32;            // K values per stage
 constexpr int kOConv = 256;         // converter threads
 constexpr int kOThreads = kOConv + 128;   // and the warpgroup of the MMA and image warps
 constexpr long kOWait = 1L << 22;
+constexpr int kOBlocks = 24;        // 16-column blocks of a CTA of the streamed kernel at most
 
 // Magnitude of an operand: `parts` words (the high words of |x|, at least 1 for
 // a nonzero x) per batch, at word off + (b0 s0 + b1 s1) parts.  img >= 0: the
@@ -80,6 +82,7 @@ struct OzParams {
   const uint8_t* images;
   OzOperand a[kMaxGroups], b[kMaxGroups];
   int total_chunks;
+  int blocks, nb16;                 // streamed kernel: 16-column blocks in all and per row tile
   int* err;
 };
 
@@ -131,16 +134,14 @@ __device__ __forceinline__ uint32_t digit_pair(uint32_t w0, uint32_t w1) {
 }
 
 // Eight consecutive K values of row r -> 16-byte chunk c (of four) of every
-// digit tile: rows of 64 bytes, 64-byte swizzle, tiles of ROWS rows.
-template <int ROWS>
-__device__ __forceinline__ void store_digits(const double* v, int emax, uint8_t* tile, int r, int c) {
+// digit tile: rows of 64 bytes, 64-byte swizzle, tiles `stride` bytes apart.
+__device__ __forceinline__ void store_digits(const double* v, int emax, uint8_t* tile, int r, int c, int stride) {
   uint32_t lo[8], hi[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) digit_bytes(v[q], emax, lo[q], hi[q]);
   uint8_t* p = tile + r * 64 + ((c ^ ((r >> 1) & 3)) << 4);
-  constexpr int kTile = ROWS * 64;
 #define TTN_OZ_DIGIT(d, w, b)                                                              \
-  *reinterpret_cast<uint4*>(p + (d) * kTile) =                                             \
+  *reinterpret_cast<uint4*>(p + (d) * stride) =                                            \
       make_uint4(digit_pair<b>(w[0], w[1]), digit_pair<b>(w[2], w[3]),                     \
                  digit_pair<b>(w[4], w[5]), digit_pair<b>(w[6], w[7]));
   TTN_OZ_DIGIT(0, hi, 3) TTN_OZ_DIGIT(1, hi, 2) TTN_OZ_DIGIT(2, hi, 1) TTN_OZ_DIGIT(3, hi, 0)
@@ -205,7 +206,7 @@ __device__ __forceinline__ void image_block(const AbsItem& it, const double* p, 
     task_pos<ROWS>(task, kf, r, c);
     double v[8];
     load8(it.s_mn, it.s_k0, it.s_k1, it.k0_log2, p, r0 + r, r0 + r < it.mn, k + 8 * c, it.k, vec, v);
-    store_digits<ROWS>(v, emax, out, r, c);
+    store_digits(v, emax, out, r, c, ROWS * 64);
   }
 }
 
@@ -349,11 +350,10 @@ __device__ __forceinline__ double* out_ptr(const GemmDesc& d, int b, int b0, int
 
 // Plain FP64 tile over the CTA's chunks (operands with infinities or NaN, or a
 // range that the digits do not cover).
-template <int BN>
-__device__ __noinline__ void plain_tile(const GemmDesc& d, int b, int b0, int b1, int split, int m0, int n0,
+__device__ __noinline__ void plain_tile(const GemmDesc& d, int b, int b0, int b1, int split, int m0, int n0, int bn,
                                         int c_lo, int c_hi) {
-  for (int e = threadIdx.x; e < kOBM * BN; e += kOThreads) {
-    const int m = m0 + e / BN, n = n0 + e % BN;
+  for (int e = threadIdx.x; e < kOBM * bn; e += kOThreads) {
+    const int m = m0 + e / bn, n = n0 + e % bn;
     if (m >= d.M || n >= d.N) continue;
     double acc = 0.0;
     int c = 0;
@@ -376,17 +376,25 @@ __device__ __noinline__ void plain_tile(const GemmDesc& d, int b, int b0, int b1
   }
 }
 
-// Combine four columns' accumulators (levels l of columns cb .. cb + 3) into
-// 96-bit integers, shifted right by sh.
-template <int BN>
-__device__ __forceinline__ void combine4(uint32_t taddr, int sh, uint32_t (&v)[4][3]) {
-  uint32_t r[kOD][4];
+// The accumulators of four columns: levels l, `cols` columns apart.  (The
+// registers hold them after ld_wait.)
+__device__ __forceinline__ void ld_levels(uint32_t taddr, int cols, uint32_t (&r)[kOD][4]) {
 #pragma unroll
   for (int l = 0; l < kOD; ++l)
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r[l][0]), "=r"(r[l][1]), "=r"(r[l][2]), "=r"(r[l][3])
-                 : "r"(taddr + l * BN));
+                 : "r"(taddr + l * cols));
+}
+// The loads of r are complete (r as operands: nothing reads it before).
+__device__ __forceinline__ void ld_wait(uint32_t (&r)[kOD][4]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int l = 0; l < kOD; ++l)
+    asm volatile("" : "+r"(r[l][0]), "+r"(r[l][1]), "+r"(r[l][2]), "+r"(r[l][3]));
+}
+
+// Combine four columns' accumulators into 96-bit integers, shifted right by sh.
+__device__ __forceinline__ void combine4(const uint32_t (&r)[kOD][4], int sh, uint32_t (&v)[4][3]) {
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     // levels 0 to 2 are at most 2^22 (digit 0 is at most 64): their integers sit
@@ -533,7 +541,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     sref = max(sref, s);
   }
   if (sref != -100000 && (sref < -1000 || sref > 900)) plain = true;
-  if (plain) plain_tile<BN>(d, b, b0, b1, split, m0, n0, c_lo, c_hi);
+  if (plain) plain_tile(d, b, b0, b1, split, m0, n0, BN, c_lo, c_hi);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
   volatile int* abort_v = &abort_flag;
@@ -644,7 +652,10 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
 #pragma unroll
       for (int cb = 0; cb < kHalf; cb += 4) {
         uint32_t v[4][3];
-        combine4<BN>(trow + cb, sh, v);
+        uint32_t r[kOD][4];
+        ld_levels(trow + cb, BN, r);
+        ld_wait(r);
+        combine4(r, sh, v);
 #pragma unroll
         for (int j = 0; j < 4; ++j)
           asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
@@ -681,11 +692,11 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
             k += kOBK;
             if (k >= d.g[g].K) { ++g; k = 0; enter(); }
           }
-          if (cb) store_digits<BN>(vb, eb, sB, cbr, cbc);
+          if (cb) store_digits(vb, eb, sB, cbr, cbc, kB);
           if (!last && b_on) load_b();
 #pragma unroll
           for (int q = 0; q < kATasks; ++q) {
-            if (ca) store_digits<kOBM>(va[q], ea, sA, car[q], cac[q]);
+            if (ca) store_digits(va[q], ea, sA, car[q], cac[q], kA);
             if (!last && a_on) load_a(q);
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -728,7 +739,10 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
 #pragma unroll 1
         for (int cb = 0; cb < kHalf; cb += 4) {
           uint32_t v[4][3];
-          combine4<BN>(trow + cb, sh, v);
+          uint32_t r[kOD][4];
+          ld_levels(trow + cb, BN, r);
+          ld_wait(r);
+          combine4(r, sh, v);
 #pragma unroll
           for (int j = 0; j < 4; j += 2)
             put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
@@ -749,6 +763,301 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   __syncthreads();
   if (warp == 8)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
+}
+
+
+// Streamed products: one chunk of K, ready digits of A, more tiles than SMs.  A
+// CTA takes an equal share of all 16-column blocks, in sub-tiles of at most 64
+// columns of one row tile: every sub-tile's first two stages are staged before
+// the one before it is combined, and no SM waits in a second round of tiles.
+// With A ready, a converter thread has one task per stage where a tile that
+// converts both operands has three.  256 tiles on 152 SMs are two rounds of 24 k
+// clocks; 112 columns per CTA (64 + 48) are 39 k.  FP64 sweep at chi = 128: 25.57
+// -> 25.29 ms, FP64 measurement of a Heisenberg chain: 3.44 -> 3.35 ms (the
+// exchange of sides alone: 25.55 and 3.41); the sums are the same.
+struct OzSub {
+  int b, m0, n0, bn;
+};
+
+__global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const GemmDesc d, const OzParams op) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int kMaxN = 64;
+  constexpr int kA = kOBM * 64;                    // bytes of one digit tile of A of a stage
+  constexpr int kStage = kOD * (kA + kMaxN * 64);
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  __shared__ __align__(8) uint64_t full_bar[2], empty_bar[2], done_bar, free_bar, drain_bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ int abort_flag, plain_flag;
+  __shared__ OzSub subs[kOBlocks];
+  __shared__ int eb_s[kOBlocks], sref_s[kOBlocks];   // exponents of a sub-tile's B and of its sums
+
+  if (desc_skipped(d)) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int blk_lo = static_cast<int>(static_cast<long long>(op.blocks) * blockIdx.x / gridDim.x);
+  const int blk_hi = static_cast<int>(static_cast<long long>(op.blocks) * (blockIdx.x + 1) / gridDim.x);
+  const int tiles_m = (d.M + kOBM - 1) / kOBM;
+  auto sub_at = [&](int blk, OzSub& u) {
+    const int row = blk / op.nb16, nb = blk - row * op.nb16;
+    const int q = min(min(kMaxN / 16, op.nb16 - nb), blk_hi - blk);
+    u.b = row / tiles_m;
+    u.m0 = (row - u.b * tiles_m) * kOBM;
+    u.n0 = nb * 16;
+    u.bn = q * 16;
+    return blk + q;
+  };
+  int nsub = 0;
+  for (int blk = blk_lo; blk < blk_hi; ++nsub) {
+    OzSub u;
+    blk = sub_at(blk, u);
+    if (threadIdx.x == 0) subs[nsub] = u;
+  }
+  if (nsub == 0) return;
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(osmem(&tmem_slot)), "r"(kOD * kMaxN));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  const Group& G = d.g[0];
+  const OzOperand &oa = op.a[0], &ob = op.b[0];
+  const int nst = (G.K + kOBK - 1) / kOBK;         // at most 4
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < 2; ++s) {
+      omb_init(&full_bar[s], kOConv + 1);
+      omb_init(&empty_bar[s], 1);
+    }
+    omb_init(&done_bar, 1);
+    omb_init(&drain_bar, 1);
+    omb_init(&free_bar, kOConv);
+    abort_flag = 0;
+    plain_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+
+  // converter state: the values of the next stage (loaded a stage ahead), their
+  // row and chunk
+  const int t = threadIdx.x;
+  const bool bkf = G.b.s_k0 == 1;
+  double vb[8];
+  const double* pb = nullptr;
+  bool bvec = false, b_on = false;
+  int br = 0, bc = 0, k = 0, blk_next = 0;
+  OzSub cur{};                                      // the sub-tile whose stages are loaded
+  auto enter = [&]() {
+    pb = static_cast<const double*>(G.b.p) + (cur.b % d.B0) * G.b.s_b0 + static_cast<long long>(cur.b / d.B0) * G.b.s_b1;
+    bvec = bkf && ((reinterpret_cast<uintptr_t>(pb) & 15) == 0) && ((G.b.s_mn | G.b.s_k1) & 1) == 0;
+    b_on = t < cur.bn * 4;
+    // K contiguous: eight rows by four chunks per warp; MN contiguous: consecutive rows of one chunk
+    if (bkf) {
+      br = t >> 2;
+      bc = t & 3;
+    } else {
+      bc = t / cur.bn;
+      br = t - bc * cur.bn;
+    }
+  };
+  auto load_b = [&]() {
+    if (b_on)
+      load8(G.b.s_mn, G.b.s_k0, G.b.s_k1, G.k0_log2, pb, cur.n0 + br, cur.n0 + br < d.N, k + 8 * bc, G.K, bvec, vb);
+  };
+  if (warp < 8) {
+    blk_next = sub_at(blk_lo, cur);
+    enter();
+    load_b();
+  }
+  __syncthreads();
+  // magnitudes: the exponents of every sub-tile's operands (a batch once)
+  for (int u = warp; u < nsub; u += kOThreads / 32) {
+    const int b0 = subs[u].b % d.B0, b1 = subs[u].b / d.B0;
+    unsigned w[2];
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const OzOperand& o = side ? ob : oa;
+      const unsigned* p = op.words + o.off + static_cast<long long>(b0 * o.s0 + b1 * o.s1) * o.parts;
+      unsigned m = 0;
+      for (int q = lane; q < o.parts; q += 32) m = max(m, __ldcg(p + q));
+      w[side] = __reduce_max_sync(0xffffffffu, m);
+    }
+    if (lane == 0) {
+      const int ea = w[0] >> 20, eb = w[1] >> 20;
+      // the scale of the digit products is 2^(ea + eb - 68); an all-zero operand gives zero digits
+      const bool zero = w[0] == 0u || w[1] == 0u;
+      const int sref = zero ? -100000 : ea + eb - 2 * 1022 - 68;
+      eb_s[u] = w[1] ? eb : 1023;
+      sref_s[u] = sref;
+      if (ea >= 0x7FF || eb >= 0x7FF || (!zero && (ea < 80 || eb < 80 || sref < -1000 || sref > 900))) plain_flag = 1;
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  const bool plain = plain_flag != 0;
+  if (plain)
+    for (int u = 0; u < nsub; ++u)
+      plain_tile(d, subs[u].b, subs[u].b % d.B0, subs[u].b / d.B0, 0, subs[u].m0, subs[u].n0, subs[u].bn, 0, 1);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+  volatile int* abort_v = &abort_flag;
+
+  if (plain) {
+    // (the tiles are done)
+  } else if (warp == 8) {
+    if (lane == 0) {
+      // ---- MMA issuer ----
+      bool ok = true;
+      int it = 0;
+      const uint32_t base = osmem(smem);
+      for (int u = 0; u < nsub && ok; ++u) {
+        const int bn = subs[u].bn;
+        if (u > 0 && !omb_wait(&free_bar, (u - 1) & 1, abort_v)) { ok = false; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        for (int st = 0; st < nst; ++st, ++it) {
+          const int s = it & 1;
+          if (!omb_wait(&full_bar[s], (it >> 1) & 1, abort_v)) { ok = false; break; }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t sa = base + s * kStage, sb = sa + kOD * kA;
+#pragma unroll 1
+          for (int j = 0; j < 2; ++j) {
+#pragma unroll
+            for (int i = 0; i < kOD; ++i) {
+              const uint64_t ad = odesc(sa + i * kA + j * 32);
+              const uint32_t acc = (st > 0 || j > 0 || i > 0) ? 1u : 0u;
+              // digits 0 .. 7 - i of B in pieces of at most 256 columns
+              const int cols = (kOD - i) * bn;
+              omma(tmem + i * bn, ad, odesc(sb + j * 32), oidesc(min(256, cols)), acc);
+              if (cols > 256)
+                omma(tmem + i * bn + 256, ad, odesc(sb + 256 * 64 + j * 32), oidesc(cols - 256), acc);
+            }
+          }
+          ocommit(&empty_bar[s]);
+        }
+        ocommit(&done_bar);
+      }
+      if (!ok) {
+        *abort_v = 1;
+        if (op.err) atomicOr(op.err, 1);
+        // the MMAs issued so far must be complete before TMEM is freed
+        ocommit(&drain_bar);
+        omb_wait(&drain_bar, 0, nullptr);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 9) {
+    if (lane == 0) {
+      // ---- A: one bulk copy of ready digits per stage ----
+      bool ok = true;
+      int it = 0;
+      const uint32_t base = osmem(smem);
+      for (int u = 0; u < nsub && ok; ++u) {
+        const int b0 = subs[u].b % d.B0, b1 = subs[u].b / d.B0;
+        const uint8_t* src = op.images + oa.img +
+            (static_cast<long long>(b0 * oa.s0 + b1 * oa.s1) * oa.nrt + subs[u].m0 / kOBM) * oa.nks * (kOD * kA);
+        for (int st = 0; st < nst; ++st, ++it) {
+          const int s = it & 1;
+          if (it >= 2 && !omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v)) { ok = false; break; }
+          omb_expect(&full_bar[s], kOD * kA);
+          bulk_load(base + s * kStage, src + st * (kOD * kA), kOD * kA, &full_bar[s]);
+        }
+      }
+      if (!ok) *abort_v = 1;
+      // copies in flight land before the CTA exits, also after an abort
+      for (int q = max(0, it - 2); q < it; ++q) omb_wait(&full_bar[q & 1], (q >> 1) & 1, nullptr);
+    }
+    __syncwarp();
+  } else if (warp < 8) {
+    // ---- converters; each sub-tile is combined and stored once two stages of the next are staged ----
+    const int quarter = warp & 3, half = warp >> 2;
+    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+    bool ok = true;
+    auto flush = [&](int u) {
+      ok = __all_sync(0xffffffffu, ok && omb_wait(&done_bar, u & 1, abort_v));
+      if (!ok) return;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const OzSub w = subs[u];
+      const int sref = sref_s[u], hc = w.bn >> 1;     // this warp's columns: 8, 16, 24 or 32
+      const uint32_t tcol = trow + half * hc;
+      const int m = w.m0 + quarter * 32 + lane, nf = w.n0 + half * hc;
+      double* row = out_ptr(d, w.b, w.b % d.B0, w.b / d.B0, 0, m, nf);
+      const long long sn = d.sc_n;
+      const int nv = m < d.M ? min(hc, d.N - nf) : 0;
+      const bool vec = sn == 1 && nv == hc && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
+      float* row32 = d.c32 ? d.c32 + (row - static_cast<double*>(d.C)) : nullptr;
+      auto put = [&](int j, double x, double y) {
+        if (row32) {
+          if (j < nv) row32[j * sn] = f64b::to_f32(x);
+          if (j + 1 < nv) row32[(j + 1) * sn] = f64b::to_f32(y);
+        }
+        if (vec) {
+          *reinterpret_cast<double2*>(row + j) = make_double2(x, y);
+        } else {
+          if (j < nv) row[j * sn] = x;
+          if (j + 1 < nv) row[(j + 1) * sn] = y;
+        }
+      };
+      auto put4 = [&](int cb, const uint32_t (&r)[kOD][4]) {
+        uint32_t v[4][3];
+        combine4(r, 0, v);
+#pragma unroll
+        for (int j = 0; j < 4; j += 2)
+          put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
+      };
+      // the next four columns are on their way while four are combined
+      uint32_t ra[kOD][4], rb[kOD][4];
+      ld_levels(tcol, w.bn, ra);
+#pragma unroll 1
+      for (int cb = 0; cb < hc; cb += 8) {
+        ld_wait(ra);
+        ld_levels(tcol + cb + 4, w.bn, rb);
+        put4(cb, ra);
+        ld_wait(rb);
+        if (cb + 8 < hc) {
+          ld_levels(tcol + cb + 8, w.bn, ra);
+        } else {
+          // (all accumulators are in registers)
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          omb_arrive(&free_bar);
+        }
+        put4(cb + 4, rb);
+      }
+    };
+    int it = 0;
+    for (int u = 0; u < nsub && ok; ++u) {
+      const int eb = eb_s[u], stride = cur.bn * 64;
+#pragma unroll 1
+      for (int st = 0; st < nst; ++st, ++it) {
+        const int s = it & 1;
+        if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v));
+        if (!ok) break;
+        if (b_on) store_digits(vb, eb, smem + s * kStage + kOD * kA, br, bc, stride);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        omb_arrive(&full_bar[s]);
+        // the next stage's values
+        k += kOBK;
+        if (st + 1 == nst) {
+          k = 0;
+          if (blk_next < blk_hi) {
+            blk_next = sub_at(blk_next, cur);
+            enter();
+          } else {
+            b_on = false;
+          }
+        }
+        load_b();
+        if (u > 0 && st == min(1, nst - 1)) {
+          flush(u - 1);
+          if (!ok) break;
+        }
+      }
+    }
+    if (ok) flush(nsub - 1);
+    if (!ok) {
+      *abort_v = 1;
+      if (op.err && t == 0) atomicOr(op.err, 1);
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 8)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kOD * kMaxN));
 }
 
 template <int BN>
@@ -801,6 +1110,7 @@ struct OzPlan {
   OzParams op;
   int blocks;
   long long words, image_bytes;
+  bool stream;
 };
 
 void plan_product(const GemmDesc& d, OzPlan& pl) {
@@ -855,6 +1165,27 @@ void plan_product(const GemmDesc& d, OzPlan& pl) {
       w.nks = it.nks;
       w.img = ap.it[at].img;
     }
+  // (at most as many tiles as SMs: one round of tiles is as short)
+  pl.stream = d.ngroups == 1 && d.g[0].K <= kOChunk && bn == 64 && pl.op.a[0].img >= 0 && pl.op.b[0].img < 0 &&
+              tm * tn * nb > device_sm_count() && tm * tn * nb < (1LL << 28);
+}
+
+// C^T = B^T A^T: the same sums with the sides exchanged.
+GemmDesc exchanged(const GemmDesc& d) {
+  GemmDesc e = d;
+  std::swap(e.M, e.N);
+  std::swap(e.sc_m, e.sc_n);
+  for (int g = 0; g < e.ngroups; ++g) std::swap(e.g[g].a, e.g[g].b);
+  return e;
+}
+
+// A large operand times a small one (more tiles than SMs, one chunk of K): the
+// side that is ready in memory becomes A, whatever the caller named it, so that
+// every value of the large one is cut into digits once; a tile has 128 rows of
+// A, so an exchange that leaves more than half of one empty is not made.
+bool exchange_sides(const GemmDesc& d) {
+  const int rest = d.N % kOBM;
+  return d.ngroups == 1 && d.g[0].K <= kOChunk && d.splits <= 1 && d.M > d.N && (rest == 0 || rest > kOBM / 2);
 }
 
 }  // namespace
@@ -890,13 +1221,28 @@ size_t oz_scratch(const GemmDesc& d) {
   if (!gemm_oz_supported(d)) return 0;
   static thread_local OzPlan pl;
   plan_product(d, pl);
-  return words_bytes(pl.words) + static_cast<size_t>(pl.image_bytes);
+  size_t bytes = words_bytes(pl.words) + static_cast<size_t>(pl.image_bytes);
+  if (exchange_sides(d)) {
+    plan_product(exchanged(d), pl);
+    bytes = std::max(bytes, words_bytes(pl.words) + static_cast<size_t>(pl.image_bytes));
+  }
+  return bytes;
 }
 
 // Returns the launches, or -1 when the scratch is too small (nothing launched).
-int gemm_oz_launch(const GemmDesc& d, cudaStream_t s) {
+int gemm_oz_launch(const GemmDesc& d0, cudaStream_t s) {
   static thread_local OzPlan pl;
-  plan_product(d, pl);
+  GemmDesc d = d0;
+  bool planned = false;
+  if (exchange_sides(d0)) {
+    d = exchanged(d0);
+    plan_product(d, pl);
+    planned = pl.stream;
+  }
+  if (!planned) {
+    d = d0;
+    plan_product(d, pl);
+  }
   if (words_bytes(pl.words) + static_cast<size_t>(pl.image_bytes) > d.words_bytes) return -1;
   pl.ap.words = d.words;
   pl.ap.images = reinterpret_cast<uint8_t*>(d.words) + words_bytes(pl.words);
@@ -907,6 +1253,15 @@ int gemm_oz_launch(const GemmDesc& d, cudaStream_t s) {
   pl.op.images = pl.ap.images;
   pl.op.total_chunks = oz_chunks(d);
   pl.op.err = d.err;
+  if (pl.stream && d.splits <= 1) {
+    // one CTA per SM, or more when a CTA's share would exceed kOBlocks
+    pl.op.nb16 = (d.N + 15) / 16;
+    const long long blocks = static_cast<long long>((d.M + kOBM - 1) / kOBM) * d.B0 * d.B1 * pl.op.nb16;
+    const long long sms = device_sm_count(), waves = (blocks + sms * kOBlocks - 1) / (sms * kOBlocks);
+    pl.op.blocks = static_cast<int>(blocks);
+    launch_attr(true, gemm_oz_stream_kernel, dim3(static_cast<unsigned>(waves * sms)), kOThreads, oz_smem<64>(), s, d, pl.op);
+    return 2;
+  }
   const int bn = oz_bn(d);
   dim3 grid(((d.M + kOBM - 1) / kOBM) * ((d.N + bn - 1) / bn), d.B0 * d.B1, d.splits);
   // always with programmatic serialisation: its only predecessor is the
@@ -918,6 +1273,7 @@ int gemm_oz_launch(const GemmDesc& d, cudaStream_t s) {
 
 void gemm_oz_init() {
   cudaFuncSetAttribute(gemm_oz_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<64>());
+  cudaFuncSetAttribute(gemm_oz_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<64>());
   cudaFuncSetAttribute(gemm_oz_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<32>());
 }
 
