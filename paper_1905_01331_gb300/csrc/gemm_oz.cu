@@ -18,26 +18,32 @@
 // term.
 //
 // One CTA owns a 128 x BN output tile (BN 64 or 32); two stages of 32 K values.
-// Warps 0-7 load FP64 operands (any strides), cut them into digits with integer
+// Warps 0-15 load FP64 operands (any strides), cut them into digits with integer
 // operations and write them to shared memory in the K-major 64-byte-swizzle
 // layout; digits that oz_prepare_kernel left in memory (small operands that many
-// tiles read) arrive as one bulk copy per stage, started by a thread of warp 9;
-// one thread of warp 8 issues the MMAs.  The digits of B are stacked along N, so
+// tiles read) arrive as one bulk copy per stage, started by a thread of warp 17;
+// one thread of warp 16 issues the MMAs.  The digits of B are stacked along N, so
 // that one MMA multiplies A's digit i with B's digits 0 .. 7 - i and adds each
 // product to the accumulator of its weight: TMEM columns (i + j) BN .. of the
 // same instruction.  All waits are bounded, as in the other tensor-core kernels.
 //
 // What bounds it (clocks of a 128 x 64 tile, K = 128): the four stages' MMAs take
-// 12.4 k -- 9.2 k at the tensor rate, the rest is shared memory, which feeds them
+// 12.5 k -- 9.2 k at the tensor rate, the rest is shared memory, which feeds them
 // 106 bytes a clock beside the next stage's stores -- the combination of the
-// accumulators about 6 k, first loads and start 3 k.  128 x 64 because eight
-// accumulators of 64 columns fill TMEM.  Measured on a GB300 (P = n = 128, with the
-// preparation): F X of 128 x 128 by 128 x 16384 41 us (the FP64 kernel 547), the
-// environment's five such products in one 128 us (2674), three close products over
-// K = 16384 120 us (1931), the Gram matrix of 128 x 16384 56 us (449).  Converting
+// accumulators 7 k (100 instructions per output), first loads and start 4 k; a
+// stage that converts both operands takes 6 k, half of it its loads.  128 x 64
+// because eight accumulators of 64 columns fill TMEM.  Sixteen converter warps
+// (eight before: 2 warps a scheduler, an instruction every third clock): FP64
+// sweep at chi = 128 25.29 -> 25.05 ms, FP64 gradient of a torus at chi = 64 3.61 ->
+// 3.46 ms, measurement 3.35 -> 3.23 ms.  Measured on a GB300 (P = n = 128, with the
+// preparation): F X of 128 x 128 by 128 x 16384 35 us (the FP64 kernel 547), the
+// environment's five such products in one 131 us (2674), three close products over
+// K = 16384 119 us (1931), the Gram matrix of 128 x 16384 56 us (449).  Converting
 // both operands in every tile with BF16 digits, which take two operations more a
 // pair, and combining by eight converting instructions per output took 55, 186,
-// 123 and 59.  Relative error against extended precision 4e-17 to 2e-16 where the
+// 123 and 59; loads whose 16-byte pieces are consecutive over four threads (K
+// permuted in a stage) took 5 % more than eight consecutive values per thread.
+// Relative error against extended precision 4e-17 to 2e-16 where the
 // FP64 kernel has 2e-16 to 2e-15.  At n = 32 both kernels take 15 to 30 us
 // (latency), so kOzMinWork lies between n = 32 (2^20 multiply-adds) and n = 64
 // (2^24: 21 against 58 us).
@@ -63,8 +69,9 @@ constexpr int kOD = 8;              // digits per operand
 constexpr int kOBM = 128;
 constexpr int kOChunk = 128;        // K values per exact accumulation
 constexpr int kOBK = 32;            // K values per stage
-constexpr int kOConv = 256;         // converter threads
+constexpr int kOConv = 512;         // converter threads
 constexpr int kOThreads = kOConv + 128;   // and the warpgroup of the MMA and image warps
+constexpr int kOWork = kOConv / 32; // converter warps; the MMA warp follows them, then the image warp
 constexpr long kOWait = 1L << 22;
 constexpr int kOBlocks = 24;        // 16-column blocks of a CTA of the streamed kernel at most
 
@@ -376,8 +383,15 @@ __device__ __noinline__ void plain_tile(const GemmDesc& d, int b, int b0, int b1
   }
 }
 
-// The accumulators of four columns: levels l, `cols` columns apart.  (The
-// registers hold them after ld_wait.)
+// The accumulators of four columns (two columns): levels l, `cols` columns
+// apart.  (The registers hold them after ld_wait.)
+__device__ __forceinline__ void ld_levels(uint32_t taddr, int cols, uint32_t (&r)[kOD][2]) {
+#pragma unroll
+  for (int l = 0; l < kOD; ++l)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];"
+                 : "=r"(r[l][0]), "=r"(r[l][1])
+                 : "r"(taddr + l * cols));
+}
 __device__ __forceinline__ void ld_levels(uint32_t taddr, int cols, uint32_t (&r)[kOD][4]) {
 #pragma unroll
   for (int l = 0; l < kOD; ++l)
@@ -386,17 +400,20 @@ __device__ __forceinline__ void ld_levels(uint32_t taddr, int cols, uint32_t (&r
                  : "r"(taddr + l * cols));
 }
 // The loads of r are complete (r as operands: nothing reads it before).
-__device__ __forceinline__ void ld_wait(uint32_t (&r)[kOD][4]) {
+template <int NC>
+__device__ __forceinline__ void ld_wait(uint32_t (&r)[kOD][NC]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int l = 0; l < kOD; ++l)
-    asm volatile("" : "+r"(r[l][0]), "+r"(r[l][1]), "+r"(r[l][2]), "+r"(r[l][3]));
+#pragma unroll
+    for (int j = 0; j < NC; ++j) asm volatile("" : "+r"(r[l][j]));
 }
 
-// Combine four columns' accumulators into 96-bit integers, shifted right by sh.
-__device__ __forceinline__ void combine4(const uint32_t (&r)[kOD][4], int sh, uint32_t (&v)[4][3]) {
+// Combine the columns' accumulators into 96-bit integers, shifted right by sh.
+template <int NC>
+__device__ __forceinline__ void combine(const uint32_t (&r)[kOD][NC], int sh, uint32_t (&v)[NC][3]) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < NC; ++j) {
     // levels 0 to 2 are at most 2^22 (digit 0 is at most 64): their integers sit
     // in the low bits of x + 1.5 2^23; the others take the converting
     // instruction, a quarter of the rate of an addition
@@ -431,7 +448,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   pdl_trigger();
   constexpr int kA = kOBM * 64, kB = BN * 64;      // bytes of one digit tile of a stage
   constexpr int kStage = kOD * (kA + kB);
-  constexpr int kHalf = BN / 2;                    // columns per flush warp
+  constexpr int kPart = BN / 4;                    // columns per flush warp
   constexpr int kCols = kOD * BN;                  // TMEM columns
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -450,7 +467,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   const int c_lo = static_cast<int>(static_cast<long long>(op.total_chunks) * split / d.splits);
   const int c_hi = static_cast<int>(static_cast<long long>(op.total_chunks) * (split + 1) / d.splits);
 
-  if (warp == 8) {
+  if (warp == kOWork) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(osmem(&tmem_slot)), "r"(kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -471,7 +488,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   // converter state: the values of the next stage (loaded before the operands'
   // magnitudes arrive), their rows and chunks, the position after them
   const int t = threadIdx.x;
-  constexpr int kATasks = kOBM * 4 / kOConv;                     // 2
+  constexpr int kATasks = kOBM * 4 / kOConv;                     // 1
   double va[kATasks][8], vb[8];
   int g = g0, k = kfirst;                                        // next stage to load
   const double *pa = nullptr, *pb = nullptr;
@@ -498,7 +515,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     const Group& G = d.g[g];
     load8(G.b.s_mn, G.b.s_k0, G.b.s_k1, G.k0_log2, pb, n0 + br, n0 + br < d.N, k + 8 * bc, G.K, bvec, vb);
   };
-  if (warp < 8 && nchunks > 0) {
+  if (warp < kOWork && nchunks > 0) {
     enter();
     if (b_on) load_b();
     if (a_on) {
@@ -546,13 +563,13 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   const uint32_t tmem = tmem_slot;
   volatile int* abort_v = &abort_flag;
 
-  // registers: three warpgroups of 168 at launch -> 72 for the MMA warp's, 216
-  // for the two of the converters (2 x 216 + 72 = 3 x 168)
+  // registers: five warpgroups of 96 at launch -> 32 for the MMA warp's, 112 for
+  // the four of the converters (4 x 112 + 32 = 5 x 96)
   if (plain) {
     // (the tile is done)
-  } else if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
-    if (warp == 8 && lane == 0) {
+  } else if (warp >= kOWork) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+    if (warp == kOWork && lane == 0) {
       // ---- MMA issuer ----
       bool ok = true;
       int g = g0, k = kfirst, it = 0;
@@ -595,7 +612,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
         ocommit(&drain_bar);
         omb_wait(&drain_bar, 0, nullptr);
       }
-    } else if (warp == 9 && lane == 0) {
+    } else if (warp == kOWork + 1 && lane == 0) {
       // ---- ready digits: one bulk copy per operand and stage ----
       bool ok = true;
       int g = g0, k = kfirst, it = 0;
@@ -629,19 +646,20 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     }
     __syncwarp();
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
     // ---- converters, then the flush of every chunk ----
-    uint32_t acc[3][kHalf];
+    uint32_t acc[3][kPart];
 #pragma unroll
-    for (int j = 0; j < kHalf; ++j) acc[0][j] = acc[1][j] = acc[2][j] = 0u;
-    const int quarter = warp & 3, half = warp >> 2;
-    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + half * kHalf;
+    for (int j = 0; j < kPart; ++j) acc[0][j] = acc[1][j] = acc[2][j] = 0u;
+    const int quarter = warp & 3, part = warp >> 2;   // 32 rows, kPart columns
+    const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + part * kPart;
     bool ok = true;
     int flushed = 0;
     auto shift_of = [&](int fg) {
       const unsigned wa = ex[2 * fg], wb = ex[2 * fg + 1];
       return (wa == 0u || wb == 0u) ? 0 : sref - (static_cast<int>(wa >> 20) + static_cast<int>(wb >> 20) - 2 * 1022 - 68);
     };
+    constexpr int kF = 2;                            // columns combined together (registers)
     // add the eight accumulators of a finished chunk (of group fg) to acc
     auto flush = [&](int fg) {
       ok = __all_sync(0xffffffffu, ok && omb_wait(&done_bar, flushed & 1, abort_v));
@@ -650,14 +668,14 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int sh = shift_of(fg);
 #pragma unroll
-      for (int cb = 0; cb < kHalf; cb += 4) {
-        uint32_t v[4][3];
-        uint32_t r[kOD][4];
+      for (int cb = 0; cb < kPart; cb += kF) {
+        uint32_t v[kF][3];
+        uint32_t r[kOD][kF];
         ld_levels(trow + cb, BN, r);
         ld_wait(r);
-        combine4(r, sh, v);
+        combine(r, sh, v);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < kF; ++j)
           asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
               : "+r"(acc[0][cb + j]), "+r"(acc[1][cb + j]), "+r"(acc[2][cb + j])
               : "r"(v[j][0]), "r"(v[j][1]), "r"(v[j][2]));
@@ -676,28 +694,17 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
 #pragma unroll 1
       for (int st = 0; st < max(nst, 1); ++st, ++it) {
         const int s = it & 1;
+        bool more = false;
         if (nst) {
           if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v));
           if (!ok) break;
           uint8_t* sA = smem + s * kStage;
           uint8_t* sB = sA + kOD * kA;
-          // the positions of this stage's tasks; the next stage's loads follow each conversion
-          int car[kATasks], cac[kATasks];
+          more = !(c + 1 == nchunks && st + 1 == nst);
+          if (b_on) store_digits(vb, eb, sB, br, bc, kB);
+          if (a_on) {
 #pragma unroll
-          for (int q = 0; q < kATasks; ++q) { car[q] = ar[q]; cac[q] = ac[q]; }
-          const int cbr = br, cbc = bc;
-          const bool ca = a_on, cb = b_on;
-          const bool last = c + 1 == nchunks && st + 1 == nst;
-          if (!last) {
-            k += kOBK;
-            if (k >= d.g[g].K) { ++g; k = 0; enter(); }
-          }
-          if (cb) store_digits(vb, eb, sB, cbr, cbc, kB);
-          if (!last && b_on) load_b();
-#pragma unroll
-          for (int q = 0; q < kATasks; ++q) {
-            if (ca) store_digits(va[q], ea, sA, car[q], cac[q], kA);
-            if (!last && a_on) load_a(q);
+            for (int q = 0; q < kATasks; ++q) store_digits(va[q], ea, sA, ar[q], ac[q], kA);
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           omb_arrive(&full_bar[s]);
@@ -708,14 +715,25 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
           pend = -1;
           if (!ok) break;
         }
+        // the next stage's loads: after the combination, whose registers they
+        // would take (they have the time of the staged MMAs)
+        if (more) {
+          k += kOBK;
+          if (k >= d.g[g].K) { ++g; k = 0; enter(); }
+          if (b_on) load_b();
+          if (a_on) {
+#pragma unroll
+            for (int q = 0; q < kATasks; ++q) load_a(q);
+          }
+        }
       }
       pend = cg;
     }
     const int m = m0 + quarter * 32 + lane;
-    double* row = out_ptr(d, b, b0, b1, split, m, n0 + half * kHalf);
+    double* row = out_ptr(d, b, b0, b1, split, m, n0 + part * kPart);
     const long long sn = d.splits > 1 ? 1 : d.sc_n;
-    const int nv = m < d.M ? min(kHalf, d.N - (n0 + half * kHalf)) : 0;
-    const bool vec = sn == 1 && nv == kHalf && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
+    const int nv = m < d.M ? min(kPart, d.N - (n0 + part * kPart)) : 0;
+    const bool vec = sn == 1 && nv == kPart && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
     float* row32 = d.c32 ? d.c32 + (row - static_cast<double*>(d.C)) : nullptr;   // (splits == 1)
     auto put = [&](int j, double x, double y) {
       if (row32) {
@@ -737,12 +755,12 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int sh = shift_of(g0);
 #pragma unroll 1
-        for (int cb = 0; cb < kHalf; cb += 4) {
+        for (int cb = 0; cb < kPart; cb += 4) {
           uint32_t v[4][3];
           uint32_t r[kOD][4];
           ld_levels(trow + cb, BN, r);
           ld_wait(r);
-          combine4(r, sh, v);
+          combine(r, sh, v);
 #pragma unroll
           for (int j = 0; j < 4; j += 2)
             put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
@@ -750,7 +768,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       }
     } else if (ok) {
 #pragma unroll
-      for (int j = 0; j < kHalf; j += 2)
+      for (int j = 0; j < kPart; j += 2)
         put(j, to_double(acc[0][j], acc[1][j], acc[2][j], sref),
             to_double(acc[0][j + 1], acc[1][j + 1], acc[2][j + 1], sref));
     }
@@ -761,7 +779,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 8)
+  if (warp == kOWork)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
 }
 
@@ -771,8 +789,8 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
 // columns of one row tile: every sub-tile's first two stages are staged before
 // the one before it is combined, and no SM waits in a second round of tiles.
 // With A ready, a converter thread has one task per stage where a tile that
-// converts both operands has three.  256 tiles on 152 SMs are two rounds of 24 k
-// clocks; 112 columns per CTA (64 + 48) are 39 k.  FP64 sweep at chi = 128: 25.57
+// converts both operands has three.  256 tiles on 152 SMs are two rounds; 112
+// columns per CTA (64 + 48) take 44 k clocks.  FP64 sweep at chi = 128: 25.57
 // -> 25.29 ms, FP64 measurement of a Heisenberg chain: 3.44 -> 3.35 ms (the
 // exchange of sides alone: 25.55 and 3.41); the sums are the same.
 struct OzSub {
@@ -814,7 +832,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
     if (threadIdx.x == 0) subs[nsub] = u;
   }
   if (nsub == 0) return;
-  if (warp == 8) {
+  if (warp == kOWork) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(osmem(&tmem_slot)), "r"(kOD * kMaxN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
@@ -823,7 +841,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
   const int nst = (G.K + kOBK - 1) / kOBK;         // at most 4
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
-      omb_init(&full_bar[s], kOConv + 1);
+      omb_init(&full_bar[s], kOConv / 2 + 1);
       omb_init(&empty_bar[s], 1);
     }
     omb_init(&done_bar, 1);
@@ -834,35 +852,40 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
 
-  // converter state: the values of the next stage (loaded a stage ahead), their
-  // row and chunk
-  const int t = threadIdx.x;
+  // converter state: half of the warps converts the even stages, the other half
+  // the odd ones; each thread's cursor (cur, k) stands at its next stage, whose
+  // values it has loaded
+  const int hw = (threadIdx.x >> 8) & 1, t = threadIdx.x & 255;
   const bool bkf = G.b.s_k0 == 1;
   double vb[8];
   const double* pb = nullptr;
-  bool bvec = false, b_on = false;
+  bool bvec = false, b_on = false, fresh = true;
   int br = 0, bc = 0, k = 0, blk_next = 0;
-  OzSub cur{};                                      // the sub-tile whose stages are loaded
-  auto enter = [&]() {
-    pb = static_cast<const double*>(G.b.p) + (cur.b % d.B0) * G.b.s_b0 + static_cast<long long>(cur.b / d.B0) * G.b.s_b1;
-    bvec = bkf && ((reinterpret_cast<uintptr_t>(pb) & 15) == 0) && ((G.b.s_mn | G.b.s_k1) & 1) == 0;
-    b_on = t < cur.bn * 4;
-    // K contiguous: eight rows by four chunks per warp; MN contiguous: consecutive rows of one chunk
-    if (bkf) {
-      br = t >> 2;
-      bc = t & 3;
-    } else {
-      bc = t / cur.bn;
-      br = t - bc * cur.bn;
-    }
+  OzSub cur{};
+  auto step = [&]() {                               // the cursor to the next stage
+    k += kOBK;
+    if (k < nst * kOBK) return;
+    k = 0;
+    fresh = true;
+    if (blk_next < blk_hi) blk_next = sub_at(blk_next, cur);
+    else cur.bn = 0;                                // (no stage left)
   };
   auto load_b = [&]() {
+    if (fresh) {
+      fresh = false;
+      pb = static_cast<const double*>(G.b.p) + (cur.b % d.B0) * G.b.s_b0 + static_cast<long long>(cur.b / d.B0) * G.b.s_b1;
+      bvec = bkf && ((reinterpret_cast<uintptr_t>(pb) & 15) == 0) && ((G.b.s_mn | G.b.s_k1) & 1) == 0;
+      b_on = t < cur.bn * 4;
+      // K contiguous: eight rows by four chunks per warp; MN contiguous: consecutive rows of one chunk
+      bc = bkf ? t & 3 : t / max(cur.bn, 1);
+      br = bkf ? t >> 2 : t - bc * cur.bn;
+    }
     if (b_on)
       load8(G.b.s_mn, G.b.s_k0, G.b.s_k1, G.k0_log2, pb, cur.n0 + br, cur.n0 + br < d.N, k + 8 * bc, G.K, bvec, vb);
   };
-  if (warp < 8) {
+  if (warp < kOWork) {
     blk_next = sub_at(blk_lo, cur);
-    enter();
+    if (hw) step();
     load_b();
   }
   __syncthreads();
@@ -900,7 +923,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
 
   if (plain) {
     // (the tiles are done)
-  } else if (warp == 8) {
+  } else if (warp == kOWork) {
     if (lane == 0) {
       // ---- MMA issuer ----
       bool ok = true;
@@ -941,7 +964,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
       }
     }
     __syncwarp();
-  } else if (warp == 9) {
+  } else if (warp == kOWork + 1) {
     if (lane == 0) {
       // ---- A: one bulk copy of ready digits per stage ----
       bool ok = true;
@@ -963,9 +986,9 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
       for (int q = max(0, it - 2); q < it; ++q) omb_wait(&full_bar[q & 1], (q >> 1) & 1, nullptr);
     }
     __syncwarp();
-  } else if (warp < 8) {
+  } else if (warp < kOWork) {
     // ---- converters; each sub-tile is combined and stored once two stages of the next are staged ----
-    const int quarter = warp & 3, half = warp >> 2;
+    const int quarter = warp & 3, part = warp >> 2;
     const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     bool ok = true;
     auto flush = [&](int u) {
@@ -973,9 +996,9 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
       if (!ok) return;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const OzSub w = subs[u];
-      const int sref = sref_s[u], hc = w.bn >> 1;     // this warp's columns: 8, 16, 24 or 32
-      const uint32_t tcol = trow + half * hc;
-      const int m = w.m0 + quarter * 32 + lane, nf = w.n0 + half * hc;
+      const int sref = sref_s[u], hc = w.bn >> 2;     // this warp's columns: 4, 8, 12 or 16
+      const uint32_t tcol = trow + part * hc;
+      const int m = w.m0 + quarter * 32 + lane, nf = w.n0 + part * hc;
       double* row = out_ptr(d, w.b, w.b % d.B0, w.b / d.B0, 0, m, nf);
       const long long sn = d.sc_n;
       const int nv = m < d.M ? min(hc, d.N - nf) : 0;
@@ -993,55 +1016,35 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
           if (j + 1 < nv) row[(j + 1) * sn] = y;
         }
       };
-      auto put4 = [&](int cb, const uint32_t (&r)[kOD][4]) {
-        uint32_t v[4][3];
-        combine4(r, 0, v);
-#pragma unroll
-        for (int j = 0; j < 4; j += 2)
-          put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
-      };
-      // the next four columns are on their way while four are combined
-      uint32_t ra[kOD][4], rb[kOD][4];
-      ld_levels(tcol, w.bn, ra);
 #pragma unroll 1
-      for (int cb = 0; cb < hc; cb += 8) {
-        ld_wait(ra);
-        ld_levels(tcol + cb + 4, w.bn, rb);
-        put4(cb, ra);
-        ld_wait(rb);
-        if (cb + 8 < hc) {
-          ld_levels(tcol + cb + 8, w.bn, ra);
-        } else {
-          // (all accumulators are in registers)
+      for (int cb = 0; cb < hc; cb += 4) {
+        uint32_t r[kOD][4], v[4][3];
+        ld_levels(tcol + cb, w.bn, r);
+        ld_wait(r);
+        if (cb + 4 >= hc) {                         // (all accumulators are in registers)
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           omb_arrive(&free_bar);
         }
-        put4(cb + 4, rb);
+        combine(r, 0, v);
+#pragma unroll
+        for (int j = 0; j < 4; j += 2)
+          put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
       }
     };
     int it = 0;
     for (int u = 0; u < nsub && ok; ++u) {
-      const int eb = eb_s[u], stride = cur.bn * 64;
 #pragma unroll 1
       for (int st = 0; st < nst; ++st, ++it) {
-        const int s = it & 1;
-        if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v));
-        if (!ok) break;
-        if (b_on) store_digits(vb, eb, smem + s * kStage + kOD * kA, br, bc, stride);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        omb_arrive(&full_bar[s]);
-        // the next stage's values
-        k += kOBK;
-        if (st + 1 == nst) {
-          k = 0;
-          if (blk_next < blk_hi) {
-            blk_next = sub_at(blk_next, cur);
-            enter();
-          } else {
-            b_on = false;
-          }
+        if ((it & 1) == hw) {
+          if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[hw], ((it >> 1) - 1) & 1, abort_v));
+          if (!ok) break;
+          if (b_on) store_digits(vb, eb_s[u], smem + hw * kStage + kOD * kA, br, bc, subs[u].bn * 64);
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          omb_arrive(&full_bar[hw]);
+          step();
+          step();
+          load_b();
         }
-        load_b();
         if (u > 0 && st == min(1, nst - 1)) {
           flush(u - 1);
           if (!ok) break;
@@ -1051,12 +1054,12 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
     if (ok) flush(nsub - 1);
     if (!ok) {
       *abort_v = 1;
-      if (op.err && t == 0) atomicOr(op.err, 1);
+      if (op.err && threadIdx.x == 0) atomicOr(op.err, 1);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 8)
+  if (warp == kOWork)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kOD * kMaxN));
 }
 
