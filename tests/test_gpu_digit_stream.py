@@ -34,3 +34,19 @@ def test_gradient_of_large_layers(model, L, chi):
     for t, x in enumerate(g):
         ref = oracle.env_layer(st, t)
         assert np.abs(x.cpu().numpy() - ref).max() < 1e-11 * np.abs(ref).max(), t
+
+
+def test_environments_of_a_per_node_tree():
+    """Batches of nodes and parent indices: 16 nodes of 64 x 64 products, one
+    operator per node; the bound as above (2^12 terms)."""
+    from paper_1905_01331_gb300 import Sweeper
+    m = ti.tfim_chain(256, 1.0)
+    ws, V = ti.initial_tensors(256, m.d0, 64, 11, True)
+    st = oracle.make_state(m, ws, V, per_node=True)
+    s = Sweeper(m, 64, per_node=True)
+    s.set_isometries(0, ws, V)
+    for t in range(2, len(ws)):
+        ref = oracle.env_layer(st, t)
+        got = s.env(0, t).cpu().numpy()
+        assert np.abs(got - ref).max() < 1e-11 * max(1.0, np.abs(ref).max()), t
+    s.close()
