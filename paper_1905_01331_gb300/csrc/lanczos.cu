@@ -893,6 +893,50 @@ __device__ __forceinline__ void wide_fma_d(const float* Ls, const float* Rs, boo
   }
 }
 
+// One CTA and one tile (c <= 8, FP64): operators, vectors and Y in shared memory,
+// matrices as 8 rows of 8; one thread per output.  The sums are those of
+// tile_fma and tile_store, whose warp w holds the terms k = w: a chain of fused
+// multiply-adds per k over the terms, then the chains in the order of k.  A step
+// of the general path is a chain of L2 round trips here (operands, Y, partial
+// sums, coefficients) with a cross-warp sum per product; without them a sweep of
+// a per-node tree of 16 spins at chi = 8 takes 1.43 instead of 1.67 ms, with the
+// same bits.
+struct LzTiny {
+  const double *s0, *s1;   // 1 + 2K slabs of the left and the right top site
+  double* Y;               // 2K slabs
+};
+__device__ __forceinline__ void tiny_y(const LzTiny& ty, const double* x, int c, int K) {
+  for (int t = threadIdx.x; t < 2 * K * 64; t += kLThreads) {
+    const int i = (t >> 3) & 7, j = t & 7;
+    const double* L = ty.s0 + 64 + (t & ~63) + i * 8;
+    double p[kLT], v = 0.0;
+#pragma unroll
+    for (int k = 0; k < kLT; ++k) p[k] = k < c ? fma(L[k], x[k * 8 + j], 0.0) : 0.0;
+#pragma unroll
+    for (int k = 0; k < kLT; ++k) v += p[k];
+    ty.Y[t] = v;
+  }
+}
+__device__ __forceinline__ double tiny_hx(const LzTiny& ty, const double* x, int c, int K) {
+  const int i = threadIdx.x >> 3, j = threadIdx.x & 7;
+  double p[kLT], v = 0.0;
+#pragma unroll
+  for (int k = 0; k < kLT; ++k) p[k] = k < c ? fma(ty.s0[i * 8 + k], x[k * 8 + j], 0.0) : 0.0;
+#pragma unroll
+  for (int k = 0; k < kLT; ++k)
+    if (k < c) p[k] = fma(x[i * 8 + k], ty.s1[j * 8 + k], p[k]);
+  for (int q = 0; q < 2 * K; ++q) {
+    const double* R = ty.s1 + 64 * (q < K ? 1 + K + q : 1 + q - K) + j * 8;
+    const double* L = ty.Y + 64 * q + i * 8;
+#pragma unroll
+    for (int k = 0; k < kLT; ++k)
+      if (k < c) p[k] = fma(L[k], R[k], p[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < kLT; ++k) v += p[k];
+  return v;
+}
+
 // FP64 value and its pair at index e of a vector (pair vector: hi at P, lo at P + n)
 __device__ __forceinline__ void store_both(double* D, float* P, long long n, long long e, double v) {
   __stcg(D + e, v);
@@ -942,7 +986,8 @@ __device__ double own_dot(LzSmem& sm, const double* a, const double* b, int nown
 // 4w .. 4w+3, 4w+32 .. (their loads issued together); each sum runs over the
 // owned entries lane by lane, then a fixed butterfly.
 __device__ void own_projections(const LanczosArgs& a, const LzOwn& own, double* part, int ldp, int j,
-                                int nslot, int nown, int bid, int G, int nt, int c, long long n) {
+                                int nslot, int nown, int bid, int G, int nt, int c, long long n,
+                                double* only = nullptr) {
   constexpr int U = 4;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nv = j + 1 + (nslot >= 0 ? 1 : 0);
@@ -984,7 +1029,11 @@ __device__ void own_projections(const LanczosArgs& a, const LzOwn& own, double* 
     r += __shfl_xor_sync(0xffffffffu, h8 ? r0 : r1, 8);
     for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
     const int i = i0 + (h8 ? 2 : 0) + (h16 ? 1 : 0);
-    if ((lane & 7) == 0 && i < nv) __stcg(part + (long long)bid * ldp + (i > j ? nslot : i), r);
+    if ((lane & 7) == 0 && i < nv) {
+      // (0 + r: what the sum over one CTA gives)
+      if (only) only[i > j ? nslot : i] = 0.0 + r;
+      else __stcg(part + (long long)bid * ldp + (i > j ? nslot : i), r);
+    }
   }
 }
 
@@ -1101,6 +1150,8 @@ __device__ __forceinline__ void lz_post(const LanczosArgs& a, unsigned v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(a.job), "r"(v) : "memory");
 }
 
+// kTiny: one CTA, one tile (c <= 8), FP64: everything a step reads is in shared memory.
+template <bool kTiny>
 __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, float* lz_dyn, int G) {
   const int c = a.c, K = a.K, m = a.m;
   const long long n = (long long)c * c;
@@ -1131,6 +1182,19 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
     return lz_wait_word(sm, a.job + 1, [&](unsigned w) { return (w >> 1) == jobs; }, a.err, wlimit, true, good);
   };
   float* bp0 = df ? a.bp : nullptr;          // pairs of basis_0
+  LzTiny ty;
+  if constexpr (kTiny) {
+    double* p = own.p + (own.n + 1) * own.pitch;
+    const int slabs = 1 + 2 * K;
+    for (int t = threadIdx.x; t < 2 * slabs * 64; t += kLThreads) {
+      const int i = (t >> 3) & 7, j = t & 7, q = t >> 6;
+      const double* S = q < slabs ? a.s0 + q * n : a.s1 + (q - slabs) * n;
+      p[t] = i < c && j < c ? __ldcg(S + i * c + j) : 0.0;
+    }
+    ty.s0 = p;
+    ty.s1 = p + slabs * 64;
+    ty.Y = p + 2 * slabs * 64;
+  }
   // start: the operators as pairs (double-float mode), Vprev = V, basis_0 = V / |V|
   if (df) {
     const long long nops = (long long)(1 + 2 * K) * n;
@@ -1191,6 +1255,22 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
       const double sigma_j = j == 0 ? 0.0 : (j == 1 ? sm.sigma : sm.alpha_prev_h);
       const double* xprev = j > 0 ? x - n : nullptr;
       const double beta_j1 = j > 0 ? sm.beta_prev : 0.0;
+      if constexpr (kTiny) {
+        const double* xs = own.p + j * own.pitch;
+        tiny_y(ty, xs, c, K);
+        __syncthreads();
+        if (threadIdx.x < 64) {
+          const int r = threadIdx.x >> 3, cc = threadIdx.x & 7;
+          double v = tiny_hx(ty, xs, c, K);
+          if (r < c && cc < c) {
+            if (sigma_j != 0.0) v = fma(-sigma_j, xs[threadIdx.x], v);
+            if (beta_j1 != 0.0) v = fma(-beta_j1, xs[threadIdx.x - own.pitch], v);
+            own.p[own.wrow * own.pitch + threadIdx.x] = v;
+          }
+        }
+        __syncthreads();
+        own_projections(a, own, part, ldp, j, nslot, nown, bid, G, nt, c, n, sm.cf);
+      } else {
       // phase A: Y_b = Op_b x for the 2K operators A_k0, B_k0 (stored after o_0)
       const float* xp = df ? a.bp + 2 * (long long)j * n : nullptr;
       // wide staging: all 2K products of a tile by its CTA, the columns of x
@@ -1358,6 +1438,7 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
       // coefficients of the first Gram-Schmidt pass and |w|^2 (one warp each)
       sum_coefs(part, ldp, j + 1, nslot, G, bid, a.coef, wn2);
       if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+      }
       if (j == due) {
         // the answer to the check posted kLLag steps ago, which ran meanwhile:
         // when it passed, the cycle ends with that step's tridiagonal and the
@@ -1374,7 +1455,8 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
       // least a quarter of |w|^2 remains, one pass is accurate to rounding
       // (the second pass of "twice is enough" is needed only after heavy
       // cancellation), and the norm needs no further reduction
-      load_coefs(sm, a.coef, j + 1);
+      if constexpr (kTiny) __syncthreads();
+      else load_coefs(sm, a.coef, j + 1);
       // warp 0 takes the step's scalars (the FP64 square root and division are
       // long: eight warps repeating them cost 4 k clocks a step): the sum of
       // c_i^2 in a fixed order (lane-strided, then a butterfly), so the same
@@ -1403,7 +1485,7 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
         sm.inv = 1.0 / beta_j;
       };
       if (threadIdx.x < 32) {
-        const double w2 = __ldcg(wn2);
+        const double w2 = kTiny ? sm.cf[nslot] : __ldcg(wn2);
         double t = 0.0;
         for (int i = threadIdx.x; i <= j; i += 32) t = fma(sm.cf[i], sm.cf[i], t);
         for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
@@ -1425,16 +1507,18 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
                         if (own.wrow >= 0) own.p[own.wrow * own.pitch + q] = v;
                       });
         __syncthreads();
-        own_projections(a, own, part, ldp, j, nslot, nown, bid, G, nt, c, n);
+        own_projections(a, own, part, ldp, j, nslot, nown, bid, G, nt, c, n, kTiny ? sm.cf : nullptr);
         if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
-        sum_coefs(part, ldp, j + 1, nslot, G, bid, a.coef + ldp, a.coef + ldp + j + 1);
-        if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
-        load_coefs(sm, a.coef + ldp, j + 2);
+        if constexpr (!kTiny) {
+          sum_coefs(part, ldp, j + 1, nslot, G, bid, a.coef + ldp, a.coef + ldp + j + 1);
+          if (!lz_barrier(sm, a.bar, target, G, a.err, a.max_spin > 0 ? a.max_spin : kLMaxSpin)) return;
+          load_coefs(sm, a.coef + ldp, j + 2);
+        }
         if (threadIdx.x < 32) {
           double t = 0.0;
           for (int i = threadIdx.x; i <= j; i += 32) t = fma(sm.cf[i], sm.cf[i], t);
           for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-          if (threadIdx.x == 0) scalars(alpha1 + sm.cf[j], sqrt(fmax(sm.cf[j + 1] - t, 0.0)));
+          if (threadIdx.x == 0) scalars(alpha1 + sm.cf[j], sqrt(fmax(sm.cf[kTiny ? nslot : j + 1] - t, 0.0)));
         }
         __syncthreads();
       }
@@ -1529,6 +1613,7 @@ __device__ __forceinline__ void lanczos_body(const LanczosArgs& a, LzSmem& sm, f
     }
 }
 
+template <bool kTiny>
 __global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs a) {
   __shared__ LzSmem sm;
   extern __shared__ __align__(16) float lz_dyn[];
@@ -1537,7 +1622,7 @@ __global__ void __launch_bounds__(kLThreads, 2) lanczos_kernel(const LanczosArgs
     lz_checker(a, sm, reinterpret_cast<double*>(lz_dyn));
     return;
   }
-  lanczos_body(a, sm, lz_dyn, G);
+  lanczos_body<kTiny>(a, sm, lz_dyn, kTiny ? 1 : G);
   if (a.extra && blockIdx.x == 0 && threadIdx.x == 0) lz_post(a, kLQuit);
 }
 
@@ -1559,10 +1644,12 @@ int lanczos_grid_cap() {
     int sms = 0, occ = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     const int dyn = kLMaxDyn;
-    if (cudaFuncSetAttribute(lanczos_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) !=
-        cudaSuccess)
+    if (cudaFuncSetAttribute(lanczos_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(lanczos_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) !=
+            cudaSuccess)
       return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lanczos_kernel, kLThreads, dyn) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lanczos_kernel<false>, kLThreads, dyn) !=
         cudaSuccess)
       return 0;
     g.sms = sms;
@@ -1597,7 +1684,12 @@ int lanczos_launch(const LanczosArgs& a0, int grid, int grid_share, cudaStream_t
   a.ncache = a.m + 1 <= (kLMaxDyn / 8 - tiles) / a.own_pitch - 1 ? a.m + 1 : 0;
   // the checks run in a CTA of their own when one more is co-resident
   a.extra = grid + 1 <= lanczos_grid_cap() / std::max(1, grid_share) ? 1 : 0;
-  const size_t dyn = 8 * ((size_t)tiles + (a.ncache > 0 ? (size_t)(a.ncache + 1) * a.own_pitch : 0));
+  size_t dyn = 8 * ((size_t)tiles + (a.ncache > 0 ? (size_t)(a.ncache + 1) * a.own_pitch : 0));
+  // one CTA and one tile: the operators and Y stay in shared memory too (larger
+  // grids exchange the vectors through L2 anyway)
+  const size_t ops = 8 * 64 * (2 * (size_t)(1 + 2 * a.K) + 2 * (size_t)a.K);
+  const bool tiny = !a.df && grid == 1 && a.c <= kLT && a.ncache > 0 && dyn + ops <= kLMaxDyn;
+  if (tiny) dyn += ops;
   a.job = a.bar + 1;
   cudaMemsetAsync(a.bar, 0, 3 * sizeof(unsigned), s);
   cudaLaunchConfig_t cfg = {};
@@ -1610,7 +1702,7 @@ int lanczos_launch(const LanczosArgs& a0, int grid, int grid_share, cudaStream_t
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, lanczos_kernel, a) != cudaSuccess) return -1;
+  if (cudaLaunchKernelEx(&cfg, tiny ? lanczos_kernel<true> : lanczos_kernel<false>, a) != cudaSuccess) return -1;
   return 1;
 }
 

@@ -62,3 +62,24 @@ def test_top_energy_streams():
     E = s.sweep(1)[0]
     assert np.abs(E - refs).max() <= 1e-11 * np.abs(refs).max()
     s.close()
+
+
+@pytest.mark.parametrize("chi,L", [(2, 4), (4, 8), (8, 16)])
+def test_top_energy_one_tile(chi, L):
+    """One CTA with everything in shared memory (FP64, c <= 8): three product
+    terms, antisymmetric factors, and a top site of its own on either side."""
+    from paper_1905_01331_gb300 import Sweeper
+    m = ti.heisenberg_xxx(L)
+    ws, V = ti.initial_tensors(L, 2, chi, 22, True)
+    s = Sweeper(m, chi, per_node=True, shift=0.0, lanczos_restarts=40)
+    s.set_isometries(0, ws, V)
+    c = s.chis()[-1]
+    l, r = s.ascend(0, len(ws))[:2]
+    H = np.kron(l[0], np.eye(c)) + np.kron(np.eye(c), r[0])
+    for k in range(3):
+        H = H + np.kron(l[1 + k], r[4 + k]) + np.kron(l[4 + k], r[1 + k])
+    ref = np.linalg.eigvalsh(0.5 * (H + H.T))[0]
+    E = s.sweep(1)[0, 0]
+    assert s.top_converged
+    assert abs(E - ref) <= 1e-11 * abs(ref)
+    s.close()
