@@ -1117,7 +1117,11 @@ struct OzPlan {
 };
 
 void plan_product(const GemmDesc& d, OzPlan& pl) {
-  memset(&pl, 0, sizeof(pl));
+  // (the tables are read up to ap.n and ngroups only; clearing their 9 KB for every
+  // product cost a context's creation 0.2 ms)
+  pl.ap.n = 0;
+  pl.blocks = 0;
+  pl.words = pl.image_bytes = 0;
   const int bn = oz_bn(d);
   const long long tm = (d.M + kOBM - 1) / kOBM, tn = (d.N + bn - 1) / bn, nb = static_cast<long long>(d.B0) * d.B1;
   AbsParams& ap = pl.ap;
