@@ -825,39 +825,49 @@ __device__ void wide_cols(float* dst, const float* M, long long n, int c, int c0
 // acc += sum over this warp's K slice of L(i, k) R(j, k) in pair arithmetic:
 // L a row tile; R a row tile (R(j, k) = row j) or, with rcol, a column tile
 // (R(j, k) = M[k][c0 + j]).  Operand order, renormalisation and the final
-// renormalisation are those of tile_fma_p.
-__device__ __forceinline__ void wide_fma(const float* L, const float* R, bool rcol, int c, int ldw,
+// renormalisation are those of tile_fma_p.  Bound by the issue of 24 FP32
+// instructions and the operand loads per k: eight k at a time (the loads ahead of
+// the sums, no counter), neighbouring columns in one load.  Rolled, with four
+// loads for them, a BF16x3 Heisenberg sweep at chi = 256 took 89.9 ms and a TF32
+// torus sweep at chi = 128 12.03; now 84.3 and 11.47 (the same bits).
+template <bool kCol>
+__device__ __forceinline__ void wide_mac(const float* Lh, const float* Ll, const float* R, int j, int k, int c, int ldw,
                                          float& a0h, float& a0l, float& a1h, float& a1l) {
+  const float xh = Lh[k], xl = Ll[k];
+  float2 h, l;
+  if constexpr (kCol) {
+    h = *reinterpret_cast<const float2*>(R + k * kLT + j);
+    l = *reinterpret_cast<const float2*>(R + kLT * c + k * kLT + j);
+  } else {
+    h = make_float2(R[j * ldw + k], R[(j + 1) * ldw + k]);
+    l = make_float2(R[(kLT + j) * ldw + k], R[(kLT + j + 1) * ldw + k]);
+  }
+  pair_mac(xh, xl, h.x, l.x, a0h, a0l);
+  pair_mac(xh, xl, h.y, l.y, a1h, a1l);
+}
+template <bool kCol>
+__device__ __forceinline__ void wide_fma_t(const float* L, const float* R, int c, int ldw,
+                                           float& a0h, float& a0l, float& a1h, float& a1l) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = lane >> 2, j = (lane & 3) * 2;
   const float* Lh = L + i * ldw;
   const float* Ll = L + (kLT + i) * ldw;
-  int cnt = 0;
-  for (int k = warp; k < c; k += kLWarps) {
-    const float xh = Lh[k], xl = Ll[k];
-    float r0h, r0l, r1h, r1l;
-    if (rcol) {
-      const float* R0 = R + k * kLT + j;
-      r0h = R0[0];
-      r1h = R0[1];
-      r0l = R0[kLT * c];
-      r1l = R0[kLT * c + 1];
-    } else {
-      r0h = R[j * ldw + k];
-      r1h = R[(j + 1) * ldw + k];
-      r0l = R[(kLT + j) * ldw + k];
-      r1l = R[(kLT + j + 1) * ldw + k];
-    }
-    pair_mac(xh, xl, r0h, r0l, a0h, a0l);
-    pair_mac(xh, xl, r1h, r1l, a1h, a1l);
-    if (++cnt == 8) {
-      cnt = 0;
-      pair_renorm(a0h, a0l);
-      pair_renorm(a1h, a1l);
-    }
+  int k = warp;
+  for (; k + 7 * kLWarps < c; k += 8 * kLWarps) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) wide_mac<kCol>(Lh, Ll, R, j, k + u * kLWarps, c, ldw, a0h, a0l, a1h, a1l);
+    pair_renorm(a0h, a0l);
+    pair_renorm(a1h, a1l);
   }
+#pragma unroll 1
+  for (; k < c; k += kLWarps) wide_mac<kCol>(Lh, Ll, R, j, k, c, ldw, a0h, a0l, a1h, a1l);
   pair_renorm(a0h, a0l);
   pair_renorm(a1h, a1l);
+}
+__device__ __forceinline__ void wide_fma(const float* L, const float* R, bool rcol, int c, int ldw,
+                                         float& a0h, float& a0l, float& a1h, float& a1l) {
+  if (rcol) wide_fma_t<true>(L, R, c, ldw, a0h, a0l, a1h, a1l);
+  else wide_fma_t<false>(L, R, c, ldw, a0h, a0l, a1h, a1l);
 }
 
 // The same three for FP64 tiles (row pitch c + 2 doubles).
