@@ -327,6 +327,14 @@ int ttn_selftest_gemm(void* d_ws, size_t bytes, int prec, double* out_rel, int n
  * FP64. */
 int ttn_selftest_df(void* d_ws, size_t bytes, double* out_rel, int n_out, void* stream);
 
+/* Diagnostic: FP64 products that also write an FP32 copy of their result (the
+ * polar factor's first try in the mixed modes), on every route that writes the
+ * result: eight cases (digit products as tiles, streamed and split over K, and
+ * the FP64 kernel after a refusal).  out[2 i] = max |C - C_fp64| / max |C_fp64|,
+ * out[2 i + 1] = entries of the copy that are not C rounded to FP32
+ * (n_out >= 16); d_ws: at least ttn_selftest_bytes() of device memory. */
+int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* stream);
+
 /* Allocation-free close product, for callers that cannot allocate device
  * memory (plug-ins inside an application that owns the CUDA allocator, or code
  * where cudaMalloc is not permitted); the paper has no counterpart.

@@ -66,6 +66,8 @@ SIGNATURES = {
                                          ctypes.c_int, ctypes.c_void_p]),
     "ttn_selftest_df": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_size_t, _dp, ctypes.c_int,
                                        ctypes.c_void_p]),
+    "ttn_selftest_digits": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_size_t, _dp, ctypes.c_int,
+                                           ctypes.c_void_p]),
     "ttn_close_noalloc": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int, ctypes.c_int,
                                          ctypes.c_longlong, ctypes.c_void_p, ctypes.c_void_p]),
     "ttn_autotune": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p,

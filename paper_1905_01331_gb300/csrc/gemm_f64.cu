@@ -12,6 +12,7 @@
 
 #include "../../include/ttn.h"
 #include "common.h"
+#include "f64_bits.cuh"
 
 namespace ttn {
 
@@ -39,7 +40,9 @@ __device__ __forceinline__ void st_out(const GemmDesc& d, long long e, double ac
     *c = d.beta == 0.0 ? (float)(d.alpha * acc) : (float)(d.alpha * acc + d.beta * (double)*c);
   } else {
     double* c = static_cast<double*>(d.C) + e;
-    *c = d.beta == 0.0 ? d.alpha * acc : d.alpha * acc + d.beta * *c;
+    const double v = d.beta == 0.0 ? d.alpha * acc : d.alpha * acc + d.beta * *c;
+    *c = v;
+    if (d.c32) d.c32[e] = f64b::to_f32(v);
   }
 }
 

@@ -379,7 +379,7 @@ __device__ __noinline__ void plain_tile(const GemmDesc& d, int b, int b0, int b1
     }
     double* out = out_ptr(d, b, b0, b1, split, m, n);
     *out = acc;
-    if (d.c32) d.c32[out - static_cast<double*>(d.C)] = static_cast<float>(acc);
+    if (d.c32 && d.splits <= 1) d.c32[out - static_cast<double*>(d.C)] = static_cast<float>(acc);
   }
 }
 
@@ -734,7 +734,8 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     const long long sn = d.splits > 1 ? 1 : d.sc_n;
     const int nv = m < d.M ? min(kPart, d.N - (n0 + part * kPart)) : 0;
     const bool vec = sn == 1 && nv == kPart && (reinterpret_cast<uintptr_t>(row) & 15) == 0;
-    float* row32 = d.c32 ? d.c32 + (row - static_cast<double*>(d.C)) : nullptr;   // (splits == 1)
+    // (split products: `row` is a partial sum, and the reduction writes the copy with C)
+    float* row32 = d.c32 && d.splits <= 1 ? d.c32 + (row - static_cast<double*>(d.C)) : nullptr;
     auto put = [&](int j, double x, double y) {
       if (row32) {
         if (j < nv) row32[j * sn] = f64b::to_f32(x);

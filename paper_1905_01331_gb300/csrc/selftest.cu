@@ -51,6 +51,20 @@ __global__ void max_abs_diff(const double* a, const double* b, long long n, doub
   if (threadIdx.x == 0) { out[0] = sd[0]; out[1] = sm[0]; }
 }
 
+// out[0] = number of i < n with a[i] != fl32(b[i]) (one block)
+__global__ void count_copy_errors(const float* a, const double* b, long long n, double* out) {
+  __shared__ double sd[256];
+  double bad = 0.0;
+  for (long long i = threadIdx.x; i < n; i += blockDim.x) bad += a[i] == static_cast<float>(b[i]) ? 0.0 : 1.0;
+  sd[threadIdx.x] = bad;
+  __syncthreads();
+  for (int s = 128; s > 0; s >>= 1) {
+    if (threadIdx.x < s) sd[threadIdx.x] += sd[threadIdx.x + s];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) out[0] = sd[0];
+}
+
 Operand mk(const double* p, long long mn, long long k0, long long k1 = 0, long long b0 = 0,
            long long b1 = 0) {
   Operand o;
@@ -367,5 +381,75 @@ extern "C" int ttn_selftest_df(void* d_ws, size_t bytes, double* out_rel, int n_
     if (cudaStreamSynchronize(s) != cudaSuccess) return TTN_ECUDA;
     out_rel[4] = host[0] / std::max(host[1], 1e-300);
   }
+  return cudaGetLastError() == cudaSuccess ? TTN_OK : TTN_ECUDA;
+}
+
+// Diagnostic: FP64 products with an FP32 copy of C (GemmDesc::c32), on every
+// route that writes C: the digit engine's tiles, its streamed kernel (either
+// side the large one), split-K products of both engines, and a product whose
+// scratch the digit engine refuses.  out[2 i] = max |C - C_fp64| / max |C_fp64|,
+// out[2 i + 1] = entries of the copy that are not C rounded to FP32.
+extern "C" int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* stream) {
+  struct Case { int M, N, K, splits, scratch; };
+  const Case cases[] = {{256, 256, 256, 1, 1}, {256, 256, 256, 2, 1},   {256, 256, 256, 1, 0}, {256, 256, 256, 2, 0},
+                        {96, 400, 256, 1, 1},  {128, 16384, 128, 1, 1}, {16384, 128, 128, 1, 1}, {128, 16384, 128, 2, 1}};
+  const int nc = sizeof(cases) / sizeof(cases[0]);
+  if (!d_ws || !out || n_out < 2 * nc) return TTN_EINVAL;
+  cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  gemm_oz_init();
+  double* base = reinterpret_cast<double*>(d_ws);
+  const size_t cap = bytes / sizeof(double);
+  size_t off = 0;
+  auto take = [&](size_t n) -> double* {
+    off = (off + 31) & ~size_t(31);
+    double* p = base + off;
+    off += n;
+    return p;
+  };
+  const size_t big = 16384 * 128;
+  double* A = take(big);
+  double* B = take(big);
+  double* C1 = take(big);
+  double* C2 = take(big);
+  float* C32 = reinterpret_cast<float*>(take(big / 2));
+  double* partial = take(2 * big);
+  double* words = take(2 * big);
+  double* res = take(4);
+  int* err = reinterpret_cast<int*>(take(1));
+  if (off > cap) return TTN_ENOMEM;
+  fill_uniform<<<592, 256, 0, s>>>(A, big, 41);
+  fill_uniform<<<592, 256, 0, s>>>(B, big, 43);
+  cudaMemsetAsync(err, 0, sizeof(int), s);
+  std::vector<double> host(3);
+  for (int i = 0; i < nc; ++i) {
+    const Case& cs = cases[i];
+    const long long n = (long long)cs.M * cs.N;
+    GemmDesc d;
+    memset(&d, 0, sizeof(d));
+    d.M = cs.M; d.N = cs.N; d.B0 = 1; d.B1 = 1;
+    d.C = C1; d.sc_m = cs.N; d.sc_n = 1;
+    d.alpha = 1.0; d.splits = 1; d.partial = partial; d.err = err;
+    Group g;
+    g.a = mk(A, cs.K, 1); g.b = mk(B, 1, cs.N); g.K = cs.K; g.k0_log2 = lg(cs.K);
+    d.g[d.ngroups++] = g;
+    gemm_launch(d, s);                       // FP64 kernel
+    d.C = C2;
+    d.c32 = C32;
+    d.digits = 1;
+    d.splits = cs.splits;
+    d.words = reinterpret_cast<unsigned*>(words);
+    d.words_bytes = cs.scratch ? 2 * big * sizeof(double) : 0;
+    cudaMemsetAsync(C32, 0xFF, n * sizeof(float), s);
+    gemm_launch(d, s);
+    max_abs_diff<<<1, 256, 0, s>>>(C2, C1, n, res);
+    count_copy_errors<<<1, 256, 0, s>>>(C32, C2, n, res + 2);
+    cudaMemcpyAsync(host.data(), res, 3 * sizeof(double), cudaMemcpyDeviceToHost, s);
+    if (cudaStreamSynchronize(s) != cudaSuccess) return TTN_ECUDA;
+    out[2 * i] = host[0] / std::max(host[1], 1e-300);
+    out[2 * i + 1] = host[2];
+  }
+  int e = 0;
+  cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e) return TTN_ETIMEOUT;
   return cudaGetLastError() == cudaSuccess ? TTN_OK : TTN_ECUDA;
 }
