@@ -332,7 +332,10 @@ int ttn_selftest_df(void* d_ws, size_t bytes, double* out_rel, int n_out, void* 
  * result: eight cases (digit products as tiles, streamed and split over K, and
  * the FP64 kernel after a refusal).  out[2 i] = max |C - C_fp64| / max |C_fp64|,
  * out[2 i + 1] = entries of the copy that are not C rounded to FP32
- * (n_out >= 16); d_ws: at least ttn_selftest_bytes() of device memory. */
+ * (n_out >= 16); with n_out >= 24 four more cases whose rows and columns are
+ * scaled by powers of two from 2^0 to 2^-150, out[2 i] = the largest error over
+ * the sum of K max|a_m| max|b_n| of the output's own row and column.  d_ws: at
+ * least ttn_selftest_bytes() of device memory. */
 int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* stream);
 
 /* Allocation-free close product, for callers that cannot allocate device
@@ -346,7 +349,14 @@ int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* 
  * device looks the array up (cudaGetSymbolAddress), so make that first call
  * before any stream capture.  Calls share the array: two calls that overlap on
  * the GPU race (use one stream, or order them).  Nothing needs clearing: each
- * call overwrites every partial sum it reads.  Limits: 1 <= P, Q <= 256 and
+ * call overwrites every partial sum it reads.  Accuracy: below 2^23
+ * multiply-adds, or with P or Q below 16, plain FP64 sums; above, exact sums of
+ * 62-bit fixed-point values, every row of Y and of W scaled by its own power of
+ * two: |error of C[p][q]| <= 2^-53 |C[p][q]| per partial sum (at most 152) plus
+ * n2 2^-57 max_j |Y[p][j]| max_j |W[q][j]|.  (A row's values 2^-62 below its
+ * largest do not count: a sum that lives on products of large and such small
+ * values of both rows keeps fewer digits than FP64 sums would.)  Infinities and
+ * NaN give what FP64 sums give.  Limits: 1 <= P, Q <= 256 and
  * 1 <= n2 <= 2^30, else TTN_EINVAL.  Work is enqueued on `stream` (cudaStream_t
  * as void*); the call allocates nothing. */
 int ttn_close_noalloc(const double* d_Y, const double* d_W, int P, int Q, long long n2,

@@ -128,6 +128,9 @@ size_t gemm_partial_elems(const GemmDesc& d, int splits);
 // below which the FP64 kernel stays (at 2^20 both take 15 us, at 2^24 the
 // digit engine 24 and the FP64 kernel 62).
 constexpr double kOzMinWork = 1 << 23;
+// Parts of K at most that the magnitudes of an operand's rows are kept in (one
+// word per row and part in the scratch of a product).
+constexpr int kOzMaxParts = 128;
 int gemm_oz_launch(const GemmDesc& d, cudaStream_t stream);
 bool gemm_oz_supported(const GemmDesc& d);
 int oz_pick_splits(const GemmDesc& d);

@@ -371,9 +371,10 @@ namespace ttn {
 namespace {
 
 constexpr long long kNoAllocScratchDoubles = 1LL << 20;   // 8 MiB of FP64 partial sums
-// the last of them hold the digit engine's magnitude words
-constexpr int kNoAllocWordDoubles = 512;
 constexpr int kNoAllocMaxDim = 256;
+// the last of them hold the digit engine's magnitude words, at most kOzMaxParts
+// for each of P + Q rows (256 KiB; 15 splits of a 256 x 256 product fit before them)
+constexpr int kNoAllocWordDoubles = 2 * kNoAllocMaxDim * kOzMaxParts / 2;
 constexpr int kNoAllocMaxDevices = 64;
 
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocScratchDoubles];
@@ -419,7 +420,7 @@ extern "C" int ttn_close_noalloc(const double* d_Y, const double* d_W, int P, in
   d.ngroups = 1;
   d.digits = 1;
   d.words = reinterpret_cast<unsigned*>(scratch + kNoAllocScratchDoubles - kNoAllocWordDoubles);
-  d.words_bytes = kNoAllocWordDoubles * sizeof(double);   // (needs at most 2 x 256 words)
+  d.words_bytes = kNoAllocWordDoubles * sizeof(double);
   const long long per_split = static_cast<long long>(P) * Q;
   int splits = gemm_pick_splits(d);
   splits = static_cast<int>(std::min<long long>(splits, (kNoAllocScratchDoubles - kNoAllocWordDoubles) / per_split));

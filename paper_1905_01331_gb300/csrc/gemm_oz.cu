@@ -2,20 +2,28 @@
 //
 // GB300 has two FP64 FMA units per SM (1.1 TFLOP/s for the whole GPU), so a
 // plain FP64 product is bound by them at any shape.  Here every FP64 operand is
-// cut into eight signed base-256 digits relative to the power of two above the
-// operand's largest magnitude (62 bits: elements within 2^-9 of the largest
-// are represented exactly) -- the error-free splitting of Ozaki, Ogita, Oishi
-// and Rump, "Error-free transformations of matrix multiplication", Numer.
-// Algorithms 59 (2012), with digits in place of floating-point slices (Mukunoki
-// et al., "DGEMM using tensor cores", ISC 2020).  A digit is an integer in
-// [-128, 127], exact in FP16; a product of two digits is below 2^14, and the
+// cut into eight signed base-256 digits, every row of A and every column of B
+// relative to the power of two above its own largest magnitude (62 bits:
+// elements within 2^-9 of the largest are represented exactly) -- the error-free
+// splitting of Ozaki, Ogita, Oishi and Rump, "Error-free transformations of
+// matrix multiplication", Numer. Algorithms 59 (2012), with digits in place of
+// floating-point slices (Mukunoki et al., "DGEMM using tensor cores", ISC 2020).
+// A digit is an integer in [-128, 127], exact in FP16; a product of two digits is
+// below 2^14, and the
 // digit products of one weight (i + j = l <= 7) over 128 values of K stay below
 // 2^24, so the tensor cores' FP32 accumulation of them is exact.  The 36 digit
-// products with i + j <= 7 go to eight accumulators, one per weight; what is
-// dropped is below 2^-62 of max|A| max|B| per term.  Every 128 values of K the
-// accumulators are combined into a 96-bit integer per output, which is rounded
-// to FP64 once at the end: the result carries one rounding instead of one per
-// term.
+// products with i + j <= 7 go to eight accumulators, one per weight.  What is
+// dropped is at most 7 2^-62 of the two powers of two, 28 2^-62 of max|a_m|
+// max|b_n| (largest magnitudes of the output's row and column); with the cut of
+// both operands 2^-57 max|a_m| max|b_n| per term at most.  Every 128 values of K
+// the accumulators are combined into a 96-bit integer per output, which is
+// rounded to FP64 once at the end: the result carries one rounding instead of
+// one per term.  One power of two per operand would lose rows that are small as
+// a whole (2^-40 below the largest: 3e-6 of their products) and costs less: FP64
+// sweep at chi = 128 23.93 ms, now 24.34; gradient of a torus at chi = 64 3.50,
+// now 3.62; measurement of a Heisenberg chain at chi = 128 3.24, now 3.31; close
+// product of 96 x 80 x 10007 53.3 us, now 54.5.  (In a sum of several groups, whose
+// scales differ by output, a tenth of the product; else 1 to 2 %.)
 //
 // One CTA owns a 128 x BN output tile (BN 64 or 32); two stages of 32 K values.
 // Warps 0-15 load FP64 operands (any strides), cut them into digits with integer
@@ -36,21 +44,22 @@
 // (eight before: 2 warps a scheduler, an instruction every third clock): FP64
 // sweep at chi = 128 25.29 -> 25.05 ms, FP64 gradient of a torus at chi = 64 3.61 ->
 // 3.46 ms, measurement 3.35 -> 3.23 ms.  Measured on a GB300 (P = n = 128, with the
-// preparation): F X of 128 x 128 by 128 x 16384 35 us (the FP64 kernel 547), the
-// environment's five such products in one 131 us (2674), three close products over
-// K = 16384 119 us (1931), the Gram matrix of 128 x 16384 56 us (449).  Converting
+// preparation): F X of 128 x 128 by 128 x 16384 37 us (the FP64 kernel 547), the
+// environment's five such products in one 163 us (2674), three close products over
+// K = 16384 128 us (1931), the Gram matrix of 128 x 16384 57 us (449).  Converting
 // both operands in every tile with BF16 digits, which take two operations more a
 // pair, and combining by eight converting instructions per output took 55, 186,
-// 123 and 59; loads whose 16-byte pieces are consecutive over four threads (K
-// permuted in a stage) took 5 % more than eight consecutive values per thread.
+// 123 and 59 (all with one power of two per operand, which now takes 35, 147, 126
+// and 55); loads whose 16-byte pieces are consecutive over four threads (K permuted
+// in a stage) took 5 % more than eight consecutive values per thread.
 // Relative error against extended precision 4e-17 to 2e-16 where the
 // FP64 kernel has 2e-16 to 2e-15.  At n = 32 both kernels take 15 to 30 us
 // (latency), so kOzMinWork lies between n = 32 (2^20 multiply-adds) and n = 64
 // (2^24: 21 against 58 us).
 //
-// An operand with an infinity or NaN, or whose range would leave the normal
-// FP64 numbers, makes the CTA compute its tile with plain FP64 FMAs instead, so
-// that the result is what the FP64 kernel gives.
+// A row or column of a tile with an infinity or NaN, or whose range would leave
+// the normal FP64 numbers, makes the CTA compute its tile with plain FP64 FMAs
+// instead, so that the result is what the FP64 kernel gives.
 #include <algorithm>
 #include <cstdint>
 #include <cstring>
@@ -75,13 +84,17 @@ constexpr int kOWork = kOConv / 32; // converter warps; the MMA warp follows the
 constexpr long kOWait = 1L << 22;
 constexpr int kOBlocks = 24;        // 16-column blocks of a CTA of the streamed kernel at most
 
-// Magnitude of an operand: `parts` words (the high words of |x|, at least 1 for
-// a nonzero x) per batch, at word off + (b0 s0 + b1 s1) parts.  img >= 0: the
-// operand's digits are ready in memory (oz_prepare_kernel), block (batch, row
-// tile, K slice of 32) at byte img + ((batch nrt + row tile) nks + slice) of
-// the block size, laid out as a stage of shared memory.
+// Magnitudes of an operand's rows (columns of B): the word (the high word of |x|,
+// at least 1 for a nonzero x) of the largest value of a row among 2^len_log2
+// values of K, part by part: word off + ((b0 s0 + b1 s1) parts + part) rows + row.
+// img >= 0: the operand's digits are ready in memory (oz_prepare_kernel), cut
+// under the largest value of the whole row (one part), block (batch, row tile, K
+// slice of 32) at byte img + ((batch nrt + row tile) nks + slice) of the block
+// size, laid out as a stage of shared memory.  chunk0, chunks: the group's chunks
+// of K among all; whole: rows are cut under their value over all of K (a group
+// with ready digits), else over the chunks that a CTA sums.
 struct OzOperand {
-  int off, parts, s0, s1, nrt, nks;
+  int off, parts, len_log2, rows, s0, s1, nrt, nks, chunk0, chunks, whole;
   long long img;
 };
 struct OzParams {
@@ -95,11 +108,15 @@ struct OzParams {
 
 struct AbsItem {
   const double* p;
-  long long s_mn, s_k0, s_k1, s_b0, s_b1, count, img;
-  int flat, mn, k0_log2, k, n0, n1, parts, off, blocks_before, nrt, nks, rt;
+  long long s_mn, s_k0, s_k1, s_b0, s_b1, img;
+  int mn, k0_log2, k, n0, n1, parts, len_log2, off, blocks_before, nrt, nks, rt;
 };
-constexpr int kAbsPer = 4096;       // elements per block of a magnitude pass
-constexpr int kAbsMaxParts = 512;
+constexpr int kAbsBlocks = 512;     // blocks that a pass over an operand is divided into
+// A row's exponent is kOBias + the biased exponent of the power of two above its
+// largest value, or 0 for a row of zeros.  (The sum of a row's and a column's fits
+// 15 bits, and pairs of sums are added and compared 16 bits each; the bias keeps
+// the sums with a row or column of zeros below all others.)
+constexpr int kOBias = 10000;
 struct AbsParams {
   AbsItem it[2 * kMaxGroups];
   int n;
@@ -109,6 +126,11 @@ struct AbsParams {
   int skip_when_zero;
 };
 static_assert(sizeof(AbsParams) < 32000, "kernel parameter");
+
+__device__ __forceinline__ int word_exponent(unsigned w) { return w ? static_cast<int>(w >> 20) + kOBias : 0; }
+// The exponent that a row's values are cut under (a row of zeros: any, its digits
+// are zero).
+__device__ __forceinline__ int cut_exponent(int e) { return e ? e - kOBias : 1023; }
 
 __device__ __forceinline__ unsigned mag_word(double x) {
   const unsigned hi = static_cast<unsigned>(__double2hiint(x)) & 0x7FFFFFFFu;
@@ -202,9 +224,10 @@ __device__ __forceinline__ void load8(long long s_mn, long long s_k0, long long 
 }
 
 // The digits of one stage block (ROWS rows from r0, 32 K values from k) of a
-// small operand into memory, by the whole block.
+// small operand into memory, by the whole block; words: its rows' magnitudes.
 template <int ROWS>
-__device__ __forceinline__ void image_block(const AbsItem& it, const double* p, int r0, int k, int emax, uint8_t* out) {
+__device__ __forceinline__ void image_block(const AbsItem& it, const double* p, int r0, int k, const unsigned* words,
+                                            uint8_t* out) {
   const bool kf = it.s_k0 == 1;
   const bool vec = kf && (reinterpret_cast<uintptr_t>(p) & 15) == 0 && ((it.s_mn | it.s_k1) & 1) == 0;
 #pragma unroll 1
@@ -213,15 +236,82 @@ __device__ __forceinline__ void image_block(const AbsItem& it, const double* p, 
     task_pos<ROWS>(task, kf, r, c);
     double v[8];
     load8(it.s_mn, it.s_k0, it.s_k1, it.k0_log2, p, r0 + r, r0 + r < it.mn, k + 8 * c, it.k, vec, v);
-    store_digits(v, emax, out, r, c, ROWS * 64);
+    store_digits(v, cut_exponent(word_exponent(words[r])), out, r, c, ROWS * 64);
   }
 }
 
-// Before a product: the magnitudes of its operands, and the digits of the
+// words[r] = the largest magnitude word of row r0 + r over K values k_lo .. k_hi
+// - 1, for R rows (32, 64 or 128); words hold 0 before.  K contiguous: a warp per
+// row, lanes along K, KS steps of K and 16 / KS rows at a time; else lanes along
+// the rows and the warps share K.  Sixteen loads in flight per thread.
+template <int KS>
+__device__ __forceinline__ void row_magnitudes_k(const AbsItem& it, const double* p, int r0, int R, int k_lo, int k_hi,
+                                                 unsigned* words) {
+  constexpr int kRows = 16 / KS;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kmask = (1 << it.k0_log2) - 1;
+#pragma unroll 1
+  for (int r = warp; r < R; r += 8 * kRows) {
+    unsigned m[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) m[i] = 0u;
+#pragma unroll 1
+    for (int k = k_lo + lane; k < k_hi; k += 32 * KS) {
+      double v[kRows][KS];
+#pragma unroll
+      for (int q = 0; q < KS; ++q) {
+        const int kk = k + 32 * q;
+        const bool in = kk < k_hi;
+        const double* pk = p + (in ? (kk & kmask) + static_cast<long long>(kk >> it.k0_log2) * it.s_k1 : 0);
+#pragma unroll
+        for (int i = 0; i < kRows; ++i)
+          v[i][q] = in && r + 8 * i < R && r0 + r + 8 * i < it.mn ? pk[(r0 + r + 8 * i) * it.s_mn] : 0.0;
+      }
+#pragma unroll
+      for (int i = 0; i < kRows; ++i)
+#pragma unroll
+        for (int q = 0; q < KS; ++q) m[i] = max(m[i], mag_word(v[i][q]));
+    }
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) {
+      m[i] = __reduce_max_sync(0xffffffffu, m[i]);
+      if (lane == 0 && r + 8 * i < R) words[r + 8 * i] = m[i];
+    }
+  }
+}
+__device__ __forceinline__ void row_magnitudes(const AbsItem& it, const double* p, int r0, int R, int k_lo, int k_hi,
+                                               unsigned* words) {
+  if (it.s_k0 == 1) {
+    if (k_hi - k_lo > 64) row_magnitudes_k<4>(it, p, r0, R, k_lo, k_hi, words);
+    else if (k_hi - k_lo > 32) row_magnitudes_k<2>(it, p, r0, R, k_lo, k_hi, words);
+    else row_magnitudes_k<1>(it, p, r0, R, k_lo, k_hi, words);
+    return;
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int kmask = (1 << it.k0_log2) - 1;
+  const int groups = R >> 5, rg = warp % groups, step = 8 / groups;
+  const int row = r0 + rg * 32 + lane;
+  if (row >= it.mn) return;
+  const double* pr = p + row * it.s_mn;
+  unsigned m = 0;
+#pragma unroll 1
+  for (int k = k_lo + warp / groups; k < k_hi; k += 16 * step) {
+    double v[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int kk = k + q * step;
+      v[q] = kk < k_hi ? pr[(kk & kmask) * it.s_k0 + static_cast<long long>(kk >> it.k0_log2) * it.s_k1] : 0.0;
+    }
+#pragma unroll
+    for (int q = 0; q < 16; ++q) m = max(m, mag_word(v[q]));
+  }
+  atomicMax(&words[rg * 32 + lane], m);
+}
+
+// Before a product: the magnitudes of its operands' rows, and the digits of the
 // small operands that many of its tiles read.
-//   without an image: words[off + batch parts + part] = the largest magnitude
-//     word of that part of the batch;
-//   with one: a block per stage block; each scans its whole (small) batch.
+//   without an image: a block per 32 to 128 rows of a batch and part of K;
+//   with one: a block per stage block; each scans its (few, short) rows.
 // Bound by the read of the operands (from L2 when they were just produced).
 __global__ void __launch_bounds__(256) oz_prepare_kernel(const AbsParams ap) {
   pdl_wait();
@@ -232,45 +322,26 @@ __global__ void __launch_bounds__(256) oz_prepare_kernel(const AbsParams ap) {
   const AbsItem& it = ap.it[i];
   const int u = blockIdx.x - it.blocks_before;
   const bool image = it.img >= 0;
-  const int per = image ? it.nrt * it.nks : it.parts;
-  const int batch = u / per, part = u % per;
+  const int inner = image ? it.nks : it.parts;       // K slices, or parts of K
+  const int rt = (u / inner) % it.nrt, ks = u % inner, batch = u / (inner * it.nrt);
   const int b0 = batch % it.n0, b1 = batch / it.n0;
   const double* p = it.p + b0 * it.s_b0 + static_cast<long long>(b1) * it.s_b1;
-  const long long lo = image ? 0 : it.count * part / it.parts, hi = image ? it.count : it.count * (part + 1) / it.parts;
-  unsigned m = 0;
-  if (it.flat) {
-    long long e = lo + threadIdx.x;
-    for (; e + 15 * 256 < hi; e += 16 * 256) {
-      double v[16];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) v[q] = p[e + q * 256];
-#pragma unroll
-      for (int q = 0; q < 16; ++q) m = max(m, mag_word(v[q]));
-    }
-    for (; e < hi; e += 256) m = max(m, mag_word(p[e]));
-  } else {
-    for (long long e = lo + threadIdx.x; e < hi; e += 256) {
-      const long long k = e / it.mn, r = e - k * it.mn;
-      const long long k0 = k & ((1LL << it.k0_log2) - 1), k1 = k >> it.k0_log2;
-      m = max(m, mag_word(p[r * it.s_mn + k0 * it.s_k0 + k1 * it.s_k1]));
-    }
-  }
-  m = __reduce_max_sync(0xffffffffu, m);
-  __shared__ unsigned sh[8];
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
+  const int r0 = rt * it.rt;
+  const int k_lo = image ? 0 : ks << it.len_log2, k_hi = image ? it.k : min(it.k, k_lo + (1 << it.len_log2));
+  __shared__ unsigned words[kOBM];
+  if (threadIdx.x < kOBM) words[threadIdx.x] = 0u;
   __syncthreads();
-  for (int w = 0; w < 8; ++w) m = max(m, sh[w]);
-  if (!image) {
-    if (threadIdx.x == 0) ap.words[it.off + u] = m;
-    return;
-  }
-  if (part == 0 && threadIdx.x == 0) ap.words[it.off + batch] = m;
-  const int rt = part / it.nks, ks = part % it.nks;
+  const int rows = it.mn - r0;
+  row_magnitudes(it, p, r0, min(it.rt, rows <= 32 ? 32 : (rows <= 64 ? 64 : 128)), k_lo, k_hi, words);
+  __syncthreads();
+  if (static_cast<int>(threadIdx.x) < it.rt && r0 + static_cast<int>(threadIdx.x) < it.mn && (!image || ks == 0))
+    ap.words[it.off + (static_cast<long long>(batch) * it.parts + (image ? 0 : ks)) * it.mn + r0 + threadIdx.x] =
+        words[threadIdx.x];
+  if (!image) return;
   uint8_t* out = ap.images + it.img + static_cast<long long>(u) * kOD * it.rt * 64;
-  const int emax = m ? static_cast<int>(m >> 20) : 1023;
-  if (it.rt == 128) image_block<128>(it, p, rt * 128, ks * kOBK, emax, out);
-  else if (it.rt == 64) image_block<64>(it, p, rt * 64, ks * kOBK, emax, out);
-  else image_block<32>(it, p, rt * 32, ks * kOBK, emax, out);
+  if (it.rt == 128) image_block<128>(it, p, r0, ks * kOBK, words, out);
+  else if (it.rt == 64) image_block<64>(it, p, r0, ks * kOBK, words, out);
+  else image_block<32>(it, p, r0, ks * kOBK, words, out);
 }
 
 __device__ __forceinline__ uint32_t osmem(const void* p) {
@@ -328,10 +399,15 @@ __host__ __device__ constexpr uint32_t oidesc(int N) {
          (static_cast<uint32_t>(kOBM >> 4) << 24);
 }
 
+// A sum of digit products of a row with exponent ea and a column with exponent
+// eb is an integer times 2^(ea + eb - kOScale).
+constexpr int kOScale = 2 * kOBias + 2 * 1022 + 68;
+
 // The 96-bit integer (a2 a1 a0, two's complement) times 2^scale, rounded to
 // FP64 (the caller has checked that the result is zero or a normal number).  A
-// negative value is complemented without the one: a unit of 2^scale, 2^-124 of
-// the operands' magnitudes, below the cut of their digits.
+// negative value is complemented without the one: a unit of 2^scale, 2^-68 of
+// the powers of two above the row's and the column's largest values, below the
+// dropped digit products.
 __device__ __forceinline__ double to_double(uint32_t a0, uint32_t a1, uint32_t a2, int scale) {
   const uint32_t neg = static_cast<uint32_t>(static_cast<int>(a2) >> 31);
   a0 ^= neg; a1 ^= neg; a2 ^= neg;
@@ -409,9 +485,9 @@ __device__ __forceinline__ void ld_wait(uint32_t (&r)[kOD][NC]) {
     for (int j = 0; j < NC; ++j) asm volatile("" : "+r"(r[l][j]));
 }
 
-// Combine the columns' accumulators into 96-bit integers, shifted right by sh.
+// Combine the columns' accumulators into 96-bit integers.
 template <int NC>
-__device__ __forceinline__ void combine(const uint32_t (&r)[kOD][NC], int sh, uint32_t (&v)[NC][3]) {
+__device__ __forceinline__ void combine(const uint32_t (&r)[kOD][NC], uint32_t (&v)[NC][3]) {
 #pragma unroll
   for (int j = 0; j < NC; ++j) {
     // levels 0 to 2 are at most 2^22 (digit 0 is at most 64): their integers sit
@@ -427,22 +503,44 @@ __device__ __forceinline__ void combine(const uint32_t (&r)[kOD][NC], int sh, ui
     const long long Q = static_cast<long long>(L[4]) * (1 << 24) + (static_cast<long long>(L[5]) * (1 << 16) +
                         (static_cast<long long>(L[6]) * 256 + L[7]));
     const long long hi = H + static_cast<int>(Q >> 32);
-    uint32_t v0 = static_cast<uint32_t>(Q), v1 = static_cast<uint32_t>(hi), v2 = static_cast<uint32_t>(hi >> 32);
-    if (sh) {   // (the same in all threads of the CTA)
-      const uint32_t sg = static_cast<uint32_t>(static_cast<int>(v2) >> 31);
-      int s2 = sh;
-      if (s2 >= 32) { v0 = v1; v1 = v2; v2 = sg; s2 -= 32; }
-      if (s2 >= 32) { v0 = v1; v1 = v2; s2 -= 32; }
-      if (s2 >= 32) { v0 = sg; v1 = sg; s2 = 0; }
-      v0 = __funnelshift_r(v0, v1, s2);
-      v1 = __funnelshift_r(v1, v2, s2);
-      v2 = static_cast<uint32_t>(static_cast<int>(v2) >> s2);
-    }
-    v[j][0] = v0; v[j][1] = v1; v[j][2] = v2;
+    v[j][0] = static_cast<uint32_t>(Q);
+    v[j][1] = static_cast<uint32_t>(hi);
+    v[j][2] = static_cast<uint32_t>(hi >> 32);
   }
 }
 
-template <int BN>
+// The 96-bit integer v shifted right by 0 <= sh <= 63.
+__device__ __forceinline__ void shift96(uint32_t (&v)[3], uint32_t sh) {
+  const uint32_t sg = static_cast<uint32_t>(static_cast<int>(v[2]) >> 31);
+  const bool w = sh >= 32u;
+  const uint32_t a0 = w ? v[1] : v[0], a1 = w ? v[2] : v[1], a2 = w ? sg : v[2];
+  v[0] = __funnelshift_r(a0, a1, sh);
+  v[1] = __funnelshift_r(a1, a2, sh);
+  v[2] = static_cast<uint32_t>(static_cast<int>(a2) >> (sh & 31u));
+}
+
+// Whether the digits do not cover a tile whose nonzero rows and columns have
+// exponents within [range[0], range[1]] and [range[2], range[3]]: its results
+// could leave the normal numbers.
+__device__ __forceinline__ bool plain_range(const int* range) {
+  return range[1] && range[3] &&
+         (range[1] + range[3] - kOScale > 900 || range[0] + range[2] - kOScale < -1000);
+}
+// The exponents of 32 rows (one per lane) into a range, by lane 0.
+__device__ __forceinline__ void add_range(int* range, int e) {
+  const int hi = __reduce_max_sync(0xffffffffu, e), lo = __reduce_min_sync(0xffffffffu, e ? e : 0x7FFF);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&range[0], lo);
+    atomicMax(&range[1], hi);
+  }
+}
+// Rows with infinities, NaN or so small values that their digits would be
+// subnormal: the tile is left to plain FP64.
+__device__ __forceinline__ bool plain_row(int e) { return e >= kOBias + 0x7FF || (e && e < kOBias + 80); }
+
+// kMulti: several groups (their sums are shifted to a common scale); without, the
+// same code at run time took 2 to 4 % of a product of one group.
+template <int BN, bool kMulti>
 __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d, const OzParams op) {
   pdl_wait();
   pdl_trigger();
@@ -455,7 +553,10 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
   __shared__ __align__(8) uint64_t full_bar[2], empty_bar[2], done_bar, free_bar, drain_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  __shared__ unsigned ex[2 * kMaxGroups];
+  // exponents of the tile's rows and columns, group by group, and their range
+  constexpr int kRB = (kOBM + BN) / 32;
+  __shared__ __align__(16) short ea[kMaxGroups][kOBM], eb[kMaxGroups][BN];
+  __shared__ int range[4], plain_flag;
 
   if (desc_skipped(d)) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -523,15 +624,6 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       for (int q = 0; q < kATasks; ++q) load_a(q);
     }
   }
-  // largest magnitude of every operand
-  for (int i = warp; i < 2 * d.ngroups; i += kOThreads / 32) {
-    const OzOperand& o = (i & 1) ? op.b[i >> 1] : op.a[i >> 1];
-    const unsigned* w = op.words + o.off + static_cast<long long>(b0 * o.s0 + b1 * o.s1) * o.parts;
-    unsigned m = 0;
-    for (int q = lane; q < o.parts; q += 32) m = max(m, __ldcg(w + q));
-    m = __reduce_max_sync(0xffffffffu, m);
-    if (lane == 0) ex[i] = m;
-  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) {
       omb_init(&full_bar[s], kOConv + 1);
@@ -541,23 +633,39 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     omb_init(&drain_bar, 1);
     omb_init(&free_bar, kOConv);
     abort_flag = 0;
+    range[0] = range[2] = 0x7FFF;
+    range[1] = range[3] = 0;
+    plain_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int u = warp; u < d.ngroups * kRB; u += kOThreads / 32) {
+    const int gi = u / kRB, q = u - gi * kRB;
+    const bool isb = q >= kOBM / 32;
+    const OzOperand& o = isb ? op.b[gi] : op.a[gi];
+    const int q_lo = max(0, c_lo - o.chunk0), q_hi = min(o.chunks, c_hi - o.chunk0);   // chunks of the group
+    int p_lo = 0, p_hi = q_lo < q_hi ? o.parts : 0;
+    if (!o.whole && q_lo < q_hi) {
+      p_lo = q_lo * kOChunk >> o.len_log2;
+      p_hi = min(p_hi, ((q_hi * kOChunk - 1) >> o.len_log2) + 1);
+    }
+    const int r = (isb ? q - kOBM / 32 : q) * 32 + lane, row = (isb ? n0 : m0) + r;
+    unsigned m = 0u;
+    if (row < o.rows) {
+      const unsigned* w = op.words + o.off + static_cast<long long>(b0 * o.s0 + b1 * o.s1) * o.parts * o.rows + row;
+#pragma unroll 4
+      for (int j = p_lo; j < p_hi; ++j) m = max(m, __ldcg(w + static_cast<long long>(j) * o.rows));
+    }
+    const int e = word_exponent(m);
+    if (isb) eb[gi][r] = static_cast<short>(e);
+    else ea[gi][r] = static_cast<short>(e);
+    if (plain_row(e)) plain_flag = 1;
+    add_range(&range[isb ? 2 : 0], e);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  // the scale of a group's digit products is 2^(ea + eb - 68); all groups are
-  // added relative to the largest one
-  int sref = -100000;
-  bool plain = false;
-  for (int g = 0; g < d.ngroups; ++g) {
-    const unsigned wa = ex[2 * g], wb = ex[2 * g + 1];
-    if (wa >= 0x7FF00000u || wb >= 0x7FF00000u) plain = true;
-    if (wa == 0u || wb == 0u) continue;      // an all-zero operand
-    const int s = static_cast<int>(wa >> 20) + static_cast<int>(wb >> 20) - 2 * 1022 - 68;
-    if (wa < (80u << 20) || wb < (80u << 20)) plain = true;
-    sref = max(sref, s);
-  }
-  if (sref != -100000 && (sref < -1000 || sref > 900)) plain = true;
+  const bool plain = plain_flag || plain_range(range);
   if (plain) plain_tile(d, b, b0, b1, split, m0, n0, BN, c_lo, c_hi);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
@@ -655,10 +763,29 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + part * kPart;
     bool ok = true;
     int flushed = 0;
-    auto shift_of = [&](int fg) {
-      const unsigned wa = ex[2 * fg], wb = ex[2 * fg + 1];
-      return (wa == 0u || wb == 0u) ? 0 : sref - (static_cast<int>(wa >> 20) + static_cast<int>(wb >> 20) - 2 * 1022 - 68);
-    };
+    // A group's sums of output (m, n) are integers times 2^(ea[m] + eb[n] - kOScale);
+    // with several groups they are shifted to the largest of these scales, which
+    // the thread keeps for its outputs in shared memory after the stages (pairs of
+    // columns, 16 bits each; only this thread reads them).  A shift common to the
+    // tile would need one exponent per operand, and rows that are small as a whole
+    // would lose their digits.
+    const int orow = quarter * 32 + lane;             // of the tile
+    uint32_t* top2 = reinterpret_cast<uint32_t*>(smem + 2 * kStage) + part * (kPart / 2) * kOBM + orow;
+    auto row2 = [&](int fg) { return static_cast<uint32_t>(ea[fg][orow]) * 0x10001u; };
+    auto col2 = [&](int fg, int j) { return *reinterpret_cast<const uint32_t*>(&eb[fg][part * kPart + j]); };
+    if constexpr (kMulti) {
+      uint32_t top[kPart / 2];
+#pragma unroll
+      for (int j = 0; j < kPart / 2; ++j) top[j] = 0u;
+#pragma unroll 1
+      for (int gi = 0; gi < d.ngroups; ++gi) {
+        const uint32_t a2 = row2(gi);
+#pragma unroll
+        for (int j = 0; j < kPart / 2; ++j) top[j] = __vmaxu2(a2 + col2(gi, 2 * j), top[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < kPart / 2; ++j) top2[j * kOBM] = top[j];
+    }
     constexpr int kF = 2;                            // columns combined together (registers)
     // add the eight accumulators of a finished chunk (of group fg) to acc
     auto flush = [&](int fg) {
@@ -666,14 +793,22 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       ++flushed;
       if (!ok) return;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const int sh = shift_of(fg);
+      const uint32_t a2 = kMulti ? row2(fg) : 0u;
 #pragma unroll
       for (int cb = 0; cb < kPart; cb += kF) {
         uint32_t v[kF][3];
         uint32_t r[kOD][kF];
         ld_levels(trow + cb, BN, r);
+        static_assert(kF == 2, "a pair of columns per shift word");
+        uint32_t sh2 = 0u;
+        // (below a shift of 63, 2^-63 of the largest group's magnitudes per term)
+        if constexpr (kMulti) sh2 = __vminu2(top2[cb / 2 * kOBM] - a2 - col2(fg, cb), 0x003F003Fu);
         ld_wait(r);
-        combine(r, sh, v);
+        combine(r, v);
+        if constexpr (kMulti) {
+          shift96(v[0], sh2 & 0xFFFFu);
+          shift96(v[1], sh2 >> 16);
+        }
 #pragma unroll
         for (int j = 0; j < kF; ++j)
           asm("add.cc.u32 %0, %0, %3;\n\taddc.cc.u32 %1, %1, %4;\n\taddc.u32 %2, %2, %5;"
@@ -687,10 +822,8 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     for (int c = 0; c <= nchunks && ok; ++c) {   // (one round more: the last flush)
       const int cg = g;
       const int nst = c == nchunks ? 0 : (min(d.g[g].K, k + kOChunk) - k + kOBK - 1) / kOBK;
-      const unsigned wa = ex[2 * cg], wb = ex[2 * cg + 1];
-      // (an all-zero operand: any exponent gives zero digits)
-      const int ea = wa ? static_cast<int>(wa >> 20) : 1023, eb = wb ? static_cast<int>(wb >> 20) : 1023;
       if (nst == 0 && nchunks == 1) break;       // a single chunk is stored from TMEM below
+      // (a CTA without chunks has not entered a group: no rows)
 #pragma unroll 1
       for (int st = 0; st < max(nst, 1); ++st, ++it) {
         const int s = it & 1;
@@ -701,10 +834,10 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
           uint8_t* sA = smem + s * kStage;
           uint8_t* sB = sA + kOD * kA;
           more = !(c + 1 == nchunks && st + 1 == nst);
-          if (b_on) store_digits(vb, eb, sB, br, bc, kB);
+          if (b_on) store_digits(vb, cut_exponent(eb[cg][br]), sB, br, bc, kB);
           if (a_on) {
 #pragma unroll
-            for (int q = 0; q < kATasks; ++q) store_digits(va[q], ea, sA, ar[q], ac[q], kA);
+            for (int q = 0; q < kATasks; ++q) store_digits(va[q], cut_exponent(ea[cg][ar[q]]), sA, ar[q], ac[q], kA);
           }
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           omb_arrive(&full_bar[s]);
@@ -754,24 +887,31 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       ok = __all_sync(0xffffffffu, omb_wait(&done_bar, 0, abort_v));
       if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int sh = shift_of(g0);
+        // (with several groups the others' K ranges are empty here: no shift)
+        const int fa = ea[g0][orow] - kOScale;
 #pragma unroll 1
         for (int cb = 0; cb < kPart; cb += 4) {
           uint32_t v[4][3];
           uint32_t r[kOD][4];
           ld_levels(trow + cb, BN, r);
           ld_wait(r);
-          combine(r, sh, v);
+          combine(r, v);
+          int e[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) e[j] = fa + eb[g0][part * kPart + cb + j];
 #pragma unroll
           for (int j = 0; j < 4; j += 2)
-            put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
+            put(cb + j, to_double(v[j][0], v[j][1], v[j][2], e[j]),
+                to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], e[j + 1]));
         }
       }
     } else if (ok) {
 #pragma unroll
-      for (int j = 0; j < kPart; j += 2)
-        put(j, to_double(acc[0][j], acc[1][j], acc[2][j], sref),
-            to_double(acc[0][j + 1], acc[1][j + 1], acc[2][j + 1], sref));
+      for (int j = 0; j < kPart; j += 2) {
+        const uint32_t t = kMulti ? top2[j / 2 * kOBM] : row2(0) + col2(0, j);
+        put(j, to_double(acc[0][j], acc[1][j], acc[2][j], static_cast<int>(t & 0xFFFFu) - kOScale),
+            to_double(acc[0][j + 1], acc[1][j + 1], acc[2][j + 1], static_cast<int>(t >> 16) - kOScale));
+      }
     }
     if (!ok) {
       *abort_v = 1;
@@ -808,9 +948,10 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   __shared__ __align__(8) uint64_t full_bar[2], empty_bar[2], done_bar, free_bar, drain_bar;
   __shared__ uint32_t tmem_slot;
-  __shared__ int abort_flag, plain_flag;
+  __shared__ int abort_flag;
   __shared__ OzSub subs[kOBlocks];
-  __shared__ int eb_s[kOBlocks], sref_s[kOBlocks];   // exponents of a sub-tile's B and of its sums
+  __shared__ short ea[kOBlocks][kOBM], eb[kOBlocks][kMaxN];   // exponents of a sub-tile's rows and columns
+  __shared__ int range[4], plain_flag;               // lowest and highest of the rows', then of the columns'
 
   if (desc_skipped(d)) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -849,6 +990,8 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
     omb_init(&drain_bar, 1);
     omb_init(&free_bar, kOConv);
     abort_flag = 0;
+    range[0] = range[2] = 0x7FFF;
+    range[1] = range[3] = 0;
     plain_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -890,31 +1033,29 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
     load_b();
   }
   __syncthreads();
-  // magnitudes: the exponents of every sub-tile's operands (a batch once)
-  for (int u = warp; u < nsub; u += kOThreads / 32) {
-    const int b0 = subs[u].b % d.B0, b1 = subs[u].b / d.B0;
-    unsigned w[2];
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const OzOperand& o = side ? ob : oa;
-      const unsigned* p = op.words + o.off + static_cast<long long>(b0 * o.s0 + b1 * o.s1) * o.parts;
-      unsigned m = 0;
-      for (int q = lane; q < o.parts; q += 32) m = max(m, __ldcg(p + q));
-      w[side] = __reduce_max_sync(0xffffffffu, m);
+  // magnitudes: the exponents of every sub-tile's rows and columns
+  constexpr int kRB = (kOBM + kMaxN) / 32;
+  for (int u = warp; u < nsub * kRB; u += kOThreads / 32) {
+    const int si = u / kRB, q = u % kRB;
+    const bool isb = q >= kOBM / 32;
+    const OzOperand& o = isb ? ob : oa;
+    const OzSub w = subs[si];
+    const int r = (isb ? q - kOBM / 32 : q) * 32 + lane, row = (isb ? w.n0 : w.m0) + r;
+    unsigned m = 0;
+    if (row < o.rows && (!isb || r < w.bn)) {
+      const unsigned* p = op.words + o.off +
+          static_cast<long long>((w.b % d.B0) * o.s0 + (w.b / d.B0) * o.s1) * o.parts * o.rows + row;
+      for (int i = 0; i < o.parts; ++i) m = max(m, __ldcg(p + static_cast<long long>(i) * o.rows));
     }
-    if (lane == 0) {
-      const int ea = w[0] >> 20, eb = w[1] >> 20;
-      // the scale of the digit products is 2^(ea + eb - 68); an all-zero operand gives zero digits
-      const bool zero = w[0] == 0u || w[1] == 0u;
-      const int sref = zero ? -100000 : ea + eb - 2 * 1022 - 68;
-      eb_s[u] = w[1] ? eb : 1023;
-      sref_s[u] = sref;
-      if (ea >= 0x7FF || eb >= 0x7FF || (!zero && (ea < 80 || eb < 80 || sref < -1000 || sref > 900))) plain_flag = 1;
-    }
+    const int e = word_exponent(m);
+    if (isb) eb[si][r] = static_cast<short>(e);
+    else ea[si][r] = static_cast<short>(e);
+    if (plain_row(e)) plain_flag = 1;
+    add_range(&range[isb ? 2 : 0], e);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  const bool plain = plain_flag != 0;
+  const bool plain = plain_flag || plain_range(range);
   if (plain)
     for (int u = 0; u < nsub; ++u)
       plain_tile(d, subs[u].b, subs[u].b % d.B0, subs[u].b / d.B0, 0, subs[u].m0, subs[u].n0, subs[u].bn, 0, 1);
@@ -997,7 +1138,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
       if (!ok) return;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const OzSub w = subs[u];
-      const int sref = sref_s[u], hc = w.bn >> 2;     // this warp's columns: 4, 8, 12 or 16
+      const int fa = ea[u][quarter * 32 + lane] - kOScale, hc = w.bn >> 2;   // this warp's columns: 4, 8, 12 or 16
       const uint32_t tcol = trow + part * hc;
       const int m = w.m0 + quarter * 32 + lane, nf = w.n0 + part * hc;
       double* row = out_ptr(d, w.b, w.b % d.B0, w.b / d.B0, 0, m, nf);
@@ -1026,10 +1167,14 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
           omb_arrive(&free_bar);
         }
-        combine(r, 0, v);
+        combine(r, v);
+        int e[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) e[j] = fa + eb[u][part * hc + cb + j];
 #pragma unroll
         for (int j = 0; j < 4; j += 2)
-          put(cb + j, to_double(v[j][0], v[j][1], v[j][2], sref), to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], sref));
+          put(cb + j, to_double(v[j][0], v[j][1], v[j][2], e[j]),
+              to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], e[j + 1]));
       }
     };
     int it = 0;
@@ -1039,7 +1184,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
         if ((it & 1) == hw) {
           if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[hw], ((it >> 1) - 1) & 1, abort_v));
           if (!ok) break;
-          if (b_on) store_digits(vb, eb_s[u], smem + hw * kStage + kOD * kA, br, bc, subs[u].bn * 64);
+          if (b_on) store_digits(vb, cut_exponent(eb[u][br]), smem + hw * kStage + kOD * kA, br, bc, subs[u].bn * 64);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
           omb_arrive(&full_bar[hw]);
           step();
@@ -1065,7 +1210,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
 }
 
 template <int BN>
-constexpr int oz_smem() { return 2 * kOD * (kOBM + BN) * 64 + 1024; }
+constexpr int oz_smem() { return 2 * kOD * (kOBM + BN) * 64 + BN * kOBM * 2 + 1024; }   // stages, scales, alignment
 
 int oz_chunks(const GemmDesc& d) {
   int t = 0;
@@ -1075,27 +1220,9 @@ int oz_chunks(const GemmDesc& d) {
 
 int oz_bn(const GemmDesc& d) { return d.N > 32 ? 64 : 32; }
 
-// The elements of one batch of an operand cover a dense range: count and true,
-// else the strided walk.
-bool flat_operand(const Operand& o, int k0_log2, int K, int mn, long long* count) {
-  const long long K0 = std::min<long long>(1LL << k0_log2, K), K1 = K0 < K ? K >> k0_log2 : 1;
-  long long ext[3] = {mn, K0, K1}, str[3] = {o.s_mn, o.s_k0, o.s_k1};
-  *count = static_cast<long long>(mn) * K;
-  long long need = 1;
-  for (int step = 0; step < 3; ++step) {
-    int f = -1;
-    for (int i = 0; i < 3; ++i)
-      if (ext[i] > 1 && str[i] == need) f = i;
-    if (f < 0) break;
-    need *= ext[f];
-    ext[f] = 1;
-  }
-  return ext[0] == 1 && ext[1] == 1 && ext[2] == 1;
-}
-
 bool same_operand(const AbsItem& a, const AbsItem& b) {
   return a.p == b.p && a.s_mn == b.s_mn && a.s_k0 == b.s_k0 && a.s_k1 == b.s_k1 && a.s_b0 == b.s_b0 &&
-         a.s_b1 == b.s_b1 && a.count == b.count && a.flat == b.flat && a.mn == b.mn && a.k == b.k &&
+         a.s_b1 == b.s_b1 && a.mn == b.mn && a.k == b.k &&
          a.k0_log2 == b.k0_log2 && a.n0 == b.n0 && a.n1 == b.n1 && a.rt == b.rt && (a.img >= 0) == (b.img >= 0);
 }
 
@@ -1106,6 +1233,7 @@ bool same_operand(const AbsItem& a, const AbsItem& b) {
 // 8, so a large operand is converted by the tiles that read it.)
 constexpr int kOzReuse = 8;
 constexpr long long kOzImageMax = 4 << 20;
+constexpr long long kOzImageCount = 1 << 16;   // values of a batch
 
 // The preparation of a product: items (operands, without repeats), their words
 // and images; returns the blocks of oz_prepare_kernel.
@@ -1126,7 +1254,9 @@ void plan_product(const GemmDesc& d, OzPlan& pl) {
   const int bn = oz_bn(d);
   const long long tm = (d.M + kOBM - 1) / kOBM, tn = (d.N + bn - 1) / bn, nb = static_cast<long long>(d.B0) * d.B1;
   AbsParams& ap = pl.ap;
-  for (int g = 0; g < d.ngroups; ++g)
+  int chunk0 = 0;
+  for (int g = 0; g < d.ngroups; ++g) {
+    const int chunks = (d.g[g].K + kOChunk - 1) / kOChunk;
     for (int side = 0; side < 2; ++side) {
       const Group& G = d.g[g];
       const Operand& o = side ? G.b : G.a;
@@ -1139,40 +1269,55 @@ void plan_product(const GemmDesc& d, OzPlan& pl) {
       it.k0_log2 = G.k0_log2;
       it.n0 = o.s_b0 ? d.B0 : 1;
       it.n1 = o.s_b1 ? d.B1 : 1;
-      it.flat = flat_operand(o, G.k0_log2, G.K, it.mn, &it.count) ? 1 : 0;
       it.rt = side ? bn : kOBM;
       it.nrt = (it.mn + it.rt - 1) / it.rt;
       it.nks = (G.K + kOBK - 1) / kOBK;
       const long long batches = static_cast<long long>(it.n0) * it.n1;
       const long long bytes = batches * it.nrt * it.nks * kOD * it.rt * 64;
       const long long reuse = (side ? tm : tn) * nb / batches;
-      const bool image = reuse >= kOzReuse && bytes <= kOzImageMax && it.count <= 16 * kAbsPer;
+      const bool image = reuse >= kOzReuse && bytes <= kOzImageMax && static_cast<long long>(it.mn) * G.K <= kOzImageCount;
       it.img = image ? 0 : -1;
-      it.parts = image ? 1 : static_cast<int>(std::max<long long>(1, std::min<long long>((it.count + kAbsPer - 1) / kAbsPer, kAbsMaxParts)));
+      it.parts = 1;
+      it.len_log2 = 30;                      // (ready digits: one part, all of K)
+      if (!image) {
+        // blocks of 32 rows (64 or 128 where K is short) by a part of K, a power of
+        // two of at least a chunk: as many parts as make kAbsBlocks blocks
+        it.rt = G.K > 64 ? 32 : (G.K > 32 ? 64 : 128);
+        it.nrt = (it.mn + it.rt - 1) / it.rt;
+        const long long want = std::max<long long>(1, std::min<long long>(kOzMaxParts, kAbsBlocks / (batches * it.nrt)));
+        it.len_log2 = 7;
+        while (((G.K - 1) >> it.len_log2) + 1 > want) ++it.len_log2;
+        it.parts = ((G.K - 1) >> it.len_log2) + 1;
+      }
       int at = 0;
       while (at < ap.n && !same_operand(ap.it[at], it)) ++at;
       if (at == ap.n) {
         it.off = static_cast<int>(pl.words);
         it.blocks_before = pl.blocks;
-        pl.words += it.parts * batches;
+        pl.words += it.parts * batches * it.mn;
         if (image) {
           it.img = pl.image_bytes;
           pl.image_bytes += bytes;
-          pl.blocks += static_cast<int>(batches) * it.nrt * it.nks;
-        } else {
-          pl.blocks += static_cast<int>(batches) * it.parts;
         }
+        pl.blocks += static_cast<int>(batches) * it.nrt * (image ? it.nks : it.parts);
         ap.it[ap.n++] = it;
       }
       OzOperand& w = side ? pl.op.b[g] : pl.op.a[g];
       w.off = ap.it[at].off;
       w.parts = ap.it[at].parts;
+      w.len_log2 = ap.it[at].len_log2;
+      w.rows = it.mn;
       w.s0 = o.s_b0 ? 1 : 0;
       w.s1 = o.s_b1 ? it.n0 : 0;
       w.nrt = it.nrt;
       w.nks = it.nks;
       w.img = ap.it[at].img;
+      w.chunk0 = chunk0;
+      w.chunks = chunks;
     }
+    pl.op.a[g].whole = pl.op.b[g].whole = pl.op.a[g].img >= 0 || pl.op.b[g].img >= 0;
+    chunk0 += chunks;
+  }
   // (at most as many tiles as SMs: one round of tiles is as short)
   pl.stream = d.ngroups == 1 && d.g[0].K <= kOChunk && bn == 64 && pl.op.a[0].img >= 0 && pl.op.b[0].img < 0 &&
               tm * tn * nb > device_sm_count() && tm * tn * nb < (1LL << 28);
@@ -1199,7 +1344,7 @@ bool exchange_sides(const GemmDesc& d) {
 }  // namespace
 
 // Products the digit engine takes: FP64 in and out, K0 a whole number of
-// 16-byte digit chunks, and enough work that the launch of absmax_kernel pays.
+// 16-byte digit chunks, and enough work that the launch of oz_prepare_kernel pays.
 bool gemm_oz_supported(const GemmDesc& d) {
   if (!d.digits || d.prec != 0 || d.c_f32 || d.alpha != 1.0 || d.beta != 0.0 || d.ngroups < 1 ||
       d.ngroups > kMaxGroups || d.M < 1 || d.N < 1)
@@ -1274,15 +1419,20 @@ int gemm_oz_launch(const GemmDesc& d0, cudaStream_t s) {
   dim3 grid(((d.M + kOBM - 1) / kOBM) * ((d.N + bn - 1) / bn), d.B0 * d.B1, d.splits);
   // always with programmatic serialisation: its only predecessor is the
   // preparation, so its CTAs wait for nothing else
-  if (bn == 64) launch_attr(true, gemm_oz_kernel<64>, grid, kOThreads, oz_smem<64>(), s, d, pl.op);
-  else launch_attr(true, gemm_oz_kernel<32>, grid, kOThreads, oz_smem<32>(), s, d, pl.op);
+  const bool multi = d.ngroups > 1;
+  if (bn == 64)
+    launch_attr(true, multi ? gemm_oz_kernel<64, true> : gemm_oz_kernel<64, false>, grid, kOThreads, oz_smem<64>(), s, d, pl.op);
+  else
+    launch_attr(true, multi ? gemm_oz_kernel<32, true> : gemm_oz_kernel<32, false>, grid, kOThreads, oz_smem<32>(), s, d, pl.op);
   return 2;
 }
 
 void gemm_oz_init() {
-  cudaFuncSetAttribute(gemm_oz_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<64>());
+  cudaFuncSetAttribute(gemm_oz_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<64>());
+  cudaFuncSetAttribute(gemm_oz_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<64>());
   cudaFuncSetAttribute(gemm_oz_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<64>());
-  cudaFuncSetAttribute(gemm_oz_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<32>());
+  cudaFuncSetAttribute(gemm_oz_kernel<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<32>());
+  cudaFuncSetAttribute(gemm_oz_kernel<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, oz_smem<32>());
 }
 
 }  // namespace ttn

@@ -65,6 +65,37 @@ __global__ void count_copy_errors(const float* a, const double* b, long long n, 
   if (threadIdx.x == 0) out[0] = sd[0];
 }
 
+// Powers of two of the graded products: row m and column n of group g.
+__host__ __device__ __forceinline__ int row_grade(int m, int g) { return (7 * m + 31 * g) % 120; }
+__host__ __device__ __forceinline__ int col_grade(int n, int g) { return (11 * n + 53 * g) % 150; }
+
+// dst = src (rows x cols) with every row, or every column, scaled by its grade.
+__global__ void grade(const double* src, double* dst, int rows, long long cols, bool by_row, int g) {
+  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * cols;
+       e += (long long)gridDim.x * blockDim.x) {
+    const int r = (int)(e / cols), c = (int)(e % cols);
+    dst[e] = ldexp(src[e], by_row ? -row_grade(r, g) : -col_grade(c, g));
+  }
+}
+
+// out[0] = max |a - b| over sum_g K 2^-(grades of the entry) (one block)
+__global__ void max_graded_diff(const double* a, const double* b, int M, int N, int K, int groups, double* out) {
+  __shared__ double sd[256];
+  double d = 0.0;
+  for (long long e = threadIdx.x; e < (long long)M * N; e += blockDim.x) {
+    double t = 0.0;
+    for (int g = 0; g < groups; ++g) t += ldexp((double)K, -row_grade((int)(e / N), g) - col_grade((int)(e % N), g));
+    const double x = fabs(a[e] - b[e]) / t;
+    d = x <= d ? d : x;   // (a NaN stays)
+  }
+  sd[threadIdx.x] = d;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 256; ++i) d = sd[i] <= d ? d : sd[i];
+    out[0] = d;
+  }
+}
+
 Operand mk(const double* p, long long mn, long long k0, long long k1 = 0, long long b0 = 0,
            long long b1 = 0) {
   Operand o;
@@ -388,13 +419,19 @@ extern "C" int ttn_selftest_df(void* d_ws, size_t bytes, double* out_rel, int n_
 // route that writes C: the digit engine's tiles, its streamed kernel (either
 // side the large one), split-K products of both engines, and a product whose
 // scratch the digit engine refuses.  out[2 i] = max |C - C_fp64| / max |C_fp64|,
-// out[2 i + 1] = entries of the copy that are not C rounded to FP32.
+// out[2 i + 1] = entries of the copy that are not C rounded to FP32.  With n_out
+// >= 24 also operands whose rows and columns are graded over 2^0 to 2^-150, each
+// group in its own way: streamed (either side the large one), split over K, and
+// three groups (tiles of several exponents); out[2 i] = the largest |C - C_fp64|
+// over sum_g K max|a_m| max|b_n| of its own row and column.
 extern "C" int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* stream) {
-  struct Case { int M, N, K, splits, scratch; };
-  const Case cases[] = {{256, 256, 256, 1, 1}, {256, 256, 256, 2, 1},   {256, 256, 256, 1, 0}, {256, 256, 256, 2, 0},
-                        {96, 400, 256, 1, 1},  {128, 16384, 128, 1, 1}, {16384, 128, 128, 1, 1}, {128, 16384, 128, 2, 1}};
-  const int nc = sizeof(cases) / sizeof(cases[0]);
-  if (!d_ws || !out || n_out < 2 * nc) return TTN_EINVAL;
+  struct Case { int M, N, K, splits, scratch, graded; };   // graded: groups (0: one, not graded)
+  const Case cases[] = {{256, 256, 256, 1, 1, 0},     {256, 256, 256, 2, 1, 0},   {256, 256, 256, 1, 0, 0},
+                        {256, 256, 256, 2, 0, 0},     {96, 400, 256, 1, 1, 0},    {128, 16384, 128, 1, 1, 0},
+                        {16384, 128, 128, 1, 1, 0},   {128, 16384, 128, 2, 1, 0}, {128, 16384, 128, 1, 1, 1},
+                        {10000, 128, 64, 1, 1, 1},    {256, 256, 256, 2, 1, 1},   {130, 2500, 128, 1, 1, 3}};
+  const int nc = n_out >= 24 ? 12 : 8;
+  if (!d_ws || !out || n_out < 16) return TTN_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   gemm_oz_init();
   double* base = reinterpret_cast<double*>(d_ws);
@@ -414,6 +451,7 @@ extern "C" int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_
   float* C32 = reinterpret_cast<float*>(take(big / 2));
   double* partial = take(2 * big);
   double* words = take(2 * big);
+  double* graded = take(3 * big);
   double* res = take(4);
   int* err = reinterpret_cast<int*>(take(1));
   if (off > cap) return TTN_ENOMEM;
@@ -429,9 +467,18 @@ extern "C" int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_
     d.M = cs.M; d.N = cs.N; d.B0 = 1; d.B1 = 1;
     d.C = C1; d.sc_m = cs.N; d.sc_n = 1;
     d.alpha = 1.0; d.splits = 1; d.partial = partial; d.err = err;
-    Group g;
-    g.a = mk(A, cs.K, 1); g.b = mk(B, 1, cs.N); g.K = cs.K; g.k0_log2 = lg(cs.K);
-    d.g[d.ngroups++] = g;
+    for (int q = 0; q < std::max(1, cs.graded); ++q) {
+      double *a = A, *b = B;
+      if (cs.graded) {
+        a = graded + q * (big / 2);
+        b = graded + q * (big / 2) + (long long)cs.M * cs.K;
+        grade<<<592, 256, 0, s>>>(A, a, cs.M, cs.K, true, q);
+        grade<<<592, 256, 0, s>>>(B, b, cs.K, cs.N, false, q);
+      }
+      Group g;
+      g.a = mk(a, cs.K, 1); g.b = mk(b, 1, cs.N); g.K = cs.K; g.k0_log2 = lg(cs.K);
+      d.g[d.ngroups++] = g;
+    }
     gemm_launch(d, s);                       // FP64 kernel
     d.C = C2;
     d.c32 = C32;
@@ -441,11 +488,12 @@ extern "C" int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_
     d.words_bytes = cs.scratch ? 2 * big * sizeof(double) : 0;
     cudaMemsetAsync(C32, 0xFF, n * sizeof(float), s);
     gemm_launch(d, s);
-    max_abs_diff<<<1, 256, 0, s>>>(C2, C1, n, res);
+    if (cs.graded) max_graded_diff<<<1, 256, 0, s>>>(C2, C1, cs.M, cs.N, cs.K, cs.graded, res);
+    else max_abs_diff<<<1, 256, 0, s>>>(C2, C1, n, res);
     count_copy_errors<<<1, 256, 0, s>>>(C32, C2, n, res + 2);
     cudaMemcpyAsync(host.data(), res, 3 * sizeof(double), cudaMemcpyDeviceToHost, s);
     if (cudaStreamSynchronize(s) != cudaSuccess) return TTN_ECUDA;
-    out[2 * i] = host[0] / std::max(host[1], 1e-300);
+    out[2 * i] = cs.graded ? host[0] : host[0] / std::max(host[1], 1e-300);
     out[2 * i + 1] = host[2];
   }
   int e = 0;

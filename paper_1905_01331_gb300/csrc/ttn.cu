@@ -1063,8 +1063,11 @@ void polar(ttn_ctx* h, Instance& I, int t, int prec, const double* Gam) {
   int* run_full = try_first ? I.ppred + nT + t : nullptr;
   // The first try's products over X on the digit engine (gemm_oz.cu), where the
   // layer is large enough for it: a well-conditioned factor is the same to
-  // 1e-13, at 56 (Gram) and 41 us (apply) where the double-float products take 88
-  // and 127 (P = 128, N = 16384).  The full schedule keeps the double-float
+  // 1e-13, at 57 (Gram) and 41 us (apply) where the double-float products take 88
+  // and 127 (P = 128, N = 16384).  Every row of X and of F is cut at 2^-61 of its
+  // own largest value: values below 2^-14 of that keep fewer bits than their FP32
+  // pair, but the sums they enter carry the pairs' 2^-48 of the larger ones there
+  // and 2^-57 here.  The full schedule keeps the double-float
   // products: the directions it amplifies by up to 1e7 carry their rounding.
   const bool oz_try = try_first && oz_gram_ok(P, N);
   if (df_ok && !h->measuring && !adaptive)
@@ -1449,7 +1452,12 @@ void sweep_instance(ttn_ctx* h, Instance& I) {
     // product divided by mu = 1e-7.  It stays on the FP64 units (2.7 ms of an
     // FP64 sweep at P = n = 128), so that those directions are those of plain
     // FP64 sums; with the digit engine they differ by up to 4.5e-8 of the
-    // isometry's entries.
+    // isometry's entries.  The lower layers' environments have no such
+    // directions (two roundings of their products move no entry of an isometry
+    // by more than 8e-9 in a sweep at chi = 128), and an environment or a
+    // gradient that is itself the result divides by no mu: there the digit
+    // products are as far from extended precision as FP64 sums are (4e-17 to
+    // 2e-16 against 2e-16 to 2e-15).
     environment(h, I, t, prec, h->Gam, t == I.T - 1);
     polar(h, I, t, prec, h->Gam);
     descend(h, I, t, prec);
