@@ -334,8 +334,11 @@ int ttn_selftest_df(void* d_ws, size_t bytes, double* out_rel, int n_out, void* 
  * out[2 i + 1] = entries of the copy that are not C rounded to FP32
  * (n_out >= 16); with n_out >= 24 four more cases whose rows and columns are
  * scaled by powers of two from 2^0 to 2^-150, out[2 i] = the largest error over
- * the sum of K max|a_m| max|b_n| of the output's own row and column.  d_ws: at
- * least ttn_selftest_bytes() of device memory. */
+ * the sum of K max|a_m| max|b_n| of the output's own row and column; with n_out >=
+ * 30 three more whose internal waits expire at once (every wait still ends, and
+ * the context stays usable), out[2 i] = outputs that are numbers without an error
+ * flag, out[2 i + 1] = the flag with one.  d_ws: at least ttn_selftest_bytes() of
+ * device memory. */
 int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* stream);
 
 /* Allocation-free close product, for callers that cannot allocate device
@@ -356,7 +359,9 @@ int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* 
  * n2 2^-57 max_j |Y[p][j]| max_j |W[q][j]|.  (A row's values 2^-62 below its
  * largest do not count: a sum that lives on products of large and such small
  * values of both rows keeps fewer digits than FP64 sums would.)  Infinities and
- * NaN give what FP64 sums give.  Limits: 1 <= P, Q <= 256 and
+ * NaN give what FP64 sums give.  The kernel's internal waits are bounded; should
+ * one expire (a call cannot report it, it returns before the work runs), the
+ * outputs that it leaves are NaN.  Limits: 1 <= P, Q <= 256 and
  * 1 <= n2 <= 2^30, else TTN_EINVAL.  Work is enqueued on `stream` (cudaStream_t
  * as void*); the call allocates nothing. */
 int ttn_close_noalloc(const double* d_Y, const double* d_W, int P, int Q, long long n2,

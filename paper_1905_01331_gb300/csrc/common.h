@@ -98,6 +98,7 @@ struct GemmDesc {
   int digits;        // FP64 products: the digit engine (gemm_oz.cu) where it is supported
   unsigned* words;   // its scratch (oz_scratch(d) bytes) and the bytes there are
   size_t words_bytes;
+  int no_waits;      // digit engine: every wait expires at once (the tests of that path)
   float* c32;        // FP64 products: also the FP32 copy of C, at C's offsets (may be null);
                      // written by whatever writes C: an engine's kernel or the split-K reduction
   int occ;           // TMA-fed kernel: 2 = the 96 KB stage ring (two CTAs per

@@ -103,7 +103,8 @@ struct OzParams {
   OzOperand a[kMaxGroups], b[kMaxGroups];
   int total_chunks;
   int blocks, nb16;                 // streamed kernel: 16-column blocks in all and per row tile
-  int* err;
+  long wait;                        // tries of a wait before it expires
+  int* err;                         // raised by an expired wait; null: the outputs it leaves become NaN
 };
 
 struct AbsItem {
@@ -348,9 +349,10 @@ __device__ __forceinline__ uint32_t osmem(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-__device__ __forceinline__ bool omb_wait(uint64_t* bar, uint32_t parity, const volatile int* abort_flag) {
+__device__ __forceinline__ bool omb_wait(uint64_t* bar, uint32_t parity, const volatile int* abort_flag,
+                                         long tries = kOWait) {
   const uint32_t a = osmem(bar);
-  for (long it = 0; it < kOWait; ++it) {
+  for (long it = 0; it < tries; ++it) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -683,13 +685,13 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       int g = g0, k = kfirst, it = 0;
       const uint32_t base = osmem(smem);
       for (int c = 0; c < nchunks && ok; ++c) {
-        if (c > 0 && !omb_wait(&free_bar, (c - 1) & 1, abort_v)) { ok = false; break; }
+        if (c > 0 && !omb_wait(&free_bar, (c - 1) & 1, abort_v, op.wait)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int kend = min(d.g[g].K, k + kOChunk);
         const int nst = (kend - k + kOBK - 1) / kOBK;
         for (int st = 0; st < nst; ++st, ++it) {
           const int s = it & 1;
-          if (!omb_wait(&full_bar[s], (it >> 1) & 1, abort_v)) { ok = false; break; }
+          if (!omb_wait(&full_bar[s], (it >> 1) & 1, abort_v, op.wait)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t sa = base + s * kStage, sb = sa + kOD * kA;
 #pragma unroll
@@ -730,7 +732,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
         const OzOperand &oa = op.a[g], &ob = op.b[g];
         for (int ks = k / kOBK; ks * kOBK < kend; ++ks, ++it) {
           const int s = it & 1;
-          if (it >= 2 && !omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v)) { ok = false; break; }
+          if (it >= 2 && !omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v, op.wait)) { ok = false; break; }
           const uint32_t bytes = (oa.img >= 0 ? kOD * kA : 0) + (ob.img >= 0 ? kOD * kB : 0);
           if (!bytes) { omb_arrive(&full_bar[s]); continue; }
           omb_expect(&full_bar[s], bytes);
@@ -789,7 +791,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     constexpr int kF = 2;                            // columns combined together (registers)
     // add the eight accumulators of a finished chunk (of group fg) to acc
     auto flush = [&](int fg) {
-      ok = __all_sync(0xffffffffu, ok && omb_wait(&done_bar, flushed & 1, abort_v));
+      ok = __all_sync(0xffffffffu, ok && omb_wait(&done_bar, flushed & 1, abort_v, op.wait));
       ++flushed;
       if (!ok) return;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -829,7 +831,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
         const int s = it & 1;
         bool more = false;
         if (nst) {
-          if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v));
+          if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v, op.wait));
           if (!ok) break;
           uint8_t* sA = smem + s * kStage;
           uint8_t* sB = sA + kOD * kA;
@@ -884,7 +886,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
     if (ok && nchunks == 1) {
       // one chunk: straight from the accumulators, four columns at a time (a
       // short loop: unrolled, its instructions took longer to fetch than to run)
-      ok = __all_sync(0xffffffffu, omb_wait(&done_bar, 0, abort_v));
+      ok = __all_sync(0xffffffffu, omb_wait(&done_bar, 0, abort_v, op.wait));
       if (ok) {
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // (with several groups the others' K ranges are empty here: no shift)
@@ -914,8 +916,14 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_kernel(const GemmDesc d,
       }
     }
     if (!ok) {
+      // an expired wait: reported, or where the caller has no flag to read the
+      // warp's outputs are NaN
       *abort_v = 1;
       if (op.err && t == 0) atomicOr(op.err, 1);
+      if (!op.err) {
+        const double nan = __longlong_as_double(0x7FF8000000000000ll);
+        for (int j = 0; j < kPart; j += 2) put(j, nan, nan);
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1073,11 +1081,11 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
       const uint32_t base = osmem(smem);
       for (int u = 0; u < nsub && ok; ++u) {
         const int bn = subs[u].bn;
-        if (u > 0 && !omb_wait(&free_bar, (u - 1) & 1, abort_v)) { ok = false; break; }
+        if (u > 0 && !omb_wait(&free_bar, (u - 1) & 1, abort_v, op.wait)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         for (int st = 0; st < nst; ++st, ++it) {
           const int s = it & 1;
-          if (!omb_wait(&full_bar[s], (it >> 1) & 1, abort_v)) { ok = false; break; }
+          if (!omb_wait(&full_bar[s], (it >> 1) & 1, abort_v, op.wait)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t sa = base + s * kStage, sb = sa + kOD * kA;
 #pragma unroll 1
@@ -1118,7 +1126,7 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
             (static_cast<long long>(b0 * oa.s0 + b1 * oa.s1) * oa.nrt + subs[u].m0 / kOBM) * oa.nks * (kOD * kA);
         for (int st = 0; st < nst; ++st, ++it) {
           const int s = it & 1;
-          if (it >= 2 && !omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v)) { ok = false; break; }
+          if (it >= 2 && !omb_wait(&empty_bar[s], ((it >> 1) - 1) & 1, abort_v, op.wait)) { ok = false; break; }
           omb_expect(&full_bar[s], kOD * kA);
           bulk_load(base + s * kStage, src + st * (kOD * kA), kOD * kA, &full_bar[s]);
         }
@@ -1133,8 +1141,9 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
     const int quarter = warp & 3, part = warp >> 2;
     const uint32_t trow = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     bool ok = true;
+    int stored = 0;                                   // sub-tiles
     auto flush = [&](int u) {
-      ok = __all_sync(0xffffffffu, ok && omb_wait(&done_bar, u & 1, abort_v));
+      ok = __all_sync(0xffffffffu, ok && omb_wait(&done_bar, u & 1, abort_v, op.wait));
       if (!ok) return;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const OzSub w = subs[u];
@@ -1176,13 +1185,14 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
           put(cb + j, to_double(v[j][0], v[j][1], v[j][2], e[j]),
               to_double(v[j + 1][0], v[j + 1][1], v[j + 1][2], e[j + 1]));
       }
+      stored = u + 1;
     };
     int it = 0;
     for (int u = 0; u < nsub && ok; ++u) {
 #pragma unroll 1
       for (int st = 0; st < nst; ++st, ++it) {
         if ((it & 1) == hw) {
-          if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[hw], ((it >> 1) - 1) & 1, abort_v));
+          if (it >= 2) ok = __all_sync(0xffffffffu, omb_wait(&empty_bar[hw], ((it >> 1) - 1) & 1, abort_v, op.wait));
           if (!ok) break;
           if (b_on) store_digits(vb, cut_exponent(eb[u][br]), smem + hw * kStage + kOD * kA, br, bc, subs[u].bn * 64);
           asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1201,6 +1211,14 @@ __global__ void __launch_bounds__(kOThreads, 1) gemm_oz_stream_kernel(const Gemm
     if (!ok) {
       *abort_v = 1;
       if (op.err && threadIdx.x == 0) atomicOr(op.err, 1);
+      // (without a flag: NaN, as above)
+      for (int u = stored; u < nsub && !op.err; ++u) {
+        const OzSub w = subs[u];
+        const int hc = w.bn >> 2, m = w.m0 + quarter * 32 + lane, nf = w.n0 + part * hc;
+        double* row = out_ptr(d, w.b, w.b % d.B0, w.b / d.B0, 0, m, nf);
+        for (int j = 0; j < hc; ++j)
+          if (m < d.M && nf + j < d.N) row[j * d.sc_n] = __longlong_as_double(0x7FF8000000000000ll);
+      }
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1405,6 +1423,7 @@ int gemm_oz_launch(const GemmDesc& d0, cudaStream_t s) {
   pl.op.words = pl.ap.words;
   pl.op.images = pl.ap.images;
   pl.op.total_chunks = oz_chunks(d);
+  pl.op.wait = d.no_waits ? 0 : kOWait;
   pl.op.err = d.err;
   if (pl.stream && d.splits <= 1) {
     // one CTA per SM, or more when a CTA's share would exceed kOBlocks

@@ -69,6 +69,18 @@ __global__ void count_copy_errors(const float* a, const double* b, long long n, 
 __host__ __device__ __forceinline__ int row_grade(int m, int g) { return (7 * m + 31 * g) % 120; }
 __host__ __device__ __forceinline__ int col_grade(int n, int g) { return (11 * n + 53 * g) % 150; }
 
+// out[0] = number of i < n with a[i] not a NaN (one block)
+__global__ void count_numbers(const double* a, long long n, double* out) {
+  __shared__ int sum;
+  if (threadIdx.x == 0) sum = 0;
+  __syncthreads();
+  int c = 0;
+  for (long long i = threadIdx.x; i < n; i += blockDim.x) c += a[i] == a[i];
+  atomicAdd(&sum, c);
+  __syncthreads();
+  if (threadIdx.x == 0) out[0] = sum;
+}
+
 // dst = src (rows x cols) with every row, or every column, scaled by its grade.
 __global__ void grade(const double* src, double* dst, int rows, long long cols, bool by_row, int g) {
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < rows * cols;
@@ -423,7 +435,10 @@ extern "C" int ttn_selftest_df(void* d_ws, size_t bytes, double* out_rel, int n_
 // >= 24 also operands whose rows and columns are graded over 2^0 to 2^-150, each
 // group in its own way: streamed (either side the large one), split over K, and
 // three groups (tiles of several exponents); out[2 i] = the largest |C - C_fp64|
-// over sum_g K max|a_m| max|b_n| of its own row and column.
+// over sum_g K max|a_m| max|b_n| of its own row and column.  With n_out >= 30
+// also products whose waits expire at once, as tiles (one and two splits) and
+// streamed: out[2 i] = outputs that are numbers where the caller gave no error
+// flag, out[2 i + 1] = the flag where it gave one.
 extern "C" int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* stream) {
   struct Case { int M, N, K, splits, scratch, graded; };   // graded: groups (0: one, not graded)
   const Case cases[] = {{256, 256, 256, 1, 1, 0},     {256, 256, 256, 2, 1, 0},   {256, 256, 256, 1, 0, 0},
@@ -499,5 +514,32 @@ extern "C" int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_
   int e = 0;
   cudaMemcpy(&e, err, sizeof(int), cudaMemcpyDeviceToHost);
   if (e) return TTN_ETIMEOUT;
+  const Case expired[] = {{200, 256, 256, 1, 1, 0}, {256, 256, 256, 2, 1, 0}, {128, 16380, 128, 1, 1, 0}};
+  for (int i = 0; i < 3 && n_out >= 30; ++i) {
+    const Case& cs = expired[i];
+    const long long n = (long long)cs.M * cs.N;
+    GemmDesc d;
+    memset(&d, 0, sizeof(d));
+    d.M = cs.M; d.N = cs.N; d.B0 = 1; d.B1 = 1;
+    d.C = C2; d.sc_m = cs.N; d.sc_n = 1;
+    d.alpha = 1.0; d.splits = cs.splits; d.partial = partial;
+    d.digits = 1; d.no_waits = 1;
+    d.words = reinterpret_cast<unsigned*>(words);
+    d.words_bytes = 2 * big * sizeof(double);
+    Group g;
+    g.a = mk(A, cs.K, 1); g.b = mk(B, 1, cs.N); g.K = cs.K; g.k0_log2 = lg(cs.K);
+    d.g[d.ngroups++] = g;
+    cudaMemsetAsync(C2, 0, n * sizeof(double), s);
+    gemm_launch(d, s);
+    count_numbers<<<1, 256, 0, s>>>(C2, n, res);
+    d.err = err;
+    gemm_launch(d, s);
+    cudaMemcpyAsync(host.data(), res, sizeof(double), cudaMemcpyDeviceToHost, s);
+    cudaMemcpyAsync(&e, err, sizeof(int), cudaMemcpyDeviceToHost, s);
+    cudaMemsetAsync(err, 0, sizeof(int), s);
+    if (cudaStreamSynchronize(s) != cudaSuccess) return TTN_ECUDA;
+    out[24 + 2 * i] = host[0];
+    out[25 + 2 * i] = e;
+  }
   return cudaGetLastError() == cudaSuccess ? TTN_OK : TTN_ECUDA;
 }
