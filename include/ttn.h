@@ -353,7 +353,7 @@ int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* 
  * before any stream capture.  Calls share the array: two calls that overlap on
  * the GPU race (use one stream, or order them).  Nothing needs clearing: each
  * call overwrites every partial sum it reads.  Accuracy: below 2^23
- * multiply-adds, or with P or Q below 16, plain FP64 sums; above, exact sums of
+ * multiply-adds, or with P or Q below 16, plain FP64 sums; else mostly exact sums of
  * 62-bit fixed-point values, every row of Y and of W scaled by its own power of
  * two: |error of C[p][q]| <= 2^-53 |C[p][q]| per partial sum (at most 152) plus
  * n2 2^-57 max_j |Y[p][j]| max_j |W[q][j]|.  (A row's values 2^-62 below its

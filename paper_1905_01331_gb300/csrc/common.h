@@ -125,10 +125,7 @@ int device_sm_count();
 int gemm_pick_splits(const GemmDesc& d);
 size_t gemm_partial_elems(const GemmDesc& d, int splits);
 
-// Digit engine of the FP64 products (gemm_oz.cu).  kOzMinWork: multiply-adds
-// below which the FP64 kernel stays (at 2^20 both take 15 us, at 2^24 the
-// digit engine 24 and the FP64 kernel 62).
-constexpr double kOzMinWork = 1 << 23;
+// Digit engine of the FP64 products (gemm_oz.cu; which products: oz_rule.h).
 // Parts of K at most that the magnitudes of an operand's rows are kept in (one
 // word per row and part in the scratch of a product).
 constexpr int kOzMaxParts = 128;

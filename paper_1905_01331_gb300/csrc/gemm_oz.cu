@@ -53,9 +53,7 @@
 // and 55); loads whose 16-byte pieces are consecutive over four threads (K permuted
 // in a stage) took 5 % more than eight consecutive values per thread.
 // Relative error against extended precision 4e-17 to 2e-16 where the
-// FP64 kernel has 2e-16 to 2e-15.  At n = 32 both kernels take 15 to 30 us
-// (latency), so kOzMinWork lies between n = 32 (2^20 multiply-adds) and n = 64
-// (2^24: 21 against 58 us).
+// FP64 kernel has 2e-16 to 2e-15.
 //
 // A row or column of a tile with an infinity or NaN, or whose range would leave
 // the normal FP64 numbers, makes the CTA compute its tile with plain FP64 FMAs
@@ -69,15 +67,13 @@
 
 #include "common.h"
 #include "f64_bits.cuh"
+#include "oz_rule.h"
 
 namespace ttn {
 
 namespace {
 
 constexpr int kOD = 8;              // digits per operand
-constexpr int kOBM = 128;
-constexpr int kOChunk = 128;        // K values per exact accumulation
-constexpr int kOBK = 32;            // K values per stage
 constexpr int kOConv = 512;         // converter threads
 constexpr int kOThreads = kOConv + 128;   // and the warpgroup of the MMA and image warps
 constexpr int kOWork = kOConv / 32; // converter warps; the MMA warp follows them, then the image warp
@@ -1236,7 +1232,7 @@ int oz_chunks(const GemmDesc& d) {
   return t;
 }
 
-int oz_bn(const GemmDesc& d) { return d.N > 32 ? 64 : 32; }
+int oz_bn(const GemmDesc& d) { return oz_tile_n(d.N); }
 
 bool same_operand(const AbsItem& a, const AbsItem& b) {
   return a.p == b.p && a.s_mn == b.s_mn && a.s_k0 == b.s_k0 && a.s_k1 == b.s_k1 && a.s_b0 == b.s_b0 &&
@@ -1362,19 +1358,19 @@ bool exchange_sides(const GemmDesc& d) {
 }  // namespace
 
 // Products the digit engine takes: FP64 in and out, K0 a whole number of
-// 16-byte digit chunks, and enough work that the launch of oz_prepare_kernel pays.
+// 16-byte digit chunks, and those that it is the faster engine for (oz_rule.h).
 bool gemm_oz_supported(const GemmDesc& d) {
   if (!d.digits || d.prec != 0 || d.c_f32 || d.alpha != 1.0 || d.beta != 0.0 || d.ngroups < 1 ||
       d.ngroups > kMaxGroups || d.M < 1 || d.N < 1)
     return false;
-  double work = 0.0;
+  int K[kMaxGroups];
   for (int g = 0; g < d.ngroups; ++g) {
     const Group& G = d.g[g];
     if (G.a.f32 || G.b.f32 || G.K < 1) return false;
     if (G.k0_log2 < 3 && (G.K >> G.k0_log2) > 1) return false;
-    work += static_cast<double>(d.M) * d.N * G.K * d.B0 * d.B1;
+    K[g] = G.K;
   }
-  return d.M >= 16 && d.N >= 16 && work >= kOzMinWork;
+  return d.M >= 16 && d.N >= 16 && oz_worth(d.M, d.N, static_cast<long long>(d.B0) * d.B1, K, d.ngroups);
 }
 
 int oz_pick_splits(const GemmDesc& d) {
