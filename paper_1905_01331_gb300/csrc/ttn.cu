@@ -167,8 +167,8 @@ struct Lane {
   SubStreams sub;
 };
 
-// A captured energy or gradient pass: the first call of a kind runs eagerly, the
-// second is captured, later ones replay it.
+// A captured energy or gradient pass: the first calls of a kind run eagerly, the
+// next is captured, later ones replay it (run_pass).
 struct PassGraph {
   int calls = 0;
   cudaGraph_t graph = nullptr;
@@ -1666,15 +1666,26 @@ void destroy_passes(ttn_ctx* h) {
   h->passes.clear();
 }
 
+// Eager calls of a pass before its capture.  A replay saves 60 to 450 us of a
+// call, the capture and instantiation cost 90 to 1040: the costs of 0.8 to 3.3
+// replays (us eager, capturing call, replay: gradient of 16 spins at chi = 8
+// 514, 697, 290; of a chain of 1024 at chi = 32 1643, 2374, 1190; of a 64 x 4 torus
+// at chi = 64 3440, 4477, 3055, in 3xTF32 at chi = 128 4330, 5280, 4037; energy
+// of a Heisenberg chain at chi = 128 2955, 3275, 2790).  After three calls, the
+// eager passes have given up about what a capture costs: a context that makes
+// fewer calls than that never pays for one, and one that makes more has paid at
+// most once for what it then saves.
+constexpr int kEagerCalls = 3;
+
 // Run a pass of many small launches (`body` enqueues it on h->stream): eagerly
-// the first time, so that a context used once pays no capture; captured on the
-// second call of its kind and replayed from then on (launches of 2 us instead
-// of 4 to 5, branches in parallel).  A pass that cannot be captured stays eager.
+// in its first kEagerCalls calls, captured on the next one and replayed from then
+// on (launches of 2 us instead of 4 to 5, branches in parallel).  A pass that
+// cannot be captured stays eager.
 template <typename Body>
 int run_pass(ttn_ctx* h, int key, Body body) {
   PassGraph& pg = h->passes[key];
   ++pg.calls;
-  if (!h->opt.use_graph || pg.calls == 1 || (!pg.exec && pg.calls > 2)) {
+  if (!h->opt.use_graph || pg.calls <= kEagerCalls || (!pg.exec && pg.calls > kEagerCalls + 1)) {
     body();
     return TTN_OK;
   }
