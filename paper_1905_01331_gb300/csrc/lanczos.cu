@@ -259,41 +259,11 @@ __device__ int first_thread(LzSmem& sm, bool flag) {
   return f;
 }
 
-// The work of the tridiagonal in pair arithmetic or FP64: twisted_rows is
-// generic over the two.
-struct ArithDF {
-  typedef tdf::DF T;
-  static __device__ __forceinline__ T sub(T a, T b) { return tdf::sub(a, b); }
-  static __device__ __forceinline__ T mul(T a, T b) { return tdf::mul(a, b); }
-  static __device__ __forceinline__ T div(T a, T b) { return tdf::div(a, b); }
-  static __device__ __forceinline__ bool zero(T a) { return a.h == 0.f; }
-  static __device__ __forceinline__ T tiny() { return {1e-30f, 0.f}; }
-  static __device__ __forceinline__ T one() { return {1.f, 0.f}; }
-  static __device__ __forceinline__ double mag(T a) { return fabs((double)a.h); }
-  static __device__ __forceinline__ T from(double x) { return tdf::make(x); }
-  static __device__ __forceinline__ double to(T x) { return tdf::to_double(x); }
-};
-struct ArithD {
-  typedef double T;
-  static __device__ __forceinline__ T sub(T a, T b) { return a - b; }
-  static __device__ __forceinline__ T mul(T a, T b) { return a * b; }
-  static __device__ __forceinline__ T div(T a, T b) { return a / b; }
-  static __device__ __forceinline__ bool zero(T a) { return a == 0.0; }
-  static __device__ __forceinline__ T tiny() { return 1e-290; }
-  static __device__ __forceinline__ T one() { return 1.0; }
-  static __device__ __forceinline__ double mag(T a) { return fabs(a); }
-  static __device__ __forceinline__ T from(double x) { return x; }
-  static __device__ __forceinline__ double to(T x) { return x; }
-};
-
 // Eigenvector of the m x m tridiagonal (al, be) for the eigenvalue th, by warp
-// 0, from the twisted factorisation (Dhillon and Parlett, "Orthogonal
-// eigenvectors and relative gaps", SIAM J. Matrix Anal. Appl. 25, 2004): the
-// pivots of T - th I from both ends (lanes 0 and 1 at the same time), the
-// twist at the row where their sum less the diagonal is smallest, and the
-// vector outwards from 1 there by products alone.  One division per row in
-// each chain, where an LU with pivoting and its two substitutions need four.
-// z[0 .. m) unnormalised (FP64); scratch: 4 m values of T.
+// 0 (the twisted factorisation of tridiag_df.cuh; the two chains of pivots and
+// the two of the vector on lanes 0 and 1 at the same time).  One division per
+// row in each chain, where an LU with pivoting and its two substitutions need
+// four.  z[0 .. m) unnormalised (FP64); scratch: 4 m values of T.
 template <typename A>
 __device__ void twisted_vector(const double* al, const double* be, int m, double th, typename A::T* scratch,
                                double* z) {
@@ -301,39 +271,17 @@ __device__ void twisted_vector(const double* al, const double* be, int m, double
   const int lane = threadIdx.x;
   T* ms = scratch;           // al - th
   T* b2 = scratch + m;       // squared off-diagonal, then the multipliers
-  T* dp = scratch + 2 * m;   // pivots from the top
+  T* dp = scratch + 2 * m;   // pivots from the top, then the vector
   T* dm = scratch + 3 * m;   // pivots from the bottom
-  for (int i = lane; i < m; i += 32) {
-    ms[i] = A::sub(A::from(al[i]), A::from(th));
-    const T b = A::from(i + 1 < m ? be[i] : 0.0);
-    b2[i] = A::mul(b, b);
-  }
+  for (int i = lane; i < m; i += 32) tdf::twist_row<A>(al, be, m, th, i, ms, b2);
   __syncwarp();
-  if (lane < 2) {
-    T* d = lane == 0 ? dp : dm;
-    int i = lane == 0 ? 0 : m - 1;
-    const int step = lane == 0 ? 1 : -1;
-    T cur = ms[i];
-    d[i] = cur;
-    for (int k = 1; k < m; ++k) {
-      const T bb = b2[lane == 0 ? i : i - 1];
-      i += step;
-      const T a = ms[i];
-      if (A::zero(cur)) {
-        cur = A::tiny();
-        d[i - step] = cur;
-      }
-      cur = A::sub(a, A::div(bb, cur));
-      d[i] = cur;
-    }
-    if (A::zero(cur)) d[i] = A::tiny();
-  }
+  if (lane < 2) tdf::twist_pivots<A>(ms, b2, m, lane == 0, lane == 0 ? dp : dm);
   __syncwarp();
-  // twist row: smallest |d+ + d- - (a - th)|
+  // twist row: the smallest gap, the first of equals
   double best = 1e300;
   int r = 0;
   for (int i = lane; i < m; i += 32) {
-    const double g = A::mag(A::sub(dp[i], A::sub(ms[i], dm[i])));
+    const double g = tdf::twist_gap<A>(ms, dp, dm, i);
     if (g < best) { best = g; r = i; }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -341,24 +289,10 @@ __device__ void twisted_vector(const double* al, const double* be, int m, double
     const int orr = __shfl_xor_sync(0xffffffffu, r, o);
     if (ob < best || (ob == best && orr < r)) { best = ob; r = orr; }
   }
-  // multipliers: z_i = -(b_i / d+_i) z_{i+1} above r, z_{i+1} = -(b_i / d-_{i+1}) z_i below
-  for (int i = lane; i + 1 < m; i += 32) b2[i] = A::div(A::from(-be[i]), i < r ? dp[i] : dm[i + 1]);
+  for (int i = lane; i + 1 < m; i += 32) b2[i] = tdf::twist_multiplier<A>(be, dp, dm, r, i);
   __syncwarp();
-  if (lane < 2) {
-    T cur = A::one();
-    if (lane == 0) {
-      z[r] = 1.0;
-      for (int i = r - 1; i >= 0; --i) {
-        cur = A::mul(b2[i], cur);
-        dp[i] = cur;
-      }
-    } else {
-      for (int i = r; i + 1 < m; ++i) {
-        cur = A::mul(b2[i], cur);
-        dp[i + 1] = cur;
-      }
-    }
-  }
+  if (lane == 0) z[r] = 1.0;
+  if (lane < 2) tdf::twist_outwards<A>(b2, m, r, lane == 0, dp);
   __syncwarp();
   for (int i = lane; i < m; i += 32)
     if (i != r) z[i] = A::to(dp[i]);
@@ -483,7 +417,7 @@ __device__ bool ritz_check_df(LzSmem& sm, double* scratch, int m, double sigma, 
   const double th = lowest_value(sm, scratch, m, unscale);
   if (threadIdx.x >= 32) return false;
   double* z = sm.tri[0];
-  twisted_vector<ArithDF>(sm.al, sm.be, m, th, reinterpret_cast<tdf::DF*>(scratch), z);
+  twisted_vector<tdf::ArithDF>(sm.al, sm.be, m, th, reinterpret_cast<tdf::DF*>(scratch), z);
   double s = 0.0;
   for (int i = threadIdx.x; i < m; i += 32) s = fma(z[i], z[i], s);
   s = warp_sum(s);
@@ -503,7 +437,7 @@ __device__ void ritz_pair(LzSmem& sm, double* scratch, int m, double* y, double*
   if (threadIdx.x >= 32) return;
   const int lane = threadIdx.x;
   double* z = sm.tri[0];
-  twisted_vector<ArithDF>(sm.al, sm.be, m, th0, reinterpret_cast<tdf::DF*>(scratch), z);
+  twisted_vector<tdf::ArithDF>(sm.al, sm.be, m, th0, reinterpret_cast<tdf::DF*>(scratch), z);
   // Rayleigh quotient of (T - th0) z, added to th0
   double nn = 0.0, rq = 0.0;
   for (int i = lane; i < m; i += 32) {
@@ -515,7 +449,7 @@ __device__ void ritz_pair(LzSmem& sm, double* scratch, int m, double* y, double*
   nn = warp_sum(nn);
   rq = warp_sum(rq);
   const double th = th0 + rq / nn;
-  twisted_vector<ArithD>(sm.al, sm.be, m, th, scratch, z);
+  twisted_vector<tdf::ArithD>(sm.al, sm.be, m, th, scratch, z);
   double s = 0.0;
   for (int i = lane; i < m; i += 32) s = fma(z[i], z[i], s);
   const double inv = sqrt(warp_sum(s));

@@ -120,7 +120,8 @@ TDF_HD int sturm_below(const DF* a, const DF* b2, int m, DF x) {
 // Solve (T - th I) x = ones by LU with partial pivoting (one round of inverse
 // iteration) and return |x_{m-1}| / |x|, the last component of the
 // normalised approximate eigenvector.  dd, du, du2, dl, x: scratch arrays of
-// m pairs.
+// m pairs.  (A second way to the quantity that the convergence checks take from
+// the twisted vector below; host only.)
 TDF_HD double last_component(const DF* a, const DF* b, int m, DF th, DF* dd, DF* du, DF* du2,
                              DF* dl, DF* x) {
   const DF tiny = {1e-30f, 0.f};
@@ -172,6 +173,96 @@ TDF_HD double last_component(const DF* a, const DF* b, int m, DF th, DF* dd, DF*
     n2 += v * v;
   }
   return n2 > 0.0 ? std::fabs(to_double(x[m - 1])) / std::sqrt(n2) : 1.0;
+}
+
+// The eigenvector below in pair arithmetic or FP64.
+struct ArithDF {
+  typedef DF T;
+  static TDF_HD T sub(T a, T b) { return tdf::sub(a, b); }
+  static TDF_HD T mul(T a, T b) { return tdf::mul(a, b); }
+  static TDF_HD T div(T a, T b) { return tdf::div(a, b); }
+  static TDF_HD bool zero(T a) { return a.h == 0.f; }
+  static TDF_HD T tiny() { return {1e-30f, 0.f}; }
+  static TDF_HD T one() { return {1.f, 0.f}; }
+  static TDF_HD double mag(T a) { return fabs_hi(a); }
+  static TDF_HD T from(double x) { return make(x); }
+  static TDF_HD double to(T x) { return to_double(x); }
+};
+struct ArithD {
+  typedef double T;
+  static TDF_HD T sub(T a, T b) { return a - b; }
+  static TDF_HD T mul(T a, T b) { return a * b; }
+  static TDF_HD T div(T a, T b) { return a / b; }
+  static TDF_HD bool zero(T a) { return a == 0.0; }
+  static TDF_HD T tiny() { return 1e-290; }
+  static TDF_HD T one() { return 1.0; }
+  static TDF_HD double mag(T a) { return a < 0.0 ? -a : a; }
+  static TDF_HD T from(double x) { return x; }
+  static TDF_HD double to(T x) { return x; }
+};
+
+// Eigenvector of the m x m tridiagonal (al, be) for the eigenvalue th, from the
+// twisted factorisation (Dhillon and Parlett, "Orthogonal eigenvectors and
+// relative gaps", SIAM J. Matrix Anal. Appl. 25, 2004), in the pieces that the
+// lanes of a warp share: the pivots of T - th I from both ends, the twist at the
+// row where their sum less the diagonal is smallest, and the vector outwards from
+// 1 there by products alone.
+//
+// Row i: ms = al - th, b2 = the squared off-diagonal after it.
+template <typename A>
+TDF_HD void twist_row(const double* al, const double* be, int m, double th, int i, typename A::T* ms,
+                      typename A::T* b2) {
+  ms[i] = A::sub(A::from(al[i]), A::from(th));
+  const typename A::T b = A::from(i + 1 < m ? be[i] : 0.0);
+  b2[i] = A::mul(b, b);
+}
+// The pivots d from the top (down) or from the bottom; a zero one becomes tiny.
+template <typename A>
+TDF_HD void twist_pivots(const typename A::T* ms, const typename A::T* b2, int m, bool down, typename A::T* d) {
+  typedef typename A::T T;
+  int i = down ? 0 : m - 1;
+  const int step = down ? 1 : -1;
+  T cur = ms[i];
+  d[i] = cur;
+  for (int k = 1; k < m; ++k) {
+    const T bb = b2[down ? i : i - 1];
+    i += step;
+    const T a = ms[i];
+    if (A::zero(cur)) {
+      cur = A::tiny();
+      d[i - step] = cur;
+    }
+    cur = A::sub(a, A::div(bb, cur));
+    d[i] = cur;
+  }
+  if (A::zero(cur)) d[i] = A::tiny();
+}
+// |d+ + d- - (al - th)| of row i: the twist row has the smallest.
+template <typename A>
+TDF_HD double twist_gap(const typename A::T* ms, const typename A::T* dp, const typename A::T* dm, int i) {
+  return A::mag(A::sub(dp[i], A::sub(ms[i], dm[i])));
+}
+// z_i = multiplier_i z_{i+1} above the twist row r, z_{i+1} = multiplier_i z_i below.
+template <typename A>
+TDF_HD typename A::T twist_multiplier(const double* be, const typename A::T* dp, const typename A::T* dm, int r,
+                                      int i) {
+  return A::div(A::from(-be[i]), i < r ? dp[i] : dm[i + 1]);
+}
+// The entries of the vector above (up) or below r, from 1 at r (v[r] stays).
+template <typename A>
+TDF_HD void twist_outwards(const typename A::T* mult, int m, int r, bool up, typename A::T* v) {
+  typename A::T cur = A::one();
+  if (up) {
+    for (int i = r - 1; i >= 0; --i) {
+      cur = A::mul(mult[i], cur);
+      v[i] = cur;
+    }
+  } else {
+    for (int i = r; i + 1 < m; ++i) {
+      cur = A::mul(mult[i], cur);
+      v[i + 1] = cur;
+    }
+  }
 }
 
 }  // namespace tdf
