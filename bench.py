@@ -394,14 +394,14 @@ def run_gpu(args):
                "peak": sm_count * 128 * 2 * sm_ghz / 1e3,
                "peak_source": "152 SMs x 128 FP32 lanes x 2 flop/FMA x max SM clock (FP32 FMA peak); "
                               "the kernel's mix (8 of 12 instructions are adds) caps it at 0.625"},
-        # the double-float polar composition (P x P products between grid barriers)
+        # the double-float polar composition (P x P products, tile by tile)
         "dfc": {"bound": "alu", "kernel": "polar_compose_df_kernel (double-float composition, "
-                                          "persistent, grid barriers)",
+                                          "persistent, per-block counters)",
                 "ms": prof.get("dfc_ms", 0.0), "achieved_units": prof.get("dfc_flops", 0.0) / 2 * 15,
                 "launches": prof.get("dfc_launches", 0.0),
                 "peak": sm_count * 128 * 2 * sm_ghz / 1e3,
-                "peak_source": "FP32 FMA peak as for df; latency-bound (two grid barriers per "
-                               "Newton-Schulz step)"},
+                "peak_source": "FP32 FMA peak as for df; latency-bound (two dependent phases "
+                               "per Newton-Schulz step)"},
     }
     fam = {}
     for k, f in families.items():

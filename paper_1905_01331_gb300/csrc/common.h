@@ -100,7 +100,8 @@ struct GemmDesc {
   size_t words_bytes;
   int no_waits;      // digit engine: every wait expires at once (the tests of that path)
   float* c32;        // FP64 products: also the FP32 copy of C, at C's offsets (may be null);
-                     // written by whatever writes C: an engine's kernel or the split-K reduction
+                     // written by the digit kernels, the split-K reduction or a pass after
+                     // the FP64 kernel
   int occ;           // TMA-fed kernel: 2 = the 96 KB stage ring (two CTAs per
                      // SM), else the 192 KB ring (one CTA per SM)
 };

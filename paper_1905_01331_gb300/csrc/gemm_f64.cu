@@ -12,7 +12,6 @@
 
 #include "../../include/ttn.h"
 #include "common.h"
-#include "f64_bits.cuh"
 
 namespace ttn {
 
@@ -34,6 +33,8 @@ __device__ __forceinline__ double ld_operand(const Operand& o, int k0_log2, long
   return o.f32 ? (double)static_cast<const float*>(o.p)[e] : static_cast<const double*>(o.p)[e];
 }
 
+// kCopy: also C's FP32 copy (d.c32; FP64 outputs only).
+template <bool kCopy = false>
 __device__ __forceinline__ void st_out(const GemmDesc& d, long long e, double acc) {
   if (d.c_f32) {
     float* c = static_cast<float*>(d.C) + e;
@@ -42,7 +43,7 @@ __device__ __forceinline__ void st_out(const GemmDesc& d, long long e, double ac
     double* c = static_cast<double*>(d.C) + e;
     const double v = d.beta == 0.0 ? d.alpha * acc : d.alpha * acc + d.beta * *c;
     *c = v;
-    if (d.c32) d.c32[e] = f64b::to_f32(v);
+    if constexpr (kCopy) d.c32[e] = static_cast<float>(v);
   }
 }
 
@@ -193,6 +194,7 @@ __global__ void __launch_bounds__(kThreads) gemm_f64_kernel(const GemmDesc d, in
 // owns 32 consecutive outputs; its 8 warps each sum a contiguous eighth of the
 // splits in order (loads in flight together), and warp 0 adds the eight sums
 // in group order (a fixed order of terms).
+template <bool kCopy>
 __global__ void splitk_reduce_kernel(const GemmDesc d) {
   pdl_wait();
   pdl_trigger();
@@ -230,9 +232,24 @@ __global__ void splitk_reduce_kernel(const GemmDesc d) {
       for (int q = 0; q < 8; ++q) t += gs[q][lane];
       const int m = (int)(r / d.N), n = (int)(r % d.N);
       const int b0 = (int)(b % d.B0), b1 = (int)(b / d.B0);
-      st_out(d, b0 * d.sc_b0 + (long long)b1 * d.sc_b1 + m * d.sc_m + n * d.sc_n, t);
+      st_out<kCopy>(d, b0 * d.sc_b0 + (long long)b1 * d.sc_b1 + m * d.sc_m + n * d.sc_n, t);
     }
     __syncthreads();
+  }
+}
+
+// C's FP32 copy after an FP64 kernel that wrote C itself (the FP64 tile kernel,
+// whose store has no room for the test: 1 % of a chi = 32 sweep).
+__global__ void copy_f32_kernel(const GemmDesc d) {
+  pdl_wait();
+  pdl_trigger();
+  if (desc_skipped(d)) return;
+  const long long MN = (long long)d.M * d.N, total = MN * d.B0 * d.B1;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const int b = (int)(i / MN);
+    const long long r = i % MN;
+    const long long e = b % d.B0 * d.sc_b0 + b / d.B0 * d.sc_b1 + r / d.N * d.sc_m + r % d.N * d.sc_n;
+    d.c32[e] = static_cast<float>(static_cast<const double*>(d.C)[e]);
   }
 }
 
@@ -346,7 +363,10 @@ int gemm_launch(const GemmDesc& d0, cudaStream_t s) {
   if (d.splits > 1) {
     const long long total = (long long)d.M * d.N * d.B0 * d.B1;
     const int blocks = (int)std::min<long long>((total + 31) / 32, 8192);
-    launch_k(splitk_reduce_kernel, blocks, 256, 0, s, d);
+    launch_k(d.c32 ? splitk_reduce_kernel<true> : splitk_reduce_kernel<false>, blocks, 256, 0, s, d);
+    ++n;
+  } else if (d.c32 && oz < 0) {
+    launch_k(copy_f32_kernel, (int)std::min<long long>(((long long)d.M * d.N * d.B0 * d.B1 + 255) / 256, 1216), 256, 0, s, d);
     ++n;
   }
   return n;

@@ -1064,11 +1064,12 @@ void polar(ttn_ctx* h, Instance& I, int t, int prec, const double* Gam) {
   // The first try's products over X on the digit engine (gemm_oz.cu), where the
   // layer is large enough for it: a well-conditioned factor is the same to
   // 1e-13, at 57 (Gram) and 41 us (apply) where the double-float products take 88
-  // and 127 (P = 128, N = 16384).  Every row of X and of F is cut at 2^-61 of its
-  // own largest value: values below 2^-14 of that keep fewer bits than their FP32
-  // pair, but the sums they enter carry the pairs' 2^-48 of the larger ones there
-  // and 2^-57 here.  The full schedule keeps the double-float
-  // products: the directions it amplifies by up to 1e7 carry their rounding.
+  // and 127 (P = 128, N = 16384).  Every row (in F X: every row of F and column of
+  // X) is cut at 2^-61 of its own largest value: values below 2^-14 of that keep
+  // fewer bits than their FP32 pair, but the sums they enter carry the pairs'
+  // 2^-48 of the larger ones there and 2^-57 here.  The full schedule keeps the
+  // double-float products: the directions it amplifies by up to 1e7 carry their
+  // rounding.
   const bool oz_try = try_first && oz_gram_ok(P, N);
   if (df_ok && !h->measuring && !adaptive)
     h->launches += store_ints(full, nullptr, 1, 1, h->stream);
