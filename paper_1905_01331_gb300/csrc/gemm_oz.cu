@@ -20,10 +20,10 @@
 // rounded to FP64 once at the end: the result carries one rounding instead of
 // one per term.  One power of two per operand would lose rows that are small as
 // a whole (2^-40 below the largest: 3e-6 of their products) and costs less: FP64
-// sweep at chi = 128 23.93 ms, now 24.34; gradient of a torus at chi = 64 3.50,
-// now 3.62; measurement of a Heisenberg chain at chi = 128 3.24, now 3.31; close
-// product of 96 x 80 x 10007 53.3 us, now 54.5.  (In a sum of several groups, whose
-// scales differ by output, a tenth of the product; else 1 to 2 %.)
+// sweep at chi = 128 24.48 ms, now 24.83; gradient of a torus at chi = 64 3.48,
+// now 3.58; measurement of a Heisenberg chain at chi = 128 3.24, now 3.30; close
+// product of 96 x 80 x 10007 53.4 us, now 54.0.  (In a sum of several groups, whose
+// scales differ by output, 8 % of the product; else 0 to 1 %.)
 //
 // One CTA owns a 128 x BN output tile (BN 64 or 32); two stages of 32 K values.
 // Warps 0-15 load FP64 operands (any strides), cut them into digits with integer
@@ -44,9 +44,9 @@
 // (eight before: 2 warps a scheduler, an instruction every third clock): FP64
 // sweep at chi = 128 25.29 -> 25.05 ms, FP64 gradient of a torus at chi = 64 3.61 ->
 // 3.46 ms, measurement 3.35 -> 3.23 ms.  Measured on a GB300 (P = n = 128, with the
-// preparation): F X of 128 x 128 by 128 x 16384 37 us (the FP64 kernel 547), the
-// environment's five such products in one 163 us (2674), three close products over
-// K = 16384 128 us (1931), the Gram matrix of 128 x 16384 57 us (449).  Converting
+// preparation): F X of 128 x 128 by 128 x 16384 35 us (the FP64 kernel 547), the
+// environment's five such products in one 160 us (2674), three close products over
+// K = 16384 126 us (1931), the Gram matrix of 128 x 16384 55 us (449).  Converting
 // both operands in every tile with BF16 digits, which take two operations more a
 // pair, and combining by eight converting instructions per output took 55, 186,
 // 123 and 59 (all with one power of two per operand, which now takes 35, 147, 126
@@ -240,13 +240,17 @@ __device__ __forceinline__ void image_block(const AbsItem& it, const double* p, 
 // words[r] = the largest magnitude word of row r0 + r over K values k_lo .. k_hi
 // - 1, for R rows (32, 64 or 128); words hold 0 before.  K contiguous: a warp per
 // row, lanes along K, KS steps of K and 16 / KS rows at a time; else lanes along
-// the rows and the warps share K.  Sixteen loads in flight per thread.
-template <int KS>
-__device__ __forceinline__ void row_magnitudes_k(const AbsItem& it, const double* p, int r0, int R, int k_lo, int k_hi,
-                                                 unsigned* words) {
+// the rows and the warps share K.  Sixteen loads in flight per thread.  kFull: all
+// rows are there, the K values are whole steps of one run of K0 -- without the
+// index arithmetic and the tests per value, which take three times the
+// instructions of the loads and maxima.
+template <int KS, bool kFull>
+__device__ __forceinline__ void rows_kfast(const AbsItem& it, const double* p, int r0, int R, int k_lo, int k_hi,
+                                           unsigned* words) {
   constexpr int kRows = 16 / KS;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int kmask = (1 << it.k0_log2) - 1;
+  const double* pf = p + (k_lo & kmask) + static_cast<long long>(k_lo >> it.k0_log2) * it.s_k1 - k_lo + r0 * it.s_mn;
 #pragma unroll 1
   for (int r = warp; r < R; r += 8 * kRows) {
     unsigned m[kRows];
@@ -255,14 +259,23 @@ __device__ __forceinline__ void row_magnitudes_k(const AbsItem& it, const double
 #pragma unroll 1
     for (int k = k_lo + lane; k < k_hi; k += 32 * KS) {
       double v[kRows][KS];
+      if constexpr (kFull) {
 #pragma unroll
-      for (int q = 0; q < KS; ++q) {
-        const int kk = k + 32 * q;
-        const bool in = kk < k_hi;
-        const double* pk = p + (in ? (kk & kmask) + static_cast<long long>(kk >> it.k0_log2) * it.s_k1 : 0);
+        for (int i = 0; i < kRows; ++i) {
+          const double* pr = pf + (r + 8 * i < R ? r + 8 * i : r) * it.s_mn + k;   // (a short tile: a row again)
 #pragma unroll
-        for (int i = 0; i < kRows; ++i)
-          v[i][q] = in && r + 8 * i < R && r0 + r + 8 * i < it.mn ? pk[(r0 + r + 8 * i) * it.s_mn] : 0.0;
+          for (int q = 0; q < KS; ++q) v[i][q] = pr[32 * q];
+        }
+      } else {
+#pragma unroll
+        for (int q = 0; q < KS; ++q) {
+          const int kk = k + 32 * q;
+          const bool in = kk < k_hi;
+          const double* pk = p + (in ? (kk & kmask) + static_cast<long long>(kk >> it.k0_log2) * it.s_k1 : 0);
+#pragma unroll
+          for (int i = 0; i < kRows; ++i)
+            v[i][q] = in && r + 8 * i < R && r0 + r + 8 * i < it.mn ? pk[(r0 + r + 8 * i) * it.s_mn] : 0.0;
+        }
       }
 #pragma unroll
       for (int i = 0; i < kRows; ++i)
@@ -276,41 +289,61 @@ __device__ __forceinline__ void row_magnitudes_k(const AbsItem& it, const double
     }
   }
 }
-__device__ __forceinline__ void row_magnitudes(const AbsItem& it, const double* p, int r0, int R, int k_lo, int k_hi,
-                                               unsigned* words) {
-  if (it.s_k0 == 1) {
-    if (k_hi - k_lo > 64) row_magnitudes_k<4>(it, p, r0, R, k_lo, k_hi, words);
-    else if (k_hi - k_lo > 32) row_magnitudes_k<2>(it, p, r0, R, k_lo, k_hi, words);
-    else row_magnitudes_k<1>(it, p, r0, R, k_lo, k_hi, words);
-    return;
-  }
+template <bool kFull>
+__device__ __forceinline__ void rows_mnfast(const AbsItem& it, const double* p, int r0, int R, int k_lo, int k_hi,
+                                            unsigned* words) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int kmask = (1 << it.k0_log2) - 1;
   const int groups = R >> 5, rg = warp % groups, step = 8 / groups;
   const int row = r0 + rg * 32 + lane;
-  if (row >= it.mn) return;
+  if (!kFull && row >= it.mn) return;
   const double* pr = p + row * it.s_mn;
   unsigned m = 0;
 #pragma unroll 1
   for (int k = k_lo + warp / groups; k < k_hi; k += 16 * step) {
     double v[16];
+    const double* pk = pr + (k & kmask) * it.s_k0 + static_cast<long long>(k >> it.k0_log2) * it.s_k1;
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
-      const int kk = k + q * step;
-      v[q] = kk < k_hi ? pr[(kk & kmask) * it.s_k0 + static_cast<long long>(kk >> it.k0_log2) * it.s_k1] : 0.0;
+      if constexpr (kFull) {
+        v[q] = *pk;
+        pk += step * it.s_k0;
+      } else {
+        const int kk = k + q * step;
+        v[q] = kk < k_hi ? pr[(kk & kmask) * it.s_k0 + static_cast<long long>(kk >> it.k0_log2) * it.s_k1] : 0.0;
+      }
     }
 #pragma unroll
     for (int q = 0; q < 16; ++q) m = max(m, mag_word(v[q]));
   }
   atomicMax(&words[rg * 32 + lane], m);
 }
+__device__ __forceinline__ void row_magnitudes(const AbsItem& it, const double* p, int r0, int R, int k_lo, int k_hi,
+                                               unsigned* words) {
+  const int nk = k_hi - k_lo;
+  const bool full = r0 + R <= it.mn && ((k_lo ^ (k_hi - 1)) >> it.k0_log2) == 0;
+  if (it.s_k0 != 1) {
+    if (full && nk % (4096 / R) == 0) rows_mnfast<true>(it, p, r0, R, k_lo, k_hi, words);
+    else rows_mnfast<false>(it, p, r0, R, k_lo, k_hi, words);
+  } else if (nk > 64) {
+    if (full && nk % 128 == 0) rows_kfast<4, true>(it, p, r0, R, k_lo, k_hi, words);
+    else rows_kfast<4, false>(it, p, r0, R, k_lo, k_hi, words);
+  } else if (nk > 32) {
+    if (full && nk == 64) rows_kfast<2, true>(it, p, r0, R, k_lo, k_hi, words);
+    else rows_kfast<2, false>(it, p, r0, R, k_lo, k_hi, words);
+  } else {
+    rows_kfast<1, false>(it, p, r0, R, k_lo, k_hi, words);
+  }
+}
 
 // Before a product: the magnitudes of its operands' rows, and the digits of the
 // small operands that many of its tiles read.
 //   without an image: a block per 32 to 128 rows of a batch and part of K;
 //   with one: a block per stage block; each scans its (few, short) rows.
-// Bound by the read of the operands (from L2 when they were just produced).
-__global__ void __launch_bounds__(256) oz_prepare_kernel(const AbsParams ap) {
+// Bound by the read of the operands (from L2 when they were just produced): 20 us
+// for five operands of 128 x 16384 from DRAM, 9 to 11 for one.  Five blocks a SM: at
+// four (80 registers instead of 48) the five operands' product took 1 % longer.
+__global__ void __launch_bounds__(256, 5) oz_prepare_kernel(const AbsParams ap) {
   pdl_wait();
   pdl_trigger();
   if (ap.skip && ((*ap.skip != 0) != (ap.skip_when_zero != 0))) return;

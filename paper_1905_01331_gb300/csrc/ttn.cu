@@ -1063,7 +1063,7 @@ void polar(ttn_ctx* h, Instance& I, int t, int prec, const double* Gam) {
   int* run_full = try_first ? I.ppred + nT + t : nullptr;
   // The first try's products over X on the digit engine (gemm_oz.cu), where the
   // layer is large enough for it: a well-conditioned factor is the same to
-  // 1e-13, at 57 (Gram) and 41 us (apply) where the double-float products take 88
+  // 1e-13, at 55 (Gram) and 41 us (apply) where the double-float products take 88
   // and 127 (P = 128, N = 16384).  Every row (in F X: every row of F and column of
   // X) is cut at 2^-61 of its own largest value: values below 2^-14 of that keep
   // fewer bits than their FP32 pair, but the sums they enter carry the pairs'
