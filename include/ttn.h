@@ -355,10 +355,11 @@ int ttn_selftest_digits(void* d_ws, size_t bytes, double* out, int n_out, void* 
  * call overwrites every partial sum it reads.  Accuracy: below 2^23
  * multiply-adds, or with P or Q below 16, plain FP64 sums; else mostly exact sums of
  * 62-bit fixed-point values, every row of Y and of W scaled by its own power of
- * two: |error of C[p][q]| <= 2^-53 |C[p][q]| per partial sum (at most 152) plus
- * n2 2^-57 max_j |Y[p][j]| max_j |W[q][j]|.  (A row's values 2^-62 below its
- * largest do not count: a sum that lives on products of large and such small
- * values of both rows keeps fewer digits than FP64 sums would.)  Infinities and
+ * two over each of S <= 152 ranges of j: the error of C[p][q] is at most
+ * 2 S 2^-53 sum_j |Y[p][j]| |W[q][j]| (the roundings of the S partial sums and of
+ * their additions) plus n2 2^-57 max_j |Y[p][j]| max_j |W[q][j]|.  (A sum that
+ * lives on products of one row's largest values with values of the other far
+ * below its largest keeps fewer digits than FP64 sums would.)  Infinities and
  * NaN give what FP64 sums give.  The kernel's internal waits are bounded; should
  * one expire (a call cannot report it, it returns before the work runs), the
  * outputs that it leaves are NaN.  Limits: 1 <= P, Q <= 256 and
@@ -374,8 +375,9 @@ int ttn_close_noalloc(const double* d_Y, const double* d_W, int P, int Q, long l
  * CUDA events over `reps` launches after one warm-up launch: for tensor-core
  * products the engine (TMA-fed where eligible, thread-staged), its tile width
  * BN, the TMA-fed kernel's stage ring (192 KB, one CTA per SM, or 96 KB, two)
- * and the split count of K (powers of two up to 128); for FP64 products the
- * tile (16, 32, 64) and the split count; the split counts are limited to the
+ * and the split count of K (powers of two up to 128); for FP64 products on the
+ * FP64 units the tile (16, 32, 64) and the split count, for those on the tensor
+ * cores (exact digit products) the split count alone; the split counts are limited to the
  * context's split-K buffer.  The fastest becomes the product's configuration (the next
  * ttn_sweep captures its graph again).  The sweep updates the tensors like
  * ttn_sweep.  With blob_bytes != NULL the table is exported: blob == NULL
