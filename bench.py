@@ -384,7 +384,7 @@ def run_gpu(args):
         "fp64": {"bound": "alu", "kernel": "FP64 engine: gemm_f64_kernel + polar_compose_kernel",
                  "ms": prof["fp64_ms"], "achieved_units": prof["fp64_flops"],
                  "launches": prof["fp64_launches"], "peak": 1.10,
-                 "peak_source": "measured cuBLAS DGEMM 8192^3 on this pool's GB300 (1.10 TFLOP/s)"},
+                 "peak_source": "measured cuBLAS DGEMM 8192^3 on a GB300 (1.10 TFLOP/s)"},
         # double-float products: FP32 flops executed, 15 per multiply-add
         # (1 MUL + 3 FMA + 8 ADD), against the FP32 FMA peak from unit counts
         "df": {"bound": "alu", "kernel": "gemm_df_kernel (double-float Gram and apply products, "
